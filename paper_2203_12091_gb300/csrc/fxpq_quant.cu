@@ -319,60 +319,247 @@ __global__ void __launch_bounds__(256) quantize_batch_kernel(const __grid_consta
 
 // ------------------------------------------------------------------------------------------
 // Packed k-bit code storage: bit-plane words per group of 32 codes (see fxpq_pack_codes)
+//
+// Both directions move bytes only (2 bytes of code per plane and k / 8 of word), so the work per code has
+// to stay small: a lane takes 8 consecutive codes with one 16-byte access per plane, four lanes one group.
+// An 8 x 8 bit transpose (three delta swaps) turns a lane's 8 code bytes into one byte per bit plane, and
+// a 4 x 4 byte transpose over the four lanes (two shuffles) turns these into the plane words, lane j
+// holding planes j, j + 4, ...  About 6 instructions per code; the form with one code per lane and a
+// ballot or shuffle per plane took 30 (2^25 4-bit codes: pack 78 -> 21 us, unpack
+// 74 -> 21 us, 4.0 TB/s; 16-bit: 234 -> 36 and 177 -> 38 us).
 // ------------------------------------------------------------------------------------------
-constexpr int PACK_G = 4;  // groups per warp and iteration (their code loads are issued together)
 
-__global__ void pack_codes_kernel(const __half* __restrict__ codes, long long n, int k, int planes,
-                                  uint32_t* __restrict__ words) {
+// 8 x 8 bit matrix, byte b bit c in (lo: bytes 0-3, hi: 4-7) -> byte c bit b (Hacker's Delight, 7-3).
+__device__ __forceinline__ void bit_transpose8(uint32_t& lo, uint32_t& hi) {
+    uint32_t t;
+    t = (lo ^ (lo >> 7)) & 0x00AA00AAu;
+    lo ^= t ^ (t << 7);
+    t = (hi ^ (hi >> 7)) & 0x00AA00AAu;
+    hi ^= t ^ (t << 7);
+    t = (lo ^ (lo >> 14)) & 0x0000CCCCu;
+    lo ^= t ^ (t << 14);
+    t = (hi ^ (hi >> 14)) & 0x0000CCCCu;
+    hi ^= t ^ (t << 14);
+    t = (lo ^ (hi << 4)) & 0xF0F0F0F0u;
+    lo ^= t;
+    hi ^= t >> 4;
+}
+
+// 4 x 4 byte transpose over the lanes of a quad: byte i of lane j's result is byte j of lane i's word.
+__device__ __forceinline__ uint32_t quad_transpose(uint32_t w, int lane) {
+    w = __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 1), (lane & 1) ? 0x3715 : 0x6240);
+    return __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 2), (lane & 2) ? 0x3276 : 0x5410);
+}
+
+// Codes e .. e + 7 of one plane (zero past n) at any 2-byte alignment of the plane.  mis: elements by which
+// the plane lies past a 16-byte boundary; a shifted 16-byte piece comes from the two aligned ones that
+// hold it (the second is the next lane's first, an L1 hit), edge pieces element by element.
+__device__ __forceinline__ uint4 load8_codes(const __half* __restrict__ p, long long e, long long n, int mis) {
+    const unsigned short* q = reinterpret_cast<const unsigned short*>(p);
+    uint32_t o[4];
+    if (mis == 0 && e + 8 <= n) return __ldg(reinterpret_cast<const uint4*>(q + e));
+    if (e >= 8 && e + 16 <= n) {
+        const uint4 u = __ldg(reinterpret_cast<const uint4*>(q + e - mis)), v = __ldg(reinterpret_cast<const uint4*>(q + e - mis) + 1);
+        const uint32_t w[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+        uint32_t r[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) r[i] = (mis & 4) ? w[i + 2] : w[i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) r[i] = (mis & 2) ? r[i + 1] : r[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = (mis & 1) ? __funnelshift_r(r[i], r[i + 1], 16) : r[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t c0 = e + 2 * i < n ? q[e + 2 * i] : 0u, c1 = e + 2 * i + 1 < n ? q[e + 2 * i + 1] : 0u;
+            o[i] = c0 | (c1 << 16);
+        }
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// The warp's codes e .. e + 7 of each lane (consecutive lanes, consecutive pieces) into one plane at any
+// 2-byte alignment.  A shifted plane gets aligned 16-byte stores of the previous lane's last codes and
+// the lane's own first ones; the warp's two ends and a warp that reaches past n store element by element.
+// All 32 lanes take part.
+__device__ __forceinline__ void store8_codes(__half* __restrict__ p, long long e, long long n, int mis, uint4 v, int lane) {
+    unsigned short* q = reinterpret_cast<unsigned short*>(p);
+    const bool whole = __all_sync(0xffffffffu, e + 8 <= n);
+    if (mis == 0 && whole) {
+        *reinterpret_cast<uint4*>(q + e) = v;
+        return;
+    }
+    const uint32_t own[4] = {v.x, v.y, v.z, v.w};
+    int first = 0, last = 8;  // own codes stored element by element: [first, last)
+    if (whole) {
+        // elements 8 - mis .. 15 - mis of (previous lane's 8, own 8)
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            w[i] = __shfl_up_sync(0xffffffffu, own[i], 1);
+            w[4 + i] = own[i];
+        }
+        const int s = 8 - mis;  // 1 .. 7
+        uint32_t r[6], o[4];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) r[i] = (s & 4) ? w[i + 2] : w[i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) r[i] = (s & 2) ? r[i + 1] : r[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = (s & 1) ? __funnelshift_r(r[i], r[i + 1], 16) : r[i];
+        if (lane > 0) *reinterpret_cast<uint4*>(q + e - mis) = make_uint4(o[0], o[1], o[2], o[3]);
+        first = lane == 0 ? 0 : lane == 31 ? 8 - mis : 8;
+        last = lane == 0 ? 8 - mis : 8;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (i >= first && i < last && e + i < n) q[e + i] = (unsigned short)(own[i >> 1] >> (16 * (i & 1)));
+}
+
+// Elements by which a plane of 2-byte codes lies past a 16-byte boundary.
+__device__ __forceinline__ int misaligned8(const void* p) { return (int)((reinterpret_cast<uintptr_t>(p) >> 1) & 7); }
+
+// Two fp16 codes as 16-bit two's complement integers in one word: |code| < 2^16 plus 1.5 * 2^23 is exact
+// in fp32, with the integer in the low mantissa bits.
+__device__ __forceinline__ uint32_t codes_to_s16x2(uint32_t h) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h));
+    return __byte_perm(__float_as_uint(f.x + 12582912.0f), __float_as_uint(f.y + 12582912.0f), 0x5410);
+}
+
+// Eight bit planes (byte b of (lo, hi) = plane b of 8 codes) as fp16 values of k-bit fields, k <= 8: signed
+// fields have bit k-1 flipped (`flip`), which maps them to u = code + 2^(k-1); a byte u becomes the fp16
+// 1024 + u (0x64 over it) and one half2 subtraction of `off` = 1024 (+ 2^(k-1) if signed) leaves the code.
+__device__ __forceinline__ uint4 fields_to_f16(uint32_t lo, uint32_t hi, uint32_t flip, uint32_t off) {
+    bit_transpose8(lo, hi);
+    lo ^= flip;
+    hi ^= flip;
+    const __half2 o2 = *reinterpret_cast<const __half2*>(&off);
+    uint32_t h[4] = {__byte_perm(lo, 0x64646464u, 0x5140), __byte_perm(lo, 0x64646464u, 0x5342),
+                     __byte_perm(hi, 0x64646464u, 0x5140), __byte_perm(hi, 0x64646464u, 0x5342)};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&h[q]), o2);
+        h[q] = *reinterpret_cast<const uint32_t*>(&v);
+    }
+    return make_uint4(h[0], h[1], h[2], h[3]);
+}
+
+// Flat quantization to a two-plane code tensor: 8 codes per lane from two 16-byte loads, one 16-byte store
+// per plane.  The lo plane starts n elements after the hi plane, so for n % 8 != 0 it is off every 16-byte
+// boundary (store8_codes).  HBM-bound: 4 bytes read and 4 written per value.  2^25 + 3 12-bit values: 232 us
+// with one code per thread, 66 us.  x 16-byte aligned, out at any code.
+__global__ void __launch_bounds__(256) quantize_planes2_kernel(const float* __restrict__ x, long long n, QParams p,
+                                                               __half* __restrict__ out) {
+    bool bad = false;
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long ng = (n + 31) / 32;
-    const uint32_t mask = (1u << k) - 1;
-    for (long long g0 = warp * PACK_G; g0 < ng; g0 += nwarps * PACK_G) {
-        uint32_t f[PACK_G];
+    const int m0 = misaligned8(out), m1 = misaligned8(out + n);
+    for (long long p0 = warp; p0 * 256 < n; p0 += nwarps) {
+        const long long e = p0 * 256 + 8 * lane;
+        float v[8];
+        if (e + 8 <= n) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(x + e)), b = __ldg(reinterpret_cast<const float4*>(x + e) + 1);
+            v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+        } else {
 #pragma unroll
-        for (int j = 0; j < PACK_G; ++j) {
-            const long long e = (g0 + j) * 32 + lane;
-            f[j] = e < n ? (uint32_t)code_get(codes, e, planes, n) & mask : 0u;
+            for (int i = 0; i < 8; ++i) v[i] = e + i < n ? __ldg(x + e + i) : 0.0f;
+        }
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            __half h0, l0, h1, l1;
+            split_limbs(quant1(v[2 * i], p, bad), h0, l0);
+            split_limbs(quant1(v[2 * i + 1], p, bad), h1, l1);
+            hi[i] = (uint32_t)__half_as_ushort(h0) | ((uint32_t)__half_as_ushort(h1) << 16);
+            lo[i] = (uint32_t)__half_as_ushort(l0) | ((uint32_t)__half_as_ushort(l1) << 16);
+        }
+        store8_codes(out, e, n, m0, make_uint4(hi[0], hi[1], hi[2], hi[3]), lane);
+        store8_codes(out + n, e, n, m1, make_uint4(lo[0], lo[1], lo[2], lo[3]), lane);
+    }
+    if (bad) latch_status(p.status, FXPQ_ERR_NONFINITE);
+}
+
+constexpr int PACK_U = 2;  // 256-code pieces per warp and iteration (their loads are issued together)
+
+template <int PLANES>
+__global__ void __launch_bounds__(256) pack_codes_kernel(const __half* __restrict__ codes, long long n, int k,
+                                                         uint32_t* __restrict__ words) {
+    const int lane = threadIdx.x & 31;
+    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    const long long ng = (n + 31) / 32, np = (n + 255) / 256;
+    const int m0 = misaligned8(codes), m1 = misaligned8(codes + n);
+    for (long long p0 = warp * PACK_U; p0 < np; p0 += nwarps * PACK_U) {
+        uint4 a[PACK_U], b[PACK_U];
+#pragma unroll
+        for (int u = 0; u < PACK_U; ++u) {
+            const long long e = (p0 + u) * 256 + 8 * lane;
+            a[u] = load8_codes(codes, e, n, m0);
+            if (PLANES == 2) b[u] = load8_codes(codes + n, e, n, m1);
         }
 #pragma unroll
-        for (int j = 0; j < PACK_G; ++j) {
-            if (g0 + j >= ng) break;
-            uint32_t mine = 0;
+        for (int u = 0; u < PACK_U; ++u) {
+            if (p0 + u >= np) break;
+            uint32_t c[4] = {codes_to_s16x2(a[u].x), codes_to_s16x2(a[u].y), codes_to_s16x2(a[u].z), codes_to_s16x2(a[u].w)};
+            if (PLANES == 2) {
+                // code = 256 hi + lo, in 16-bit halves
+                const uint32_t l[4] = {codes_to_s16x2(b[u].x), codes_to_s16x2(b[u].y), codes_to_s16x2(b[u].z),
+                                       codes_to_s16x2(b[u].w)};
 #pragma unroll
-            for (int b = 0; b < 16; ++b) {
-                if (b >= k) break;
-                const uint32_t w = __ballot_sync(0xffffffffu, (f[j] >> b) & 1u);
-                if (lane == b) mine = w;
+                for (int i = 0; i < 4; ++i) c[i] = __vadd2((c[i] << 8) & 0xFF00FF00u, l[i]);
             }
-            if (lane < k) words[(g0 + j) * k + lane] = mine;
+            const long long g = (p0 + u) * 8 + (lane >> 2);
+#pragma unroll
+            for (int h = 0; h < PLANES; ++h) {  // low bytes: planes 0-7; high bytes: planes 8-15
+                uint32_t lo = __byte_perm(c[0], c[1], h ? 0x7531 : 0x6420), hi = __byte_perm(c[2], c[3], h ? 0x7531 : 0x6420);
+                bit_transpose8(lo, hi);
+                lo = quad_transpose(lo, lane);
+                hi = quad_transpose(hi, lane);
+                const int b0 = 8 * h + (lane & 3);
+                if (g < ng && b0 < k) words[g * k + b0] = lo;
+                if (g < ng && b0 + 4 < k) words[g * k + b0 + 4] = hi;
+            }
         }
     }
 }
 
-__global__ void unpack_codes_kernel(const uint32_t* __restrict__ words, long long n, int k, int is_signed,
-                                    int planes, __half* __restrict__ codes) {
+template <int PLANES>
+__global__ void __launch_bounds__(256) unpack_codes_kernel(const uint32_t* __restrict__ words, long long n, int k,
+                                                           int is_signed, __half* __restrict__ codes) {
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long ng = (n + 31) / 32;
-    for (long long g0 = warp * PACK_G; g0 < ng; g0 += nwarps * PACK_G) {
-        uint32_t w[PACK_G];
+    const long long ng = (n + 31) / 32, np = (n + 255) / 256;
+    const int m0 = misaligned8(codes), m1 = misaligned8(codes + n);
+    // the top byte's field (bits 0-7 of one plane, 8-15 of two) carries the sign
+    const int kt = PLANES == 2 ? k - 8 : k;
+    const uint32_t flip = is_signed ? 0x01010101u * (1u << (kt - 1)) : 0u;
+    const uint32_t o1 = 0x6400u + (is_signed ? (1u << (kt - 1)) : 0u), off = o1 | (o1 << 16);
+    for (long long p0 = warp * PACK_U; p0 < np; p0 += nwarps * PACK_U) {
+        uint32_t w[PACK_U][4 * PLANES / 2];  // planes lane % 4, + 4, (+ 8, + 12)
 #pragma unroll
-        for (int j = 0; j < PACK_G; ++j) w[j] = (g0 + j < ng && lane < k) ? __ldg(words + (g0 + j) * k + lane) : 0u;
+        for (int u = 0; u < PACK_U; ++u) {
+            const long long g = (p0 + u) * 8 + (lane >> 2);
 #pragma unroll
-        for (int j = 0; j < PACK_G; ++j) {
-            if (g0 + j >= ng) break;
-            int field = 0;
-#pragma unroll
-            for (int b = 0; b < 16; ++b) {
-                if (b >= k) break;
-                field |= (int)((__shfl_sync(0xffffffffu, w[j], b) >> lane) & 1u) << b;
+            for (int q = 0; q < 2 * PLANES; ++q) {
+                const int b = 4 * q + (lane & 3);
+                w[u][q] = g < ng && b < k ? __ldg(words + g * k + b) : 0u;
             }
-            if (is_signed && (field >> (k - 1))) field -= 1 << k;  // sign extension of the k-bit field
-            const long long e = (g0 + j) * 32 + lane;
-            if (e < n) code_put(codes, e, planes, n, field);
+        }
+#pragma unroll
+        for (int u = 0; u < PACK_U; ++u) {
+            if (p0 + u >= np) break;
+            const long long e = (p0 + u) * 256 + 8 * lane;
+            uint32_t x[2 * PLANES];
+#pragma unroll
+            for (int q = 0; q < 2 * PLANES; ++q) x[q] = quad_transpose(w[u][q], lane);
+            if (PLANES == 1) {
+                store8_codes(codes, e, n, m0, fields_to_f16(x[0], x[1], flip, off), lane);
+            } else {
+                store8_codes(codes, e, n, m0, fields_to_f16(x[2 * PLANES - 2], x[2 * PLANES - 1], flip, off), lane);
+                store8_codes(codes + n, e, n, m1, fields_to_f16(x[0], x[1], 0u, 0x64006400u), lane);
+            }
         }
     }
 }
@@ -455,10 +642,15 @@ extern "C" fxpq_status fxpq_quantize(const float* d_x, int64_t n, fxpq_fmt f, in
                 d_x, n, p, static_cast<uint16_t*>(d_codes));
             return after_launch("quantize_f16");
         }
+        // (planes on 16-byte boundaries: 2^25 16-bit codes 49 us here, 54 us through the kernel below)
         if (al16 && n % 8 == 0) {
             quantize_rows_vec8_kernel<<<grid_for(n / 8, T), T, 0, s>>>(reinterpret_cast<const float4*>(d_x), n / 8,
                                                                       planes_of(f), p, static_cast<uint4*>(d_codes));
             return after_launch("quantize_rows_vec8");
+        }
+        if (planes_of(f) == 2 && aligned(d_x, 16) && aligned(d_codes, 2)) {
+            quantize_planes2_kernel<<<grid_for((n + 7) / 8, T), T, 0, s>>>(d_x, n, p, static_cast<__half*>(d_codes));
+            return after_launch("quantize_planes2");
         }
         // unaligned: one code per row of one channel
         quantize_rows_f16_kernel<<<grid_for(n, T), T, 0, s>>>(d_x, n, 1, 1, planes_of(f), p,
@@ -599,10 +791,11 @@ extern "C" fxpq_status fxpq_pack_codes(const void* d_codes, int64_t n, fxpq_fmt 
     if (n < 0 || !fmt_ok1(fmt) || (n > 0 && (!d_codes || !d_words)) || !aligned(d_words, 4))
         return FXPQ_ERR_INVALID_ARG;
     if (n == 0) return FXPQ_OK;
-    const long long ng = (n + 31) / 32;
-    const int T = 256;
-    pack_codes_kernel<<<grid_for((ng + PACK_G - 1) / PACK_G * 32, T), T, 0, as_stream(stream)>>>(
-        static_cast<const __half*>(d_codes), n, fmt.bits, planes_of(fmt), d_words);
+    const int T = 256, grid = grid_for((n + 256 * PACK_U - 1) / (256 * PACK_U) * 32, T);
+    if (planes_of(fmt) == 1)
+        pack_codes_kernel<1><<<grid, T, 0, as_stream(stream)>>>(static_cast<const __half*>(d_codes), n, fmt.bits, d_words);
+    else
+        pack_codes_kernel<2><<<grid, T, 0, as_stream(stream)>>>(static_cast<const __half*>(d_codes), n, fmt.bits, d_words);
     return after_launch("pack_codes");
 }
 
@@ -630,9 +823,12 @@ extern "C" fxpq_status fxpq_unpack_codes(const uint32_t* d_words, int64_t n, fxp
     if (n < 0 || !fmt_ok1(fmt) || (n > 0 && (!d_codes || !d_words)) || !aligned(d_words, 4))
         return FXPQ_ERR_INVALID_ARG;
     if (n == 0) return FXPQ_OK;
-    const long long ng = (n + 31) / 32;
-    const int T = 256;
-    unpack_codes_kernel<<<grid_for((ng + PACK_G - 1) / PACK_G * 32, T), T, 0, as_stream(stream)>>>(
-        d_words, n, fmt.bits, fmt.is_signed, planes_of(fmt), static_cast<__half*>(d_codes));
+    const int T = 256, grid = grid_for((n + 256 * PACK_U - 1) / (256 * PACK_U) * 32, T);
+    if (planes_of(fmt) == 1)
+        unpack_codes_kernel<1><<<grid, T, 0, as_stream(stream)>>>(d_words, n, fmt.bits, fmt.is_signed,
+                                                                  static_cast<__half*>(d_codes));
+    else
+        unpack_codes_kernel<2><<<grid, T, 0, as_stream(stream)>>>(d_words, n, fmt.bits, fmt.is_signed,
+                                                                  static_cast<__half*>(d_codes));
     return after_launch("unpack_codes");
 }

@@ -365,3 +365,34 @@ def test_pack_unpack_large_sampled(F, k, S):
     for g in list(rng.integers(0, ng, size=40)) + [ng - 1]:
         seg = c[32 * g: 32 * g + 32]
         assert np.array_equal(w[g * k:(g + 1) * k], oracle.pack_codes(seg, k)), g
+
+
+@pytest.mark.parametrize("k,S", [(1, 1), (5, 0), (8, 1), (9, 0), (16, 1)])
+@pytest.mark.parametrize("n", [255, 256, 257, 1024 + 263])
+@pytest.mark.parametrize("off", [0, 1, 4, 7])
+def test_pack_unpack_quantize_any_alignment(F, k, S, n, off):
+    """Pieces of 256 codes, the ends of a warp and lo planes off every 16-byte boundary: words, codes and the
+    quantizer's two-plane codes match the oracle, and nothing outside the tensor is written."""
+    rng = np.random.default_rng(1000 * k + n + off)
+    lo, hi = (-1, 0) if (k, S) == (1, 1) else (oracle.qmin(k, S), oracle.qmax(k, S))
+    c = rng.integers(lo, hi + 1, size=n)
+    f = F.fmt(k, S, 3)
+    p = F.planes(f)
+    src = torch.full((8 + n * p + 8,), 99.0, dtype=torch.float16, device="cuda")
+    src[off:off + n * p] = _f16_codes(c, k)
+    words = torch.full((F.packed_words(n, f) + 2,), 0x5A5A5A5A, dtype=torch.int32, device="cuda")
+    F.fxpq_pack_codes(src[off:], n, f, words)
+    w = words.cpu().numpy().view(np.uint32)
+    assert np.array_equal(w[:-2], oracle.pack_codes(c, k)) and (w[-2:] == 0x5A5A5A5A).all()
+    out = torch.full_like(src, 77.0)
+    F.fxpq_unpack_codes(words, n, f, out[off:])
+    got = out.cpu()
+    assert np.array_equal(F.codes_to_int(got[off:off + n * p], f, (n,)).numpy(), c)
+    assert (got[:off] == 77).all() and (got[off + n * p:] == 77).all()
+    if k > 1:
+        x = torch.from_numpy((c / 8.0).astype(np.float32)).cuda()
+        out.fill_(77.0)
+        F.fxpq_quantize(x, f, F.DT_F16, out[off:])
+        got = out.cpu()
+        assert np.array_equal(F.codes_to_int(got[off:off + n * p], f, (n,)).numpy(), c)
+        assert (got[:off] == 77).all() and (got[off + n * p:] == 77).all()
