@@ -84,4 +84,14 @@ __device__ __forceinline__ void code_put(__half* __restrict__ t, long long idx, 
     }
 }
 
+// Two values already clipped to [-512, 511], rounded half to even, as packed fp16 codes: adding
+// 1.5 2^23 + 0x6600 rounds at the integer and leaves 0x6600 + code, the fp16 pattern of 1536 + code (the
+// binade [1024, 2048) has unit spacing), in the low half-word; one packed subtraction of 1536 leaves the code.
+__device__ __forceinline__ uint32_t f32_codes_f16x2(float c0, float c1) {
+    const uint32_t w = __byte_perm(__float_as_uint(c0 + 12609024.0f), __float_as_uint(c1 + 12609024.0f), 0x5410);
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w),
+                              __halves2half2(__ushort_as_half(0x6600), __ushort_as_half(0x6600)));
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
 }  // namespace fxpq

@@ -296,6 +296,37 @@ def test_eltwise_parity(F, mode, fa, fb, relu):
         assert np.array_equal(y.cpu().numpy().reshape(npix, C), oracle.to_f32(v, ws))
 
 
+@pytest.mark.parametrize("mode", [0, 1, 2])
+@pytest.mark.parametrize("relu", [0, 1])
+@pytest.mark.parametrize("fa,fb,fy", [((8, 0, 0), (8, 1, 15), (8, 1, 12)),    # the widest alignment of the fp32 sums
+                                      ((8, 0, 0), (8, 1, 16), (8, 1, 3)),     # one bit wider: 64-bit integers
+                                      ((8, 0, 6), (8, 0, 6), (4, 0, 2)),      # ties
+                                      ((4, 1, 3), (5, 0, 4), (8, 0, 9)),      # a left-shifting FxP-QLayer
+                                      ((2, 1, -32), (8, 0, -32), (8, 1, 8)),  # left by 40, all saturated
+                                      ((8, 1, 5), (8, 0, 4), (12, 1, 5))])    # two planes out
+@pytest.mark.parametrize("npix", [1, 5, 1031])
+def test_eltwise_vector_and_scalar(F, mode, relu, fa, fb, fy, npix):
+    """Both eltwise kernels over their alignments, extreme codes among them; pieces of 8 codes at any count."""
+    rng = np.random.default_rng(npix + mode)
+    C = 24
+    a, b = rand_codes(rng, (npix, C), fa[0], fa[1]), rand_codes(rng, (npix, C), fb[0], fb[1])
+    a.flat[:4] = b.flat[:4] = 0
+    a.flat[:2], b.flat[:2] = [oracle.qmax(*fa[:2]), oracle.qmin(*fa[:2])], [oracle.qmax(*fb[:2]), oracle.qmin(*fb[:2])]
+    dt = [torch.float16, torch.int64, torch.float32][mode]
+    FY = F.fmt(*fy)
+    y = torch.empty(npix * C * (F.planes(FY) if mode == 0 else 1), dtype=dt, device="cuda")
+    s = F.fxpq_eltwise(to_f16_planes(a, fa[0], C), F.fmt(*fa), to_f16_planes(b, fb[0], C), F.fmt(*fb), npix, C, relu, mode,
+                       FY, y)
+    v, ws = oracle.eltwise_add(a, fa[2], b, fb[2], relu)
+    assert s == ws
+    if mode == 0:
+        assert np.array_equal(F.codes_to_int(y.cpu(), FY, (npix, C)).numpy(), oracle.requant(v, ws, *fy))
+    elif mode == 1:
+        assert np.array_equal(y.cpu().numpy().reshape(npix, C), v)
+    else:
+        assert np.array_equal(y.cpu().numpy().reshape(npix, C), oracle.to_f32(v, ws))
+
+
 @pytest.mark.parametrize("s,fy", [(20, (8, 0, 6)), (11, (16, 1, 3)), (5, (4, 1, 9)), (30, (8, 1, 30)), (0, (6, 1, -2))])
 def test_qlayer_parity(F, s, fy):
     rng = np.random.default_rng(s + 100)
