@@ -396,3 +396,28 @@ def test_pack_unpack_quantize_any_alignment(F, k, S, n, off):
         got = out.cpu()
         assert np.array_equal(F.codes_to_int(got[off:off + n * p], f, (n,)).numpy(), c)
         assert (got[:off] == 77).all() and (got[off + n * p:] == 77).all()
+
+
+@pytest.mark.parametrize("k,S,fl", [(8, 0, 5), (8, 1, 5), (9, 1, 4), (16, 0, 13), (16, 1, 12), (2, 1, 40), (16, 1, -32)])
+@pytest.mark.parametrize("N,hw", [(1, 1), (3, 13), (2, 33), (5, 17)])
+def test_quantize_rgb_images(F, k, S, fl, N, hw):
+    """Three-channel images: blocks of 1024 pixels that span images and end inside one, every level, ties."""
+    x = _adv(k + N, N * 3 * hw * hw)[: N * 3 * hw * hw].reshape(N, 3, hw, hw)
+    f = F.fmt(k, S, fl)
+    out = torch.full((N * hw * hw * 8 * F.planes(f),), 55.0, dtype=torch.float16, device="cuda")
+    F.fxpq_quantize_images(torch.from_numpy(x).cuda(), f, 8, out)
+    got = F.codes_to_int(out.cpu(), f, (N, hw, hw, 8)).numpy()
+    want = oracle.quantize(np.ascontiguousarray(np.transpose(x, (0, 2, 3, 1))), k, S, fl).reshape(N, hw, hw, 3)
+    assert np.array_equal(got[..., :3], want) and np.all(got[..., 3:] == 0)
+
+
+def test_quantize_rgb_images_nonfinite(F):
+    x = torch.ones(1, 3, 4, 4, device="cuda")
+    x[0, 1, 2, 3] = float("nan")
+    x[0, 2, 0, 0] = float("-inf")
+    out = torch.empty(16 * 8, dtype=torch.float16, device="cuda")
+    F.fxpq_get_device_status()
+    F.fxpq_quantize_images(x, F.fmt(8, 1, 3), 8, out)
+    assert F.fxpq_get_device_status() == 3
+    got = out.cpu().reshape(4, 4, 8)
+    assert got[2, 3, 1] == 0 and got[0, 0, 2] == 0 and got[0, 0, 0] == 8
