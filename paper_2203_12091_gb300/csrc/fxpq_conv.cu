@@ -213,6 +213,8 @@ fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, con
     a.s_out = s;
     a.has_bias = bias != nullptr;
     a.v32 = 0;
+    a.vf = 0;
+    a.vf_c = a.vf_lo = a.vf_hi = 0.0f;
     if (d.out_mode == FXPQ_OUT_CODES) {
         a.sh = s - d.fmt_y.fl;
         if (a.sh > 62) return FXPQ_ERR_RANGE;
@@ -232,6 +234,13 @@ fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, con
                  a.delta <= 30)
                     ? 1
                     : 0;
+        // fp32 path (fepi_bias): the aligned bias and the sums below 2^23, or every larger sum clipped
+        const double b_al = bb * ldexp(1.0, a.delta), top = (double)(a.hi > -a.lo ? a.hi : -a.lo) + 1.0;
+        a.vf = !a.has_scale && a.py == 1 && a.sh32 >= 1 && a.sh32 <= 30 && a.delta >= -30 && a.delta <= 30 &&
+               b_al <= ldexp(1.0, 22) && (top * ldexp(1.0, a.sh32) <= ldexp(1.0, 23) || bound + b_al + 1.0 <= ldexp(1.0, 23));
+        a.vf_c = ldexpf(1.0f, -a.sh32);
+        a.vf_lo = a.relu && a.lo < 0 ? 0.0f : (float)a.lo;
+        a.vf_hi = (float)a.hi;
     } else {
         a.sh = 0;
         a.lo = a.hi = 0;

@@ -23,6 +23,8 @@ struct ConvArgs {
     int v32;           // 1: qlayer_code32 applies (the host checked its 32-bit bounds)
     int bsh;           // bias shift of the 32-bit path (= delta)
     int sh32;          // right shift of the 32-bit path, relative to the accumulator's scale
+    int vf;            // 1: the fp32 form of the FxP-QLayer applies to sums that are exact fp32 integers
+    float vf_c, vf_lo, vf_hi;  // 2^-sh32 and the clip levels (lower one 0 under a ReLU)
     const int32_t* scale;  // Scale layer aleph1 codes [K] (has_scale)
     const int32_t* shift;  // Scale layer aleph2 codes [K]
     int has_scale;
@@ -103,6 +105,17 @@ __host__ __device__ __forceinline__ int qlayer_code32(const ConvArgs& a, int acc
     const bool up = rem > half || (rem == half && (phi || (q & 1)));
     const int c = max(q + (up ? 1 : 0), (int)a.lo);
     return min(c, (int)a.hi);
+}
+
+// The same in fp32 (valid when a.vf, for |acc| < 2^24): the code is acc 2^-sh32 + t, clipped, rounded half to
+// even, with the channel's constant t = (aligned bias) 2^-sh32.  A bias finer than the accumulator enters as
+// floor(B / 2^d) + 1/2 when bits fall below: with sh32 >= 1 no tie lies between the true fraction and 1/2.
+// acc + bias is exact in fp32 below 2^23 in magnitude; the host proves that, or that every larger value is
+// clipped (rounding is monotone, so it stays clipped).  Clipping first is immaterial: the levels are integers.
+__host__ __device__ __forceinline__ float fepi_bias(const ConvArgs& a, int32_t b) {
+    if (a.bsh >= 0) return (float)(b << a.bsh) * a.vf_c;
+    const int d = -a.bsh;
+    return ((float)(b >> d) + ((b & ((1 << d) - 1)) ? 0.5f : 0.0f)) * a.vf_c;
 }
 
 // Bias alignment, ReLU and the FxP-QLayer for one output value of row m, channel k.

@@ -18,7 +18,7 @@ std::mutex g_tc_mu;
 // allows them (by default only while they compute few extra rows), "tc_bn128" never takes
 // 256-column tiles and "tc_bn256" takes them wherever the layer allows (by default they also need
 // enough tiles to keep every SM busy), "tc_win64" keeps window mode's two-limb epilogue in 64-bit
-// arithmetic.
+// arithmetic, "tc_win32" in 32-bit integers, "tc_iepi" the one-group layers' epilogue in integers.
 bool conv_path_is(const char* name) {
     const char* e = getenv("FXPQ_CONV_PATH");
     return e && strcmp(e, name) == 0;
@@ -167,6 +167,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         P.rows_tma = 0;
         P.w32 = 0;
         P.wf32 = 0;
+        P.win_eps = P.win_c[0] = P.win_c[1] = P.win_c[2] = 0.0f;
         P.nacc = 1;
         // window mode for 8-channel stride-1 layers with at most 64 output channels: 8 x 16 output
         // patches, one input window per tile and limb plane, weights resident in shared memory, one
@@ -221,11 +222,11 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
                     // 32-bit epilogue of two-limb x and w (v = 2^16 T + Lo, see the kernel): every limb
                     // sum covers R * S2 * 8 products; L = 2^8 (S_hl + S_lh) + S_ll + Lo(B') and T must stay
                     // below 2^31, the aligned bias must not be finer than the sums (delta >= 0), and
-                    // sh - 16 in [0, 30]; the per-channel bias table takes the last 512 bytes of the B region
+                    // sh - 16 in [0, 30]; the per-channel bias tables take the last 768 bytes of the B region
                     const bool codes32 = a.out_mode == FXPQ_OUT_CODES && a.py == 1 && a.sh >= 16 && a.sh <= 46;
                     const bool image32 = a.out_mode == FXPQ_OUT_F32 && a.K % 4 == 0;  // the fp32 image
                     if (a.px == 2 && a.pw == 2 && !a.has_scale && a.delta >= 0 && (codes32 || image32) &&
-                        a.pw * a.R * (S2 / 2) * 64 * 32 + 512 <= tc_stages(64) * 64 * TC_BK * 2) {
+                        a.pw * a.R * (S2 / 2) * 64 * 32 + 768 <= tc_stages(64) * 64 * TC_BK * 2) {
                         const double taps = (double)a.R * S2 * 8;
                         const double hh = (double)limb_max(d.fmt_x, 0) * limb_max(d.fmt_w, 0) * taps;
                         const double hl = (double)limb_max(d.fmt_x, 0) * limb_max(d.fmt_w, 1) * taps;
@@ -237,6 +238,17 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
                         const bool ok32 = Lb < ldexp(1.0, 31) && Tb < ldexp(1.0, 31) && !conv_path_is("tc_win64");
                         P.w32 = ok32 && codes32;
                         P.wf32 = ok32 && image32;
+                        if (P.w32) {
+                            // t = hh 2^(16-sh) + B' 2^-sh, + mid 2^(8-sh), + ll 2^-sh: every step is off by at
+                            // most 2^-24 of its result, which for a t inside the clip levels (widened by one)
+                            // is at most `top`, plus the terms still to come; so are mid and the constant.
+                            // Beyond one 64th the exact arithmetic would run too often.
+                            const double u = ldexp(1.0, -a.sh), top = (double)(a.hi > -a.lo ? a.hi : -a.lo) + 2.0;
+                            const double tm = (hl + lh) * 256.0 * u, tl = ll * u;
+                            const double eps = ldexp(1.0, -24) * ((top + tm + tl) + tm + (top + tl) + top + bb * u) * 1.25;
+                            for (int i = 0; i < 3; ++i) P.win_c[i] = (float)ldexp(u, 16 - 8 * i);
+                            P.win_eps = eps < 1.0 / 64 && !conv_path_is("tc_win32") ? (float)eps : 0.0f;
+                        }
                     }
                 }
             }
@@ -406,6 +418,8 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         }
     }
     P.n_units = P.n_tiles * P.ksplit;
+    P.fepi = a.vf && P.fast_store && P.n_groups == 1 && P.g[0].shift == 0 && P.patch != 3 && P.ksplit == 1 && !acc64 &&
+             !conv_path_is("tc_iepi");
     {
         std::lock_guard<std::mutex> lk(g_tc_mu);
         if (!g_tc_attr_set) {

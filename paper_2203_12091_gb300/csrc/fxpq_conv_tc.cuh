@@ -123,6 +123,9 @@ struct TcParams {
     int WW, WH, S2;      // window mode: window width / height in pixels, taps per row rounded up to even
     int w32;             // window mode, two-limb x and w, one-plane codes out: the 32-bit epilogue (the
                          // host proved its bounds; see the epilogue), with m = sh - 16 in [0, 30]
+    int fepi;            // the fp32 FxP-QLayer (a.vf; one exact group, no split, fast_store)
+    float win_c[3], win_eps;  // w32 in fp32: 2^(16 - sh), 2^(8 - sh), 2^-sh; the most that the fp32 sum is off
+                              // (0: integer arithmetic throughout)
     int wf32;            // the same window instance writing the fp32 image of v = 2^16 T + Lo
     int win_bytes;       // window mode: bytes of one window (128-byte aligned; patch 4: 16-byte aligned)
     int w64_slot0;       // patch 4: offset of window slot 0 (after the resident weights)
@@ -540,6 +543,28 @@ __device__ __forceinline__ void epilogue_block32_staged(const ConvArgs& a, long 
     }
 }
 
+// 32 one-plane codes per lane (row m, channels k0 ..) through a 2 KB shared-memory slice of the warp: each
+// lane puts its row's 64 bytes there (16-byte pieces rotated against bank conflicts), then every store
+// instruction writes whole 64-byte row segments of eight rows.  One-plane codes have K % 8 == 0, so a
+// 16-byte piece lies wholly inside or past K.  Rows with m < 0 store nothing.
+__device__ __forceinline__ void store_codes_direct(const ConvArgs& a, long long m, int k0, const uint32_t (&w)[16],
+                                                   unsigned char* wbuf, int lane) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<uint4*>(wbuf + lane * 64 + 16 * (q ^ ((lane >> 1) & 3))) =
+            make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int r = (lane >> 2) + 8 * it, pc = lane & 3;
+        const long long mr = __shfl_sync(0xffffffffu, m, r);
+        const uint4 v = *reinterpret_cast<const uint4*>(wbuf + r * 64 + 16 * (pc ^ ((r >> 1) & 3)));
+        const int kk = k0 + pc * 8;
+        if (mr >= 0 && kk < a.K) *reinterpret_cast<uint4*>(static_cast<__half*>(a.y) + mr * a.K + kk) = v;
+    }
+    __syncwarp();
+}
+
 // Uniform constants of the 32-bit FxP-QLayer epilogue (the same arithmetic as qlayer_code32, with
 // the bias alignment split into a left and a right shift so that it has no branches).
 struct Epi32 {
@@ -625,6 +650,44 @@ __device__ __forceinline__ uint32_t pack_codes_f16(int c0, int c1) {
     const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&bits), __halves2half2(__ushort_as_half(0x6600),
                                                                                         __ushort_as_half(0x6600)));
     return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// One code of the two-limb window epilogue in exact 32-bit arithmetic (see the generic window epilogue): bt the
+// aligned bias (high and low 16 bits), m = sh - 16, half = 2^(m-1), mmask = 2^m - 1.
+__device__ __forceinline__ int win_code(uint32_t fhh, uint32_t fhl, uint32_t flh, uint32_t fll, int2 bt, int m, int half,
+                                        int mmask, int relu, int lo, int hi) {
+    const int mid = __float2int_rn(__uint_as_float(fhl)) + __float2int_rn(__uint_as_float(flh));
+    const int L = mid * 256 + __float2int_rn(__uint_as_float(fll)) + bt.y;
+    const int T = __float2int_rn(__uint_as_float(fhh)) + bt.x + (L >> 16);
+    const int Lo = L & 0xFFFF;
+    int q, up;
+    if (m > 0) {
+        q = T >> m;
+        const int rem = T & mmask;
+        up = (rem > half) | ((rem == half) & ((Lo != 0) | (q & 1)));
+    } else {
+        q = T;
+        up = (Lo > 0x8000) | ((Lo == 0x8000) & (q & 1));
+    }
+    return min(max((relu && T < 0) ? 0 : q + up, lo), hi);
+}
+
+// Two accumulators to packed codes in fp32 (fepi_bias): one packed fused multiply-add, clip, the packed
+// rounding addition of f32_codes_f16x2.  About 4.5 instructions per code, none of them a conversion (those
+// run at a quarter of the rate); the integer form took 20 to 30.
+__device__ __forceinline__ uint32_t fepi_pair(uint32_t a0, uint32_t a1, uint64_t cc, float t0, float t1, float lo, float hi) {
+    uint64_t av, tv, v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(av) : "r"(a0), "r"(a1));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(tv) : "f"(t0), "f"(t1));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(av), "l"(cc), "l"(tv));
+    float x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+    return f32_codes_f16x2(fminf(fmaxf(x, lo), hi), fminf(fmaxf(y, lo), hi));
+}
+__device__ __forceinline__ uint64_t f32x2_splat(float c) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(c));
+    return v;
 }
 
 // ------------------------------------------------------------------ kernel
@@ -755,10 +818,12 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     // window mode, 32-bit epilogue: per output channel the aligned bias B' = b 2^delta split as
     // (B' >> 16, B' & 0xFFFF), in the last 512 bytes of the B region (the resident weights stay below)
     int2* wtab = reinterpret_cast<int2*>(sB + TC_STAGES * B_BYTES - 512);
+    float* wtabf = reinterpret_cast<float*>(sB + TC_STAGES * B_BYTES - 768);  // B' 2^-sh, the 256 bytes before it
     if (BN == 64 && sizeof(ACC) == 8 && !SC && P.patch == 3 && (P.w32 || P.wf32) && warp == 1) {
         for (int k = lane; k < 64; k += 32) {
             const long long bb = (a.has_bias && k < a.K) ? ((long long)__ldg(a.bias + k) << (a.delta > 0 ? a.delta : 0)) : 0;
             wtab[k] = make_int2((int)(bb >> 16), (int)(bb & 0xFFFF));
+            wtabf[k] = (float)bb * P.win_c[2];
         }
     }
     tc_fence_before();
@@ -1051,19 +1116,21 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         const int half = m > 0 ? 1 << (m - 1) : 0;
         const int mmask = (int)((1u << m) - 1u);
         const int lo = (int)a.lo, hi = (int)a.hi;
+        const float flo = a.relu && lo < 0 ? 0.0f : (float)lo, fhi = (float)hi;
         const int per_img = P.tiles_p * P.tiles_q;
         const bool f32out = a.out_mode == FXPQ_OUT_F32;  // the fp32 image (calibration) instead of codes
         // W64, 32-bit codes: a thread's 16 output channels are the same in every tile, so their aligned
         // bias terms and the flags of bias bits below the accumulator's scale are formed once
         const Epi32 e32w = make_epi32(a);
-        int btw[16];
+        int btw[16];  // (P.fepi: the fp32 terms' bits)
         uint32_t phiw = 0u;
+        const uint64_t cc2 = f32x2_splat(a.vf_c);
         if (W64) {
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const int k = cw * 16 + j;
                 const int32_t b = (a.has_bias && k < a.K) ? __ldg(a.bias + k) : 0;
-                btw[j] = (b << e32w.bsl) >> e32w.bsr;
+                btw[j] = P.fepi ? __float_as_int(a.has_bias ? fepi_bias(a, b) : 0.0f) : (b << e32w.bsl) >> e32w.bsr;
                 phiw |= ((b & e32w.fmask) != 0 ? 1u : 0u) << j;
             }
         }
@@ -1094,7 +1161,12 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         w[j] = __float_as_uint(__ll2float_rn(cblock_value<false>(a, k, (long long)acc, b)) * a.f32_scale);
                     }
                 }
-                if (!f32out && a.v32) {
+                if (P.fepi) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        w[j] = fepi_pair(f[2 * j], f[2 * j + 1], cc2, __int_as_float(btw[2 * j]),
+                                         __int_as_float(btw[2 * j + 1]), a.vf_lo, a.vf_hi);
+                } else if (!f32out && a.v32) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         int c2[2];
@@ -1149,30 +1221,36 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     w[jj] = __float_as_uint(__ll2float_rn(v) * a.f32_scale);
                 }
             }
+            // codes: in fp32 first, t = v / 2^sh within P.win_eps; only a value that close to a rounding
+            // boundary (about one in a thousand) is decided by the exact 32-bit arithmetic of win_code
 #pragma unroll
             for (int j = 0; j < ((WIN && !f32out) ? 8 : 0); ++j) {
-                int c2[2];
+                if (P.win_eps > 0.0f) {
+                    float tv[2];
+                    bool near = false;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int jj = 2 * j + h;
-                    const int2 bt = wtab[cw * 16 + jj];
-                    const int mid = __float2int_rn(__uint_as_float(fhl[jj])) + __float2int_rn(__uint_as_float(flh[jj]));
-                    const int L = mid * 256 + __float2int_rn(__uint_as_float(fll[jj])) + bt.y;
-                    const int T = __float2int_rn(__uint_as_float(fhh[jj])) + bt.x + (L >> 16);
-                    const int Lo = L & 0xFFFF;
-                    int q, up;
-                    if (m > 0) {
-                        q = T >> m;
-                        const int rem = T & mmask;
-                        up = (rem > half) | ((rem == half) & ((Lo != 0) | (q & 1)));
-                    } else {
-                        q = T;
-                        up = (Lo > 0x8000) | ((Lo == 0x8000) & (q & 1));
+                    for (int h = 0; h < 2; ++h) {
+                        const int jj = 2 * j + h;
+                        float x = fmaf(__uint_as_float(fhh[jj]), P.win_c[0], wtabf[cw * 16 + jj]);
+                        x = fmaf(__uint_as_float(fhl[jj]) + __uint_as_float(flh[jj]), P.win_c[1], x);
+                        x = fmaf(__uint_as_float(fll[jj]), P.win_c[2], x);
+                        x = fminf(fmaxf(x, flo), fhi);
+                        const float r = (x + 12582912.0f) - 12582912.0f;
+                        near |= fabsf(x - r) > 0.5f - P.win_eps;
+                        tv[h] = x;
                     }
-                    const int cc = (a.relu && T < 0) ? 0 : q + up;
-                    c2[h] = min(max(cc, lo), hi);
+                    w[j] = f32_codes_f16x2(tv[0], tv[1]);
+                    if (near)
+                        w[j] = pack_codes_f16(win_code(fhh[2 * j], fhl[2 * j], flh[2 * j], fll[2 * j], wtab[cw * 16 + 2 * j],
+                                                       m, half, mmask, a.relu, lo, hi),
+                                              win_code(fhh[2 * j + 1], fhl[2 * j + 1], flh[2 * j + 1], fll[2 * j + 1],
+                                                       wtab[cw * 16 + 2 * j + 1], m, half, mmask, a.relu, lo, hi));
+                } else {
+                    w[j] = pack_codes_f16(win_code(fhh[2 * j], fhl[2 * j], flh[2 * j], fll[2 * j], wtab[cw * 16 + 2 * j], m,
+                                                   half, mmask, a.relu, lo, hi),
+                                          win_code(fhh[2 * j + 1], fhl[2 * j + 1], flh[2 * j + 1], fll[2 * j + 1],
+                                                   wtab[cw * 16 + 2 * j + 1], m, half, mmask, a.relu, lo, hi));
                 }
-                w[j] = pack_codes_f16(c2[0], c2[1]);
             }
             if (f32out) {
                 // fp32 image out: this row's 16 values are 64 contiguous bytes of the output row
@@ -1388,6 +1466,53 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         }
                         continue;
                     }
+                    if (sizeof(ACC) == 4 && !SC && !SPLIT && !PK && P.fepi) {
+                        // one exact group: codes straight from the fp32 sums
+                        uint32_t f0[16], f1[16], w[16];
+                        tmem_ld16_nw(lane_base + buf * BN + cb * 32, f0);
+                        tmem_ld16_nw(lane_base + buf * BN + cb * 32 + 16, f1);
+                        // the chunk's 32 channel constants, one per lane, to every lane through shared
+                        // memory that this warp overwrites with the codes afterwards
+                        const int kl = k0 + lane;
+                        const float t = a.has_bias && kl < a.K ? fepi_bias(a, __ldg(a.bias + kl)) : 0.0f;
+                        unsigned char* wbuf = sO + (warp - 4) * 2048;                     // DIRECT
+                        unsigned char* half_buf = sO + (cb >> 1) * (TC_BM * 128);         // staged tile
+                        // four constants 4 q .. 4 q + 3
+                        auto tab = [&](int q) {
+                            return DIRECT ? wbuf + 16 * q
+                                          : half_buf + (quad * 32 + (q >> 2)) * 128 + ((((cb & 1) * 4 + (q & 3)) ^ (q >> 2)) << 4);
+                        };
+                        *reinterpret_cast<float*>(tab(lane >> 2) + 4 * (lane & 3)) = t;
+                        __syncwarp();
+                        tmem_wait_ld();
+                        reg_fence(f0);
+                        reg_fence(f1);
+                        if (c == CPW - 1) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(accempty0 + 8 * buf);
+                        }
+                        const uint64_t cc = f32x2_splat(a.vf_c);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float4 tq = *reinterpret_cast<const float4*>(tab(q));
+                            const uint32_t* f = q < 4 ? f0 + 4 * q : f1 + 4 * (q - 4);
+                            w[2 * q] = fepi_pair(f[0], f[1], cc, tq.x, tq.y, a.vf_lo, a.vf_hi);
+                            w[2 * q + 1] = fepi_pair(f[2], f[3], cc, tq.z, tq.w, a.vf_lo, a.vf_hi);
+                        }
+                        __syncwarp();
+                        if (DIRECT) {
+                            store_codes_direct(a, m, k0, w, wbuf, lane);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const int chunk = (cb & 1) * 4 + q;
+                                *reinterpret_cast<uint4*>(half_buf + row * 128 + ((chunk ^ (row & 7)) << 4)) =
+                                    make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+                            }
+                        }
+                        continue;
+                    }
                     // One TMEM round trip per load batch: the fp32 group sums and, after the first group,
                     // the integer running sums are loaded together; the running-sum stores share one
                     // completion wait.
@@ -1573,26 +1698,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                             }
                         }
                         if (DIRECT) {
-                            // through the warp's 2 KB slice of the staging region: each lane puts its row's
-                            // 64 bytes there (16-byte pieces rotated against bank conflicts), then every
-                            // store instruction writes whole 64-byte row segments of eight rows.  One-plane
-                            // codes have K % 8 == 0, so a 16-byte piece lies wholly inside or past K.
-                            unsigned char* wbuf = sO + (warp - 4) * 2048;
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                *reinterpret_cast<uint4*>(wbuf + lane * 64 + 16 * (q ^ ((lane >> 1) & 3))) =
-                                    make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-                            __syncwarp();
-#pragma unroll
-                            for (int it = 0; it < 4; ++it) {
-                                const int r = (lane >> 2) + 8 * it, pc = lane & 3;
-                                const long long mr = __shfl_sync(0xffffffffu, m, r);
-                                const uint4 v = *reinterpret_cast<const uint4*>(wbuf + r * 64 + 16 * (pc ^ ((r >> 1) & 3)));
-                                const int kk = k0 + pc * 8;
-                                if (mr >= 0 && kk < a.K)
-                                    *reinterpret_cast<uint4*>(static_cast<__half*>(a.y) + mr * a.K + kk) = v;
-                            }
-                            __syncwarp();
+                            store_codes_direct(a, m, k0, w, sO + (warp - 4) * 2048, lane);
                             continue;
                         }
                         unsigned char* half_buf = sO + (cb >> 1) * (TC_BM * 128);

@@ -227,6 +227,68 @@ def test_window_epilogue_alternatives(F, case, alt):
         os.environ["FXPQ_CONV_PATH"] = "tc"
 
 
+@pytest.mark.parametrize("K", [24, 64, 72, 264])  # 64-channel window, ragged 128- and 256-column tiles
+@pytest.mark.parametrize("sh", [1, 8, 15, 16, 17])  # 8-bit codes: every sum at or above 2^23 is clipped up to 15
+@pytest.mark.parametrize("finer", [-3, 0, 9])  # bias coarser, equal, finer than the accumulator
+@pytest.mark.parametrize("relu,ty", [(True, (8, 0)), (False, (8, 1)), (False, (4, 1))])
+def test_fp32_epilogue(F, K, sh, finer, relu, ty):
+    """One exact group: the FxP-QLayer in fp32 on random sums, sums near 2^24 of both signs, rounding ties and
+    biases with bits below the accumulator's scale, and the integer form on the same layer."""
+    if os.environ.get("FXPQ_CONV_PATH") not in ("tc", "tc_bn256"):
+        pytest.skip("an epilogue of the tensor-core path")
+    N, H, C, R = 2, 9, 64, 3
+    rng = np.random.default_rng(K + 10 * sh + finer)
+    fx, fw = F.fmt(8, 0, 6), F.fmt(8, 1, 9)
+    fb, fy = F.fmt(16, 1, 15 + finer), F.fmt(*ty, 15 - sh)
+    x, w = rand_codes(rng, (N, H, H, C), 8, 0), rng.integers(-3, 4, size=(K, R, R, C))
+    x[0, :4] = 255
+    w[0], w[1] = 0, 0
+    w[0].reshape(-1)[:515], w[1].reshape(-1)[:516] = 127, -127  # up to 2^24 - 40000
+    w[2] = 0
+    w[2, 1, 1, 0] = 1 << min(max(sh - 1, 0), 6)                 # ties of x 2^(sh - 1)
+    b = rand_codes(rng, (K,), 16, 1)
+    b[2], b[3] = 0, 1
+    l1 = int(np.abs(w).reshape(K, -1).sum(axis=1).max())
+    assert 255 * l1 < 1 << 24
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, 1, 1, relu, 0, fy)
+    old = os.environ["FXPQ_CONV_PATH"]
+    for path in (old, "tc_iepi"):
+        os.environ["FXPQ_CONV_PATH"] = path
+        try:
+            got, s = run_conv(F, x, fx, w, fw, b, fb, 1, 1, relu, 0, fy, C, l1)
+        finally:
+            os.environ["FXPQ_CONV_PATH"] = old
+        assert s == ws and np.array_equal(got, want), path
+
+
+@pytest.mark.parametrize("sh", [16, 17, 20, 24])
+@pytest.mark.parametrize("relu,ty", [(True, (8, 0)), (False, (6, 1))])
+def test_window_fp32_epilogue_ties(F, sh, relu, ty):
+    """Two-limb window layers: sums on and next to rounding ties (one unit of 2^-30 of the output step away) are
+    decided by the exact arithmetic behind the fp32 one."""
+    if os.environ.get("FXPQ_CONV_PATH") != "tc":
+        pytest.skip("an epilogue of the default tensor-core path")
+    rng = np.random.default_rng(sh)
+    N, H, C, K = 1, 16, 3, 64
+    x = rng.integers(-32768, 32768, size=(N, H, H, C))
+    w = np.zeros((K, 3, 3, C), np.int64)
+    w[: K // 2] = rng.integers(-300, 300, size=(K // 2, 3, 3, C))
+    w[K // 2:, 1, 1, 0] = 1 << (sh - 9)
+    x[..., 0] = 256 * rng.integers(-100, 100, size=x.shape[:3])
+    x[0, ::2, :, 0] += 1  # just above the ties of the even rows
+    fx, fw, fb, fy = F.fmt(16, 1, 12), F.fmt(16, 1, 14), F.fmt(16, 1, 26), F.fmt(*ty, 26 - sh)
+    b = rng.integers(-200, 200, size=K)
+    b[K // 2:] = 0
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, 1, 1, relu, 0, fy)
+    for path in ("tc", "tc_win32"):
+        os.environ["FXPQ_CONV_PATH"] = path
+        try:
+            got, s = run_conv(F, x, fx, w, fw, b, fb, 1, 1, relu, 0, fy, 8)
+        finally:
+            os.environ["FXPQ_CONV_PATH"] = "tc"
+        assert s == ws and np.array_equal(got, want), path
+
+
 def test_code_l1max(F):
     """max over rows of sum |code| on one-plane fp16 codes, against numpy; the zero-row case."""
     rng = np.random.default_rng(11)
