@@ -174,27 +174,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// The non-blocking probe, for the thread that issues the MMAs: a try_wait there stalls the issuing
-// thread until its queued MMAs have drained (about 230 cycles per k-block of four 128-column MMAs, half
-// the tensor rate), a test_wait costs about 45.
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// The copy- and MMA-issuing instructions below are executed by a whole, converged warp and carry their own
+// elect.sync predicate: one (always the same) lane issues.  The operands then stay in uniform registers and
+// the loops around them in uniform control flow.  Issued from a branch of one thread instead, every operand
+// was moved there per instruction: 44 cycles per MMA and about 230 more after each barrier probe (four
+// M = 128, N = 128 MMAs, a commit and a wait: 472 cycles, 256 in this form, the tensor core's own rate), and
+// about 1300 cycles per pair of tensor copies.
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes) : "memory");
 }
 
 // 2-D tiled TMA store from shared memory (bulk-group completion).
@@ -221,8 +214,9 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, int x, int 
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
                                             int c4, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5, %6}], [%7];" ::"r"(dst),
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5, %6}], [%7];\n\t}" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
         : "memory");
 }
@@ -231,8 +225,9 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
                                             uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5}], [%6];" ::"r"(dst),
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5}], [%6];\n\t}" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
         : "memory");
 }
@@ -254,8 +249,9 @@ __device__ __forceinline__ long long tile_row(const TcParams& P, int tm, int i) 
 // 3-D tiled TMA load (coordinates innermost first) completing on mbarrier `bar`.
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];" ::"r"(dst),
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];\n\t}" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
 }
@@ -263,9 +259,11 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 // 1-D bulk copy global -> shared completing on mbarrier `bar` (both addresses 16-byte aligned, bytes a
 // multiple of 16).
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(bar)
+        : "memory");
 }
 
 // Bit-plane bytes -> fp16 codes.  (lo, hi): an 8 x 8 bit matrix, byte b = plane b (bytes 0-3 in lo,
@@ -343,12 +341,9 @@ __device__ __forceinline__ void pk_convert_stage(const uint32_t* pk, unsigned ch
 
 // Bounded wait for the phase of `bar` with the given parity.  Returns false (and latches the
 // timeout status, sets the CTA abort flag) if it gave up or another role already aborted.
-// TEST: the first probe does not block (the MMA-issuing thread's fast path); the retries suspend in
-// try_wait rather than spin, which would take issue slots from the epilogue warps.
-template <bool TEST = false>
 __device__ __forceinline__ bool wait_bounded_for(uint32_t bar, uint32_t parity, volatile int* abort, int* status,
                                                  long long limit) {
-    if (TEST ? mbar_test_wait(bar, parity) : mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (true) {
         if (mbar_try_wait(bar, parity)) return true;
@@ -364,9 +359,20 @@ __device__ __forceinline__ bool wait_bounded_for(uint32_t bar, uint32_t parity, 
 __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
     return wait_bounded_for(bar, parity, abort, status, TC_WAIT_CYCLES);
 }
-// the same for the MMA-issuing thread (a non-blocking first probe)
-__device__ __forceinline__ bool wait_mma(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
-    return wait_bounded_for<true>(bar, parity, abort, status, TC_WAIT_CYCLES);
+// The same for a whole converged warp (the MMA- and copy-issuing ones); the result is uniform by votes, which
+// keeps the caller's control flow uniform.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort, int* status) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    while (true) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, *abort)) return false;
+        if (__any_sync(0xffffffffu, clock64() - t0 > TC_WAIT_CYCLES)) {
+            *abort = 1;
+            latch_status(status, FXPQ_ERR_TIMEOUT);
+            return false;
+        }
+    }
 }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
@@ -415,16 +421,18 @@ __host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
 __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                        uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        : "memory");
 }
 
 // Loads / stores without their completion wait, so that several TMEM accesses share one round trip.
@@ -784,7 +792,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     const uint32_t pkfull0 = smem_u32(bars + 2 * TC_STAGES + 10);
     unsigned char* sP = sO;  // PK: packed stages of BN * 64 bytes (k <= 8 words per 32 codes)
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // warp: uniform
     const ConvArgs& a = P.a;
 
     if (threadIdx.x == 0) {
@@ -838,7 +846,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         // window of the 16 x 8 patch shifted by s pixels, TH + R - 1 rows of 8 pixels of 64 channels (one
         // swizzle pattern per row, padding zero filled), is one box into window slot (tile count mod 2):
         // every tap's A operand then starts on a pattern boundary.
-        if (threadIdx.x == 0) {
+        if (warp == 0) {
             mbar_arrive_expect_tx(wbar, (uint32_t)(a.R * a.S) * 8192u);
             for (int t = 0; t < a.R * a.S; ++t)
                 tma_load_3d(smem_u32(sA) + (uint32_t)t * 8192u, &P.tmap_w, t * TC_BK, 0, 0, wbar);
@@ -849,7 +857,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
             for (int t = blockIdx.x; t < P.n_tiles && ok; t += gridDim.x) {
                 const int n_img = t / per_img, r = t - n_img * per_img;
                 const int hp0 = (r / P.tiles_q) * P.TH - a.pad, wq0 = (r % P.tiles_q) * P.TW - a.pad;
-                if (!wait_bounded(empty0 + 8 * stage, phase ^ 1, abort, P.status)) {
+                if (!wait_warp(empty0 + 8 * stage, phase ^ 1, abort, P.status)) {
                     ok = false;
                     break;
                 }
@@ -881,7 +889,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         // one box {8 ch, BN out ch} per tap and plane, taps past S zero filled); per tile, one box per
         // x limb plane holds the input window of TH + R - 1 rows by TW + S2 - 1 pixels (padding zero
         // filled).
-        if (threadIdx.x == 0) {
+        if (warp == 0) {
             const int np = P.S2 / 2;
             const uint32_t tapb = (uint32_t)(BN * 16);  // one tap of one plane
             mbar_arrive_expect_tx(wbar, (uint32_t)(a.pw * a.R * np * 2) * tapb);
@@ -900,7 +908,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 const int tm = t / P.tiles_n;
                 const int n_img = tm / per_img, r = tm - n_img * per_img;
                 const int hp0 = (r / P.tiles_q) * P.TH - a.pad, wq0 = (r % P.tiles_q) * P.TW - a.pad;
-                if (!wait_bounded(empty0 + 8 * stage, phase ^ 1, abort, P.status)) {
+                if (!wait_warp(empty0 + 8 * stage, phase ^ 1, abort, P.status)) {
                     ok = false;
                     break;
                 }
@@ -935,7 +943,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         // Cp == 8: a k-block is 8 taps of 8 channels; tap tl's box {8, TW, TH} lands at byte
         // 2048 tl of the stage (a 16-byte K column of the no-swizzle layout), and taps past R*S
         // are boxes wholly outside the tensor (zero filled).
-        if (lane == 0 && warp < TC_PRODUCERS) {
+        if (warp < TC_PRODUCERS) {
             // k-block it goes to producer (it % TC_STAGES) % TC_PRODUCERS: one thread's latency per k-block
             // (barrier wait, two TMA instructions) would bound the stage rate
             const int me = warp;
@@ -961,7 +969,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
                         if ((int)((it % TC_STAGES) % TC_PRODUCERS) == me) {
                             const uint32_t stage = it % TC_STAGES, phase = (it / TC_STAGES) & 1;
-                            if (!wait_bounded(empty0 + 8 * stage, phase ^ 1, abort, P.status)) {
+                            if (!wait_warp(empty0 + 8 * stage, phase ^ 1, abort, P.status)) {
                                 ok = false;
                                 break;
                             }
@@ -1048,12 +1056,13 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 for (int kb = g.kb0; kb < g.kb1; ++kb) {
                     const int stage = it % TC_STAGES;
                     const uint32_t ph = (it / TC_STAGES) & 1;
-                    if (!wait_bounded(empty0 + 8 * stage, ph ^ 1, abort, P.status)) {
+                    if (!wait_warp(empty0 + 8 * stage, ph ^ 1, abort, P.status)) {
                         ok = false;
                         break;
                     }
                     const uint32_t dA = smem_u32(sA + stage * A_BYTES);
-                    if (threadIdx.x == 0) {  // the weight tile: one TMA, zero-filled past K and R*S*Cp
+                    if (warp == 0) {  // the weight tile: one TMA, zero-filled past K and R*S*Cp
+                        __syncwarp();
                         mbar_arrive_expect_tx(full0 + 8 * stage, (uint32_t)B_BYTES);
                         tma_load_3d(smem_u32(sB + stage * B_BYTES), &P.tmap_w, kb * TC_BK, tn * BN, g.w_plane,
                                     full0 + 8 * stage);
@@ -1747,19 +1756,19 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     } else if (PK && warp > MMA_WARP) {
         // ============================================================ packed-weight converters
         pk_convert_loop<BN, SPLIT>(P, 3 + (warp - MMA_WARP - 1), lane, sP, sB, pkfull0, full0, abort);
-    } else if (!WIN && lane == 0 && P.patch == 4) {
+    } else if (!WIN && P.patch == 4) {
         // ============================================================ MMA issue, 64-channel window mode
         // Per tile, tap (r, s) and 16-channel step kk: one MMA.  A is window copy s from row r: rows 128
         // bytes apart, the 8-row groups (patch rows, TW = 8) one pattern (1 KiB) apart; B the resident tap
         // block (a B stage's layout).  One barrier round per tile.
         const uint32_t copyb = (uint32_t)P.WH * 1024u;
         uint32_t stage = 0, phase = 0, gcount = 0;
-        bool ok = wait_mma(wbar, 0, abort, P.status);
+        bool ok = wait_warp(wbar, 0, abort, P.status);
         tc_fence_after();
         for (int t = blockIdx.x; t < P.n_tiles && ok; t += gridDim.x) {
             const uint32_t buf = gcount & 1;
-            if (!wait_mma(accempty0 + 8 * buf, ((gcount >> 1) & 1) ^ 1, abort, P.status) ||
-                !wait_mma(full0 + 8 * stage, phase, abort, P.status)) {
+            if (!wait_warp(accempty0 + 8 * buf, ((gcount >> 1) & 1) ^ 1, abort, P.status) ||
+                !wait_warp(full0 + 8 * stage, phase, abort, P.status)) {
                 ok = false;
                 break;
             }
@@ -1790,7 +1799,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         const long long t0 = clock64();
         while (!mbar_try_wait(done_bar, 0) && clock64() - t0 < TC_WAIT_CYCLES) {
         }
-    } else if (!W64 && lane == 0 && P.patch == 3) {
+    } else if (!W64 && P.patch == 3) {
         // ============================================================ MMA issue, window mode
         // Per tile and limb pair (ia, iw): R * S2/2 MMAs of K = 16 (two taps of 8 channels).  The A
         // operand of taps (r, 2sp), (r, 2sp + 1) is the window shifted by (r, 2sp) pixels: K-major
@@ -1810,14 +1819,14 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
             aoff[i] = (uint32_t)((r * P.WW + 2 * sp) * 16) >> 4;
         }
         uint32_t stage = 0, phase = 0, gcount = 0;
-        bool ok = wait_mma(wbar, 0, abort, P.status);
+        bool ok = wait_warp(wbar, 0, abort, P.status);
         tc_fence_after();
         for (int ut = blockIdx.x; ut < (SPLIT ? P.n_units : P.n_tiles) && ok; ut += gridDim.x) {
             const int t = SPLIT ? ut / P.ksplit : ut, sp = SPLIT ? ut - t * P.ksplit : 0;
             (void)sp;
             const uint32_t buf = gcount & 1;
-            if (!wait_mma(accempty0 + 8 * buf, ((gcount >> 1) & 1) ^ 1, abort, P.status) ||
-                !wait_mma(full0 + 8 * stage, phase, abort, P.status)) {
+            if (!wait_warp(accempty0 + 8 * buf, ((gcount >> 1) & 1) ^ 1, abort, P.status) ||
+                !wait_warp(full0 + 8 * stage, phase, abort, P.status)) {
                 ok = false;
                 break;
             }
@@ -1846,8 +1855,8 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         const long long t0 = clock64();
         while (!mbar_try_wait(done_bar, 0) && clock64() - t0 < TC_WAIT_CYCLES) {
         }
-    } else if (!WEPI && lane == 0) {
-        // ============================================================ MMA issue (one thread of MMA_WARP)
+    } else if (!WEPI) {
+        // ============================================================ MMA issue (MMA_WARP, one elected lane)
         // Descriptors of stage 0; a stage or a 16-element k step moves the start-address field
         // (address >> 4, 14 bits) without carry since shared addresses stay below 256 KB.
         // 8-channel patch tiles: no-swizzle A, one 16-element k step = two taps = 4096 bytes
@@ -1864,7 +1873,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 const TcGroup g = P.g[gi];
                 const uint32_t buf = P.nbuf == 2 ? (gcount & 1) : 0;
                 const uint32_t par = P.nbuf == 2 ? ((gcount >> 1) & 1) : (gcount & 1);
-                if (!wait_mma(accempty0 + 8 * buf, par ^ 1, abort, P.status)) {
+                if (!wait_warp(accempty0 + 8 * buf, par ^ 1, abort, P.status)) {
                     ok = false;
                     break;
                 }
@@ -1872,7 +1881,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 const uint32_t d = tmem + buf * BN;
                 uint32_t accum = 0;
                 for (int kb = g.kb0; kb < g.kb1; ++kb) {
-                    if (!wait_mma(full0 + 8 * stage, phase, abort, P.status)) {
+                    if (!wait_warp(full0 + 8 * stage, phase, abort, P.status)) {
                         ok = false;
                         break;
                     }
