@@ -48,12 +48,40 @@ long long limb_max(const fxpq_fmt& f, int plane) {
 
 }  // namespace
 
-// Builds the group table; returns false if the tensor-core path cannot keep the sums exact.
-bool plan_tc(const ConvArgs& a, const fxpq_conv_desc& d, TcParams& P, bool& acc64) {
+// Patch shape of a layer's output: TW x TH pixels of TN images, at most 128, with the fewest tiles (a 7 x 7 map
+// of 128 images takes 49 tiles like its 6272 rows do, not 128).  Only widths and heights that divide the map
+// into equal counts matter; among equals the fewest images and the widest rows.
+struct PatchShape {
+    int TW = 0, TH = 0, TN = 0;
+    long long tiles = 0;
+};
+static PatchShape patch_shape(const ConvArgs& a, int max_tn) {
+    PatchShape s;
+    const long long ideal = (a.M + TC_BM - 1) / TC_BM;
+    const int span = (256 - 1) / a.stride + 1;  // a TMA box spans at most 256 input positions
+    for (int i = 1, tw = 0; i <= a.Q; ++i) {
+        const int w = (a.Q + i - 1) / i;
+        if (w == tw || w > TC_BM || w > span) continue;
+        tw = w;
+        for (int j = 1, th = 0; j <= a.P; ++j) {
+            const int h = (a.P + j - 1) / j;
+            if (h == th || (long long)h * tw > TC_BM || h > span) continue;
+            th = h;
+            int tn = TC_BM / (th * tw);
+            if (tn > a.N) tn = a.N;
+            if (tn > max_tn) tn = max_tn;
+            const long long t = (long long)((a.N + tn - 1) / tn) * ((a.P + th - 1) / th) * ((a.Q + tw - 1) / tw);
+            if (s.TW == 0 || t < s.tiles || (t == s.tiles && tn < s.TN)) s.TW = tw, s.TH = th, s.TN = tn, s.tiles = t;
+            if (s.tiles == ideal && s.TN == 1) return s;
+        }
+    }
+    return s;
+}
+
+// Builds the group table over n_kb k-blocks; returns false if the tensor-core path cannot keep the sums exact.
+bool plan_tc(const ConvArgs& a, const fxpq_conv_desc& d, TcParams& P, bool& acc64, int n_kb) {
     P.a = a;
     P.RSC = a.R * a.S * a.Cp;
-    const int n_kb = (P.RSC + TC_BK - 1) / TC_BK;
-    P.cp64 = (a.Cp % TC_BK) == 0;
     const int pa = planes_of(d.fmt_x), pw = planes_of(d.fmt_w);
     int ng = 0;
     bool shifted = false;
@@ -113,12 +141,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     launched = false;
     TcParams P;
     bool acc64 = false;
-    if (!plan_tc(a, d, P, acc64)) return FXPQ_OK;
     const int sms = num_sms();
-    // 64-column tiles for int64 sums and for layers with at most 64 output channels; 256-column tiles
-    // (one MMA instruction covers twice the work of a 128-column one, which hides its issue cost) for
-    // wide layers with enough tiles
-    int BN = 128;
     const long long row_tiles_est = (a.M + TC_BM - 1) / TC_BM;
     // Layers whose im2col matrix is the stored activations themselves: 1x1 stride-1 convolutions
     // without padding ([M][Cp] per plane) and kernels covering the whole unpadded map (P = Q = 1,
@@ -127,16 +150,42 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     const bool whole_map = a.R == a.H && a.S == a.W && a.pad == 0 && a.P == 1 && a.Q == 1;
     const bool rows_geom = (one_by_one || whole_map) && a.M > 0 && a.M < (1LL << 31) - TC_BM &&
                            !conv_path_is("tc_rows") && !conv_path_is("tc_patch");
+    // Patch tiles for every other layer whose stride a TMA box can traverse and whose channel count fills its
+    // 64-channel blocks well enough: up to four times the k-blocks of the flattened reduction of the
+    // gathered row tiles, which take about six times as long per k-block (2600 cycles against 410; a 7 x 7
+    // 512-channel layer of 128 images 95 us gathered, 31 us as patches); 8-channel stride-1 inputs take boxes
+    // of one tap each (narrow)
+    const bool narrow = a.Cp == 8;
+    PatchShape ps;
+    if (!rows_geom && a.P > 0 && a.Q > 0 && a.N > 0 && a.stride <= (narrow ? 1 : 8) && !conv_path_is("tc_rows"))
+        ps = patch_shape(a, TC_BM);
+    const int kbt = (a.Cp + TC_BK - 1) / TC_BK;
+    const int kb_flat = (a.R * a.S * a.Cp + TC_BK - 1) / TC_BK;
+    const bool use_patch = ps.TW > 0 && (narrow || conv_path_is("tc_patch") ||
+                                         (double)ps.tiles * a.R * a.S * kbt <= 4.0 * (double)row_tiles_est * kb_flat);
+    P.kbt = kbt;
+    if (!plan_tc(a, d, P, acc64, use_patch && !narrow ? a.R * a.S * kbt : kb_flat)) return FXPQ_OK;
     // ... with few row tiles (FC layers at small batches) they take 256-column tiles and a split
     // reduction fills the SMs: the MMA thread's fixed cost per k-block is then hidden, and the weights
     // stream at the memory's rate
     const bool wide_split = rows_geom && !acc64 && !a.has_scale && ws && a.K > 128 && !conv_path_is("tc_bn128") &&
                             !conv_path_is("tc_nosplit") && row_tiles_est * ((a.K + 255) / 256) * 2 <= sms;
-    if (acc64 || a.K <= 64)
+    // Tile width: 64 columns for int64 sums and at most 64 output channels, else the width whose whole rounds
+    // over the SMs take the fewest cycles.  A k-block costs what its stage takes from L2 at about 80 bytes
+    // per cycle and SM (24, 32 and 48 KB: 300, 410 and 615 cycles; the MMAs 228, 256 and 512); a 256-column
+    // tile of several exact groups has one accumulator buffer, whose drain is not hidden.
+    const long long tiles_m_est = use_patch ? ps.tiles : row_tiles_est;
+    int BN = 64;
+    if (acc64 || a.K <= 64) {
         BN = 64;
-    else if (wide_split || (a.K > 128 && !conv_path_is("tc_bn128") &&
-                            (conv_path_is("tc_bn256") || (a.K % 256 == 0 && row_tiles_est * (a.K / 256) >= sms))))
+    } else if (wide_split || (a.K > 128 && conv_path_is("tc_bn256"))) {
         BN = 256;
+    } else {
+        auto rounds = [&](int bn) { return (double)((tiles_m_est * ((a.K + bn - 1) / bn) + sms - 1) / sms); };
+        const double c64 = rounds(64) * 300, c128 = rounds(128) * 410, c256 = rounds(256) * (P.n_groups > 1 ? 1100 : 615);
+        BN = c128 <= c64 ? 128 : 64;
+        if (a.K > 128 && !conv_path_is("tc_bn128") && c256 <= (BN == 128 ? c128 : c64)) BN = 256;
+    }
     // packed k-bit weights (k <= 8, one plane) are read by the 256-column TMA-row instances of the
     // split (FC) layers, whose weights stream through once; elsewhere every weight tile is expanded
     // once per row tile and the fp16 codes are read instead
@@ -146,9 +195,6 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     P.wk = d.fmt_w.bits;
     P.wsigned = d.fmt_w.is_signed;
     P.K_pad = (a.K + 255) / 256 * 256;
-    // too few 128-column tiles to occupy every SM (small batches, FC layers): 64-column tiles double
-    // the CTA count
-    if (BN == 128 && row_tiles_est * ((a.K + 127) / 128) < sms) BN = 64;
     // BN = 256 fills TMEM with two accumulator buffers; with several exact groups per tile it keeps one
     // buffer and the integer running sums
     P.nbuf = (BN == 256 && P.n_groups > 1) ? 1 : 2;
@@ -169,6 +215,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         P.wf32 = 0;
         P.win_eps = P.win_c[0] = P.win_c[1] = P.win_c[2] = 0.0f;
         P.nacc = 1;
+        P.TN = 1;
         // window mode for 8-channel stride-1 layers with at most 64 output channels: 8 x 16 output
         // patches, one input window per tile and limb plane, weights resident in shared memory, one
         // exact fp32 accumulator per limb pair (R * S2 * 8 products each)
@@ -300,42 +347,24 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
                 P.rows_tma = 1;
         }
-        // patch tiles for stride-1 layers whose taps are whole 64-channel blocks, or 8-channel inputs
-        // (a k-block of 8 taps)
-        const bool narrow = a.Cp == 8;
-        if (P.patch == 0 && !P.rows_tma && a.stride == 1 && (P.cp64 || narrow) && a.P > 0 && a.Q > 0 && a.N > 0 &&
-            !conv_path_is("tc_rows")) {
-            int best_tw = 0, best_th = 0;
-            long long best = 0;
-            for (int tw = a.Q < TC_BM ? a.Q : TC_BM; tw >= 1; --tw) {
-                const int th = TC_BM / tw < a.P ? TC_BM / tw : a.P;
-                const long long cost = (long long)((a.P + th - 1) / th) * ((a.Q + tw - 1) / tw);
-                if (best_tw == 0 || cost < best) best = cost, best_tw = tw, best_th = th;
-            }
-            // take patches unless they need more than twice as many tiles as 128-row tiles of N*P*Q:
-            // one TMA box per k-block against 128 gathered rows pays for a good deal of idle MMA rows
-            // (3x3 layers, 14x14 maps: 2 patches of 126 rows per image, 1.3x the row tiles, 1.7-2x
-            // faster; 7x7 maps: 2.6x the row tiles, 6% slower)
-            const long long row_tiles = (a.M + TC_BM - 1) / TC_BM;
-            if ((double)a.N * best <= 2.0 * (double)row_tiles + 1e-9 || conv_path_is("tc_patch")) {
-                const cuuint64_t xdims[5] = {(cuuint64_t)a.Cp, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.N,
-                                             (cuuint64_t)a.px};
-                const cuuint64_t xstrides[4] = {(cuuint64_t)a.Cp * 2, (cuuint64_t)a.W * a.Cp * 2,
-                                                (cuuint64_t)a.H * a.W * a.Cp * 2, (cuuint64_t)a.x_ps * 2};
-                const cuuint32_t xbox[5] = {(cuuint32_t)(narrow ? 8 : TC_BK), (cuuint32_t)best_tw,
-                                            (cuuint32_t)best_th, 1, 1};
-                const cuuint32_t es5[5] = {1, 1, 1, 1, 1};
-                if (enc(&P.tmap_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, const_cast<__half*>(a.x), xdims, xstrides,
-                        xbox, es5, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        narrow ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
-                    P.patch = narrow ? 2 : 1;
-                    P.TW = best_tw;
-                    P.TH = best_th;
-                    P.tiles_p = (a.P + best_th - 1) / best_th;
-                    P.tiles_q = (a.Q + best_tw - 1) / best_tw;
-                }
-            }
+        if (P.patch == 0 && !P.rows_tma && use_patch) {
+            const cuuint64_t xdims[5] = {(cuuint64_t)a.Cp, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.N, (cuuint64_t)a.px};
+            const cuuint64_t xstrides[4] = {(cuuint64_t)a.Cp * 2, (cuuint64_t)a.W * a.Cp * 2,
+                                            (cuuint64_t)a.H * a.W * a.Cp * 2, (cuuint64_t)a.x_ps * 2};
+            const cuuint32_t st = (cuuint32_t)a.stride;
+            const cuuint32_t xbox[5] = {(cuuint32_t)(narrow ? 8 : TC_BK), (ps.TW - 1) * st + 1, (ps.TH - 1) * st + 1,
+                                        (cuuint32_t)ps.TN, 1};
+            const cuuint32_t es5[5] = {1, st, st, 1, 1};
+            if (enc(&P.tmap_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, const_cast<__half*>(a.x), xdims, xstrides, xbox, es5,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, narrow ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                return FXPQ_OK;  // the groups are in patch order: the CUDA-core kernel runs instead
+            P.patch = narrow ? 2 : 1;
+            P.TW = ps.TW;
+            P.TH = ps.TH;
+            P.TN = ps.TN;
+            P.tiles_p = (a.P + ps.TH - 1) / ps.TH;
+            P.tiles_q = (a.Q + ps.TW - 1) / ps.TW;
         }
         if (!P.rows_tma) P.pk = 0;
         if (P.w32 && !(a.out_mode == FXPQ_OUT_CODES && a.py == 1)) P.w32 = 0;
@@ -349,7 +378,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
                 const cuuint64_t ydims[4] = {(cuuint64_t)a.K, (cuuint64_t)a.Q, (cuuint64_t)a.P, (cuuint64_t)a.N};
                 const cuuint64_t ystrides[3] = {(cuuint64_t)a.K * 2, (cuuint64_t)a.Q * a.K * 2,
                                                 (cuuint64_t)a.P * a.Q * a.K * 2};
-                const cuuint32_t ybox[4] = {64, (cuuint32_t)P.TW, (cuuint32_t)P.TH, 1};
+                const cuuint32_t ybox[4] = {64, (cuuint32_t)P.TW, (cuuint32_t)P.TH, (cuuint32_t)P.TN};
                 const cuuint32_t es4[4] = {1, 1, 1, 1};
                 r = enc(&P.tmap_y, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, a.y, ydims, ystrides, ybox, es4,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
@@ -366,7 +395,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         }
         if (!P.fast_store) P.w32 = 0;  // the 32-bit window epilogue writes through the staging tile
     }
-    P.tiles_m = P.patch ? a.N * P.tiles_p * P.tiles_q : (int)((a.M + TC_BM - 1) / TC_BM);
+    P.tiles_m = P.patch ? (a.N + P.TN - 1) / P.TN * P.tiles_p * P.tiles_q : (int)((a.M + TC_BM - 1) / TC_BM);
     P.tiles_n = (a.K + BN - 1) / BN;
     P.n_tiles = P.tiles_m * P.tiles_n;
     if (P.n_tiles == 0) {

@@ -16,9 +16,9 @@
 //              (BN channels x 64 taps) always comes by TMA.  The A tile takes one of two forms:
 //              row tiles (128 consecutive output pixels): cp.async gather by 128 threads, with
 //              zero fill for padding and ragged edges;
-//              patch tiles (stride 1, Cp % 64 == 0): a TH x TW patch of output pixels of one
-//              image, whose input window for one tap and 64 channels is a single 5-D TMA box
-//              (the hardware zero-fills the padding); one thread issues both copies.
+//              patch tiles: a TH x TW patch of output pixels of TN images, whose inputs for one tap
+//              and 64 channels are a single 5-D TMA box, strided like the convolution (the
+//              hardware zero-fills the padding); one warp issues both copies.
 //   warp  4-7  epilogue: drain TMEM (tcgen05.ld), integer running sums, final bias / ReLU /
 //              FxP-QLayer (shared with the CUDA-core kernel).
 //   warp  8    TMEM allocation and the single MMA-issuing thread.
@@ -107,8 +107,8 @@ struct TcParams {
                          // [planes][N][H][W * 8], box {8 WW, WH, 1, 1} (a window row is one 16 WW-byte run)
     int fast_store;      // 1: one-plane codes staged in shared memory and written by TMA stores
     int nbuf;            // fp32 accumulator buffers in TMEM: 2, or 1 when BN = 256 needs running sums
-    int patch;           // a tile is a TH x TW patch of one image and the A tile comes by TMA:
-                         // 1: Cp % 64 == 0 (one 64-channel box per k-block, 128-byte swizzle);
+    int patch;           // a tile is a TH x TW patch of TN images and the A tile comes by TMA:
+                         // 1: one 64-channel box per k-block (128-byte swizzle), kbt k-blocks per tap;
                          // 2: Cp == 8 (one 8-channel box per tap, 8 taps per k-block, no swizzle);
                          // 3: Cp == 8, window mode (one input window per tile and limb plane, taps as
                          //    shifted descriptors, weights resident in shared memory)
@@ -130,8 +130,9 @@ struct TcParams {
     int win_bytes;       // window mode: bytes of one window (128-byte aligned; patch 4: 16-byte aligned)
     int w64_slot0;       // patch 4: offset of window slot 0 (after the resident weights)
     int w64_slot_stride; // bytes between the two window slots (S copies of WH KiB)
-    int TH, TW;          // patch shape (TH * TW = 128)
+    int TH, TW, TN;      // patch shape: TH x TW pixels of TN images (TH * TW * TN <= 128)
     int tiles_p, tiles_q;  // patches per image along P and Q
+    int kbt;             // patch 1: k-blocks per tap (the 64-channel blocks of Cp, the last one zero filled)
     ConvArgs a;
     int RSC;       // R * S * Cp: reduction length of one plane
     int tiles_m, tiles_n, n_tiles;
@@ -143,7 +144,6 @@ struct TcParams {
     int ksplit, n_units;
     int gs[TC_MAX_SPLIT + 1];
     void* part;
-    int cp64;      // Cp % 64 == 0: a k-block never straddles a tap
     // Packed weights (pk = 1, one plane of wk <= 8 bits, wsigned): fxpq_pack_weights' tiles, words
     // [ceil(R*S*Cp / 64)][K_pad / 256][wk][256][2]: word (kb, t, b, o, h) bit i = bit b of code
     // 64 kb + 32 h + i of output channel 256 t + o.
@@ -238,11 +238,12 @@ __device__ __forceinline__ long long tile_row(const TcParams& P, int tm, int i) 
         const long long m = (long long)tm * 128 + i;
         return m < P.a.M ? m : -1;
     }
-    if (i >= P.TH * P.TW) return -1;
-    const int per_img = P.tiles_p * P.tiles_q;
-    const int n = tm / per_img, r = tm - n * per_img;
-    const int p = (r / P.tiles_q) * P.TH + i / P.TW, q = (r % P.tiles_q) * P.TW + i % P.TW;
-    if (p >= P.a.P || q >= P.a.Q) return -1;
+    const int per_img = P.tiles_p * P.tiles_q, pix = P.TH * P.TW;
+    const int ti = i / pix, j = i - ti * pix;
+    if (ti >= P.TN) return -1;
+    const int ng = tm / per_img, r = tm - ng * per_img, n = ng * P.TN + ti;
+    const int p = (r / P.tiles_q) * P.TH + j / P.TW, q = (r % P.tiles_q) * P.TW + j % P.TW;
+    if (n >= P.a.N || p >= P.a.P || q >= P.a.Q) return -1;
     return ((long long)n * P.a.P + p) * P.a.Q + q;
 }
 
@@ -938,8 +939,10 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         }
     } else if (!WEPI && warp < 4 && (P.patch || P.rows_tma)) {
         // ============================================================ producer, patch tiles
-        // Stride 1 and Cp % 64 == 0: the A tile of tap (r, s) and channels c0..c0+63 is the box
-        // {64, TW, TH} of the input at (c0, q0 + s - pad, p0 + r - pad); the padding reads as zeros.
+        // The A tile of tap (r, s) and channels c0..c0+63 is the box {64, TW, TH, TN} of the input at
+        // (c0, q0 st + s - pad, p0 st + r - pad, n0), traversed with the convolution's stride; the padding
+        // and channels past Cp read as zeros, so that the weight columns of the next tap, which the B box
+        // then holds in their place, count for nothing.
         // Cp == 8: a k-block is 8 taps of 8 channels; tap tl's box {8, TW, TH} lands at byte
         // 2048 tl of the stage (a 16-byte K column of the no-swizzle layout), and taps past R*S
         // are boxes wholly outside the tensor (zero filled).
@@ -948,7 +951,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
             // (barrier wait, two TMA instructions) would bound the stage rate
             const int me = warp;
             const bool narrow = P.patch == 2;
-            const uint32_t a_bytes = P.rows_tma ? (uint32_t)(TC_BM * 128) : (uint32_t)(P.TH * P.TW * (narrow ? 8 * 16 : 128));
+            const uint32_t a_bytes = P.rows_tma ? (uint32_t)(TC_BM * 128) : (uint32_t)(P.TH * P.TW * P.TN * (narrow ? 8 * 16 : 128));
             const int per_img = P.rows_tma ? 1 : P.tiles_p * P.tiles_q;
             uint32_t it = 0;
             bool ok = true;
@@ -956,16 +959,17 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 const int t = SPLIT ? ut / P.ksplit : ut, sp = SPLIT ? ut - t * P.ksplit : 0;
                 (void)sp;
                 const int tm = t / P.tiles_n, tn = t % P.tiles_n;
-                const int n_img = tm / per_img, r = tm - n_img * per_img;
+                const int ng = tm / per_img, r = tm - ng * per_img, n_img = ng * P.TN;
                 const int tq = P.rows_tma ? 1 : P.tiles_q;
-                const int hp0 = (r / tq) * P.TH - a.pad, wq0 = (r % tq) * P.TW - a.pad;
+                const int hp0 = (r / tq) * P.TH * a.stride - a.pad, wq0 = (r % tq) * P.TW * a.stride - a.pad;
                 for (int gi = SPLIT ? P.gs[sp] : 0; gi < (SPLIT ? P.gs[sp + 1] : P.n_groups) && ok; ++gi) {
                     const TcGroup g = P.g[gi];
                     // tap (rr, ss) and channel offset cc of the group's first k-block, then stepped by
-                    // TC_BK channels (Cp % 64 == 0: a k-block never straddles a tap)
-                    const int tp0 = g.kb0 * TC_BK / a.Cp;
-                    int cc = g.kb0 * TC_BK - tp0 * a.Cp;
+                    // TC_BK channels; wx: the weights' column
+                    const int tp0 = g.kb0 / P.kbt;
+                    int cc = (g.kb0 - tp0 * P.kbt) * TC_BK;
                     int rr = tp0 / a.S, ss = tp0 - rr * a.S;
+                    int wx = P.patch == 1 ? tp0 * a.Cp + cc : g.kb0 * TC_BK;
                     for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
                         if ((int)((it % TC_STAGES) % TC_PRODUCERS) == me) {
                             const uint32_t stage = it % TC_STAGES, phase = (it / TC_STAGES) & 1;
@@ -995,12 +999,13 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                                 bulk_load(smem_u32(sP + stage * (BN * 64)),
                                           P.wpack + ((size_t)kb * P.K_pad + (size_t)tn * BN) * 2 * P.wk, pk_bytes, fb);
                             else
-                                tma_load_3d(smem_u32(sB + stage * B_BYTES), &P.tmap_w, kb * TC_BK, tn * BN, g.w_plane,
-                                            fb);
+                                tma_load_3d(smem_u32(sB + stage * B_BYTES), &P.tmap_w, wx, tn * BN, g.w_plane, fb);
                         }
+                        wx += TC_BK;
                         if (!narrow) {
                             cc += TC_BK;
                             if (cc >= a.Cp) {
+                                if (P.patch == 1) wx += a.Cp - cc;  // the next tap's first column
                                 cc = 0;
                                 if (++ss == a.S) {
                                     ss = 0;
@@ -1737,7 +1742,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         }
                         if (P.patch) {
                             const int per_img = P.tiles_p * P.tiles_q;
-                            const int n_img = tm / per_img, r = tm - n_img * per_img;
+                            const int ng = tm / per_img, r = tm - ng * per_img, n_img = ng * P.TN;
                             for (int hb = 0; hb < BN / 64; ++hb)
                                 tma_store_4d(&P.tmap_y, tn * BN + hb * 64, (r % P.tiles_q) * P.TW,
                                              (r / P.tiles_q) * P.TH, n_img, smem_u32(sO + hb * (TC_BM * 128)));
@@ -1880,6 +1885,11 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 tc_fence_after();
                 const uint32_t d = tmem + buf * BN;
                 uint32_t accum = 0;
+                // patch 1: a tap's last channel block has ksteps 16-channel steps, the others (and every
+                // k-block of the other forms) four
+                int cb = P.patch == 1 ? g.kb0 % P.kbt : 0;
+                const int cb_last = P.patch == 1 ? P.kbt - 1 : -1;
+                const int ksteps = (a.Cp - (P.kbt - 1) * TC_BK + 15) / 16;
                 for (int kb = g.kb0; kb < g.kb1; ++kb) {
                     if (!wait_warp(full0 + 8 * stage, phase, abort, P.status)) {
                         ok = false;
@@ -1888,9 +1898,11 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     tc_fence_after();
                     const uint64_t ad = adesc0 + (uint64_t)((stage * A_BYTES) >> 4);
                     const uint64_t bd = bdesc0 + (uint64_t)((stage * B_BYTES) >> 4);
+                    const int ns = cb == cb_last ? ksteps : TC_BK / 16;
+                    if (++cb > cb_last) cb = 0;
 #pragma unroll
                     for (int kk = 0; kk < TC_BK / 16; ++kk) {
-                        tc_mma(d, ad + a_kstep * kk, bd + 2 * kk, IDESC, accum);
+                        if (kk < ns) tc_mma(d, ad + a_kstep * kk, bd + 2 * kk, IDESC, accum);
                         accum = 1;
                     }
                     tc_commit(empty0 + 8 * stage);
