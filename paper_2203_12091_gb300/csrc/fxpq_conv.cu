@@ -101,6 +101,68 @@ __global__ void __launch_bounds__(NT) conv_simt_kernel(ConvArgs a) {
     }
 }
 
+// Codes of a strided 8-channel layer to the space-to-depth form (S2dPlan): blocks [0, xb) one thread per pixel of
+// x2 and plane, the rest one thread per 8 weights.  HBM-bound (16 bytes read per pixel and plane, st st C2 / (8 C)
+// times less written): 128 224 x 224 images, stride 2, 60 us.
+__global__ void __launch_bounds__(256) s2d_kernel(const __half* __restrict__ x, const __half* __restrict__ w, int N, int H,
+                                                  int W, int K, int R, int S, int pad, long long x_ps, long long w_ps,
+                                                  S2dPlan p, int px, int pw, unsigned xb, uint4* __restrict__ x2,
+                                                  uint4* __restrict__ w2) {
+    const int c8 = p.C2 / 8;
+    if (blockIdx.x < xb) {
+        const long long npix = (long long)N * p.H2 * p.W2;
+        const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+        if (i >= npix * px) return;
+        const int pl = (int)(i / npix);
+        const long long pix = i - pl * npix;
+        const int n = (int)(pix / (p.H2 * p.W2)), r = (int)(pix - (long long)n * p.H2 * p.W2);
+        const int h0 = (r / p.W2) * p.st - pad, w0 = (r % p.W2) * p.st - pad;
+        const unsigned short* src = reinterpret_cast<const unsigned short*>(x) + pl * x_ps;
+        uint32_t o[4] = {0u, 0u, 0u, 0u};
+        int e = 0;  // codes gathered so far
+        for (int dy = 0; dy < p.st; ++dy)
+            for (int dx = 0; dx < p.st; ++dx) {
+                const int h = h0 + dy, ww = w0 + dx;
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if ((unsigned)h < (unsigned)H && (unsigned)ww < (unsigned)W)
+                    v = __ldg(reinterpret_cast<const uint4*>(src + (((long long)n * H + h) * W + ww) * 8));
+                const uint32_t q[4] = {v.x, v.y, v.z, v.w};
+                for (int c = 0; c < p.C; ++c, ++e) {
+                    const uint32_t code = (q[c >> 1] >> (16 * (c & 1))) & 0xFFFFu;
+                    const int s = e & 7;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (k == (s >> 1)) o[k] |= code << (16 * (s & 1));
+                    if (s == 7) {
+                        x2[i * c8 + (e >> 3)] = make_uint4(o[0], o[1], o[2], o[3]);
+                        o[0] = o[1] = o[2] = o[3] = 0u;
+                    }
+                }
+            }
+        if (e & 7) x2[i * c8 + (e >> 3)] = make_uint4(o[0], o[1], o[2], o[3]);
+    } else {
+        const long long n8 = (long long)K * p.R2 * p.S2 * c8;
+        const long long i = (long long)(blockIdx.x - xb) * 256 + threadIdx.x;
+        if (i >= n8 * pw) return;
+        const int pl = (int)(i / n8);
+        const long long j = i - pl * n8;
+        const int g = (int)(j % c8);
+        const int s2 = (int)((j / c8) % p.S2), r2 = (int)((j / ((long long)c8 * p.S2)) % p.R2);
+        const int k = (int)(j / ((long long)c8 * p.S2 * p.R2));
+        uint32_t o[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const int e = 8 * g + t, c = e % p.C, d = e / p.C;
+            const int r = r2 * p.st + d / p.st, s = s2 * p.st + d % p.st;
+            if (d < p.st * p.st && r < R && s < S) {
+                const uint32_t v = __half_as_ushort(w[pl * w_ps + (((long long)k * R + r) * S + s) * 8 + c]);
+                o[t >> 1] |= v << (16 * (t & 1));
+            }
+        }
+        w2[i] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
+
 template <typename ACC>
 __global__ void splitk_reduce_kernel(const ConvArgs a, const ACC* __restrict__ part, int ks) {
     const long long total = a.M * a.K;
@@ -135,6 +197,35 @@ size_t conv_split_ws_bytes(long long M, int K) {
     return 16 * one < cap ? 16 * one : cap;
 }
 
+S2dPlan s2d_plan(const fxpq_conv_desc& d) {
+    S2dPlan p = {};
+    if (d.Cp != 8 || d.stride < 2 || d.stride > 4 || d.R < d.stride || d.S < d.stride || d.C < 1 || d.C > 8 || d.N < 1 ||
+        d.pad < 0 || d.K < 1)
+        return p;
+    const long long P = ((long long)d.H + 2 * d.pad - d.R) / d.stride + 1, Q = ((long long)d.W + 2 * d.pad - d.S) / d.stride + 1;
+    if (d.H + 2 * d.pad < d.R || d.W + 2 * d.pad < d.S || P > (1 << 24) || Q > (1 << 24)) return p;
+    p.st = d.stride;
+    p.C = d.C;
+    p.R2 = (d.R + d.stride - 1) / d.stride;
+    p.S2 = (d.S + d.stride - 1) / d.stride;
+    p.C2 = (d.stride * d.stride * d.C + 7) / 8 * 8;
+    p.H2 = (int)P + p.R2 - 1;
+    p.W2 = (int)Q + p.S2 - 1;
+    p.flat = (p.S2 * p.C2 + 63) / 64 < p.S2 * ((p.C2 + 63) / 64);
+    p.x_bytes = ((size_t)d.N * p.H2 * p.W2 * p.C2 * 2 * planes_of(d.fmt_x) + 255) / 256 * 256;
+    p.w_bytes = ((size_t)d.K * p.R2 * p.S2 * p.C2 * 2 * planes_of(d.fmt_w) + 255) / 256 * 256;
+    p.ok = (long long)d.N * p.H2 * p.W2 * 2 < (1LL << 31) * 128;
+    return p;
+}
+
+size_t conv_ws_bytes(const fxpq_conv_desc& d) {
+    if (d.N < 1 || d.stride < 1 || d.R < 1 || d.S < 1) return 0;
+    const int P = (d.H + 2 * d.pad - d.R) / d.stride + 1, Q = (d.W + 2 * d.pad - d.S) / d.stride + 1;
+    if (P < 1 || Q < 1) return 0;
+    const S2dPlan p = s2d_plan(d);
+    return (p.ok ? p.x_bytes + p.w_bytes : 0) + conv_split_ws_bytes((long long)d.N * P * Q, d.K);
+}
+
 // Host-side planning shared by conv and gemm: fills ConvArgs, checks the integer bounds.
 fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, const int32_t* bias, void* y,
                       ConvArgs& a, int32_t* out_scale, bool& need64) {
@@ -166,6 +257,7 @@ fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, con
     a.M = (long long)d.N * P * Q;
     a.x_ps = (long long)d.N * d.H * d.W * d.Cp;
     a.w_ps = (long long)d.K * d.R * d.S * d.Cp;
+    a.x_sw = d.Cp, a.x_sh = (long long)d.W * d.Cp, a.x_sn = (long long)d.H * d.W * d.Cp;
     a.px = planes_of(d.fmt_x);
     a.pw = planes_of(d.fmt_w);
     a.relu = d.relu;
@@ -257,12 +349,56 @@ static bool tc_path_enabled() {
     return !(e && strcmp(e, "simt") == 0);
 }
 
+// FXPQ_CONV_PATH=tc_rows / tc_nos2d keep strided 8-channel layers on their own codes.
+static bool s2d_enabled() {
+    const char* e = getenv("FXPQ_CONV_PATH");
+    return !(e && (strcmp(e, "tc_rows") == 0 || strcmp(e, "tc_nos2d") == 0));
+}
+
+// The layer's arguments in the space-to-depth form.
+static ConvArgs s2d_args(const ConvArgs& a, const S2dPlan& p, const __half* x2, const __half* w2) {
+    ConvArgs b = a;
+    b.x = x2;
+    b.w = w2;
+    b.H = p.H2;
+    b.W = p.flat ? a.Q : p.W2;  // flat: one overlapping pixel of S2 C2 channels per output column
+    b.Cp = p.flat ? p.S2 * p.C2 : p.C2;
+    b.R = p.R2;
+    b.S = p.flat ? 1 : p.S2;
+    b.stride = 1;
+    b.pad = 0;
+    b.x_ps = (long long)a.N * p.H2 * p.W2 * p.C2;
+    b.w_ps = (long long)a.K * p.R2 * p.S2 * p.C2;
+    b.x_sw = p.C2;
+    b.x_sh = (long long)p.W2 * p.C2;
+    b.x_sn = (long long)p.H2 * p.W2 * p.C2;
+    return b;
+}
+
 fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64, cudaStream_t st, void* ws,
                         size_t ws_bytes) {
     const long long M = (long long)a.N * a.P * a.Q;
     if (M == 0) return FXPQ_OK;
     if (tc_path_enabled()) {
         bool launched = false;
+        // A strided 8-channel layer runs in the space-to-depth form when the workspace holds it: its taps are
+        // then whole runs of a pixel row, where gathered rows cost about 2600 cycles per 8 taps (ResNet conv1,
+        // 7 x 7 / 2 of 128 images, 455 -> 216 us with its copy; AlexNet conv1, 11 x 11 / 4 of 256, 431 -> 336)
+        const S2dPlan p = s2d_plan(d);
+        if (p.ok && ws && ws_bytes >= p.x_bytes + p.w_bytes && s2d_enabled()) {
+            char* base = static_cast<char*>(ws);
+            const long long npix = (long long)a.N * p.H2 * p.W2 * a.px, nw = (long long)a.K * p.R2 * p.S2 * (p.C2 / 8) * a.pw;
+            const unsigned xb = (unsigned)((npix + 255) / 256), wb = (unsigned)((nw + 255) / 256);
+            s2d_kernel<<<xb + wb, 256, 0, st>>>(a.x, a.w, a.N, a.H, a.W, a.K, a.R, a.S, a.pad, a.x_ps, a.w_ps, p, a.px, a.pw,
+                                                xb, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + p.x_bytes));
+            fxpq_status s = after_launch("s2d");
+            if (s != FXPQ_OK) return s;
+            const ConvArgs b = s2d_args(a, p, reinterpret_cast<const __half*>(base),
+                                        reinterpret_cast<const __half*>(base + p.x_bytes));
+            const size_t used = p.x_bytes + p.w_bytes;
+            s = launch_conv_tc(b, d, st, launched, ws_bytes > used ? base + used : nullptr, ws_bytes - used);
+            if (s != FXPQ_OK || launched) return s;
+        }
         fxpq_status s = launch_conv_tc(a, d, st, launched, ws, ws_bytes);
         if (s != FXPQ_OK || launched) return s;
     }
@@ -279,11 +415,7 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
 using namespace fxpq;
 
 extern "C" size_t fxpq_conv_workspace(const fxpq_conv_desc* h_desc) {
-    if (!h_desc || h_desc->N < 1 || h_desc->stride < 1 || h_desc->R < 1 || h_desc->S < 1) return 0;
-    const int P = (h_desc->H + 2 * h_desc->pad - h_desc->R) / h_desc->stride + 1;
-    const int Q = (h_desc->W + 2 * h_desc->pad - h_desc->S) / h_desc->stride + 1;
-    if (P < 1 || Q < 1) return 0;
-    return conv_split_ws_bytes((long long)h_desc->N * P * Q, h_desc->K);
+    return h_desc ? conv_ws_bytes(*h_desc) : 0;
 }
 
 extern "C" fxpq_status fxpq_conv_fwd(const fxpq_conv_desc* h_desc, const void* d_x, const void* d_w,

@@ -13,6 +13,8 @@ struct ConvArgs {
     int N, H, W, Cp, K, R, S, stride, pad, P, Q;
     long long M;       // N * P * Q output rows
     long long x_ps, w_ps;  // plane strides (elements) of x and w
+    long long x_sw, x_sh, x_sn;  // strides of x (elements) between pixels, rows and images: Cp, W Cp, H W Cp,
+                                 // except for the space-to-depth form (overlapping pixels)
     int px, pw, py;
     int relu, out_mode, has_bias;
     int delta;         // bias alignment: s_acc - fl_b
@@ -143,5 +145,19 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
 fxpq_status launch_splitk_reduce(const ConvArgs& a, const void* part, int ks, bool acc64, cudaStream_t st);
 // Scratch bytes a conv may use for its split reduction (0: never split).
 size_t conv_split_ws_bytes(long long M, int K);
+
+// Space-to-depth form of a strided layer with 8 stored channels (the first layer of a network): st x st input
+// pixels of C true channels become one pixel of C2 = st st C (rounded up to 8) channels, in which the layer has
+// stride 1, no padding and R2 x S2 taps.  x: [planes][N][H2][W2][C2], zero outside the map; w: [planes][K][R2]
+// [S2][C2], zero for taps past R, S.  A tap row's S2 C2 values are contiguous in both, so a row whose values
+// fill fewer 64-channel blocks together than tap by tap runs as one tap of S2 C2 channels (flat).
+struct S2dPlan {
+    bool ok, flat;
+    int st, C, R2, S2, C2, H2, W2;
+    size_t x_bytes, w_bytes;  // 256-byte multiples
+};
+S2dPlan s2d_plan(const fxpq_conv_desc& d);
+// Scratch bytes a conv may use: the space-to-depth copies, then the split reduction's shares.
+size_t conv_ws_bytes(const fxpq_conv_desc& d);
 
 }  // namespace fxpq

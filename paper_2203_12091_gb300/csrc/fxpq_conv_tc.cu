@@ -146,7 +146,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     // Layers whose im2col matrix is the stored activations themselves: 1x1 stride-1 convolutions
     // without padding ([M][Cp] per plane) and kernels covering the whole unpadded map (P = Q = 1,
     // FC layers: [N][H W Cp]).  A 128-row A tile is then one 2-D box of [M][R S Cp].
-    const bool one_by_one = a.R == 1 && a.S == 1 && a.stride == 1 && a.pad == 0;
+    const bool one_by_one = a.R == 1 && a.S == 1 && a.stride == 1 && a.pad == 0 && a.x_sw == a.Cp;
     const bool whole_map = a.R == a.H && a.S == a.W && a.pad == 0 && a.P == 1 && a.Q == 1;
     const bool rows_geom = (one_by_one || whole_map) && a.M > 0 && a.M < (1LL << 31) - TC_BM &&
                            !conv_path_is("tc_rows") && !conv_path_is("tc_patch");
@@ -223,7 +223,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
             const int S2 = (a.S + 1) & ~1;
             const int WW = 8 + S2 - 1, WH = 16 + a.R - 1;
             const int win_bytes = (WW * WH * 16 + 127) / 128 * 128;
-            bool ok = a.stride == 1 && a.Cp == 8 && a.K <= 64 && a.N > 0 && a.R * S2 <= 16 && 8 * WW <= 256 &&
+            bool ok = a.stride == 1 && a.Cp == 8 && a.x_sw == 8 && a.K <= 64 && a.N > 0 && a.R * S2 <= 16 && 8 * WW <= 256 &&
                       WH <= 256 && a.px * win_bytes <= TC_BM * TC_BK * 2 &&
                       a.pw * a.R * (S2 / 2) * 64 * 32 <= tc_stages(64) * 64 * TC_BK * 2 && !conv_path_is("tc_rows") &&
                       !conv_path_is("tc_nowin");
@@ -315,8 +315,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
             const long long wb = (long long)a.R * a.S * 8192;
             if (wb + 2 * slot <= TC_W64_SO) {
                 const cuuint64_t xdims[4] = {(cuuint64_t)a.Cp, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.N};
-                const cuuint64_t xstrides[3] = {(cuuint64_t)a.Cp * 2, (cuuint64_t)a.W * a.Cp * 2,
-                                                (cuuint64_t)a.H * a.W * a.Cp * 2};
+                const cuuint64_t xstrides[3] = {(cuuint64_t)a.x_sw * 2, (cuuint64_t)a.x_sh * 2, (cuuint64_t)a.x_sn * 2};
                 const cuuint32_t xbox[4] = {64, 8, (cuuint32_t)WH, 1};
                 const cuuint32_t es4[4] = {1, 1, 1, 1};
                 CUtensorMap mx;
@@ -349,8 +348,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         }
         if (P.patch == 0 && !P.rows_tma && use_patch) {
             const cuuint64_t xdims[5] = {(cuuint64_t)a.Cp, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.N, (cuuint64_t)a.px};
-            const cuuint64_t xstrides[4] = {(cuuint64_t)a.Cp * 2, (cuuint64_t)a.W * a.Cp * 2,
-                                            (cuuint64_t)a.H * a.W * a.Cp * 2, (cuuint64_t)a.x_ps * 2};
+            const cuuint64_t xstrides[4] = {(cuuint64_t)a.x_sw * 2, (cuuint64_t)a.x_sh * 2, (cuuint64_t)a.x_sn * 2, (cuuint64_t)a.x_ps * 2};
             const cuuint32_t st = (cuuint32_t)a.stride;
             const cuuint32_t xbox[5] = {(cuuint32_t)(narrow ? 8 : TC_BK), (ps.TW - 1) * st + 1, (ps.TH - 1) * st + 1,
                                         (cuuint32_t)ps.TN, 1};

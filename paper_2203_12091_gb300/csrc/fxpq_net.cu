@@ -96,15 +96,17 @@ fxpq_status plan_net(const fxpq_net* net, int32_t batch, std::vector<Slot>& slot
     return FXPQ_OK;
 }
 
-// Largest split-reduction scratch any conv op of the list may use at this batch.
+// Largest scratch any conv op of the list may use at this batch.
 size_t net_conv_ws(const fxpq_net* net, const std::vector<Slot>& slots, int32_t batch) {
     size_t m = 0;
     for (int i = 0; i < net->n_ops; ++i) {
         const fxpq_op_desc& o = net->ops[i];
         if (o.op != FXPQ_OP_CONV) continue;
         const Slot& s0 = slots[o.src0];
-        const int P = (s0.H + 2 * o.pad - o.R) / o.stride + 1, Q = (s0.W + 2 * o.pad - o.S) / o.stride + 1;
-        const size_t b = fxpq::conv_split_ws_bytes((long long)batch * P * Q, o.K);
+        fxpq_conv_desc d = {};
+        d.N = batch, d.H = s0.H, d.W = s0.W, d.C = s0.C, d.Cp = s0.Cp, d.K = o.K, d.R = o.R, d.S = o.S;
+        d.stride = o.stride, d.pad = o.pad, d.fmt_x = s0.fmt, d.fmt_w = o.fmt_w;
+        const size_t b = fxpq::conv_ws_bytes(d);
         if (b > m) m = b;
     }
     return align256(m);
@@ -165,7 +167,7 @@ extern "C" fxpq_status fxpq_net_forward(const fxpq_net* h_net, const float* d_im
     char* base = static_cast<char*>(d_ws);
     auto ptr = [&](int slot) { return static_cast<void*>(base + slots[slot].offset); };
     if (batch == 0) return FXPQ_OK;
-    // the convs' split-reduction scratch follows the slots when the caller provided it
+    // the convs' scratch follows the slots when the caller provided it
     const size_t cws = net_conv_ws(h_net, slots, batch);
     void* conv_ws = (cws && ws_bytes >= total + cws) ? static_cast<void*>(base + total) : nullptr;
 
@@ -182,7 +184,7 @@ extern "C" fxpq_status fxpq_net_forward(const fxpq_net* h_net, const float* d_im
                 d.N = batch;
                 d.H = s0.H;
                 d.W = s0.W;
-                d.C = s0.Cp;
+                d.C = s0.C;
                 d.Cp = s0.Cp;
                 d.K = o.K;
                 d.R = o.R;
@@ -402,7 +404,7 @@ extern "C" fxpq_status fxpq_net_calibrate(const fxpq_net* h_net, const float* d_
                 cd.N = n_calib;
                 cd.H = s0.H;
                 cd.W = s0.W;
-                cd.C = s0.Cp;
+                cd.C = s0.C;
                 cd.Cp = s0.Cp;
                 cd.K = o.K;
                 cd.R = o.R;

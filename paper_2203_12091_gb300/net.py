@@ -233,7 +233,7 @@ class QNet:
             sH, sW, sCp = self.shapes[src]
             wq, bq = self.q[nm]
             sq, hq = self.qs.get(nm, (None, None))
-            d = F.conv_desc(N, sH, sW, sCp, sCp, L_["K"], L_["R"], L_["R"], L_["stride"], L_["pad"], L_["relu"],
+            d = F.conv_desc(N, sH, sW, L_["C"], sCp, L_["K"], L_["R"], L_["R"], L_["stride"], L_["pad"], L_["relu"],
                             out_mode, fx, self.fmts[nm]["w"], self.fmts[nm].get("b"), fy, self.w_l1.get(nm, 0),
                             scale=sq, fmt_scale=self.fmts[nm].get("s"), shift=hq, fmt_shift=self.fmts[nm].get("h"),
                             wpacked=self.qp.get(nm))

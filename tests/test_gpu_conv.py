@@ -619,3 +619,44 @@ def test_conv_packed_weights(F, case, tw):
         assert np.array_equal(got2, want)
     else:
         assert np.array_equal(got2, want2)
+
+
+@pytest.mark.parametrize("H,C,K,R,st,pad", [(31, 3, 64, 7, 2, 3), (39, 3, 96, 11, 4, 2), (23, 1, 24, 3, 2, 1), (17, 4, 40, 5, 2, 2),
+                                            (20, 8, 72, 3, 3, 0), (12, 3, 136, 4, 4, 0), (9, 5, 8, 9, 2, 4), (16, 2, 64, 6, 3, 5)])
+@pytest.mark.parametrize("kx,kw", [(8, 7), (16, 16)])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_space_to_depth_parity(F, H, C, K, R, st, pad, kx, kw, mode):
+    """Strided layers on 8 stored channels: the space-to-depth form (taps cut off by the block grid, blocks that
+    reach past the map, partial 64-channel blocks, two limbs), and the same call without its workspace."""
+    if os.environ.get("FXPQ_CONV_PATH") not in ("tc", "tc_bn256"):
+        pytest.skip("a form of the tensor-core path")
+    rng = np.random.default_rng(H * C + K)
+    fx, fw, fb = F.fmt(kx, 1, kx - 3), F.fmt(kw, 1, kw - 1), F.fmt(16, 1, 18)
+    fy = F.fmt(8, 0, 2) if mode == 0 else None
+    x, w, b = rand_codes(rng, (3, H, H, C), kx, 1), rand_codes(rng, (K, R, R, C), kw, 1), rand_codes(rng, (K,), 16, 1)
+    got, s = run_conv(F, x, fx, w, fw, b, fb, st, pad, True, mode, fy, 8)
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, st, pad, True, mode, fy)
+    assert s == ws and np.array_equal(got, want)
+    old = os.environ["FXPQ_CONV_PATH"]
+    os.environ["FXPQ_CONV_PATH"] = "tc_nos2d"
+    try:
+        got, s = run_conv(F, x, fx, w, fw, b, fb, st, pad, True, mode, fy, 8)
+    finally:
+        os.environ["FXPQ_CONV_PATH"] = old
+    assert s == ws and np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("N,H,C,K,R,st,pad", [(5, 7, 64, 64, 3, 1, 1), (130, 3, 64, 72, 3, 1, 1), (3, 14, 96, 256, 5, 1, 2),
+                                              (4, 15, 16, 128, 3, 2, 1), (2, 30, 128, 136, 1, 2, 0), (2, 33, 24, 64, 3, 3, 1),
+                                              (1, 70, 40, 64, 3, 7, 2), (7, 5, 200, 384, 3, 1, 1), (2, 19, 64, 64, 3, 8, 1)])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_patch_shapes_parity(F, N, H, C, K, R, st, pad, mode):
+    """Patches over several images, strided boxes (up to the box limits) and channel counts off 64: the last
+    image group, ragged maps and the zero-filled channels of every tap."""
+    rng = np.random.default_rng(N * H + K)
+    fx, fw, fb = F.fmt(7, 0, 3), F.fmt(6, 1, 6), F.fmt(16, 1, 14)
+    fy = F.fmt(8, 0, 1) if mode == 0 else None
+    x, w, b = rand_codes(rng, (N, H, H, C), 7, 0), rand_codes(rng, (K, R, R, C), 6, 1), rand_codes(rng, (K,), 16, 1)
+    got, s = run_conv(F, x, fx, w, fw, b, fb, st, pad, True, mode, fy, C, int(np.abs(w).reshape(K, -1).sum(axis=1).max()))
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, st, pad, True, mode, fy)
+    assert s == ws and np.array_equal(got, want)
