@@ -307,6 +307,9 @@ fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, con
     a.v32 = 0;
     a.vf = 0;
     a.vf_c = a.vf_lo = a.vf_hi = 0.0f;
+    a.vi = d.out_mode == FXPQ_OUT_F32 && !a.has_scale && (!bias || d.fmt_b.bits <= 24);
+    a.vi_c = ldexpf(1.0f, -(d.fmt_x.fl + d.fmt_w.fl));
+    a.vi_b = bias ? ldexpf(1.0f, -d.fmt_b.fl) : 0.0f;
     if (d.out_mode == FXPQ_OUT_CODES) {
         a.sh = s - d.fmt_y.fl;
         if (a.sh > 62) return FXPQ_ERR_RANGE;

@@ -27,6 +27,8 @@ struct ConvArgs {
     int sh32;          // right shift of the 32-bit path, relative to the accumulator's scale
     int vf;            // 1: the fp32 form of the FxP-QLayer applies to sums that are exact fp32 integers
     float vf_c, vf_lo, vf_hi;  // 2^-sh32 and the clip levels (lower one 0 under a ReLU)
+    int vi;            // 1: fepi_image gives the fp32 image of sums that are exact fp32 integers
+    float vi_c, vi_b;  // 2^-(fl_x + fl_w) and 2^-fl_b
     const int32_t* scale;  // Scale layer aleph1 codes [K] (has_scale)
     const int32_t* shift;  // Scale layer aleph2 codes [K]
     int has_scale;
@@ -118,6 +120,13 @@ __host__ __device__ __forceinline__ float fepi_bias(const ConvArgs& a, int32_t b
     if (a.bsh >= 0) return (float)(b << a.bsh) * a.vf_c;
     const int d = -a.bsh;
     return ((float)(b >> d) + ((b & ((1 << d) - 1)) ? 0.5f : 0.0f)) * a.vf_c;
+}
+
+// The fp32 nearest-even image of a C-Block output in one fused multiply-add (valid when a.vi, for |acc| < 2^24):
+// acc 2^-(fl_x + fl_w) and t = b 2^-fl_b are exact in fp32, their sum is rounded once, whichever is finer.
+__host__ __device__ __forceinline__ float fepi_image(const ConvArgs& a, float acc, float t) {
+    const float v = fmaf(acc, a.vi_c, t);
+    return a.relu ? fmaxf(v, 0.0f) : v;
 }
 
 // Bias alignment, ReLU and the FxP-QLayer for one output value of row m, channel k.

@@ -215,7 +215,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         P.wf32 = 0;
         P.win_eps = P.win_c[0] = P.win_c[1] = P.win_c[2] = 0.0f;
         P.nacc = 1;
-        P.TN = 1;
+        P.TH = P.TW = P.TN = P.tiles_p = P.tiles_q = 1;
         // window mode for 8-channel stride-1 layers with at most 64 output channels: 8 x 16 output
         // patches, one input window per tile and limb plane, weights resident in shared memory, one
         // exact fp32 accumulator per limb pair (R * S2 * 8 products each)
@@ -445,8 +445,8 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         }
     }
     P.n_units = P.n_tiles * P.ksplit;
-    P.fepi = a.vf && P.fast_store && P.n_groups == 1 && P.g[0].shift == 0 && P.patch != 3 && P.ksplit == 1 && !acc64 &&
-             !conv_path_is("tc_iepi");
+    P.fepi = ((a.vf && P.fast_store) || (a.vi && a.K % 4 == 0)) && P.n_groups == 1 && P.g[0].shift == 0 && P.patch != 3 &&
+             P.ksplit == 1 && !P.pk && !acc64 && !a.has_scale && !conv_path_is("tc_iepi");
     {
         std::lock_guard<std::mutex> lk(g_tc_mu);
         if (!g_tc_attr_set) {
@@ -458,6 +458,12 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
                                      (int)tc_smem_bytes<64>()) != cudaSuccess ||
                 cudaFuncSetAttribute(conv_tc_kernel<64, int, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes<64>()) != cudaSuccess ||
+                cudaFuncSetAttribute(conv_tc_kernel<64, int, false, false, false, false, false, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes<64>()) != cudaSuccess ||
+                cudaFuncSetAttribute(conv_tc_kernel<128, int, false, false, false, false, false, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes<128>()) != cudaSuccess ||
+                cudaFuncSetAttribute(conv_tc_kernel<256, int, false, false, false, false, false, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes<256>()) != cudaSuccess ||
                 cudaFuncSetAttribute(conv_tc_kernel<128, int, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes<128>()) != cudaSuccess ||
                 cudaFuncSetAttribute(conv_tc_kernel<256, int, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -470,7 +476,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
                                      (int)tc_smem_bytes<256, true>()) != cudaSuccess ||
                 cudaFuncSetAttribute(conv_tc_kernel<64, long long, false, false, false, true>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(tc_smem_bytes<64>() + 64 * TC_BM * 2)) != cudaSuccess ||
+                                     (int)(tc_smem_bytes<64>())) != cudaSuccess ||
                 cudaFuncSetAttribute(conv_tc_kernel<64, int, false, false, false, false, true>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_w64()) != cudaSuccess)
                 return FXPQ_ERR_CUDA;
@@ -478,11 +484,12 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         }
     }
     const int grid = P.n_units < sms ? P.n_units : sms;
+    TileIter::split(P, grid, P.step_n, P.step_q, P.step_p, P.step_g);
     launched = true;
     if (a.has_scale) return launch_conv_tc_scaled(P, BN, acc64, grid, st);  // never split
     if (P.patch == 3 && (P.w32 || P.wf32))  // window mode, 32-bit two-limb epilogue: its own instance (never split)
         conv_tc_kernel<64, long long, false, false, false, true>
-            <<<grid, tc_threads_win(), tc_smem_bytes<64>() + 64 * TC_BM * 2, st>>>(P);
+            <<<grid, tc_threads_win(), tc_smem_bytes<64>(), st>>>(P);
     else if (P.patch == 4 && (P.fast_store || a.out_mode == FXPQ_OUT_F32))
         // 64-channel window mode: the instance with its own shared-memory layout and 16 epilogue warps
         conv_tc_kernel<64, int, false, false, false, false, true><<<grid, tc_threads_win(), tc_smem_w64(), st>>>(P);
@@ -500,6 +507,12 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         conv_tc_kernel<64, long long, false, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
     else if (P.ksplit > 1)
         conv_tc_kernel<64, int, false, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+    else if (P.fepi && BN == 64)
+        conv_tc_kernel<64, int, false, false, false, false, false, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+    else if (P.fepi && BN == 128)
+        conv_tc_kernel<128, int, false, false, false, false, false, true><<<grid, tc_threads(128), tc_smem_bytes<128>(), st>>>(P);
+    else if (P.fepi)
+        conv_tc_kernel<256, int, false, false, false, false, false, true><<<grid, tc_threads(256), tc_smem_bytes<256>(), st>>>(P);
     else if (acc64)
         conv_tc_kernel<64, long long, false><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
     else if (BN == 64)

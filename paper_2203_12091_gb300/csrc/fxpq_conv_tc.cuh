@@ -43,15 +43,17 @@ namespace tc {
 
 constexpr int TC_BM = 128;
 constexpr int TC_BK = 64;  // fp16 elements per k-block row = 128 bytes (one swizzle atom row)
-// Pipeline depth: 6 stages of 32 KB (BN <= 128); 4 of 48 KB for BN = 256, whose one-plane codes are
+// Pipeline depth: 6 stages of 24 or 32 KB (BN <= 128); 4 of 48 KB for BN = 256, whose one-plane codes are
 // stored through per-warp 2 KB slices (no TMA-store staging of the whole tile) so that the output
 // staging keeps only 32 KB; 3 for the packed-weight instance, whose packed stages take the 64 KB
 // staging region.  (The 256-column layers lose about a fifth of their speed from 3 stages to 2: the
 // copies' latency, not the tensor pipe, bounds them at this depth.)
 __host__ __device__ constexpr int tc_stages(int BN, bool PK = false) { return BN == 256 ? (PK ? 3 : 4) : 6; }
-// Output staging bytes: BN / 64 boxes of 128 rows x 128 bytes for the TMA-store epilogue, 32 KB where
+// Output staging: tiles of BN / 64 boxes of 128 rows x 128 bytes for the TMA-store epilogue, two of them for
+// BN = 64 (the sixth stage is worth more than a second 32 KB tile for BN = 128), 32 KB where
 // the codes are stored directly (BN = 256 without packed weights).
-__host__ __device__ constexpr int tc_out_bytes(int BN, bool PK = false) { return (BN == 256 && !PK) ? 32768 : BN * TC_BM * 2; }
+__host__ __device__ constexpr int tc_out_bytes(int BN, bool PK = false) { return (BN == 256 && PK) ? 65536 : 32768; }
+__host__ __device__ constexpr int tc_stg_tiles(int BN) { return BN == 64 ? 2 : 1; }
 // Row-tile producers arrive on a stage this many k-blocks after issuing its copies (cp.async groups
 // in flight).  It must stay below the stage count: a producer waiting for a stage to be consumed
 // must already have arrived on it.
@@ -59,7 +61,8 @@ __host__ __device__ constexpr int tc_lag(int BN, bool PK = false) { return tc_st
 // Warps: 4 producers, epilogue warps (four per 32-column chunk group: one per TMEM lane quadrant;
 // BN / 8 of them up to 16, each then draining BN / 128 chunks), one MMA / TMEM-allocation warp.
 __host__ __device__ constexpr int tc_epi_warps(int BN) { return BN / 8 < 16 ? BN / 8 : 16; }
-__host__ __device__ constexpr int tc_threads(int BN) { return (5 + tc_epi_warps(BN)) * 32; }
+// and, where whole tiles are stored by TMA (BN <= 128), one warp that issues these stores.
+__host__ __device__ constexpr int tc_threads(int BN) { return (5 + (BN <= 128 ? 1 : 0) + tc_epi_warps(BN)) * 32; }
 // Packed weights (PK instances, BN = 256 only): the weights arrive as k-bit records (k <= 8) and these
 // extra warps after the MMA warp, with producer warps 1-3, expand every k-block's records into the
 // fp16 B stage.  The packed stages live in the output staging region, which PK layers do not use.
@@ -74,7 +77,7 @@ constexpr int TC_WIN_EPI_WARPS = 16;
 // at W64_SO.
 constexpr int TC_W64_SO = 180 * 1024;
 constexpr size_t tc_smem_w64() { return 1024 + TC_W64_SO + 2 * 64 * TC_BM * 2 + 256; }
-__host__ __device__ constexpr int tc_threads_win() { return (5 + TC_WIN_EPI_WARPS) * 32; }
+__host__ __device__ constexpr int tc_threads_win() { return (6 + TC_WIN_EPI_WARPS) * 32; }
 // Dynamic shared memory: barriers, the stages (A and B tiles), the output staging tile.
 template <int BN, bool PK = false>
 constexpr size_t tc_smem_bytes() {
@@ -85,11 +88,13 @@ static_assert(tc_smem_bytes<256>() <= 232448 && tc_smem_bytes<256, true>() <= 23
 constexpr int TC_MAX_GROUPS = 64;
 constexpr int TC_MAX_SPLIT = 16;
 constexpr long long TC_WAIT_CYCLES = 4000000000LL;  // ~2 s at 2 GHz
-// TMA-issuing threads of patch tiles (lane 0 of warps 0 .. n-1).  Producer p issues the k-blocks of the
-// stages s with s % n == p (n divides the stage count), so every use of a stage comes from one thread, in
+// TMA-issuing warps of patch and TMA row tiles (warps 0 .. n-1).  Producer p issues the k-blocks of the
+// stages s with s % n == p (n divides the stage count), so every use of a stage comes from one warp, in
 // order, and its parity wait on the stage's `empty` barrier is never more than one phase ahead of it.
 // (A parity wait two phases ahead reads as complete: with k-blocks dealt round-robin, more producers
-// than stages could refill a stage before its data was consumed.)
+// than stages could refill a stage before its data was consumed.)  A warp's latency per k-block (the
+// barrier round, two copies) would bound the rate: one warp for the A and one for the B boxes of every
+// stage took 880 cycles per k-block of 128-column tiles where two that share the stages take 650.
 __host__ __device__ constexpr int tc_producers(int BN, bool PK = false) {
     return tc_stages(BN, PK) <= 4 ? tc_stages(BN, PK) : 2;
 }
@@ -123,7 +128,7 @@ struct TcParams {
     int WW, WH, S2;      // window mode: window width / height in pixels, taps per row rounded up to even
     int w32;             // window mode, two-limb x and w, one-plane codes out: the 32-bit epilogue (the
                          // host proved its bounds; see the epilogue), with m = sh - 16 in [0, 30]
-    int fepi;            // the fp32 FxP-QLayer (a.vf; one exact group, no split, fast_store)
+    int fepi;            // the fp32 epilogue (codes: a.vf and fast_store; fp32 image: a.vi; one exact group, no split)
     float win_c[3], win_eps;  // w32 in fp32: 2^(16 - sh), 2^(8 - sh), 2^-sh; the most that the fp32 sum is off
                               // (0: integer arithmetic throughout)
     int wf32;            // the same window instance writing the fp32 image of v = 2^16 T + Lo
@@ -131,7 +136,8 @@ struct TcParams {
     int w64_slot0;       // patch 4: offset of window slot 0 (after the resident weights)
     int w64_slot_stride; // bytes between the two window slots (S copies of WH KiB)
     int TH, TW, TN;      // patch shape: TH x TW pixels of TN images (TH * TW * TN <= 128)
-    int tiles_p, tiles_q;  // patches per image along P and Q
+    int tiles_p, tiles_q;  // patches per image along P and Q (128-row tiles: 1)
+    int step_n, step_q, step_p, step_g;  // the grid size in the tile index's digits (TileIter)
     int kbt;             // patch 1: k-blocks per tap (the 64-channel blocks of Cp, the last one zero filled)
     ConvArgs a;
     int RSC;       // R * S * Cp: reduction length of one plane
@@ -230,6 +236,52 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         "%5}], [%6];\n\t}" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
         : "memory");
+}
+
+// Position of a CTA's current tile, stepped by the grid size with carries instead of divisions: tile index
+// = ((image group * tiles_p + patch row) * tiles_q + patch column) * tiles_n + column tile (128-row tiles: the
+// row tile takes the image group's place).  A division is about 30 instructions, and every epilogue warp
+// would need five per tile.
+struct TileIter {
+    int tn, iq, ip, ng;
+    __device__ __forceinline__ TileIter(const TcParams& P, int t0) { split(P, t0, tn, iq, ip, ng); }
+    static __host__ __device__ __forceinline__ void split(const TcParams& P, int t, int& n, int& q, int& p, int& g) {
+        n = t % P.tiles_n;
+        t /= P.tiles_n;
+        q = t % P.tiles_q;
+        t /= P.tiles_q;
+        p = t % P.tiles_p;
+        g = t / P.tiles_p;
+    }
+    __device__ __forceinline__ void next(const TcParams& P) {
+        tn += P.step_n;
+        int c = tn >= P.tiles_n;
+        tn -= c ? P.tiles_n : 0;
+        iq += P.step_q + c;
+        c = iq >= P.tiles_q;
+        iq -= c ? P.tiles_q : 0;
+        ip += P.step_p + c;
+        c = ip >= P.tiles_p;
+        ip -= c ? P.tiles_p : 0;
+        ng += P.step_g + c;
+    }
+};
+
+// A tile row's place within its tile, decoded once per thread: image, row and column offsets of a patch pixel
+// in bytes 2, 1 and 0 (each below 128), or -1 for a row past the patch.
+__device__ __forceinline__ int row_in_tile(const TcParams& P, int row) {
+    const int pix = P.TH * P.TW, ti = row / pix, r = row - ti * pix, j = r / P.TW;
+    return ti < P.TN ? (ti << 16) | (j << 8) | (r - j * P.TW) : -1;
+}
+// Linear output row of that place in the tile at T (`row` itself in 128-row tiles), or -1 outside the map.
+__device__ __forceinline__ long long row_at(const TcParams& P, const TileIter& T, int place, int row) {
+    if (!P.patch) {
+        const long long m = (long long)T.ng * TC_BM + row;
+        return m < P.a.M ? m : -1;
+    }
+    const int n = T.ng * P.TN + (place >> 16), p = T.ip * P.TH + ((place >> 8) & 255), q = T.iq * P.TW + (place & 255);
+    if (place < 0 || n >= P.a.N || p >= P.a.P || q >= P.a.Q) return -1;
+    return ((long long)n * P.a.P + p) * P.a.Q + q;
 }
 
 // Output row (linear index into N*P*Q, or -1 when outside the map) of tile row i.
@@ -464,8 +516,10 @@ __device__ __forceinline__ void tmem_st16_nw(uint32_t taddr, const uint32_t (&r)
 }
 // Final epilogue of 32 consecutive output channels k0.. of row m (generic outputs: two-plane codes,
 // int64 accumulators, fp32 calibration images): bias alignment, ReLU, FxP-QLayer.
+// (This and the next are calls, their values passed in local memory: inlined, they made the 128-column kernels
+// spill 1.2 KB around every path, the codes of several groups among them.)
 template <typename ACC, bool SC>
-__device__ __forceinline__ void epilogue_block32(const ConvArgs& a, long long m, int k0, const ACC (&acc)[32]) {
+__device__ __noinline__ void epilogue_block32(const ConvArgs& a, long long m, int k0, const ACC (&acc)[32]) {
     if (a.out_mode == FXPQ_OUT_CODES) {
         __half* y = static_cast<__half*>(a.y);
         const long long base = m * a.K + k0;
@@ -502,7 +556,7 @@ __device__ __forceinline__ void epilogue_block32(const ConvArgs& a, long long m,
 // value per lane.  All 32 lanes take part; rows with m < 0 (outside the output) store nothing.  Needs K %
 // 4 == 0 (fp32) or K % 2 == 0 (int64), so that a 16-byte piece is wholly inside or past K.
 template <typename ACC, bool SC>
-__device__ __forceinline__ void epilogue_block32_staged(const ConvArgs& a, long long m, int k0, const ACC (&acc)[32],
+__device__ __noinline__ void epilogue_block32_staged(const ConvArgs& a, long long m, int k0, const ACC (&acc)[32],
                                                         unsigned char* wbuf, int lane) {
     const bool f32 = a.out_mode == FXPQ_OUT_F32;
     const int per = f32 ? 16 : 8;  // values per round: 64 bytes of a row
@@ -572,6 +626,30 @@ __device__ __forceinline__ void store_codes_direct(const ConvArgs& a, long long 
         if (mr >= 0 && kk < a.K) *reinterpret_cast<uint4*>(static_cast<__half*>(a.y) + mr * a.K + kk) = v;
     }
     __syncwarp();
+}
+
+// The same for 32 fp32 values per lane (channels k0 ..), in two rounds of 64 bytes of a row.  K % 4 == 0.
+__device__ __forceinline__ void store_f32_direct(const ConvArgs& a, long long m, int k0, const float (&v)[32],
+                                                 unsigned char* wbuf, int lane) {
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = 16 * hf + 4 * q;
+            *reinterpret_cast<float4*>(wbuf + lane * 64 + 16 * (q ^ ((lane >> 1) & 3))) =
+                make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const int r = (lane >> 2) + 8 * it, pc = lane & 3;
+            const long long mr = __shfl_sync(0xffffffffu, m, r);
+            const uint4 x = *reinterpret_cast<const uint4*>(wbuf + r * 64 + 16 * (pc ^ ((r >> 1) & 3)));
+            const int kk = k0 + 16 * hf + pc * 4;
+            if (mr >= 0 && kk < a.K) *reinterpret_cast<uint4*>(static_cast<float*>(a.y) + mr * a.K + kk) = x;
+        }
+        __syncwarp();
+    }
 }
 
 // Uniform constants of the 32-bit FxP-QLayer epilogue (the same arithmetic as qlayer_code32, with
@@ -681,6 +759,12 @@ __device__ __forceinline__ int win_code(uint32_t fhh, uint32_t fhl, uint32_t flh
     return min(max((relu && T < 0) ? 0 : q + up, lo), hi);
 }
 
+__device__ __forceinline__ uint64_t f32x2_splat(float c) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(c));
+    return v;
+}
+
 // Two accumulators to packed codes in fp32 (fepi_bias): one packed fused multiply-add, clip, the packed
 // rounding addition of f32_codes_f16x2.  About 4.5 instructions per code, none of them a conversion (those
 // run at a quarter of the rate); the integer form took 20 to 30.
@@ -691,12 +775,16 @@ __device__ __forceinline__ uint32_t fepi_pair(uint32_t a0, uint32_t a1, uint64_t
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(av), "l"(cc), "l"(tv));
     float x, y;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-    return f32_codes_f16x2(fminf(fmaxf(x, lo), hi), fminf(fmaxf(y, lo), hi));
-}
-__device__ __forceinline__ uint64_t f32x2_splat(float c) {
-    uint64_t v;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(c));
-    return v;
+    x = fminf(fmaxf(x, lo), hi);
+    y = fminf(fmaxf(y, lo), hi);
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(v) : "l"(f32x2_splat(12609024.0f)));
+    uint32_t r0, r1;
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(r0), "=r"(r1) : "l"(v));
+    const uint32_t w = __byte_perm(r0, r1, 0x5410);
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w),
+                              __halves2half2(__ushort_as_half(0x6600), __ushort_as_half(0x6600)));
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 // ------------------------------------------------------------------ kernel
@@ -739,7 +827,9 @@ __device__ __forceinline__ void pk_convert_loop(const TcParams& P, int cid, int 
 // WIN: the window-mode instance of the 32-bit two-limb epilogue (P.patch == 3, P.w32): 16 epilogue warps and
 // two staging tiles; only window mode's roles are compiled into it.
 // W64: the same for the 64-channel window mode (P.patch == 4) with one-plane codes out.
-template <int BN, typename ACC, bool SC, bool SPLIT = false, bool PK = false, bool WIN = false, bool W64 = false>
+// FE: the instance of layers whose epilogue is the fp32 FxP-QLayer (P.fepi): nothing else is compiled into it,
+// which keeps its epilogue out of local memory (beside the integer forms the 128-column one spilled 320 bytes).
+template <int BN, typename ACC, bool SC, bool SPLIT = false, bool PK = false, bool WIN = false, bool W64 = false, bool FE = false>
 __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_pk(BN, PK), 1)
     conv_tc_kernel(const __grid_constant__ TcParams P) {
     constexpr int TC_STAGES = tc_stages(BN, PK);
@@ -750,17 +840,20 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     static_assert(TC_LAG >= 1 && TC_LAG < TC_STAGES, "producer lag must be below the stage count");
     static_assert(!PK || (BN == 256 && sizeof(ACC) == 4 && !SC), "packed weights: 256-column int32 tiles only");
     static_assert(!PK || TC_STAGES * BN * 64 <= tc_out_bytes(BN, PK), "packed stages must fit the staging region");
-    // PK: one issuing thread (producer warp 0), so its stage waits are in order by construction
+    // PK: one issuing warp (producer warp 0), so its stage waits are in order by construction
     constexpr int TC_PRODUCERS = PK ? 1 : tc_producers(BN, PK);
     static_assert(TC_STAGES % TC_PRODUCERS == 0 && TC_PRODUCERS <= 4,
-                  "each stage must have one producer thread among warps 0..3");
+                  "each stage must have one producer among warps 0..3");
+    constexpr int NSTG = tc_stg_tiles(BN);  // staging tiles of the TMA stores
     static_assert(!WIN || (BN == 64 && sizeof(ACC) == 8 && !SC && !SPLIT && !PK), "window instance: BN = 64, int64");
     static_assert(!W64 || (BN == 64 && sizeof(ACC) == 4 && !SC && !SPLIT && !PK && !WIN), "W64 instance: BN = 64, int32");
+    static_assert(!FE || (sizeof(ACC) == 4 && !SC && !SPLIT && !PK && !WIN && !W64), "fp32 epilogue: plain int32 instances");
     constexpr bool WEPI = WIN || W64;  // the window instances' epilogue (16 warps, two staging tiles)
     constexpr int EPI_WARPS = WEPI ? TC_WIN_EPI_WARPS : tc_epi_warps(BN);
-    constexpr int EPI_THREADS = 32 * EPI_WARPS;
-    static_assert(WEPI || tc_out_bytes(BN, PK) >= EPI_WARPS * 2048, "the staged fp32 / int64 epilogue takes 2 KB per warp");
+    static_assert(tc_out_bytes(BN, PK) >= EPI_WARPS * 2048 || WEPI, "the staged fp32 / int64 epilogue takes 2 KB per warp");
     constexpr int MMA_WARP = 4 + EPI_WARPS;
+    constexpr bool STORE_WARP = BN <= 128;  // warp MMA_WARP + 1 stores the staged tiles
+    constexpr int STG_BYTES = BN * TC_BM * 2;  // one staging tile
     constexpr int CPW = WEPI ? 1 : (BN / 32) / (EPI_WARPS / 4);  // 32-column chunks per epilogue warp
     constexpr int A_BYTES = TC_BM * TC_BK * 2;  // 16 KB
     constexpr int B_BYTES = BN * TC_BK * 2;
@@ -776,7 +869,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     unsigned char* sB = base + TC_STAGES * A_BYTES;
     unsigned char* sO = W64 ? base + TC_W64_SO : sB + TC_STAGES * B_BYTES;  // output staging: BN/64 halves of
                                                                          // [128 rows][64 codes]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sO + (WEPI ? 2 * BN * TC_BM * 2 : tc_out_bytes(BN, PK)));  // WEPI: two staging tiles
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sO + tc_out_bytes(BN, PK));
     // bars: full[STAGES], empty[STAGES], accfull[2], accempty[2], done
     volatile int* abort = reinterpret_cast<volatile int*>(bars + 2 * TC_STAGES + 5);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * TC_STAGES + 6);
@@ -786,7 +879,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     const uint32_t stg_full = smem_u32(bars + 2 * TC_STAGES + 7);  // staging written by every epilogue warp
     const uint32_t stg_free = smem_u32(bars + 2 * TC_STAGES + 8);  // staging read by the previous TMA store
     const uint32_t wbar = smem_u32(bars + 2 * TC_STAGES + 9);      // window mode: resident weights loaded
-    const uint32_t stg_full2 = smem_u32(bars + 2 * TC_STAGES + 10);  // WIN: the second staging tile
+    const uint32_t stg_full2 = smem_u32(bars + 2 * TC_STAGES + 10);  // the second staging tile
     const uint32_t stg_free2 = smem_u32(bars + 2 * TC_STAGES + 11);
     // PK: pkfull[s] completes when stage s's A box and packed weight records have landed; the
     // converters then fill the B stage and arrive on full[s]
@@ -798,8 +891,8 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < TC_STAGES; ++s) {
-            // patch tiles: one expect_tx arrival for both TMAs; row tiles: one arrival per producer
-            // warp + the weight TMA's expect_tx
+            // patch and TMA row tiles: one expect_tx arrival for both TMAs; gathered row tiles: one arrival per
+            // producer warp + the weight TMA's expect_tx
             mbar_init(full0 + 8 * s, PK ? TC_PK_CONVERTERS : (P.patch || P.rows_tma) ? 1 : 4 + 1);
             mbar_init(empty0 + 8 * s, 1);
             if (PK) mbar_init(pkfull0 + 8 * s, 1);
@@ -811,7 +904,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         mbar_init(done_bar, 1);
         mbar_init(stg_full, EPI_WARPS);
         mbar_init(stg_free, 1);
-        if (WEPI) {
+        if (STORE_WARP) {
             mbar_init(stg_full2, EPI_WARPS);
             mbar_init(stg_free2, 1);
         }
@@ -947,21 +1040,18 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         // 2048 tl of the stage (a 16-byte K column of the no-swizzle layout), and taps past R*S
         // are boxes wholly outside the tensor (zero filled).
         if (warp < TC_PRODUCERS) {
-            // k-block it goes to producer (it % TC_STAGES) % TC_PRODUCERS: one thread's latency per k-block
-            // (barrier wait, two TMA instructions) would bound the stage rate
-            const int me = warp;
+            const uint32_t me = warp;
             const bool narrow = P.patch == 2;
             const uint32_t a_bytes = P.rows_tma ? (uint32_t)(TC_BM * 128) : (uint32_t)(P.TH * P.TW * P.TN * (narrow ? 8 * 16 : 128));
-            const int per_img = P.rows_tma ? 1 : P.tiles_p * P.tiles_q;
-            uint32_t it = 0;
+            uint32_t it = 0, stage = 0, phase = 0;
             bool ok = true;
+            TileIter T(P, SPLIT ? 0 : blockIdx.x);
             for (int ut = blockIdx.x; ut < (SPLIT ? P.n_units : P.n_tiles) && ok; ut += gridDim.x) {
-                const int t = SPLIT ? ut / P.ksplit : ut, sp = SPLIT ? ut - t * P.ksplit : 0;
-                (void)sp;
-                const int tm = t / P.tiles_n, tn = t % P.tiles_n;
-                const int ng = tm / per_img, r = tm - ng * per_img, n_img = ng * P.TN;
-                const int tq = P.rows_tma ? 1 : P.tiles_q;
-                const int hp0 = (r / tq) * P.TH * a.stride - a.pad, wq0 = (r % tq) * P.TW * a.stride - a.pad;
+                const int sp = SPLIT ? ut % P.ksplit : 0;
+                if (SPLIT) TileIter::split(P, ut / P.ksplit, T.tn, T.iq, T.ip, T.ng);
+                const int tm = T.ng, tn = T.tn, n_img = T.ng * P.TN;  // tm: TMA row tiles
+                const int hp0 = T.ip * P.TH * a.stride - a.pad, wq0 = T.iq * P.TW * a.stride - a.pad;
+                if (!SPLIT) T.next(P);
                 for (int gi = SPLIT ? P.gs[sp] : 0; gi < (SPLIT ? P.gs[sp + 1] : P.n_groups) && ok; ++gi) {
                     const TcGroup g = P.g[gi];
                     // tap (rr, ss) and channel offset cc of the group's first k-block, then stepped by
@@ -971,8 +1061,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     int rr = tp0 / a.S, ss = tp0 - rr * a.S;
                     int wx = P.patch == 1 ? tp0 * a.Cp + cc : g.kb0 * TC_BK;
                     for (int kb = g.kb0; kb < g.kb1; ++kb, ++it) {
-                        if ((int)((it % TC_STAGES) % TC_PRODUCERS) == me) {
-                            const uint32_t stage = it % TC_STAGES, phase = (it / TC_STAGES) & 1;
+                        if (stage % TC_PRODUCERS == me) {
                             if (!wait_warp(empty0 + 8 * stage, phase ^ 1, abort, P.status)) {
                                 ok = false;
                                 break;
@@ -1000,6 +1089,10 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                                           P.wpack + ((size_t)kb * P.K_pad + (size_t)tn * BN) * 2 * P.wk, pk_bytes, fb);
                             else
                                 tma_load_3d(smem_u32(sB + stage * B_BYTES), &P.tmap_w, wx, tn * BN, g.w_plane, fb);
+                        }
+                        if (++stage == TC_STAGES) {
+                            stage = 0;
+                            phase ^= 1;
                         }
                         wx += TC_BK;
                         if (!narrow) {
@@ -1124,14 +1217,12 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         // tile's store is then in flight).
         const int quad = warp & 3, cw = (warp - 4) >> 2;
         const int row = quad * 32 + lane;
-        const bool leader = threadIdx.x == 128;  // waits for and issues the TMA stores
         const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
         const int m = a.sh - 16;
         const int half = m > 0 ? 1 << (m - 1) : 0;
         const int mmask = (int)((1u << m) - 1u);
         const int lo = (int)a.lo, hi = (int)a.hi;
         const float flo = a.relu && lo < 0 ? 0.0f : (float)lo, fhi = (float)hi;
-        const int per_img = P.tiles_p * P.tiles_q;
         const bool f32out = a.out_mode == FXPQ_OUT_F32;  // the fp32 image (calibration) instead of codes
         // W64, 32-bit codes: a thread's 16 output channels are the same in every tile, so their aligned
         // bias terms and the flags of bias bits below the accumulator's scale are formed once
@@ -1144,7 +1235,9 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
             for (int j = 0; j < 16; ++j) {
                 const int k = cw * 16 + j;
                 const int32_t b = (a.has_bias && k < a.K) ? __ldg(a.bias + k) : 0;
-                btw[j] = P.fepi ? __float_as_int(a.has_bias ? fepi_bias(a, b) : 0.0f) : (b << e32w.bsl) >> e32w.bsr;
+                btw[j] = !P.fepi  ? (b << e32w.bsl) >> e32w.bsr
+                         : f32out ? __float_as_int((float)b * a.vi_b)
+                                  : __float_as_int(a.has_bias ? fepi_bias(a, b) : 0.0f);
                 phiw |= ((b & e32w.fmask) != 0 ? 1u : 0u) << j;
             }
         }
@@ -1166,7 +1259,11 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(accempty0 + 8 * buf);
-                if (f32out) {
+                if (f32out && P.fepi) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        w[j] = __float_as_uint(fepi_image(a, __uint_as_float(f[j]), __int_as_float(btw[j])));
+                } else if (f32out) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         const int k = cw * 16 + j;
@@ -1175,7 +1272,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         w[j] = __float_as_uint(__ll2float_rn(cblock_value<false>(a, k, (long long)acc, b)) * a.f32_scale);
                     }
                 }
-                if (P.fepi) {
+                if (!f32out && P.fepi) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
                         w[j] = fepi_pair(f[2 * j], f[2 * j + 1], cc2, __int_as_float(btw[2 * j]),
@@ -1280,15 +1377,10 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
             }
             const uint32_t sb = u & 1, n = u >> 1;  // staging tile and its use count
             const uint32_t sfull = sb ? stg_full2 : stg_full, sfree = sb ? stg_free2 : stg_free;
-            if (n > 0) {
-                if (leader) {
-                    bulk_wait_read1();  // the store of tile u - 2 (this staging tile) has read it
-                    mbar_arrive(sfree);
-                }
-                if (!wait_bounded(sfree, (n - 1) & 1, abort, P.status)) {
-                    ok = false;
-                    break;
-                }
+            // the store of tile u - 2 (this staging tile) must have read it
+            if (n > 0 && !wait_bounded(sfree, (n - 1) & 1, abort, P.status)) {
+                ok = false;
+                break;
             }
             unsigned char* sbuf = sO + sb * (TC_BM * 128);
 #pragma unroll
@@ -1300,17 +1392,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(sfull);
-            if (leader) {
-                if (!wait_bounded(sfull, n & 1, abort, P.status)) {
-                    ok = false;
-                    break;
-                }
-                const int n_img = t / per_img, r = t - n_img * per_img;
-                tma_store_4d(&P.tmap_y, 0, (r % P.tiles_q) * P.TW, (r / P.tiles_q) * P.TH, n_img, smem_u32(sbuf));
-                bulk_commit();
-            }
         }
-        if (leader) bulk_wait0();  // every output store has completed
     } else if (warp < MMA_WARP) {
         // ============================================================ epilogue
         // Warp w drains TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31 (the quadrant a warp may access) and
@@ -1318,7 +1400,6 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         const int quad = warp & 3;
         const int cw = (warp - 4) >> 2;
         const int row = quad * 32 + lane;
-        const bool leader = threadIdx.x == 128;  // waits for and issues the tile's TMA stores
         const int nbuf = P.nbuf;
         uint32_t gcount = 0;
         bool ok = true;
@@ -1326,12 +1407,17 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         // [nbuf BN, nbuf BN + BN * words), words = 1 (int32) or 2 (int64 as lo / hi column blocks).
         const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
         const uint32_t run_base = (uint32_t)(nbuf * BN);
-        uint32_t u = 0;  // tiles written through the staging buffer so far
+        uint32_t u = 0;  // tiles written through the staging tiles so far
+        const int place = row_in_tile(P, row);
+        TileIter T(P, SPLIT ? 0 : blockIdx.x);
         for (int ut = blockIdx.x; ut < (SPLIT ? P.n_units : P.n_tiles) && ok; ut += gridDim.x) {
-            const int t = SPLIT ? ut / P.ksplit : ut, sp = SPLIT ? ut - t * P.ksplit : 0;
-            (void)sp;
-            const int tm = t / P.tiles_n, tn = t % P.tiles_n;
-            const long long m = tile_row(P, tm, row);  // -1: row outside the output
+            const int sp = SPLIT ? ut % P.ksplit : 0;
+            if (SPLIT) TileIter::split(P, ut / P.ksplit, T.tn, T.iq, T.ip, T.ng);
+            const int tn = T.tn;
+            // -1: row outside the output (not needed where the TMA store clips)
+            const long long m = FE && !DIRECT && P.fast_store ? 0 : row_at(P, T, place, row);
+            if (!SPLIT) T.next(P);
+            unsigned char* const stg = sO + (NSTG == 2 ? (u & 1) * STG_BYTES : 0);  // this tile's staging tile
             const int g_lo = SPLIT ? P.gs[sp] : 0, g_hi = SPLIT ? P.gs[sp + 1] : P.n_groups;
             for (int gi = g_lo; gi < g_hi; ++gi) {
                 const int shift = P.g[gi].shift;
@@ -1343,22 +1429,18 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     break;
                 }
                 tc_fence_after();
-                if (!DIRECT && last && P.fast_store && u > 0) {
-                    // the previous tile's TMA store must have read the staging buffer
-                    if (leader) {
-                        bulk_wait_read0();
-                        mbar_arrive(stg_free);
-                    }
-                    if (!wait_bounded(stg_free, (u - 1) & 1, abort, P.status)) {
-                        ok = false;
-                        break;
-                    }
+                // the store of tile u - NSTG must have read this tile's staging tile
+                if (STORE_WARP && last && P.fast_store && u >= NSTG &&
+                    !wait_bounded(NSTG == 2 && (u & 1) ? stg_free2 : stg_free, (u / NSTG - 1) & 1, abort, P.status)) {
+                    ok = false;
+                    break;
                 }
 #pragma unroll 1
                 for (int c = 0; c < CPW; ++c) {
                     const int cb = cw * CPW + c;
                     const int k0 = tn * BN + cb * 32;
                     const uint32_t run_col = run_base + cb * 32;
+                    if constexpr (!FE) {
                     if (BN == 64 && sizeof(ACC) == 8 && !SC && P.patch == 3 && P.w32) {
                         // window mode, two-limb x and w, 32-bit arithmetic.  With the limb sums S_hh,
                         // S_mid = S_hl + S_lh, S_ll and the aligned bias B' = 2^16 Bh + Bl (0 <= Bl < 2^16):
@@ -1418,7 +1500,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                                 w[8 * hf + j] = pack_codes_f16(c2[0], c2[1]);
                             }
                         }
-                        unsigned char* half_buf = sO + (cb >> 1) * (TC_BM * 128);
+                        unsigned char* half_buf = stg + (cb >> 1) * (TC_BM * 128);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int chunk = (cb & 1) * 4 + q;
@@ -1471,7 +1553,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                                 w[8 * hf + j] = pack_codes_f16(c2[0], c2[1]);
                             }
                         }
-                        unsigned char* half_buf = sO + (cb >> 1) * (TC_BM * 128);
+                        unsigned char* half_buf = stg + (cb >> 1) * (TC_BM * 128);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int chunk = (cb & 1) * 4 + q;
@@ -1480,7 +1562,8 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         }
                         continue;
                     }
-                    if (sizeof(ACC) == 4 && !SC && !SPLIT && !PK && P.fepi) {
+                    }
+                    if constexpr (FE) {
                         // one exact group: codes straight from the fp32 sums
                         uint32_t f0[16], f1[16], w[16];
                         tmem_ld16_nw(lane_base + buf * BN + cb * 32, f0);
@@ -1488,12 +1571,14 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         // the chunk's 32 channel constants, one per lane, to every lane through shared
                         // memory that this warp overwrites with the codes afterwards
                         const int kl = k0 + lane;
-                        const float t = a.has_bias && kl < a.K ? fepi_bias(a, __ldg(a.bias + kl)) : 0.0f;
-                        unsigned char* wbuf = sO + (warp - 4) * 2048;                     // DIRECT
-                        unsigned char* half_buf = sO + (cb >> 1) * (TC_BM * 128);         // staged tile
+                        const bool image = a.out_mode == FXPQ_OUT_F32;
+                        const int32_t b = a.has_bias && kl < a.K ? __ldg(a.bias + kl) : 0;
+                        const float t = image ? (float)b * a.vi_b : a.has_bias ? fepi_bias(a, b) : 0.0f;
+                        unsigned char* wbuf = sO + (warp - 4) * 2048;                     // DIRECT, fp32 image
+                        unsigned char* half_buf = stg + (cb >> 1) * (TC_BM * 128);         // staged tile
                         // four constants 4 q .. 4 q + 3
                         auto tab = [&](int q) {
-                            return DIRECT ? wbuf + 16 * q
+                            return DIRECT || image ? wbuf + 16 * q
                                           : half_buf + (quad * 32 + (q >> 2)) * 128 + ((((cb & 1) * 4 + (q & 3)) ^ (q >> 2)) << 4);
                         };
                         *reinterpret_cast<float*>(tab(lane >> 2) + 4 * (lane & 3)) = t;
@@ -1505,6 +1590,21 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                             tc_fence_before();
                             __syncwarp();
                             if (lane == 0) mbar_arrive(accempty0 + 8 * buf);
+                        }
+                        if (image) {
+                            float v[32];
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                const float4 tq = *reinterpret_cast<const float4*>(tab(q));
+                                const uint32_t* f = q < 4 ? f0 + 4 * q : f1 + 4 * (q - 4);
+                                v[4 * q] = fepi_image(a, __uint_as_float(f[0]), tq.x);
+                                v[4 * q + 1] = fepi_image(a, __uint_as_float(f[1]), tq.y);
+                                v[4 * q + 2] = fepi_image(a, __uint_as_float(f[2]), tq.z);
+                                v[4 * q + 3] = fepi_image(a, __uint_as_float(f[3]), tq.w);
+                            }
+                            __syncwarp();
+                            store_f32_direct(a, m, k0, v, wbuf, lane);
+                            continue;
                         }
                         const uint64_t cc = f32x2_splat(a.vf_c);
 #pragma unroll
@@ -1525,8 +1625,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                                     make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
                             }
                         }
-                        continue;
-                    }
+                    } else {
                     // One TMEM round trip per load batch: the fp32 group sums and, after the first group,
                     // the integer running sums are loaded together; the running-sum stores share one
                     // completion wait.
@@ -1715,7 +1814,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                             store_codes_direct(a, m, k0, w, sO + (warp - 4) * 2048, lane);
                             continue;
                         }
-                        unsigned char* half_buf = sO + (cb >> 1) * (TC_BM * 128);
+                        unsigned char* half_buf = stg + (cb >> 1) * (TC_BM * 128);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const int chunk = (cb & 1) * 4 + q;
@@ -1724,40 +1823,57 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         }
                     } else if (!PK && (a.out_mode == FXPQ_OUT_F32 ? a.K % 4 == 0 : (a.out_mode == FXPQ_OUT_ACC64 && a.K % 2 == 0))) {
                         // fp32 / int64 outputs through the warp's 2 KiB of the (unused) staging tile
-                        epilogue_block32_staged<ACC, SC>(a, m, k0, acc, sO + (warp - 4) * 2048, lane);
+                        ACC v[32];
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] = acc[j];
+                        epilogue_block32_staged<ACC, SC>(a, m, k0, v, sO + (warp - 4) * 2048, lane);
                     } else if (m >= 0) {
-                        epilogue_block32<ACC, SC>(a, m, k0, acc);
+                        ACC v[32];
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] = acc[j];
+                        epilogue_block32<ACC, SC>(a, m, k0, v);
+                    }
                     }
                 }
                 ++gcount;
-                if (!DIRECT && last && P.fast_store) {
-                    // make the staging writes visible to the async proxy, then one thread stores the tile
+                if (STORE_WARP && last && P.fast_store) {
+                    // make the staging writes visible to the async proxy, then hand the tile to the store warp
                     fence_proxy_async();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(stg_full);
-                    if (leader) {
-                        if (!wait_bounded(stg_full, u & 1, abort, P.status)) {
-                            ok = false;
-                            break;
-                        }
-                        if (P.patch) {
-                            const int per_img = P.tiles_p * P.tiles_q;
-                            const int ng = tm / per_img, r = tm - ng * per_img, n_img = ng * P.TN;
-                            for (int hb = 0; hb < BN / 64; ++hb)
-                                tma_store_4d(&P.tmap_y, tn * BN + hb * 64, (r % P.tiles_q) * P.TW,
-                                             (r / P.tiles_q) * P.TH, n_img, smem_u32(sO + hb * (TC_BM * 128)));
-                        } else {
-                            for (int hb = 0; hb < BN / 64; ++hb)
-                                tma_store_2d(&P.tmap_y, tn * BN + hb * 64, tm * TC_BM,
-                                             smem_u32(sO + hb * (TC_BM * 128)));
-                        }
-                        bulk_commit();
-                    }
+                    if (lane == 0) mbar_arrive(NSTG == 2 && (u & 1) ? stg_full2 : stg_full);
                     ++u;
                 }
             }
         }
-        if (leader) bulk_wait0();  // every output store has completed
+    } else if (STORE_WARP && warp > MMA_WARP) {
+        // ============================================================ tile stores (one thread)
+        // Tile u goes out of staging tile u % NSTG once every epilogue warp has written it.  The tile is free
+        // again when the store has read it; with two tiles that is waited for with the next store in flight.
+        if (lane == 0 && P.fast_store) {
+            TileIter T(P, blockIdx.x);
+            uint32_t u = 0;
+            for (int t = blockIdx.x; t < P.n_tiles; t += gridDim.x, ++u) {
+                const uint32_t sb = u % NSTG;
+                if (!wait_bounded(sb ? stg_full2 : stg_full, (u / NSTG) & 1, abort, P.status)) break;
+                for (int hb = 0; hb < BN / 64; ++hb) {
+                    const uint32_t src = smem_u32(sO + sb * STG_BYTES + hb * (TC_BM * 128));
+                    if (P.patch)
+                        tma_store_4d(&P.tmap_y, T.tn * BN + hb * 64, T.iq * P.TW, T.ip * P.TH, T.ng * P.TN, src);
+                    else
+                        tma_store_2d(&P.tmap_y, T.tn * BN + hb * 64, T.ng * TC_BM, src);
+                }
+                bulk_commit();
+                if (NSTG == 1) {
+                    bulk_wait_read0();
+                    mbar_arrive(stg_free);
+                } else if (u >= 1) {
+                    bulk_wait_read1();  // the store of tile u - 1 has read the other staging tile
+                    mbar_arrive(sb ? stg_free : stg_free2);
+                }
+                T.next(P);
+            }
+            bulk_wait0();  // every output store has completed
+        }
     } else if (PK && warp > MMA_WARP) {
         // ============================================================ packed-weight converters
         pk_convert_loop<BN, SPLIT>(P, 3 + (warp - MMA_WARP - 1), lane, sP, sB, pkfull0, full0, abort);
