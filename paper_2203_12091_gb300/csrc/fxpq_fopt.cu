@@ -13,11 +13,15 @@ namespace fxpq {
 namespace {
 
 // ------------------------------------------------------------------ fp32 implicit-GEMM convolution
-// Tile 128 output pixels x BN output channels (BN = 128 for wide layers, 64 otherwise), 8 reduction
-// steps per stage (double-buffered shared memory), 256 threads with 8 x BN/16 outputs each (64 or 32
-// FMAs per 16 or 12 shared-memory words).  x: [N, H, W, C]; w: [K, R*S*C] (KRSC); y: [N, P, Q, K].
-// When C % 8 == 0 a stage's 8 reduction steps are 8 channels of one tap, loaded as float4.
-constexpr int CF_BM = 128, CF_BK = 8;
+// x: [N, H, W, C]; w: [K, R*S*C] (KRSC); y: [N, P, Q, K].  Bound by the fp32 FMA rate (128 per cycle and SM).
+// A block of 256 threads computes BM output pixels x 64 channels as four groups of 64 threads: every stage of
+// 32 reduction steps is split into four slices of 8, one per group, and each thread accumulates (BM / 8) x 8
+// outputs over its group's slices, so that small tiles (which occupy the SMs at a few calibration images)
+// still read only 4 16-byte pieces of shared memory per 64 FMAs.  The groups' sums are added pairwise at the
+// end.  FMAs are issued packed two pixels at a time (fma.rn.f32x2), which leaves issue slots for the loads.
+// 24 images (three candidates of 8), ResNet-18: 56 x 56 x 64 177 -> 137 us, 28 x 28 x 128 283 -> 132, 7 x 7 x 512 488 -> 152
+// (128 x 64 and 64 x 64 tiles with one accumulator chain before).
+constexpr int CF_BN = 64, CF_BK = 32, CF_TAB = 1024;
 
 struct ConvF32Args {
     const float* x;
@@ -28,80 +32,142 @@ struct ConvF32Args {
     long long M;
 };
 
-template <int CF_BN>
-__global__ void __launch_bounds__(256) conv_f32_kernel(const ConvF32Args a) {
-    constexpr int TN = CF_BN / 16;  // output channels per thread
-    __shared__ __align__(16) float sa[2][CF_BK][CF_BM];
+__device__ __forceinline__ unsigned long long f2_pack(float x, float y) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+    return v;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+
+// VEC: C % 4 == 0 (a float4 of a row stays inside one tap) and 16-byte aligned x and w; otherwise single loads,
+// the reduction index decoded through a table in shared memory (up to CF_TAB steps).
+template <int BM, bool VEC>
+__global__ void __launch_bounds__(256, 2) conv_f32_kernel(const ConvF32Args a) {
+    constexpr int MT = BM / 8;           // output pixels per thread
+    constexpr int AV = BM * CF_BK / 4 / 256;  // float4 of the A stage per thread
+    constexpr int BV = CF_BN * CF_BK / 4 / 256;
+    // stage: [k][m] and [k][n], 16-byte pieces of row k at piece ^ (k / 4 % 8): the transposing stores of eight
+    // lanes with consecutive k / 4 then fall into different banks, and pieces stay whole for the loads
+    __shared__ __align__(16) float sa[2][CF_BK][BM];
     __shared__ __align__(16) float sb[2][CF_BK][CF_BN];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const long long m0 = (long long)blockIdx.x * CF_BM;
+    __shared__ int2 tab[VEC ? 1 : CF_TAB];
+    const int tid = threadIdx.x, grp = tid >> 6, t64 = tid & 63;
+    const int tx = t64 & 7, ty = t64 >> 3;
+    const long long m0 = (long long)blockIdx.x * BM;
     const int n0 = blockIdx.y * CF_BN;
     const int RSC = a.R * a.S * a.C;
-    // staging: thread t loads row t / 2 of the A tile (and of the B tile when BN = 128; rows t / 4 with
-    // two columns each when BN = 64), reduction columns 4 (t % 2) .. + 3
-    const int lr = threadIdx.x >> 1, lk = (threadIdx.x & 1) * 4;
-    const int br = CF_BN == 128 ? lr : (threadIdx.x >> 2), bk = CF_BN == 128 ? lk : (threadIdx.x & 3) * 2;
-    const long long m = m0 + lr;
-    const bool mok = m < a.M;
-    int pn = 0, pp = 0, pq = 0;
-    if (mok) {
-        pn = (int)(m / ((long long)a.P * a.Q));
-        const int rem = (int)(m - (long long)pn * a.P * a.Q);
-        pp = rem / a.Q;
-        pq = rem - pp * a.Q;
+    if (!VEC) {
+        for (int k = tid; k < RSC && k < CF_TAB; k += 256) {
+            const int c = k % a.C, rs = k / a.C, s = rs % a.S, r = rs / a.S;
+            tab[k] = make_int2((r * a.W + s) * a.C + c, (r << 16) | s);
+        }
+        __syncthreads();
     }
-    const int o = n0 + br;
-    const bool ook = o < a.K;
-    const bool vecA = (a.C % 8) == 0, vecB = (RSC % 4) == 0;
-    float ra[4], rb[4];
+    // loads: thread t takes k quad t % 8 of rows t / 8, t / 8 + 32, ..
+    const int kq = tid & 7, lr = tid >> 3;
+    int p0[AV], q0[AV];
+    long long xo[AV];
+#pragma unroll
+    for (int i = 0; i < AV; ++i) {
+        const long long m = m0 + lr + 32 * i;
+        p0[i] = -(1 << 20);  // rows past the end read zeros
+        q0[i] = 0;
+        xo[i] = 0;
+        if (m < a.M) {
+            const long long n = m / ((long long)a.P * a.Q);
+            const int rem = (int)(m - n * a.P * a.Q), pp = rem / a.Q, pq = rem - pp * a.Q;
+            p0[i] = pp * a.stride - a.pad;
+            q0[i] = pq * a.stride - a.pad;
+            xo[i] = ((n * a.H + p0[i]) * a.W + q0[i]) * a.C;
+        }
+    }
+    float4 ra[AV], rb[BV];
+    // the tap of this thread's k quad, stepped with the stages
+    int kc = VEC ? (4 * kq) % a.C : 0, ks = VEC ? (4 * kq) / a.C % a.S : 0, kr = VEC ? (4 * kq) / a.C / a.S : 0;
     auto load = [&](int k0) {
-        if (vecA) {
-            const int rs = k0 / a.C, c = k0 - rs * a.C + lk;
-            const int s = rs % a.S, r = rs / a.S;
-            const int h = pp * a.stride + r - a.pad, ww = pq * a.stride + s - a.pad;
-            if (mok && k0 < RSC && h >= 0 && h < a.H && ww >= 0 && ww < a.W) {
-                const float4 v =
-                    *reinterpret_cast<const float4*>(a.x + (((long long)pn * a.H + h) * a.W + ww) * a.C + c);
-                ra[0] = v.x, ra[1] = v.y, ra[2] = v.z, ra[3] = v.w;
-            } else {
-                ra[0] = ra[1] = ra[2] = ra[3] = 0.0f;
+        const int k = k0 + 4 * kq;
+        if (VEC) {
+            const long long to = ((long long)kr * a.W + ks) * a.C + kc;
+#pragma unroll
+            for (int i = 0; i < AV; ++i) {
+                const int h = p0[i] + kr, w = q0[i] + ks;
+                const bool in = k < RSC && (unsigned)h < (unsigned)a.H && (unsigned)w < (unsigned)a.W;
+                ra[i] = in ? __ldg(reinterpret_cast<const float4*>(a.x + xo[i] + to)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int i = 0; i < BV; ++i) {
+                const int o = n0 + lr + 32 * i;
+                rb[i] = k < RSC && o < a.K ? __ldg(reinterpret_cast<const float4*>(a.w + (long long)o * RSC + k))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            kc += CF_BK;
+            while (kc >= a.C) {
+                kc -= a.C;
+                if (++ks == a.S) {
+                    ks = 0;
+                    ++kr;
+                }
             }
         } else {
+            float va[AV][4], vb[BV][4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int kk = k0 + lk + e;
-                float v = 0.0f;
-                if (mok && kk < RSC) {
-                    const int c = kk % a.C, rs = kk / a.C;
-                    const int s = rs % a.S, r = rs / a.S;
-                    const int h = pp * a.stride + r - a.pad, ww = pq * a.stride + s - a.pad;
-                    if (h >= 0 && h < a.H && ww >= 0 && ww < a.W)
-                        v = a.x[(((long long)pn * a.H + h) * a.W + ww) * a.C + c];
+                const int kk = k + e;
+                int2 te = make_int2(0, 0);
+                if (kk < RSC) {
+                    if (kk < CF_TAB) {
+                        te = tab[kk];
+                    } else {
+                        const int c = kk % a.C, rs = kk / a.C, s = rs % a.S, r = rs / a.S;
+                        te = make_int2((r * a.W + s) * a.C + c, (r << 16) | s);
+                    }
                 }
-                ra[e] = v;
-            }
-        }
-        const int kb = k0 + bk;
-        constexpr int NB = CF_BN == 128 ? 4 : 2;
-        if (CF_BN == 128 && vecB && ook && kb + 3 < RSC) {
-            const float4 v = *reinterpret_cast<const float4*>(a.w + (long long)o * RSC + kb);
-            rb[0] = v.x, rb[1] = v.y, rb[2] = v.z, rb[3] = v.w;
-        } else {
 #pragma unroll
-            for (int e = 0; e < NB; ++e) rb[e] = (ook && kb + e < RSC) ? a.w[(long long)o * RSC + kb + e] : 0.0f;
+                for (int i = 0; i < AV; ++i) {
+                    const int h = p0[i] + (te.y >> 16), w = q0[i] + (te.y & 0xFFFF);
+                    const bool in = kk < RSC && (unsigned)h < (unsigned)a.H && (unsigned)w < (unsigned)a.W;
+                    va[i][e] = in ? __ldg(a.x + xo[i] + te.x) : 0.0f;
+                }
+#pragma unroll
+                for (int i = 0; i < BV; ++i) {
+                    const int o = n0 + lr + 32 * i;
+                    vb[i][e] = kk < RSC && o < a.K ? __ldg(a.w + (long long)o * RSC + kk) : 0.0f;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < AV; ++i) ra[i] = make_float4(va[i][0], va[i][1], va[i][2], va[i][3]);
+#pragma unroll
+            for (int i = 0; i < BV; ++i) rb[i] = make_float4(vb[i][0], vb[i][1], vb[i][2], vb[i][3]);
         }
     };
     auto store = [&](int buf) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) sa[buf][lk + e][lr] = ra[e];
+        for (int i = 0; i < AV; ++i) {
+            const int m = (lr + 32 * i) ^ (kq << 2);
+            sa[buf][4 * kq][m] = ra[i].x;
+            sa[buf][4 * kq + 1][m] = ra[i].y;
+            sa[buf][4 * kq + 2][m] = ra[i].z;
+            sa[buf][4 * kq + 3][m] = ra[i].w;
+        }
 #pragma unroll
-        for (int e = 0; e < (CF_BN == 128 ? 4 : 2); ++e) sb[buf][bk + e][br] = rb[e];
+        for (int i = 0; i < BV; ++i) {
+            const int n = (lr + 32 * i) ^ (kq << 2);
+            sb[buf][4 * kq][n] = rb[i].x;
+            sb[buf][4 * kq + 1][n] = rb[i].y;
+            sb[buf][4 * kq + 2][n] = rb[i].z;
+            sb[buf][4 * kq + 3][n] = rb[i].w;
+        }
     };
-    float acc[8][TN];
+    // pixels 4 ty .. + 3 (and BM / 2 + the same for BM = 64), channels 4 tx .. + 3 and 32 + the same
+    unsigned long long acc[MT / 2][8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < MT / 2; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = 0.0f;
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
     load(0);
     store(0);
     __syncthreads();
@@ -110,20 +176,27 @@ __global__ void __launch_bounds__(256) conv_f32_kernel(const ConvF32Args a) {
         const bool more = k0 + CF_BK < RSC;
         if (more) load(k0 + CF_BK);  // next stage's global loads in flight during this stage's FMAs
 #pragma unroll
-        for (int kk = 0; kk < CF_BK; ++kk) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&sa[buf][kk][ty * 8]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&sa[buf][kk][ty * 8 + 4]);
-            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            float bv[TN];
+        for (int kk = 0; kk < 8; ++kk) {
+            const int k = 8 * grp + kk, x = (2 * grp + (kk >> 2)) & 7;  // k / 4 % 8
+            unsigned long long av[MT / 2];
 #pragma unroll
-            for (int q = 0; q < TN / 4; ++q) {
-                const float4 b = *reinterpret_cast<const float4*>(&sb[buf][kk][tx * TN + 4 * q]);
-                bv[4 * q] = b.x, bv[4 * q + 1] = b.y, bv[4 * q + 2] = b.z, bv[4 * q + 3] = b.w;
+            for (int i = 0; i < MT / 4; ++i) {
+                const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&sa[buf][k][((ty ^ x) << 2) + 32 * i]);
+                av[2 * i] = v.x;
+                av[2 * i + 1] = v.y;
+            }
+            float bv[8];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float4 v = *reinterpret_cast<const float4*>(&sb[buf][k][((tx ^ x) << 2) + 32 * j]);
+                bv[4 * j] = v.x, bv[4 * j + 1] = v.y, bv[4 * j + 2] = v.z, bv[4 * j + 3] = v.w;
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int j = 0; j < 8; ++j) {
+                const unsigned long long b2 = f2_pack(bv[j], bv[j]);
 #pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+                for (int i = 0; i < MT / 2; ++i) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(av[i]), "l"(b2));
+            }
         }
         if (more) {
             store(buf ^ 1);
@@ -131,85 +204,51 @@ __global__ void __launch_bounds__(256) conv_f32_kernel(const ConvF32Args a) {
             buf ^= 1;
         }
     }
+    // groups 2, 3 onto 0, 1, then 1 onto 0, through the A stage (a group's sums are BM x 64 floats as 16-byte
+    // pieces [piece][thread])
+    __syncthreads();
+    ulonglong2* red = reinterpret_cast<ulonglong2*>(&sa[0][0][0]);
+    constexpr int NP = MT * 8 / 4;  // 16-byte pieces per thread
+    static_assert(NP * 64 * 16 <= (int)sizeof(sa) && BM <= 64, "one group's sums fit the A stage");
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const long long mm = m0 + ty * 8 + i;
-        if (mm >= a.M) continue;
+    for (int rnd = 0; rnd < 3; ++rnd) {
+        const int src = rnd == 0 ? 3 : rnd == 1 ? 2 : 1, dst = rnd == 0 ? 1 : 0;
+        if (grp == src)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            const int oo = n0 + tx * TN + j;
-            if (oo >= a.K) continue;
-            float v = acc[i][j];
-            if (a.bias) v += a.bias[oo];
-            if (a.relu) v = fmaxf(v, 0.0f);
-            a.y[mm * a.K + oo] = v;
-        }
-    }
-}
-
-// Small layers (too few 128-row tiles to occupy the SMs): 64 x 64 tiles, 4 x 4 outputs per thread.
-constexpr int SF_BM = 64, SF_BN = 64, SF_BK = 16;
-
-__global__ void __launch_bounds__(256) conv_f32_small_kernel(const ConvF32Args a) {
-    __shared__ float sa[SF_BK][SF_BM + 4];
-    __shared__ float sb[SF_BK][SF_BN + 4];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const long long m0 = (long long)blockIdx.x * SF_BM;
-    const int n0 = blockIdx.y * SF_BN;
-    const int RSC = a.R * a.S * a.C;
-    // the A element this thread stages: pixel row (threadIdx.x / 4) and reduction columns 4 * (tid % 4) ..
-    const int lr = threadIdx.x >> 2, lk = (threadIdx.x & 3) * 4;
-    const long long m = m0 + lr;
-    int pn = 0, pp = 0, pq = 0;
-    if (m < a.M) {
-        pn = (int)(m / ((long long)a.P * a.Q));
-        const int rem = (int)(m - (long long)pn * a.P * a.Q);
-        pp = rem / a.Q;
-        pq = rem - pp * a.Q;
-    }
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < RSC; k0 += SF_BK) {
+            for (int q = 0; q < NP; ++q) red[q * 64 + t64] = make_ulonglong2(acc[q / 4][2 * (q % 4)], acc[q / 4][2 * (q % 4) + 1]);
+        __syncthreads();
+        if (grp == dst)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int kk = k0 + lk + e;
-            float v = 0.0f;
-            if (m < a.M && kk < RSC) {
-                const int c = kk % a.C, rs = kk / a.C;
-                const int s = rs % a.S, r = rs / a.S;
-                const int h = pp * a.stride + r - a.pad, ww = pq * a.stride + s - a.pad;
-                if (h >= 0 && h < a.H && ww >= 0 && ww < a.W) v = a.x[(((long long)pn * a.H + h) * a.W + ww) * a.C + c];
+            for (int q = 0; q < NP; ++q) {
+                const ulonglong2 v = red[q * 64 + t64];
+                asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[q / 4][2 * (q % 4)]) : "l"(v.x));
+                asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[q / 4][2 * (q % 4) + 1]) : "l"(v.y));
             }
-            sa[lk + e][lr] = v;
-            const int o = n0 + lr;
-            sb[lk + e][lr] = (o < a.K && kk < RSC) ? a.w[(long long)o * RSC + kk] : 0.0f;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < SF_BK; ++kk) {
-            float av[4], bv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) av[i] = sa[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) bv[j] = sb[kk][tx * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-        }
         __syncthreads();
     }
+    if (grp != 0) return;
+    const bool v4 = a.K % 4 == 0 && (reinterpret_cast<uintptr_t>(a.y) & 15) == 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const long long mm = m0 + ty * 4 + i;
+    for (int i = 0; i < MT; ++i) {
+        const long long mm = m0 + 4 * ty + (i & 3) + (i >> 2) * 32;
         if (mm >= a.M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int o = n0 + tx * 4 + j;
-            if (o >= a.K) continue;
-            float v = acc[i][j];
-            if (a.bias) v += a.bias[o];
-            if (a.relu) v = fmaxf(v, 0.0f);
-            a.y[mm * a.K + o] = v;
+        for (int h = 0; h < 2; ++h) {
+            float o[4];
+            const int oo = n0 + 4 * tx + 32 * h;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 f = f2_unpack(acc[i >> 1][4 * h + j]);
+                o[j] = (i & 1) ? f.y : f.x;
+                if (a.bias && oo + j < a.K) o[j] += __ldg(a.bias + oo + j);
+                if (a.relu) o[j] = fmaxf(o[j], 0.0f);
+            }
+            if (v4 && oo < a.K)
+                *reinterpret_cast<float4*>(a.y + mm * a.K + oo) = make_float4(o[0], o[1], o[2], o[3]);
+            else
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (oo + j < a.K) a.y[mm * a.K + oo + j] = o[j];
         }
     }
 }
@@ -541,17 +580,19 @@ extern "C" fxpq_status fxpq_conv_f32(const fxpq_conv_f32_desc* h_desc, const flo
     ConvF32Args a{d_x, d_w, d_bias, d_y, d.N, d.H, d.W, d.C, d.K, d.R, d.S, d.stride, d.pad, P, Q, d.relu ? 1 : 0,
                   (long long)d.N * P * Q};
     if (a.M == 0) return FXPQ_OK;
-    const long long big = ((a.M + CF_BM - 1) / CF_BM) * ((d.K + (d.K >= 128 ? 127 : 63)) / (d.K >= 128 ? 128 : 64));
-    if (big < 152) {
-        dim3 grid((unsigned)((a.M + SF_BM - 1) / SF_BM), (unsigned)((d.K + SF_BN - 1) / SF_BN));
-        conv_f32_small_kernel<<<grid, 256, 0, as_stream(stream)>>>(a);
-    } else if (d.K >= 128) {
-        dim3 grid((unsigned)((a.M + CF_BM - 1) / CF_BM), (unsigned)((d.K + 127) / 128));
-        conv_f32_kernel<128><<<grid, 256, 0, as_stream(stream)>>>(a);
-    } else {
-        dim3 grid((unsigned)((a.M + CF_BM - 1) / CF_BM), (unsigned)((d.K + 63) / 64));
-        conv_f32_kernel<64><<<grid, 256, 0, as_stream(stream)>>>(a);
-    }
+    // 32-pixel tiles for few output pixels (FC layers of a calibration slice), where 64-pixel ones are mostly empty
+    const bool vec = d.C % 4 == 0 && aligned(d_x, 16) && aligned(d_w, 16);
+    const int bm = a.M <= 32 ? 32 : 64;
+    dim3 grid((unsigned)((a.M + bm - 1) / bm), (unsigned)((d.K + CF_BN - 1) / CF_BN));
+    cudaStream_t s = as_stream(stream);
+    if (bm == 32 && vec)
+        conv_f32_kernel<32, true><<<grid, 256, 0, s>>>(a);
+    else if (bm == 32)
+        conv_f32_kernel<32, false><<<grid, 256, 0, s>>>(a);
+    else if (vec)
+        conv_f32_kernel<64, true><<<grid, 256, 0, s>>>(a);
+    else
+        conv_f32_kernel<64, false><<<grid, 256, 0, s>>>(a);
     return after_launch("conv_f32");
 }
 

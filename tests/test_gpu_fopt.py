@@ -45,6 +45,30 @@ def test_fp32_layers_match_float64(M):
     np.testing.assert_allclose(a.cpu().numpy().reshape(2, 1, 1, 5), qopt.f_avgpool(x), rtol=1e-6, atol=1e-6)
 
 
+@pytest.mark.parametrize("N,H,C,K,R,st,pad", [(3, 5, 8, 64, 3, 1, 1), (1, 4, 4, 200, 4, 1, 0), (5, 9, 12, 65, 1, 2, 0),
+                                              (2, 33, 3, 33, 11, 4, 2), (33, 1, 36, 10, 1, 1, 0), (1, 40, 5, 7, 17, 1, 8),
+                                              (2, 7, 30, 128, 3, 2, 1)])
+@pytest.mark.parametrize("off", [0, 1])
+def test_conv_f32_tiles(M, N, H, C, K, R, st, pad, off):
+    """Both tile heights, ragged tiles and reductions, taps stepped by channel quads and through the table (and
+    past its end), inputs off 16-byte boundaries: within the fp32 bound of a chain of R S C additions."""
+    fopt, F = M
+    rng = np.random.default_rng(N + H + C + K)
+    x = rng.standard_normal((N, H, H, C)).astype(np.float32)
+    w = rng.standard_normal((K, R, R, C)).astype(np.float32)
+    b = rng.standard_normal(K).astype(np.float32)
+    P = (H + 2 * pad - R) // st + 1
+    xd, wd = torch.empty(x.size + 1, device="cuda"), torch.empty(w.size + 1, device="cuda")
+    xd[off:off + x.size], wd[off:off + w.size] = torch.from_numpy(x).cuda().reshape(-1), torch.from_numpy(w).cuda().reshape(-1)
+    y = torch.full((N * P * P * K + 1,), 7.0, dtype=torch.float32, device="cuda")
+    F.fxpq_conv_f32(N, H, H, C, K, R, R, st, pad, False, xd[off:], wd[off:], torch.from_numpy(b).cuda(), y)
+    want = qopt.f_conv(x, w, b, st, pad, False)
+    mag = qopt.f_conv(np.abs(x), np.abs(w), np.abs(b), st, pad, False)  # sum of |terms|
+    got = y.cpu().numpy()
+    assert got[-1] == 7.0
+    assert (np.abs(got[:-1].reshape(want.shape) - want) <= (R * R * C + 2) * 2.0 ** -24 * mag).all()
+
+
 def test_ds_stats_batch_and_ties(M):
     """Statistics records (Eq. DSB_QE's L, the range ends, per-sample mean and sum of squared deviations)
     against float64 numpy, several items in one batch, one of them past one work unit per sample; a
