@@ -374,6 +374,46 @@ __device__ __forceinline__ double ds_block_sum(double v, double* red) {
     return t;  // valid in thread 0
 }
 
+// The sums of these kernels run in triples of fp32: every addition's rounding error is carried into the next
+// word (TwoSum), so that a thread's chain keeps about 70 bits, and it meets fp64 once, at the end.  fp64
+// arithmetic has 1/64 of the fp32 rate here (two operations per cycle and SM): the twelve operations per
+// element of the direct fp64 form were these kernels' time (95 M values of three ResNet-18 candidates: sums
+// 555 -> 132 us, deviations 2950 -> 608 us), and its rounding per addition was the larger one.
+constexpr int DS_U = 8;  // values per thread and step (their loads are issued together)
+
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+    const float t = a + b, z = t - a, r = (a - (t - z)) + (b - z);
+    err = r;
+    return t;
+}
+struct Sum3 {
+    float a = 0.0f, b = 0.0f, c = 0.0f;
+    __device__ __forceinline__ void low(float v) {  // v well below the terms of add
+        float e;
+        b = two_sum(b, v, e);
+        c += e;
+    }
+    __device__ __forceinline__ void add(float v) {
+        float e;
+        a = two_sum(a, v, e);
+        low(e);
+    }
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+
+// f(value) for a unit's values, DS_U per thread and step, consecutive threads in consecutive places.
+template <typename F>
+__device__ __forceinline__ void ds_walk(const float* __restrict__ xs, long long i0, long long i1, F f) {
+    for (long long i = i0 + threadIdx.x; i < i1; i += (long long)DS_U * DS_T) {
+        float v[DS_U];
+#pragma unroll
+        for (int j = 0; j < DS_U; ++j) v[j] = i + (long long)j * DS_T < i1 ? __ldg(xs + i + (long long)j * DS_T) : 0.0f;
+#pragma unroll
+        for (int j = 0; j < DS_U; ++j)
+            if (i + (long long)j * DS_T < i1) f(v[j]);
+    }
+}
+
 __global__ void __launch_bounds__(DS_T) ds_sum_kernel(const __grid_constant__ DsBatchDev B, DsUnit* units) {
     __shared__ double red[DS_T / 32];
     const int u = blockIdx.x;
@@ -381,9 +421,9 @@ __global__ void __launch_bounds__(DS_T) ds_sum_kernel(const __grid_constant__ Ds
     const int rel = u - it.unit0, s = rel / it.chunks, c = rel % it.chunks;
     const float* xs = it.x + (long long)s * it.nu;
     const long long i0 = (long long)c * DS_CHUNK, i1 = min(i0 + DS_CHUNK, it.nu);
-    double acc = 0.0;
-    for (long long i = i0 + threadIdx.x; i < i1; i += DS_T) acc += (double)xs[i];
-    const double t = ds_block_sum(acc, red);
+    Sum3 acc;
+    ds_walk(xs, i0, i1, [&](float v) { acc.add(v); });
+    const double t = ds_block_sum(acc.value(), red);
     if (threadIdx.x == 0) units[u].sum = t;
 }
 
@@ -403,19 +443,49 @@ __global__ void __launch_bounds__(DS_T) ds_dev_kernel(const __grid_constant__ Ds
     const double scale = ldexp(1.0, it.fl), inv = ldexp(1.0, -it.fl);
     const double lo = it.S ? -ldexp(1.0, it.k - 1) : 0.0, hi = ldexp(1.0, it.k - it.S) - 1.0;
     const bool binary = it.k == 1 && it.S == 1;
-    double m2 = 0.0, l2 = 0.0;
+    // In units of 2^-fl (y = x 2^fl), for k <= 16: the code q and r = y - q are exact in fp32 when y is zero or
+    // 2^-40 <= |y| < 2^24 (a smaller one's square could leave fp32's range), r^2 and y less the mean (mh + ml + mq)
+    // are exact as pairs, but for the last bits of the smaller word.  Other values take the fp64 form.
+    const float fscale = (float)scale, flo = (float)lo, fhi = (float)hi;
+    const double my = mean * scale;
+    const float mh = (float)my, ml = (float)(my - (double)mh), mq = (float)(my - (double)mh - (double)ml);
+    const bool narrow = it.k <= 16 && !binary && fabs(my) < 16777216.0 && (my == 0.0 || fabs(my) > 0x1p-40);
+    double m2 = 0.0, l2 = 0.0;  // the fp64 form's sums, in units of x
+    Sum3 m2y, l2y;              // in units of y
     unsigned mn = 0xFFFFFFFFu, mx = 0u;
-    for (long long i = i0 + threadIdx.x; i < i1; i += DS_T) {
-        const float v = xs[i];
-        const double d = (double)v;
-        const double q = binary ? (v < 0.0f ? -inv : inv) : fmin(fmax(nearbyint(d * scale), lo), hi) * inv;
-        const double e = d - q, dv = d - mean;
-        l2 += e * e;
-        m2 += dv * dv;
+    ds_walk(xs, i0, i1, [&](float v) {
         const unsigned key = ord_key(v);
         mn = min(mn, key);
         mx = max(mx, key);
-    }
+        const float y = v * fscale, ay = fabsf(y);
+        if (narrow && (v == 0.0f || (ay < 16777216.0f && ay > 0x1p-40f))) {
+            const float q = (fminf(fmaxf(y, flo), fhi) + 12582912.0f) - 12582912.0f;
+            // (_rn: products are not contracted into the sums)
+            const float r = y - q, p = __fmul_rn(r, r);
+            l2y.add(p);
+            l2y.low(fmaf(r, r, -p));
+            // y - mean = d + e + g, each below half a unit of the last place of the one before; its square
+            // d^2 + 2 d e + (2 d g + e^2)
+            float e, g;
+            float d = two_sum(y, -mh, e);
+            e = two_sum(e, -ml, g);
+            d = two_sum(d, e, e);
+            g -= mq;
+            const float w = __fmul_rn(d, d), d2 = 2.0f * d, c = __fmul_rn(d2, e);
+            m2y.add(w);
+            m2y.low(fmaf(d, d, -w));
+            m2y.low(c);
+            m2y.c += fmaf(d2, e, -c) + fmaf(d2, g, __fmul_rn(e, e));
+        } else {
+            const double x = (double)v;
+            const double q = binary ? (v < 0.0f ? -inv : inv) : fmin(fmax(nearbyint(x * scale), lo), hi) * inv;
+            const double e = x - q, dv = x - mean;
+            l2 += e * e;
+            m2 += dv * dv;
+        }
+    });
+    l2 += l2y.value() * inv * inv;
+    m2 += m2y.value() * inv * inv;
     if (threadIdx.x == 0) {
         kmn = 0xFFFFFFFFu;
         kmx = 0u;
@@ -441,14 +511,21 @@ __device__ __forceinline__ float ds_key_value(unsigned k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
 
-// One thread per item: its record from its units, in unit order.
-__global__ void ds_finish_kernel(const __grid_constant__ DsBatchDev B, const DsUnit* units) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B.n) return;
-    const DsItemDev& it = B.it[i];
+// One block per item: its record from its units, a thread per sample adding the sample's units in order, then
+// thread 0 the threads' shares of L in order.
+constexpr int DF_T = 64;
+__global__ void __launch_bounds__(DF_T) ds_finish_kernel(const __grid_constant__ DsBatchDev B, const DsUnit* units) {
+    __shared__ double l2s[DF_T];
+    __shared__ unsigned kmn, kmx;
+    const DsItemDev& it = B.it[blockIdx.x];
+    if (threadIdx.x == 0) {
+        kmn = 0xFFFFFFFFu;
+        kmx = 0u;
+    }
+    __syncthreads();
     double l2 = 0.0;
     unsigned mn = 0xFFFFFFFFu, mx = 0u;
-    for (int s = 0; s < it.n_samples; ++s) {
+    for (int s = threadIdx.x; s < it.n_samples; s += DF_T) {
         double sum = 0.0, m2 = 0.0;
         for (int c = 0; c < it.chunks; ++c) {
             const DsUnit& q = units[it.unit0 + s * it.chunks + c];
@@ -461,9 +538,16 @@ __global__ void ds_finish_kernel(const __grid_constant__ DsBatchDev B, const DsU
         it.out[3 + 2 * s] = sum / (double)it.nu;
         it.out[4 + 2 * s] = m2;
     }
-    it.out[0] = l2;
-    it.out[1] = (double)ds_key_value(mn);
-    it.out[2] = (double)ds_key_value(mx);
+    l2s[threadIdx.x] = l2;
+    atomicMin(&kmn, mn);
+    atomicMax(&kmx, mx);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double t = 0.0;
+    for (int i = 0; i < DF_T && i < it.n_samples; ++i) t += l2s[i];
+    it.out[0] = t;
+    it.out[1] = (double)ds_key_value(kmn);
+    it.out[2] = (double)ds_key_value(kmx);
 }
 
 // ---------------------------------------------------------------- the cost F of Alg. 1
@@ -477,13 +561,16 @@ struct CostTerms {
     CostTermDev t[COST_MAX_TERMS];
 };
 
-// One block per candidate; thread 0 adds the terms in order (a few dozen per network).
+// One block per candidate: a thread per term forms its sigma nu (square roots and divisions in fp64, one per
+// sample, are the kernel's time), then thread 0 adds the terms in order (a few dozen per network).
 __global__ void fopt_cost_kernel(const double* __restrict__ stats, long long cand_stride,
                                  const __grid_constant__ CostTerms T, const int* __restrict__ ties, int N,
                                  int n_classes, double* __restrict__ cost) {
     const int c = blockIdx.x;
     const double* base = stats + (long long)c * cand_stride;
     __shared__ unsigned n_tied, extra;
+    __shared__ double snu[COST_MAX_TERMS];  // the terms' sigma nu
+    __shared__ double lr[COST_MAX_TERMS];   // and L / R (0 where R = 0)
     if (threadIdx.x == 0) n_tied = extra = 0u;
     __syncthreads();
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
@@ -491,32 +578,28 @@ __global__ void fopt_cost_kernel(const double* __restrict__ stats, long long can
         if (k > 1) atomicAdd(&n_tied, 1u);
         atomicAdd(&extra, (unsigned)(k - 1));
     }
+    for (int t = threadIdx.x; t < T.n; t += blockDim.x) {
+        const CostTermDev& q = T.t[t];
+        const double* r = base + q.offset;
+        double sig = 0.0;
+        for (int s = 0; s < q.n_samples; ++s) sig += sqrt(r[4 + 2 * s] / (double)q.nu);
+        snu[t] = sig / q.n_samples * (double)q.nu;
+        const double R = r[2] - r[1];
+        lr[t] = R == 0.0 ? 0.0 : r[0] / R;
+    }
     __syncthreads();
     if (threadIdx.x != 0) return;
     double E = 0.0;
     int t0 = 0;
     while (t0 < T.n) {
         int t1 = t0;
-        double den = 0.0;
+        double den = 0.0, sum = 0.0;
         while (t1 < T.n && T.t[t1].layer == T.t[t0].layer) {  // one layer: sum of sigma nu
-            const CostTermDev& q = T.t[t1];
-            const double* r = base + q.offset;
-            double sig = 0.0;
-            for (int s = 0; s < q.n_samples; ++s) sig += sqrt(r[4 + 2 * s] / (double)q.nu);
-            den += sig / q.n_samples * (double)q.nu;
+            den += snu[t1];
+            sum += snu[t1] * lr[t1];
             ++t1;
         }
-        if (den > 0.0) {
-            for (int t = t0; t < t1; ++t) {
-                const CostTermDev& q = T.t[t];
-                const double* r = base + q.offset;
-                const double R = r[2] - r[1];
-                if (R == 0.0) continue;
-                double sig = 0.0;
-                for (int s = 0; s < q.n_samples; ++s) sig += sqrt(r[4 + 2 * s] / (double)q.nu);
-                E += (sig / q.n_samples * (double)q.nu / den) * r[0] / R;
-            }
-        }
+        if (den > 0.0) E += sum / den;
         t0 = t1;
     }
     const double uc = (double)n_tied / N, mp = (double)extra / ((double)N * n_classes);
@@ -701,7 +784,7 @@ extern "C" fxpq_status fxpq_ds_stats_batch(const fxpq_ds_item* h_items, int32_t 
         ds_dev_kernel<<<(unsigned)u, DS_T, 0, s>>>(B, units);
         st = after_launch("ds_dev");
         if (st != FXPQ_OK) return st;
-        ds_finish_kernel<<<(B.n + 127) / 128, 128, 0, s>>>(B, units);
+        ds_finish_kernel<<<B.n, DF_T, 0, s>>>(B, units);
         st = after_launch("ds_finish");
         if (st != FXPQ_OK) return st;
     }

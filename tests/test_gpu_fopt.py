@@ -6,6 +6,8 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
+
 import synth
 from oracle import qopt
 
@@ -67,6 +69,37 @@ def test_conv_f32_tiles(M, N, H, C, K, R, st, pad, off):
     got = y.cpu().numpy()
     assert got[-1] == 7.0
     assert (np.abs(got[:-1].reshape(want.shape) - want) <= (R * R * C + 2) * 2.0 ** -24 * mag).all()
+
+
+@pytest.mark.parametrize("fmt", [(8, 1, 5), (8, 0, 30), (16, 1, -3), (4, 1, -20), (24, 1, 10), (1, 1, 2)])
+@pytest.mark.parametrize("kind", ["normal", "relu", "wide", "offset", "constant"])
+def test_ds_stats_against_exact_sums(M, fmt, kind):
+    """The statistics' sums against exact ones (math.fsum over terms exact in fp64 or better): values inside and
+    outside the range of the paired fp32 form, saturated, tiny, huge and constant ones, odd counts."""
+    import math
+    from fractions import Fraction
+    fopt, F = M
+    rng = np.random.default_rng(5)
+    n = 3001
+    x = {"normal": rng.standard_normal(n), "relu": np.maximum(rng.standard_normal(n), 0),
+         "wide": rng.standard_normal(n) * 2.0 ** rng.integers(-60, 40, n), "offset": 1000 + 1e-3 * rng.standard_normal(n),
+         "constant": np.full(n, 0.1)}[kind].astype(np.float32)
+    out = torch.empty(5, dtype=torch.float64, device="cuda")
+    F.fxpq_ds_stats_batch([(torch.from_numpy(x).cuda(), 1, n, F.fmt(*fmt), out)])
+    h = out.cpu().numpy()
+    k, S, fl = fmt
+    xs = [Fraction(float(v)) for v in x]
+    if (k, S) == (1, 1):
+        q = [Fraction(-1 if v < 0 else 1) * Fraction(2) ** -fl for v in x]
+    else:
+        q = [Fraction(int(c)) * Fraction(2) ** -fl for c in np.clip(np.rint(x.astype(np.float64) * 2.0 ** fl), oracle.qmin(k, S), oracle.qmax(k, S))]
+    err = sum((a - b) ** 2 for a, b in zip(xs, q))
+    mean = sum(xs) / n
+    dev = sum((a - mean) ** 2 for a in xs)
+    assert h[0] == pytest.approx(float(err), rel=1e-15)
+    assert abs(h[3] - float(mean)) <= 4e-16 * math.fsum(abs(float(v)) for v in x) / n
+    # the deviations are taken from the mean rounded to fp64: n times the square of its error on top
+    assert abs(h[4] - float(dev)) <= 1e-15 * float(dev) + n * (4e-16 * float(np.abs(x).max())) ** 2 + 1e-300
 
 
 def test_ds_stats_batch_and_ties(M):
