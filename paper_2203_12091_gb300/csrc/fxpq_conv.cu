@@ -342,6 +342,33 @@ fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, con
         a.py = 1;
     }
     a.f32_scale = ldexpf(1.0f, -s);
+    // Scale layers in fp32 (fepi_scale): the factors' codes exact in fp32, every power of two well inside its range
+    a.vs = 0;
+    a.vs_m = a.vs_b = a.vs_h = a.vs_eps = 0.0f;
+    if (a.has_scale && a.py == 1 && d.out_mode != FXPQ_OUT_ACC64 && d.fmt_scale.bits <= 24 && d.fmt_shift.bits <= 24) {
+        const int fy = d.out_mode == FXPQ_OUT_CODES ? d.fmt_y.fl : 0;
+        const int em = fy - d.fmt_x.fl - d.fmt_w.fl - d.fmt_scale.fl, eb = bias ? fy - d.fmt_b.fl - d.fmt_scale.fl : 0,
+                  eh = fy - d.fmt_shift.fl;
+        const bool fits = em >= -90 && em <= 30 && eb >= -90 && eb <= 30 && eh >= -90 && eh <= 30;
+        const double mb = ldexp(1.0, d.fmt_scale.bits - d.fmt_scale.is_signed);
+        const double tb = (bias ? ldexp(1.0, d.fmt_b.bits - d.fmt_b.is_signed) * mb * ldexp(1.0, eb) : 0.0) +
+                          ldexp(1.0, d.fmt_shift.bits - d.fmt_shift.is_signed) * ldexp(1.0, eh);
+        a.vs_m = ldexpf(1.0f, em);
+        a.vs_b = bias ? ldexpf(1.0f, eb) : 0.0f;
+        a.vs_h = ldexpf(1.0f, eh);
+        if (d.out_mode == FXPQ_OUT_CODES) {
+            // half a unit of the last place of x (inside the clip levels, widened by one) and of t, whose three
+            // roundings (with a bias) count, with a margin
+            const double top = (double)(a.hi > -a.lo ? a.hi : -a.lo) + 2.0;
+            const double eps = ldexp(1.0, -24) * (top + (bias ? 3.0 * tb : 0.0)) * 1.25;
+            a.vs = fits && a.sh >= 1 && eps < 1.0 / 64 && (!bias || d.fmt_b.bits <= 24);
+            a.vs_eps = (float)eps;
+            a.vf_lo = a.relu && a.lo < 0 ? 0.0f : (float)a.lo;
+            a.vf_hi = (float)a.hi;
+        } else {
+            a.vs = fits && !bias;  // t is exact: the fused multiply-add rounds the exact value once
+        }
+    }
     if (out_scale) *out_scale = s;
     return FXPQ_OK;
 }

@@ -29,6 +29,8 @@ struct ConvArgs {
     float vf_c, vf_lo, vf_hi;  // 2^-sh32 and the clip levels (lower one 0 under a ReLU)
     int vi;            // 1: fepi_image gives the fp32 image of sums that are exact fp32 integers
     float vi_c, vi_b;  // 2^-(fl_x + fl_w) and 2^-fl_b
+    int vs;            // 1: the fp32 form of a Scale layer's epilogue applies (fepi_scale)
+    float vs_m, vs_b, vs_h, vs_eps;  // output units per unit of acc aleph1, of b aleph1 and of aleph2; its error bound
     const int32_t* scale;  // Scale layer aleph1 codes [K] (has_scale)
     const int32_t* shift;  // Scale layer aleph2 codes [K]
     int has_scale;
@@ -122,10 +124,19 @@ __host__ __device__ __forceinline__ float fepi_bias(const ConvArgs& a, int32_t b
     return ((float)(b >> d) + ((b & ((1 << d) - 1)) ? 0.5f : 0.0f)) * a.vf_c;
 }
 
+// A Scale layer's output in units of the FxP-QLayer's step (or of 1 for the fp32 image): x = acc m + t with the
+// channel's constants m = aleph1 vs_m and t = b aleph1 vs_b + aleph2 vs_h.  Valid when a.vs, for |acc| < 2^24: acc m
+// is exact before the one rounding of the fused multiply-add, so x is within vs_eps of the exact value wherever
+// that lies inside the clip levels, and a value further than that from a rounding boundary has the exact code.
+__host__ __device__ __forceinline__ float2 fepi_scale(const ConvArgs& a, int32_t b, int32_t m, int32_t h) {
+    return make_float2((float)m * a.vs_m, (float)b * ((float)m * a.vs_b) + (float)h * a.vs_h);
+}
+
 // The fp32 nearest-even image of a C-Block output in one fused multiply-add (valid when a.vi, for |acc| < 2^24):
-// acc 2^-(fl_x + fl_w) and t = b 2^-fl_b are exact in fp32, their sum is rounded once, whichever is finer.
-__host__ __device__ __forceinline__ float fepi_image(const ConvArgs& a, float acc, float t) {
-    const float v = fmaf(acc, a.vi_c, t);
+// acc c (c = 2^-(fl_x + fl_w)) and t = b 2^-fl_b are exact, their sum is rounded once, whichever is finer (a Scale
+// layer: c and t of fepi_scale).
+__host__ __device__ __forceinline__ float fepi_image(const ConvArgs& a, float acc, float c, float t) {
+    const float v = fmaf(acc, c, t);
     return a.relu ? fmaxf(v, 0.0f) : v;
 }
 

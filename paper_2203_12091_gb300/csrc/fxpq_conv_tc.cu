@@ -169,7 +169,8 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     // reduction fills the SMs: the MMA thread's fixed cost per k-block is then hidden, and the weights
     // stream at the memory's rate
     const bool wide_split = rows_geom && !acc64 && !a.has_scale && ws && a.K > 128 && !conv_path_is("tc_bn128") &&
-                            !conv_path_is("tc_nosplit") && row_tiles_est * ((a.K + 255) / 256) * 2 <= sms;
+                            !conv_path_is("tc_nosplit") && row_tiles_est * ((a.K + 255) / 256) * 2 <= sms &&
+                            (kb_flat * a.px * a.pw >= 32 || d.d_wpacked);  // (shorter ones are not split, see below)
     // Tile width: 64 columns for int64 sums and at most 64 output channels, else the width whose whole rounds
     // over the SMs take the fewest cycles.  A k-block costs what its stage takes from L2 at about 80 bytes
     // per cycle and SM (24, 32 and 48 KB: 300, 410 and 615 cycles; the MMAs 228, 256 and 512); a 256-column
@@ -407,9 +408,9 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     P.part = nullptr;
     P.gs[0] = 0;
     P.gs[1] = P.n_groups;
-    // (64-column tiles, and 256-column TMA-row tiles, without a Scale layer: the instantiations that carry
-    // the split)
-    if (P.patch != 3 && P.patch != 4 && (BN == 64 || (BN == 256 && P.rows_tma && !acc64)) && !a.has_scale && ws &&
+    // (64-column tiles and 256-column TMA-row tiles: the instantiations that carry the split; a Scale layer is
+    // applied by the second kernel)
+    if (P.patch != 3 && P.patch != 4 && (BN == 64 || (BN == 256 && P.rows_tma && !acc64)) && ws &&
         P.n_tiles * 2 <= sms && !conv_path_is("tc_nosplit")) {
         const int ng = P.n_groups;
         int min_len = 1 << 30;
@@ -418,8 +419,14 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         const int cap = std::min(sms / P.n_tiles, (int)std::min<size_t>(ws_bytes / share, TC_MAX_SPLIT));
         // long groups: each share takes a sub-range of every group (at least four k-blocks); many short
         // groups (two-limb layers): each share takes whole groups
-        const int ks_sub = std::min(cap, std::min(min_len / 4, TC_MAX_GROUPS / ng));
-        const int ks_whole = std::min(cap, ng);
+        int ks_sub = std::min(cap, std::min(min_len / 4, TC_MAX_GROUPS / ng));
+        int ks_whole = std::min(cap, ng);
+        // the second kernel costs about 3 us, a k-block of a tile that has its SM to itself 0.15 us (1 image,
+        // ResNet-18: 21 us for 72 k-blocks, 11 for 1): the split has to shorten the chain by 24
+        int total = 0;
+        for (int gi = 0; gi < ng; ++gi) total += P.g[gi].kb1 - P.g[gi].kb0;
+        if (total - total / std::max(ks_sub, 1) < 24) ks_sub = 1;
+        if (total - total / std::max(ks_whole, 1) < 24) ks_whole = 1;
         if (ks_sub >= 2 && ks_sub >= ks_whole) {
             TcGroup g0[TC_MAX_GROUPS];
             for (int gi = 0; gi < ng; ++gi) g0[gi] = P.g[gi];
@@ -445,8 +452,9 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         }
     }
     P.n_units = P.n_tiles * P.ksplit;
-    P.fepi = ((a.vf && P.fast_store) || (a.vi && a.K % 4 == 0)) && P.n_groups == 1 && P.g[0].shift == 0 && P.patch != 3 &&
-             P.ksplit == 1 && !P.pk && !acc64 && !a.has_scale && !conv_path_is("tc_iepi");
+    P.fepi = ((a.vf && P.fast_store) || (a.vi && a.K % 4 == 0) ||
+              (a.vs && (P.fast_store || (a.out_mode == FXPQ_OUT_F32 && a.K % 4 == 0)))) && P.n_groups == 1 && P.g[0].shift == 0 && P.patch != 3 &&
+             P.ksplit == 1 && !P.pk && !acc64 && !conv_path_is("tc_iepi");
     {
         std::lock_guard<std::mutex> lk(g_tc_mu);
         if (!g_tc_attr_set) {
@@ -486,7 +494,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     const int grid = P.n_units < sms ? P.n_units : sms;
     TileIter::split(P, grid, P.step_n, P.step_q, P.step_p, P.step_g);
     launched = true;
-    if (a.has_scale) return launch_conv_tc_scaled(P, BN, acc64, grid, st);  // never split
+    if (a.has_scale && P.ksplit == 1) return launch_conv_tc_scaled(P, BN, acc64, grid, st);
     if (P.patch == 3 && (P.w32 || P.wf32))  // window mode, 32-bit two-limb epilogue: its own instance (never split)
         conv_tc_kernel<64, long long, false, false, false, true>
             <<<grid, tc_threads_win(), tc_smem_bytes<64>(), st>>>(P);

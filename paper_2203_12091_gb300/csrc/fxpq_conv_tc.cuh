@@ -787,6 +787,24 @@ __device__ __forceinline__ uint32_t fepi_pair(uint32_t a0, uint32_t a1, uint64_t
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+// One output of a Scale layer in exact 64-bit arithmetic, for the rare value next to a rounding boundary.
+static __device__ __noinline__ int scale_code_exact(const ConvArgs& a, int k, uint32_t f) {
+    const Epi64 e = make_epi64(a);
+    const int32_t b = (e.has_bias && k < a.K) ? __ldg(a.bias + k) : 0;
+    return epi64_code<true>(e, (long long)__float2int_rn(__uint_as_float(f)), b, scale_code(a, k), shift_code(a, k));
+}
+// Two outputs (channels k, k + 1) of a Scale layer to packed codes: fepi_scale, exact arithmetic within vs_eps of a
+// rounding boundary (one value in some ten thousand).
+__device__ __forceinline__ uint32_t fepi_scale_pair(const ConvArgs& a, int k, uint32_t f0, uint32_t f1, float m0, float m1,
+                                                    float t0, float t1) {
+    const float x = fminf(fmaxf(fmaf(__uint_as_float(f0), m0, t0), a.vf_lo), a.vf_hi);
+    const float y = fminf(fmaxf(fmaf(__uint_as_float(f1), m1, t1), a.vf_lo), a.vf_hi);
+    const float rx = (x + 12582912.0f) - 12582912.0f, ry = (y + 12582912.0f) - 12582912.0f;
+    if (fmaxf(fabsf(x - rx), fabsf(y - ry)) > 0.5f - a.vs_eps)
+        return pack_codes_f16(scale_code_exact(a, k, f0), scale_code_exact(a, k + 1, f1));
+    return f32_codes_f16x2(x, y);
+}
+
 // ------------------------------------------------------------------ kernel
 // PK converter warp `cid` (of TC_PK_CONVERTERS): walks the same k-block sequence as the issuing thread;
 // for each k-block waits until its A box and packed records have landed (pkfull), expands its share of
@@ -847,7 +865,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     constexpr int NSTG = tc_stg_tiles(BN);  // staging tiles of the TMA stores
     static_assert(!WIN || (BN == 64 && sizeof(ACC) == 8 && !SC && !SPLIT && !PK), "window instance: BN = 64, int64");
     static_assert(!W64 || (BN == 64 && sizeof(ACC) == 4 && !SC && !SPLIT && !PK && !WIN), "W64 instance: BN = 64, int32");
-    static_assert(!FE || (sizeof(ACC) == 4 && !SC && !SPLIT && !PK && !WIN && !W64), "fp32 epilogue: plain int32 instances");
+    static_assert(!FE || (sizeof(ACC) == 4 && !SPLIT && !PK && !WIN && !W64), "fp32 epilogue: plain int32 instances");
     constexpr bool WEPI = WIN || W64;  // the window instances' epilogue (16 warps, two staging tiles)
     constexpr int EPI_WARPS = WEPI ? TC_WIN_EPI_WARPS : tc_epi_warps(BN);
     static_assert(tc_out_bytes(BN, PK) >= EPI_WARPS * 2048 || WEPI, "the staged fp32 / int64 epilogue takes 2 KB per warp");
@@ -1262,7 +1280,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 if (f32out && P.fepi) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
-                        w[j] = __float_as_uint(fepi_image(a, __uint_as_float(f[j]), __int_as_float(btw[j])));
+                        w[j] = __float_as_uint(fepi_image(a, __uint_as_float(f[j]), a.vi_c, __int_as_float(btw[j])));
                 } else if (f32out) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
@@ -1573,15 +1591,23 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         const int kl = k0 + lane;
                         const bool image = a.out_mode == FXPQ_OUT_F32;
                         const int32_t b = a.has_bias && kl < a.K ? __ldg(a.bias + kl) : 0;
-                        const float t = image ? (float)b * a.vi_b : a.has_bias ? fepi_bias(a, b) : 0.0f;
+                        float t, ms = 0.0f;  // the channel's constants
+                        if constexpr (SC) {
+                            const float2 mt = fepi_scale(a, b, scale_code(a, kl), shift_code(a, kl));
+                            ms = mt.x;
+                            t = mt.y;
+                        } else {
+                            t = image ? (float)b * a.vi_b : a.has_bias ? fepi_bias(a, b) : 0.0f;
+                        }
                         unsigned char* wbuf = sO + (warp - 4) * 2048;                     // DIRECT, fp32 image
                         unsigned char* half_buf = stg + (cb >> 1) * (TC_BM * 128);         // staged tile
-                        // four constants 4 q .. 4 q + 3
+                        // four constants 4 q .. 4 q + 3 (8 + q: the second set)
                         auto tab = [&](int q) {
                             return DIRECT || image ? wbuf + 16 * q
                                           : half_buf + (quad * 32 + (q >> 2)) * 128 + ((((cb & 1) * 4 + (q & 3)) ^ (q >> 2)) << 4);
                         };
                         *reinterpret_cast<float*>(tab(lane >> 2) + 4 * (lane & 3)) = t;
+                        if constexpr (SC) *reinterpret_cast<float*>(tab(8 + (lane >> 2)) + 4 * (lane & 3)) = ms;
                         __syncwarp();
                         tmem_wait_ld();
                         reg_fence(f0);
@@ -1597,10 +1623,12 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                             for (int q = 0; q < 8; ++q) {
                                 const float4 tq = *reinterpret_cast<const float4*>(tab(q));
                                 const uint32_t* f = q < 4 ? f0 + 4 * q : f1 + 4 * (q - 4);
-                                v[4 * q] = fepi_image(a, __uint_as_float(f[0]), tq.x);
-                                v[4 * q + 1] = fepi_image(a, __uint_as_float(f[1]), tq.y);
-                                v[4 * q + 2] = fepi_image(a, __uint_as_float(f[2]), tq.z);
-                                v[4 * q + 3] = fepi_image(a, __uint_as_float(f[3]), tq.w);
+                                float4 mq = make_float4(a.vi_c, a.vi_c, a.vi_c, a.vi_c);
+                                if constexpr (SC) mq = *reinterpret_cast<const float4*>(tab(8 + q));
+                                v[4 * q] = fepi_image(a, __uint_as_float(f[0]), mq.x, tq.x);
+                                v[4 * q + 1] = fepi_image(a, __uint_as_float(f[1]), mq.y, tq.y);
+                                v[4 * q + 2] = fepi_image(a, __uint_as_float(f[2]), mq.z, tq.z);
+                                v[4 * q + 3] = fepi_image(a, __uint_as_float(f[3]), mq.w, tq.w);
                             }
                             __syncwarp();
                             store_f32_direct(a, m, k0, v, wbuf, lane);
@@ -1611,6 +1639,12 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         for (int q = 0; q < 8; ++q) {
                             const float4 tq = *reinterpret_cast<const float4*>(tab(q));
                             const uint32_t* f = q < 4 ? f0 + 4 * q : f1 + 4 * (q - 4);
+                            if constexpr (SC) {
+                                const float4 mq = *reinterpret_cast<const float4*>(tab(8 + q));
+                                w[2 * q] = fepi_scale_pair(a, k0 + 4 * q, f[0], f[1], mq.x, mq.y, tq.x, tq.y);
+                                w[2 * q + 1] = fepi_scale_pair(a, k0 + 4 * q + 2, f[2], f[3], mq.z, mq.w, tq.z, tq.w);
+                                continue;
+                            }
                             w[2 * q] = fepi_pair(f[0], f[1], cc, tq.x, tq.y, a.vf_lo, a.vf_hi);
                             w[2 * q + 1] = fepi_pair(f[2], f[3], cc, tq.z, tq.w, a.vf_lo, a.vf_hi);
                         }

@@ -22,6 +22,12 @@ fxpq_status launch_conv_tc_scaled(const TcParams& P, int BN, bool acc64, int gri
                                      (int)tc_smem_bytes<64>()) != cudaSuccess ||
                 cudaFuncSetAttribute(conv_tc_kernel<64, int, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes<64>()) != cudaSuccess ||
+                cudaFuncSetAttribute(conv_tc_kernel<64, int, true, false, false, false, false, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes<64>()) != cudaSuccess ||
+                cudaFuncSetAttribute(conv_tc_kernel<128, int, true, false, false, false, false, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes<128>()) != cudaSuccess ||
+                cudaFuncSetAttribute(conv_tc_kernel<256, int, true, false, false, false, false, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes<256>()) != cudaSuccess ||
                 cudaFuncSetAttribute(conv_tc_kernel<128, int, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tc_smem_bytes<128>()) != cudaSuccess ||
                 cudaFuncSetAttribute(conv_tc_kernel<256, int, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -30,7 +36,13 @@ fxpq_status launch_conv_tc_scaled(const TcParams& P, int BN, bool acc64, int gri
             g_sc_attr_set = true;
         }
     }
-    if (acc64)
+    if (P.fepi && BN == 64)
+        conv_tc_kernel<64, int, true, false, false, false, false, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+    else if (P.fepi && BN == 128)
+        conv_tc_kernel<128, int, true, false, false, false, false, true><<<grid, tc_threads(128), tc_smem_bytes<128>(), st>>>(P);
+    else if (P.fepi)
+        conv_tc_kernel<256, int, true, false, false, false, false, true><<<grid, tc_threads(256), tc_smem_bytes<256>(), st>>>(P);
+    else if (acc64)
         conv_tc_kernel<64, long long, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
     else if (BN == 64)
         conv_tc_kernel<64, int, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);

@@ -660,3 +660,39 @@ def test_patch_shapes_parity(F, N, H, C, K, R, st, pad, mode):
     got, s = run_conv(F, x, fx, w, fw, b, fb, st, pad, True, mode, fy, C, int(np.abs(w).reshape(K, -1).sum(axis=1).max()))
     want, ws = oracle_conv(x, fx, w, fw, b, fb, st, pad, True, mode, fy)
     assert s == ws and np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("N,H,C,K,R,st,l1", [(2, 9, 64, 64, 3, 1, 1), (3, 12, 64, 136, 3, 2, 1), (2, 8, 128, 264, 3, 1, 1),
+                                             (1, 7, 512, 72, 3, 1, 1), (1, 7, 256, 64, 7, 1, 0)])  # the last two split
+@pytest.mark.parametrize("mode,relu,ty", [(0, True, (8, 0, 2)), (0, False, (5, 1, 1)), (2, True, None), (2, False, None), (1, False, None)])
+@pytest.mark.parametrize("bias", [0, 1])
+def test_scale_fp32_epilogue(F, N, H, C, K, R, st, l1, mode, relu, ty, bias):
+    """Scale layers of one exact group in fp32 with the exact arithmetic behind it (products on and next to rounding
+    boundaries), both forms, the fp32 image, and Scale layers behind a split reduction."""
+    if os.environ.get("FXPQ_CONV_PATH") not in ("tc", "tc_bn256"):
+        pytest.skip("an epilogue of the tensor-core path")
+    rng = np.random.default_rng(K + H + mode)
+    fx, fw, fb = F.fmt(8, 0, 6), F.fmt(6, 1, 7), F.fmt(16, 1, 17)
+    fs, fh = F.fmt(16, 1, 13), F.fmt(16, 1, 14)
+    fy = F.fmt(*ty) if ty else None
+    x, w = rand_codes(rng, (N, H, H, C), 8, 0), rng.integers(-2, 3, size=(K, R, R, C))
+    b = rand_codes(rng, (K,), 16, 1) if bias else None
+    m, h = rand_codes(rng, (K,), 16, 1), rng.integers(-9000, 9000, size=K)
+    # channel 5: sums 2 x[.., 0] times 2^12 on ties of the output step 2^(6 + 7 + 13 - fl_y), some of them one
+    # aleph2 unit off
+    w[5] = 0
+    w[5, R // 2, R // 2, 0] = 2
+    m[5] = 1 << 12
+    h[5] = 0 if K % 16 else 1
+    scale = (m, fs, h, fh)
+    pad = R // 2 if R == 3 else 0
+    bound = int(np.abs(w).reshape(K, -1).sum(axis=1).max()) if l1 else 0
+    want, ws = oracle_conv(x, fx, w, fw, b, fb if bias else None, st, pad, relu, mode, fy, scale=scale)
+    old = os.environ["FXPQ_CONV_PATH"]
+    for path in (old, "tc_iepi"):
+        os.environ["FXPQ_CONV_PATH"] = path
+        try:
+            got, s = run_conv(F, x, fx, w, fw, b, fb if bias else None, st, pad, relu, mode, fy, C, bound, scale=scale)
+        finally:
+            os.environ["FXPQ_CONV_PATH"] = old
+        assert s == ws and np.array_equal(got, want), path
