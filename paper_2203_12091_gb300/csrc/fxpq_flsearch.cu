@@ -627,19 +627,21 @@ __device__ __forceinline__ U128 mul128_64(U128 a, u64 m) {
 constexpr int BW = 12;
 constexpr int BBASE = -320;
 
-struct Big {
-    u64 w[BW];
-};
-
-// A cell's exact sum is gathered in 24 signed 64-bit columns in shared memory, column c weighing
-// 2^(32 c + BBASE): every term is cut into 32-bit pieces added to their columns (shared-memory
-// atomics, so the lanes of a warp share one set), and one carry pass turns the columns into the
-// 768-bit two's complement value.  A column takes well under 2^31 pieces, so it cannot overflow;
-// pieces above column 23 weigh multiples of 2^(768 + BBASE) and drop, as modulo 2^768 they must.
+// A cell's exact sum is gathered in 24 columns in shared memory, column c weighing 2^(32 c + BBASE): every term
+// is cut into 32-bit pieces added to their columns, and one carry pass turns the columns into the 768-bit
+// two's complement value.  A column is two signed 32-bit words, the sums of the pieces' low and high halves,
+// because 32-bit shared reductions are native while 64-bit ones are compare-and-swap loops; COL_COPIES copies
+// of the columns, by lane, keep lanes that meet in a column mostly apart (every lane of a warp scores keys of
+// neighbouring exponents).  A copy's word takes at most 512 / COL_COPIES keys of 10 terms of 3 pieces below 2^16:
+// below 2^27.  Pieces above column 23 weigh multiples of 2^(768 + BBASE) and drop, as modulo 2^768 they must.
+// The finalize kernel of a one-row search took 29 us with 64-bit columns and one lane per cell carrying and
+// rounding; 12.5 us with these and the warp-wide rounding below.
 constexpr int NCOL = 2 * BW;
+constexpr int COL_COPIES = 8;
+constexpr int COL_WORDS = NCOL * 2 * COL_COPIES;  // words of a warp's columns: [column][half][copy]
 
-// col += (neg ? -1 : 1) * v * 2^e for a 128-bit magnitude v
-__device__ __forceinline__ void col_add(u64* col, U128 v, int e, bool neg) {
+// columns += (neg ? -1 : 1) * v * 2^e for a 128-bit magnitude v (col: the lane's copy)
+__device__ __forceinline__ void col_add(int* col, U128 v, int e, bool neg) {
     if ((v.lo | v.hi) == 0ull) return;
     const int pos = e - BBASE;
     const int ci = pos >> 5;
@@ -650,77 +652,96 @@ __device__ __forceinline__ void col_add(u64* col, U128 v, int e, bool neg) {
                            __funnelshift_l(x2, x3, b), __funnelshift_l(x3, 0u, b)};
 #pragma unroll
     for (int j = 0; j < 5; ++j)
-        if (c[j] && ci + j < NCOL) atomicAdd(&col[ci + j], neg ? (u64)(-(long long)c[j]) : (u64)c[j]);
+        if (c[j] && ci + j < NCOL) {
+            int* p = col + (ci + j) * 2 * COL_COPIES;
+            const int lo = (int)(c[j] & 0xFFFFu), hi = (int)(c[j] >> 16);
+            atomicAdd(p, neg ? -lo : lo);
+            atomicAdd(p + COL_COPIES, neg ? -hi : hi);
+        }
 }
 
-// The columns' value as a 768-bit two's complement number.
-__device__ void col_to_big(const u64* col, Big& a) {
-    long long carry = 0;
+// The columns' value as a 768-bit two's complement number: lane c < 24 adds the copies of column c, lane 0 of the
+// warp carries through them.  All lanes take part; w (shared, 12 words) receives the number.
+__device__ __forceinline__ void col_to_big(const int* cols, u64* w, int lane) {
+    long long v = 0;
+    if (lane < NCOL) {
+        const int4* p = reinterpret_cast<const int4*>(cols + lane * 2 * COL_COPIES);
+        long long lo = 0, hi = 0;
 #pragma unroll
-    for (int i = 0; i < BW; ++i) {
-        const long long t0 = (long long)col[2 * i] + carry;
-        const long long t1 = (long long)col[2 * i + 1] + (t0 >> 32);
-        carry = t1 >> 32;
-        a.w[i] = (u64)(unsigned)t0 | ((u64)(unsigned)t1 << 32);
+        for (int q = 0; q < COL_COPIES / 4; ++q) {
+            const int4 a = p[q], b = p[COL_COPIES / 4 + q];
+            lo += (long long)a.x + a.y + a.z + a.w;
+            hi += (long long)b.x + b.y + b.z + b.w;
+        }
+        v = lo + hi * 65536;
     }
+    long long carry = 0;
+    unsigned even = 0u;
+#pragma unroll
+    for (int c = 0; c < NCOL; ++c) {
+        const long long t = __shfl_sync(0xFFFFFFFFu, v, c) + carry;
+        carry = t >> 32;
+        if (c & 1) {
+            if (lane == 0) w[c >> 1] = (u64)even | ((u64)(unsigned)t << 32);
+        } else {
+            even = (unsigned)t;
+        }
+    }
+    __syncwarp();
 }
 
 // a += (neg ? -1 : 1) * m * 2^e * (the three-limb bin at p).  The top limb is signed: the histogram
 // kernel's remainder sums leave out the sum of L^2 that its exponent band carries, so one key's
 // share of a cell may be negative.
-__device__ __forceinline__ void col_add_L3(u64* a, const u64* p, int e, bool neg, u64 m = 1ull) {
+__device__ __forceinline__ void col_add_L3(int* a, const u64* p, int e, bool neg, u64 m = 1ull) {
     col_add(a, mul128_64(U128{p[0], 0ull}, m), e, neg);
     col_add(a, mul128_64(U128{p[1], 0ull}, m), e + 32, neg);
     const long long w2 = (long long)p[2];
     if (w2) col_add(a, mul128_64(U128{w2 < 0 ? (u64)(-w2) : (u64)w2, 0ull}, m), e + 64, neg != (w2 < 0));
 }
 
-__device__ u64 big_bits64(const Big& a, int pos) {  // bits [pos, pos + 64), zero below bit 0
+__device__ u64 big_bits64(const u64* w, int pos) {  // bits [pos, pos + 64), zero below bit 0
     const int wi = pos >= 0 ? (pos >> 6) : -((-pos + 63) >> 6);
     const int b = pos - wi * 64;
-    const u64 lo = (wi >= 0 && wi < BW) ? a.w[wi] : 0ull;
-    const u64 hi = (wi + 1 >= 0 && wi + 1 < BW) ? a.w[wi + 1] : 0ull;
+    const u64 lo = (wi >= 0 && wi < BW) ? w[wi] : 0ull;
+    const u64 hi = (wi + 1 >= 0 && wi + 1 < BW) ? w[wi + 1] : 0ull;
     return b ? ((lo >> b) | (hi << (64 - b))) : lo;
 }
 
-__device__ bool big_any_below(const Big& a, int pos) {
-    if (pos <= 0) return false;
-    const int wi = pos >> 6, b = pos & 63;
-    for (int i = 0; i < wi && i < BW; ++i)
-        if (a.w[i]) return true;
-    return wi < BW && b && (a.w[wi] & ((1ull << b) - 1ull));
-}
-
-// round a non-negative accumulator to nearest-even double (negative -> -1, a sentinel)
-__device__ double big_to_double(const Big& a) {
-    if ((long long)a.w[BW - 1] < 0) return -1.0;
-    int h = -1;
-    for (int i = BW - 1; i >= 0; --i)
-        if (a.w[i]) {
-            h = i;
-            break;
-        }
-    if (h < 0) return 0.0;
-    const int top = 64 * h + 63 - __clzll(a.w[h]);
-    const u64 win = big_bits64(a, top - 63);
+// Round the 768-bit number w (shared, 12 words) to the nearest-even double, by a whole warp (lane i < 12 holds
+// word i); neg_ok: negative numbers too, otherwise they give -1, a sentinel.  The result is in every lane.
+__device__ double big_to_double(u64* w, int lane, bool neg_ok) {
+    const bool neg = (long long)w[BW - 1] < 0;
+    if (neg) {
+        if (!neg_ok) return -1.0;
+        // negate: complement, plus one up to and including the lowest non-zero word
+        const u64 x = lane < BW ? w[lane] : 0ull;
+        const unsigned nz = __ballot_sync(0xFFFFFFFFu, x != 0ull);
+        const int first = __ffs(nz) - 1;
+        __syncwarp();
+        if (lane < BW) w[lane] = lane < first ? 0ull : lane == first ? 0ull - x : ~x;
+        __syncwarp();
+    }
+    const u64 x = lane < BW ? w[lane] : 0ull;
+    const unsigned nz = __ballot_sync(0xFFFFFFFFu, x != 0ull);
+    if (nz == 0u) return 0.0;
+    const int h = 31 - __clz(nz);
+    const int top = 64 * h + 63 - __clzll(w[h]);
+    const u64 win = big_bits64(w, top - 63);
+    // any bit below the 64-bit window
+    const int pos = top - 63, wi = pos >> 6, b = pos & 63;
+    const bool mine = pos > 0 && lane < BW && (lane < wi ? x != 0ull : lane == wi && (x & ((1ull << b) - 1ull)) != 0ull);
+    const bool below = __any_sync(0xFFFFFFFFu, mine);
     u64 mant = win >> 11;
     const bool rb = (win >> 10) & 1ull;
-    const bool sticky = (win & 0x3FFull) != 0ull || big_any_below(a, top - 63);
+    const bool sticky = (win & 0x3FFull) != 0ull || below;
     if (rb && (sticky || (mant & 1ull))) mant += 1ull;
-    return ldexp((double)mant, top - 52 + BBASE);
-}
-
-__device__ void big_negate(Big& a) {
-    u64 c = 1ull;
-    for (int i = 0; i < BW; ++i) {
-        const u64 t = ~a.w[i] + c;
-        c = (c && t == 0ull) ? 1ull : 0ull;
-        a.w[i] = t;
-    }
+    const double v = ldexp((double)mant, top - 52 + BBASE);
+    return neg ? -v : v;
 }
 
 // saturated set with moments (n, s1, s2) at exponent E: s2 2^(2(E-23)) - 2 T s1 2^(E-23-fl) + T^2 n 2^(-2fl)
-__device__ void add_sat(u64* acc, u64 n, const u64* s1, const u64* s2, int E, int fl, u64 T) {
+__device__ void add_sat(int* acc, u64 n, const u64* s1, const u64* s2, int E, int fl, u64 T) {
     col_add_L3(acc, s2, 2 * (E - 23), false);
     if (T) {
         col_add_L3(acc, s1, E - 23 - fl, true, 2ull * T);
@@ -729,7 +750,7 @@ __device__ void add_sat(u64* acc, u64 n, const u64* s1, const u64* s2, int E, in
 }
 
 // ------------------------------------------------------------------ finalize: scores, argmin, stats
-constexpr int FIN_T = 256;            // threads per finalize block
+constexpr int FIN_T = 128;            // threads per finalize block
 constexpr int FIN_WARPS = FIN_T / 32;  // cells per finalize block, one per warp
 
 // The keys with elements and the non-zero exponent sums of squares of one item, staged per block,
@@ -742,7 +763,8 @@ struct FinSmem {
     u64 s2[NKEY][3];
     unsigned beb[256];
     u64 band[256][3];
-    u64 col[FIN_WARPS][NCOL];
+    u64 big[FIN_WARPS][BW];
+    __align__(16) int col[FIN_WARPS][COL_WORDS];
 };
 
 __device__ void fin_stage(FinSmem& sm, const FsGlobal* g) {
@@ -774,7 +796,7 @@ __device__ void fin_stage(FinSmem& sm, const FsGlobal* g) {
 
 // The exact value of one cell (candidate (S, k, FL), or the two stats cells) added to a warp's
 // columns: the lanes split the staged keys.
-__device__ void fin_cell(u64* acc, const FinSmem& sm, const FsGlobal* g, const FsFinal& F, int cell, int ncell,
+__device__ void fin_cell(int* acc, const FinSmem& sm, const FsGlobal* g, const FsFinal& F, int cell, int ncell,
                          int lane, int nlanes) {
     // the exponent-indexed sums of squares that belong to every L2 cell and to the sum of squares
     const bool with_band = cell == ncell + 1 || (cell < ncell && !F.l1);
@@ -878,26 +900,22 @@ __global__ void __launch_bounds__(FIN_T) fl_search_final_kernel(const __grid_con
     const int ncell = (F.S_hi - F.S_lo + 1) * F.nk * F.nfl;
     const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cell = ((int)blockIdx.x - B.fin0[item]) * FIN_WARPS + warp;
-    u64* col = sm.col[warp];
-    if (lane < NCOL) col[lane] = 0ull;
+    for (int i = lane; i < COL_WORDS; i += 32) sm.col[warp][i] = 0;
     fin_stage(sm, g);
     if (cell < ncell + 2) {  // warp-uniform
-        fin_cell(col, sm, g, F, cell, ncell, lane, 32);
+        fin_cell(sm.col[warp] + (lane & (COL_COPIES - 1)), sm, g, F, cell, ncell, lane, 32);
         __syncwarp();
+        col_to_big(sm.col[warp], sm.big[warp], lane);
+        const double v = big_to_double(sm.big[warp], lane, cell == ncell);
         if (lane == 0) {
-            Big acc;
-            col_to_big(col, acc);
             if (cell == ncell) {
-                const bool neg = (long long)acc.w[BW - 1] < 0;
-                if (neg) big_negate(acc);
-                const double v = big_to_double(acc);
-                g->stat_sum = neg ? -v : v;
+                g->stat_sum = v;
             } else if (cell == ncell + 1) {
-                g->stat_sumsq = big_to_double(acc);
+                g->stat_sumsq = v;
             } else {
                 const int S = F.S_lo + cell / (F.nk * F.nfl);
                 const int rem = cell % (F.nk * F.nfl);
-                g->cells[S][F.k_lo + rem / F.nfl - 1][rem % F.nfl] = big_to_double(acc);
+                g->cells[S][F.k_lo + rem / F.nfl - 1][rem % F.nfl] = v;
             }
             __threadfence();
         }

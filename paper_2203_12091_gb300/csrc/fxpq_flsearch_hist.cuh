@@ -83,8 +83,29 @@ __host__ __device__ inline bool hs_fits(const FsParams& P) { return P.hs_w <= HS
 
 struct HsLane {
     u64 acc0, acc1;   // sum (L 2^e)^2 for E - band in [0, 8) (e = E - band) and [8, 16) (e = E - band - 8)
-    unsigned mn, mx;  // order keys (non-finite values are corrected for after the chunk)
+    // extremes of the bit patterns: as signed integers the largest, as unsigned ones the largest and the
+    // smallest (non-finite values are corrected for after the chunk)
+    int smax;
+    unsigned umax, umin;
 };
+
+// Order keys of the smallest and the largest value from the pattern extremes: floats without a sign order like
+// integers, those with one the other way round.
+__device__ __forceinline__ void hs_extremes(int smax, unsigned umax, unsigned umin, unsigned& kmn, unsigned& kmx) {
+    kmn = umax & 0x80000000u ? ~umax : umin | 0x80000000u;  // any sign: the largest pattern is the smallest value
+    kmx = smax >= 0 ? (unsigned)smax | 0x80000000u : ~umin;  // all with a sign: the smallest pattern is the largest
+}
+__device__ __forceinline__ void hs_minmax(unsigned u, HsLane& st) {
+    st.smax = max(st.smax, (int)u);
+    st.umax = max(st.umax, u);
+    st.umin = min(st.umin, u);
+}
+// of two elements (three-input maxima: half the instructions)
+__device__ __forceinline__ void hs_minmax2(unsigned a, unsigned b, HsLane& st) {
+    st.smax = __vimax3_s32(st.smax, (int)a, (int)b);
+    st.umax = __vimax3_u32(st.umax, a, b);
+    st.umin = __vimin3_u32(st.umin, a, b);
+}
 
 // Per-item constants of the hot loop.
 struct HsK {
@@ -119,9 +140,6 @@ __device__ __forceinline__ bool hs_elem(unsigned u, unsigned* cnt, const HsK& K,
     const unsigned L1 = eo - 8u < K.lim1 ? Le : 0u;
     st.acc0 += (u64)L0 * L0;
     st.acc1 += (u64)L1 * L1;
-    const unsigned ok = u ^ (sgm | 0x80000000u);
-    st.mn = min(st.mn, ok);
-    st.mx = max(st.mx, ok);
     return eo >= K.span && z != 0u;  // the band lies inside the window
 }
 
@@ -437,8 +455,9 @@ __global__ void __launch_bounds__(HS_T, 1) fl_search_hist_kernel(const __grid_co
     const long long nfull = end > start ? (end - start) / HS_ITER : 0;
     HsLane st;
     st.acc0 = st.acc1 = 0ull;
-    st.mn = 0xFFFFFFFFu;
-    st.mx = 0u;
+    st.smax = INT_MIN;
+    st.umax = 0u;
+    st.umin = 0xFFFFFFFFu;
     unsigned nout = 0u;
 
     uint4 va[4], vb[4];
@@ -495,6 +514,8 @@ __global__ void __launch_bounds__(HS_T, 1) fl_search_hist_kernel(const __grid_co
             cm |= hs_elem(v[q].y, hs_smem, K, st) ? 2u << (4 * q) : 0u;
             cm |= hs_elem(v[q].z, hs_smem, K, st) ? 4u << (4 * q) : 0u;
             cm |= hs_elem(v[q].w, hs_smem, K, st) ? 8u << (4 * q) : 0u;
+            hs_minmax2(v[q].x, v[q].y, st);
+            hs_minmax2(v[q].z, v[q].w, st);
         }
         cold(v, cm);
     };
@@ -513,17 +534,25 @@ __global__ void __launch_bounds__(HS_T, 1) fl_search_hist_kernel(const __grid_co
         unsigned cm = 0u;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            if ((ma >> (4 * q)) & 1u) cm |= hs_elem(va[q].x, hs_smem, K, st) ? 1u << (4 * q) : 0u;
-            if ((ma >> (4 * q)) & 2u) cm |= hs_elem(va[q].y, hs_smem, K, st) ? 2u << (4 * q) : 0u;
-            if ((ma >> (4 * q)) & 4u) cm |= hs_elem(va[q].z, hs_smem, K, st) ? 4u << (4 * q) : 0u;
-            if ((ma >> (4 * q)) & 8u) cm |= hs_elem(va[q].w, hs_smem, K, st) ? 8u << (4 * q) : 0u;
+            const unsigned w4[4] = {va[q].x, va[q].y, va[q].z, va[q].w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if ((ma >> (4 * q + c)) & 1u) {
+                    cm |= hs_elem(w4[c], hs_smem, K, st) ? 1u << (4 * q + c) : 0u;
+                    hs_minmax(w4[c], st);
+                }
         }
         cold(va, cm);
     }
 
     // per-lane results: stats, band sums, elements outside the window that were not zeros
     {
-        const unsigned mn = __reduce_min_sync(0xFFFFFFFFu, st.mn), mx = __reduce_max_sync(0xFFFFFFFFu, st.mx);
+        unsigned mn = 0xFFFFFFFFu, mx = 0u;
+        {
+            const int smax = __reduce_max_sync(0xFFFFFFFFu, st.smax);
+            const unsigned umax = __reduce_max_sync(0xFFFFFFFFu, st.umax), umin = __reduce_min_sync(0xFFFFFFFFu, st.umin);
+            if (umax >= umin) hs_extremes(smax, umax, umin, mn, mx);  // (the warp had elements)
+        }
         const unsigned no = __reduce_add_sync(0xFFFFFFFFu, nout);
         const u64 a0 = warp_sum64(st.acc0), a1 = warp_sum64(st.acc1);  // < 2^61 per warp
         if (lane == 0) {
@@ -595,12 +624,16 @@ __global__ void __launch_bounds__(HS_T, 1) fl_search_hist_kernel(const __grid_co
         }
         __syncthreads();
     }
-    // convert the bins, one key per warp
-    for (int ks = (int)warp; ks < Ly.nkeys; ks += HS_T / 32) {
-        if (P.hs_s == 15)
-            hs_convert_key<L1, 8>(P, hs_smem, ovf_sum, misc + HM_OVF_IDX, novf, ks, lane);
-        else
-            hs_convert_key<L1, 7>(P, hs_smem, ovf_sum, misc + HM_OVF_IDX, novf, ks, lane);
+    // convert the bins, one key per warp and turn; the two signs' keys start half the warps apart, so that the few
+    // exponents that hold most values of either sign meet different warps
+    for (int i = 0; i < 2; ++i) {
+        for (int d = (int)((warp + 16u * i) & (HS_T / 32 - 1)); d < P.hs_w; d += HS_T / 32) {
+            const int ks = d + i * P.hs_w;
+            if (P.hs_s == 15)
+                hs_convert_key<L1, 8>(P, hs_smem, ovf_sum, misc + HM_OVF_IDX, novf, ks, lane);
+            else
+                hs_convert_key<L1, 7>(P, hs_smem, ovf_sum, misc + HM_OVF_IDX, novf, ks, lane);
+        }
     }
 }
 
