@@ -141,8 +141,9 @@ __host__ __device__ __forceinline__ float fepi_image(const ConvArgs& a, float ac
 }
 
 // Bias alignment, ReLU and the FxP-QLayer for one output value of row m, channel k.
+template <bool SC = true>
 __device__ __forceinline__ void cblock_epilogue_store(const ConvArgs& a, long long m, int k, long long v) {
-    v = cblock_value(a, k, v, a.has_bias ? a.bias[k] : 0);
+    v = cblock_value<SC>(a, k, v, a.has_bias ? __ldg(a.bias + k) : 0);
     if (a.out_mode == FXPQ_OUT_CODES) {
         code_put(static_cast<__half*>(a.y), m * a.K + k, a.py, a.M * a.K, qlayer_code(a, v));
     } else if (a.out_mode == FXPQ_OUT_ACC64) {

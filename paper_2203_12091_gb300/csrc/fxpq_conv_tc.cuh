@@ -517,36 +517,16 @@ __device__ __forceinline__ void tmem_st16_nw(uint32_t taddr, const uint32_t (&r)
 // Final epilogue of 32 consecutive output channels k0.. of row m (generic outputs: two-plane codes,
 // int64 accumulators, fp32 calibration images): bias alignment, ReLU, FxP-QLayer.
 // (This and the next are calls, their values passed in local memory: inlined, they made the 128-column kernels
-// spill 1.2 KB around every path, the codes of several groups among them.)
+// spill 1.2 KB around every path, the codes of several groups among them.  They run in short loops: unrolled over
+// the 32 channels, the int64 logits of a 512 -> 1000 layer, one tile per CTA and each instruction run once,
+// took 25 us, most of it for fetching code and re-reading parameters; 13 us now.)
 template <typename ACC, bool SC>
 __device__ __noinline__ void epilogue_block32(const ConvArgs& a, long long m, int k0, const ACC (&acc)[32]) {
-    if (a.out_mode == FXPQ_OUT_CODES) {
-        __half* y = static_cast<__half*>(a.y);
-        const long long base = m * a.K + k0;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            const int k = k0 + j;
-            if (k < a.K) {
-                const int32_t b = a.has_bias ? __ldg(a.bias + k) : 0;
-                code_put(y, base + j, a.py, a.M * a.K, qlayer_code(a, cblock_value<SC>(a, k, (long long)acc[j], b)));
-            }
-        }
-    } else if (a.out_mode == FXPQ_OUT_ACC64) {
-        long long* y = static_cast<long long*>(a.y) + m * a.K + k0;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            const int k = k0 + j;
-            if (k < a.K) y[j] = cblock_value<SC>(a, k, (long long)acc[j], a.has_bias ? __ldg(a.bias + k) : 0);
-        }
-    } else {
-        float* y = static_cast<float*>(a.y) + m * a.K + k0;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            const int k = k0 + j;
-            if (k < a.K)
-                y[j] = __ll2float_rn(cblock_value<SC>(a, k, (long long)acc[j], a.has_bias ? __ldg(a.bias + k) : 0)) *
-                       a.f32_scale;
-        }
+#pragma unroll 1
+    for (int j = 0; j < 32; ++j) {
+        const int k = k0 + j;
+        if (k >= a.K) break;
+        cblock_epilogue_store<SC>(a, m, k, (long long)acc[j]);
     }
 }
 
@@ -559,48 +539,48 @@ template <typename ACC, bool SC>
 __device__ __noinline__ void epilogue_block32_staged(const ConvArgs& a, long long m, int k0, const ACC (&acc)[32],
                                                         unsigned char* wbuf, int lane) {
     const bool f32 = a.out_mode == FXPQ_OUT_F32;
-    const int per = f32 ? 16 : 8;  // values per round: 64 bytes of a row
+    const int esz = f32 ? 4 : 8;
+    const int per = 64 / esz;  // values per round: 64 bytes of a row
+    const int K = a.K;         // (copies: a lies in memory here, and every store below may alias it)
+    unsigned char* const y = static_cast<unsigned char*>(a.y);
+    const float f32_scale = a.f32_scale;
+    // lane j holds the bias of channel k0 + j, aligned: its one load serves the chunk, and a value costs a shift,
+    // an addition and a shuffle (cblock_value decides on delta, bias and ReLU anew for every one)
+    const int dr = a.has_bias && a.delta < 0 ? -a.delta : 0;
+    const long long bl = a.has_bias && k0 + lane < K ? (long long)__ldg(a.bias + k0 + lane) << max(a.delta, 0) : 0;
+    const long long floor = a.relu ? 0ll : LLONG_MIN;
+    auto value = [&](int j) -> long long {
+        const int k = min(k0 + j, K - 1);
+        if constexpr (SC) return cblock_value<SC>(a, k, (long long)acc[j], a.has_bias ? __ldg(a.bias + k) : 0);
+        return max(((long long)acc[j] << dr) + __shfl_sync(0xffffffffu, bl, j), floor);
+    };
+#pragma unroll 1
+    for (int c0 = 0; c0 < 32 && k0 + c0 < K; c0 += per) {
 #pragma unroll
-    for (int c0 = 0; c0 < 32; c0 += 8) {
-        if (c0 % per) continue;  // fp32 rounds start at 0 and 16
-        uint32_t wv[16];
-        if (f32) {
+        for (int q = 0; q < 4; ++q) {
+            // one 16-byte piece: four fp32 images or two int64 sums
+            uint32_t wv[4];
+            if (f32) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int k = k0 + c0 + j;
-                float v = 0.0f;
-                if (m >= 0 && k < a.K && c0 + j < 32)
-                    v = __ll2float_rn(cblock_value<SC>(a, k, (long long)acc[(c0 + j) & 31], a.has_bias ? __ldg(a.bias + k) : 0)) *
-                        a.f32_scale;
-                wv[j] = __float_as_uint(v);
+                for (int e = 0; e < 4; ++e) wv[e] = __float_as_uint(__ll2float_rn(value(c0 + 4 * q + e)) * f32_scale);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const long long v = value(c0 + 2 * q + e);
+                    wv[2 * e] = (uint32_t)(unsigned long long)v;
+                    wv[2 * e + 1] = (uint32_t)((unsigned long long)v >> 32);
+                }
             }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int k = k0 + c0 + j;
-                long long v = 0;
-                if (m >= 0 && k < a.K) v = cblock_value<SC>(a, k, (long long)acc[c0 + j], a.has_bias ? __ldg(a.bias + k) : 0);
-                wv[2 * j] = (uint32_t)(unsigned long long)v;
-                wv[2 * j + 1] = (uint32_t)((unsigned long long)v >> 32);
-            }
+            *reinterpret_cast<uint4*>(wbuf + lane * 64 + 16 * (q ^ ((lane >> 1) & 3))) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4*>(wbuf + lane * 64 + 16 * (q ^ ((lane >> 1) & 3))) =
-                make_uint4(wv[4 * q], wv[4 * q + 1], wv[4 * q + 2], wv[4 * q + 3]);
         __syncwarp();
 #pragma unroll
         for (int it = 0; it < 4; ++it) {
             const int r = (lane >> 2) + 8 * it, pc = lane & 3;
             const long long mr = __shfl_sync(0xffffffffu, m, r);
             const uint4 v = *reinterpret_cast<const uint4*>(wbuf + r * 64 + 16 * (pc ^ ((r >> 1) & 3)));
-            const int kk = k0 + c0 + pc * (f32 ? 4 : 2);
-            if (mr >= 0 && kk < a.K) {
-                if (f32)
-                    *reinterpret_cast<uint4*>(static_cast<float*>(a.y) + mr * a.K + kk) = v;
-                else
-                    *reinterpret_cast<uint4*>(static_cast<long long*>(a.y) + mr * a.K + kk) = v;
-            }
+            const int kk = k0 + c0 + pc * (per / 4);
+            if (mr >= 0 && kk < K) *reinterpret_cast<uint4*>(y + (mr * K + kk) * esz) = v;
         }
         __syncwarp();
     }
