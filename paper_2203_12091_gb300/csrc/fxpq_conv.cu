@@ -415,7 +415,11 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
         // then whole runs of a pixel row, where gathered rows cost about 2600 cycles per 8 taps (ResNet conv1,
         // 7 x 7 / 2 of 128 images, 455 -> 216 us with its copy; AlexNet conv1, 11 x 11 / 4 of 256, 431 -> 336)
         const S2dPlan p = s2d_plan(d);
-        if (p.ok && ws && ws_bytes >= p.x_bytes + p.w_bytes && s2d_enabled()) {
+        // Rewriting the input is a launch of its own: worth it where the gathered form's row tiles take more than one
+        // round over the SMs (7 x 7 / 2, 98 tiles: 14.0 us rewritten, 11.5 gathered; 196 tiles: 15.0 / 17.3);
+        // a chosen alternative takes this form at any size
+        const bool rounds = (M + 127) / 128 * ((a.K + 63) / 64) > num_sms() || getenv("FXPQ_CONV_PATH");
+        if (p.ok && rounds && ws && ws_bytes >= p.x_bytes + p.w_bytes && s2d_enabled()) {
             char* base = static_cast<char*>(ws);
             const long long npix = (long long)a.N * p.H2 * p.W2 * a.px, nw = (long long)a.K * p.R2 * p.S2 * (p.C2 / 8) * a.pw;
             const unsigned xb = (unsigned)((npix + 255) / 256), wb = (unsigned)((nw + 255) / 256);

@@ -153,6 +153,8 @@ __device__ __forceinline__ void cblock_epilogue_store(const ConvArgs& a, long lo
     }
 }
 
+int num_sms();  // of the current device
+
 fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, const int32_t* bias, void* y,
                       ConvArgs& a, int32_t* out_scale, bool& need64);
 fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64, cudaStream_t st, void* ws,

@@ -25,17 +25,6 @@ bool conv_path_is(const char* name) {
 }
 bool g_tc_attr_set = false;
 
-int num_sms() {
-    std::lock_guard<std::mutex> lk(g_tc_mu);
-    if (g_num_sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (g_num_sms <= 0) g_num_sms = 1;
-    }
-    return g_num_sms;
-}
-
 
 // Largest |limb| of a format's codes: the only plane (k <= 8) or the hi / lo limb (k > 8).
 long long limb_max(const fxpq_fmt& f, int plane) {
@@ -47,6 +36,17 @@ long long limb_max(const fxpq_fmt& f, int plane) {
 }
 
 }  // namespace
+
+int num_sms() {
+    std::lock_guard<std::mutex> lk(g_tc_mu);
+    if (g_num_sms == 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
+        if (g_num_sms <= 0) g_num_sms = 1;
+    }
+    return g_num_sms;
+}
 
 // Patch shape of a layer's output: TW x TH pixels of TN images, at most 128, with the fewest tiles (a 7 x 7 map
 // of 128 images takes 49 tiles like its 6272 rows do, not 128).  Only widths and heights that divide the map
@@ -161,8 +161,23 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         ps = patch_shape(a, TC_BM);
     const int kbt = (a.Cp + TC_BK - 1) / TC_BK;
     const int kb_flat = (a.R * a.S * a.Cp + TC_BK - 1) / TC_BK;
-    const bool use_patch = ps.TW > 0 && (narrow || conv_path_is("tc_patch") ||
-                                         (double)ps.tiles * a.R * a.S * kbt <= 4.0 * (double)row_tiles_est * kb_flat);
+    // How many of its k-blocks a layer may spend as patches for one of the flattened reduction (K = 64 / 256, 3x3,
+    // 588 row tiles, us as patches and gathered): 32 channels, 1.8 times as many, 15.8 / 22.4 and 31.5 / 35.2; 16
+    // channels, 3 times, 25.3 / 19.4 and 37.3 / 29.4.  Pixels that are not whole 32-byte sectors cost their boxes
+    // double: 120 channels, 1.06 times, 37.6 / 46.2; 136 channels, 1.35 times, 55.7 / 49.3; 24 channels 63.9 / 35.2.
+    // Where each tile has an SM to itself the latency of a k-block decides instead, and patches win longer (24
+    // channels, 21 tiles: 8.9 / 9.9).  Two-limb reductions drain a group per limb pair, which hides less of the
+    // patches' k-blocks (32 channels, 1.8 times: 68 / 62; 80 channels, 1.5 times: 99.5 / 103; 16-bit 24 channels, 5 x 5,
+    // 2.5 times: 272 / 103).
+    // Eight-channel patches take the gathered form's k-blocks, a box per tap: one-limb layers 1.1 to 1.4 times faster,
+    // two-limb ones only with few taps (128 channels, 3 x 3, 1568 tiles: 134 / 140; 64 channels, 7 x 7: 132 / 114).
+    // (The space-to-depth form has no more k-blocks as patches.)
+    const bool two_limb = a.px * a.pw > 1, lone = row_tiles_est * ((a.K + 63) / 64) <= sms;
+    const bool any_patch = conv_path_is("tc") || conv_path_is("tc_bn256") || a.x_sw != a.Cp;
+    const double most = any_patch ? 4.0 : a.Cp % 16 ? (lone && !two_limb ? 2.3 : 1.15) : two_limb ? 1.55 : lone ? 4.0 : 2.0;
+    const bool use_patch =
+        ps.TW > 0 && (conv_path_is("tc_patch") || (narrow ? any_patch || !two_limb || (!lone && a.R * a.S <= 16)
+                                                          : (double)ps.tiles * a.R * a.S * kbt <= most * (double)row_tiles_est * kb_flat));
     P.kbt = kbt;
     if (!plan_tc(a, d, P, acc64, use_patch && !narrow ? a.R * a.S * kbt : kb_flat)) return FXPQ_OK;
     // ... with few row tiles (FC layers at small batches) they take 256-column tiles and a split
@@ -219,12 +234,14 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         P.TH = P.TW = P.TN = P.tiles_p = P.tiles_q = 1;
         // window mode for 8-channel stride-1 layers with at most 64 output channels: 8 x 16 output
         // patches, one input window per tile and limb plane, weights resident in shared memory, one
-        // exact fp32 accumulator per limb pair (R * S2 * 8 products each)
+        // exact fp32 accumulator per limb pair (R * S2 * 8 products each); with several limb pairs, as one
+        // pair's sums take the fp32 epilogue of the patch tiles (3 x 3, 64 channels, 8-bit, 6272 tiles: 188 us as
+        // windows, 130 as patches; 16-bit, 1568 tiles: 23 / 103)
         {
             const int S2 = (a.S + 1) & ~1;
             const int WW = 8 + S2 - 1, WH = 16 + a.R - 1;
             const int win_bytes = (WW * WH * 16 + 127) / 128 * 128;
-            bool ok = a.stride == 1 && a.Cp == 8 && a.x_sw == 8 && a.K <= 64 && a.N > 0 && a.R * S2 <= 16 && 8 * WW <= 256 &&
+            bool ok = two_limb && a.stride == 1 && a.Cp == 8 && a.x_sw == 8 && a.K <= 64 && a.N > 0 && a.R * S2 <= 16 && 8 * WW <= 256 &&
                       WH <= 256 && a.px * win_bytes <= TC_BM * TC_BK * 2 &&
                       a.pw * a.R * (S2 / 2) * 64 * 32 <= tc_stages(64) * 64 * TC_BK * 2 && !conv_path_is("tc_rows") &&
                       !conv_path_is("tc_nowin");

@@ -646,6 +646,26 @@ def test_space_to_depth_parity(F, H, C, K, R, st, pad, kx, kw, mode):
     assert s == ws and np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("N,H,C,K,R,st,kx", [(2, 30, 16, 64, 3, 1, 7), (26, 30, 16, 64, 3, 1, 7), (2, 30, 24, 64, 5, 1, 7),
+                                             (26, 30, 24, 64, 3, 1, 7), (26, 30, 120, 64, 3, 1, 7), (2, 30, 32, 64, 3, 1, 16),
+                                             (2, 30, 80, 64, 3, 1, 16), (2, 30, 3, 64, 5, 1, 16), (26, 30, 3, 72, 3, 1, 16),
+                                             (2, 30, 3, 64, 3, 1, 7), (2, 30, 3, 64, 3, 2, 7), (90, 30, 3, 64, 3, 2, 7)])
+def test_chosen_form_parity(F, N, H, C, K, R, st, kx):
+    """The form that a layer takes by itself, patches, gathered rows or space-to-depth, on both sides of its lines."""
+    if os.environ.get("FXPQ_CONV_PATH") != "tc":
+        pytest.skip("once")
+    rng = np.random.default_rng(N * C + R)
+    fx, fw, fb, fy = F.fmt(kx, 0, kx - 3), F.fmt(kx, 1, kx - 1), F.fmt(16, 1, 14), F.fmt(8, 0, 2)
+    x, w, b = rand_codes(rng, (N, H, H, C), kx, 0), rand_codes(rng, (K, R, R, C), kx, 1), rand_codes(rng, (K,), 16, 1)
+    del os.environ["FXPQ_CONV_PATH"]
+    try:
+        got, s = run_conv(F, x, fx, w, fw, b, fb, st, R // 2, True, 0, fy, (C + 7) // 8 * 8)
+    finally:
+        os.environ["FXPQ_CONV_PATH"] = "tc"
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, st, R // 2, True, 0, fy)
+    assert s == ws and np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("N,H,C,K,R,st,pad", [(5, 7, 64, 64, 3, 1, 1), (130, 3, 64, 72, 3, 1, 1), (3, 14, 96, 256, 5, 1, 2),
                                               (4, 15, 16, 128, 3, 2, 1), (2, 30, 128, 136, 1, 2, 0), (2, 33, 24, 64, 3, 3, 1),
                                               (1, 70, 40, 64, 3, 7, 2), (7, 5, 200, 384, 3, 1, 1), (2, 19, 64, 64, 3, 8, 1)])
