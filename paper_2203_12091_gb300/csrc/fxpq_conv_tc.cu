@@ -225,6 +225,15 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return FXPQ_OK;
+        P.rows2 = a.K % BN ? (a.K % BN + 7) / 8 * 8 : 0;
+        P.idesc2 = make_idesc(TC_BM, (P.rows2 + 15) / 16 * 16);
+        if (P.rows2) {
+            const cuuint32_t box2[3] = {(cuuint32_t)TC_BK, (cuuint32_t)P.rows2, 1};
+            if (enc(&P.tmap_w2, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half*>(a.w), dims, strides, box2, es,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                return FXPQ_OK;
+        }
         P.patch = 0;
         P.rows_tma = 0;
         P.w32 = 0;

@@ -107,6 +107,9 @@ struct TcGroup {
 
 struct TcParams {
     CUtensorMap tmap_w;  // weights as [planes][K][R*S*Cp] fp16, box {64, BN, 1}, 128-byte swizzle
+    CUtensorMap tmap_w2; // rows2 > 0: the same with a box of rows2 channels, for the last column tile (a TMA box is
+    int rows2;           // slow where it lies outside the tensor: 72 channels of 3 x 3 x 64, 1568 row tiles, 54.9 us with
+    uint32_t idesc2;     // 56 of a box's 64 rows past the end, NEWX without); idesc2: MMAs of rows2 columns, rounded to 16
     CUtensorMap tmap_y;  // output codes: [M][K] box {64, 128} (linear tiles) or [N][P][Q][K] box {64, TW, TH, 1}
     CUtensorMap tmap_x;  // patch tiles: activations [planes][N][H][W][Cp], box {64, TW, TH, 1, 1}; window mode:
                          // [planes][N][H][W * 8], box {8 WW, WH, 1, 1} (a window row is one 16 WW-byte run)
@@ -1049,6 +1052,9 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 if (SPLIT) TileIter::split(P, ut / P.ksplit, T.tn, T.iq, T.ip, T.ng);
                 const int tm = T.ng, tn = T.tn, n_img = T.ng * P.TN;  // tm: TMA row tiles
                 const int hp0 = T.ip * P.TH * a.stride - a.pad, wq0 = T.iq * P.TW * a.stride - a.pad;
+                const bool last_n = P.rows2 && tn == P.tiles_n - 1;
+                const CUtensorMap* const mw = last_n ? &P.tmap_w2 : &P.tmap_w;
+                const uint32_t b_bytes = last_n ? (uint32_t)P.rows2 * (TC_BK * 2) : (uint32_t)B_BYTES;
                 if (!SPLIT) T.next(P);
                 for (int gi = SPLIT ? P.gs[sp] : 0; gi < (SPLIT ? P.gs[sp + 1] : P.n_groups) && ok; ++gi) {
                     const TcGroup g = P.g[gi];
@@ -1066,7 +1072,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                             }
                             const uint32_t fb = PK ? pkfull0 + 8 * stage : full0 + 8 * stage;
                             const uint32_t pk_bytes = PK ? (uint32_t)(BN * 8 * P.wk) : 0u;
-                            mbar_arrive_expect_tx(fb, a_bytes + (PK ? pk_bytes : (uint32_t)B_BYTES));
+                            mbar_arrive_expect_tx(fb, a_bytes + (PK ? pk_bytes : b_bytes));
                             if (narrow) {
                                 for (int tl = 0; tl < 8; ++tl) {
                                     const int tap = kb * 8 + tl;
@@ -1086,7 +1092,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                                 bulk_load(smem_u32(sP + stage * (BN * 64)),
                                           P.wpack + ((size_t)kb * P.K_pad + (size_t)tn * BN) * 2 * P.wk, pk_bytes, fb);
                             else
-                                tma_load_3d(smem_u32(sB + stage * B_BYTES), &P.tmap_w, wx, tn * BN, g.w_plane, fb);
+                                tma_load_3d(smem_u32(sB + stage * B_BYTES), mw, wx, tn * BN, g.w_plane, fb);
                         }
                         if (++stage == TC_STAGES) {
                             stage = 0;
@@ -1133,6 +1139,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
             const int t = SPLIT ? ut / P.ksplit : ut, sp = SPLIT ? ut - t * P.ksplit : 0;
             (void)sp;
             const int tm = t / P.tiles_n, tn = t % P.tiles_n;
+            const bool last_n = P.rows2 && tn == P.tiles_n - 1;
             long long rowoff[AR];  // element offset of the (r, s) = (0, 0) tap of each row (may be negative)
             int p0[AR], q0[AR];
 #pragma unroll
@@ -1157,11 +1164,11 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         break;
                     }
                     const uint32_t dA = smem_u32(sA + stage * A_BYTES);
-                    if (warp == 0) {  // the weight tile: one TMA, zero-filled past K and R*S*Cp
+                    if (warp == 0) {  // the weight tile: one TMA, zero-filled past R*S*Cp
                         __syncwarp();
-                        mbar_arrive_expect_tx(full0 + 8 * stage, (uint32_t)B_BYTES);
-                        tma_load_3d(smem_u32(sB + stage * B_BYTES), &P.tmap_w, kb * TC_BK, tn * BN, g.w_plane,
-                                    full0 + 8 * stage);
+                        mbar_arrive_expect_tx(full0 + 8 * stage, last_n ? (uint32_t)P.rows2 * (TC_BK * 2) : (uint32_t)B_BYTES);
+                        tma_load_3d(smem_u32(sB + stage * B_BYTES), last_n ? &P.tmap_w2 : &P.tmap_w, kb * TC_BK, tn * BN,
+                                    g.w_plane, full0 + 8 * stage);
                     }
                     const int f = kb * TC_BK + 8 * c;  // this thread's chunk of the flattened (r, s, c) index
                     const bool fvalid = f < P.RSC;
@@ -1438,6 +1445,14 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     const int cb = cw * CPW + c;
                     const int k0 = tn * BN + cb * 32;
                     const uint32_t run_col = run_base + cb * 32;
+                    if (!WEPI && k0 >= a.K) {  // no channel of this chunk is stored
+                        if (c == CPW - 1) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(accempty0 + 8 * buf);
+                        }
+                        continue;
+                    }
                     if constexpr (!FE) {
                     if (BN == 64 && sizeof(ACC) == 8 && !SC && P.patch == 3 && P.w32) {
                         // window mode, two-limb x and w, 32-bit arithmetic.  With the limb sums S_hh,
@@ -2004,6 +2019,8 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         for (int ut = blockIdx.x; ut < (SPLIT ? P.n_units : P.n_tiles) && ok; ut += gridDim.x) {
             const int t = SPLIT ? ut / P.ksplit : ut, sp = SPLIT ? ut - t * P.ksplit : 0;
             (void)sp;
+            // (channels past the last tile's rows2 are whatever the stage holds; their sums are never stored)
+            const uint32_t idesc = !PK && P.rows2 && t % P.tiles_n == P.tiles_n - 1 ? P.idesc2 : IDESC;
             for (int gi = SPLIT ? P.gs[sp] : 0; gi < (SPLIT ? P.gs[sp + 1] : P.n_groups) && ok; ++gi) {
                 const TcGroup g = P.g[gi];
                 const uint32_t buf = P.nbuf == 2 ? (gcount & 1) : 0;
@@ -2032,7 +2049,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     if (++cb > cb_last) cb = 0;
 #pragma unroll
                     for (int kk = 0; kk < TC_BK / 16; ++kk) {
-                        if (kk < ns) tc_mma(d, ad + a_kstep * kk, bd + 2 * kk, IDESC, accum);
+                        if (kk < ns) tc_mma(d, ad + a_kstep * kk, bd + 2 * kk, idesc, accum);
                         accum = 1;
                     }
                     tc_commit(empty0 + 8 * stage);

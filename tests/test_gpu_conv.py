@@ -646,6 +646,20 @@ def test_space_to_depth_parity(F, H, C, K, R, st, pad, kx, kw, mode):
     assert s == ws and np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("K,mode", [(8, 0), (24, 0), (72, 0), (120, 0), (136, 0), (200, 0), (264, 0), (2, 1), (10, 2), (77, 2), (130, 1)])
+@pytest.mark.parametrize("N,H,C,R,kx", [(3, 12, 64, 3, 7), (3, 12, 72, 1, 7), (5, 1, 700, 1, 8), (2, 9, 24, 3, 16), (40, 20, 64, 3, 8)])
+def test_last_column_tile_parity(F, K, mode, N, H, C, R, kx):
+    """Channel counts off every tile width: the last column tile's shorter weight box and MMA, after a full tile and
+    alone, in patch, row, split and two-limb tiles (the last shape in several tiles per CTA and exact groups)."""
+    rng = np.random.default_rng(K * C + R)
+    fx, fw, fb = F.fmt(kx, 0, kx - 3), F.fmt(kx, 1, kx - 1), F.fmt(16, 1, 14)
+    fy = F.fmt(8, 0, 2) if mode == 0 else None
+    x, w, b = rand_codes(rng, (N, H, H, C), kx, 0), rand_codes(rng, (K, R, R, C), kx, 1), rand_codes(rng, (K,), 16, 1)
+    got, s = run_conv(F, x, fx, w, fw, b, fb, 1, R // 2, True, mode, fy, (C + 7) // 8 * 8)
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, 1, R // 2, True, mode, fy)
+    assert s == ws and np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("N,H,C,K,R,st,kx", [(2, 30, 16, 64, 3, 1, 7), (26, 30, 16, 64, 3, 1, 7), (2, 30, 24, 64, 5, 1, 7),
                                              (26, 30, 24, 64, 3, 1, 7), (26, 30, 120, 64, 3, 1, 7), (2, 30, 32, 64, 3, 1, 16),
                                              (2, 30, 80, 64, 3, 1, 16), (2, 30, 3, 64, 5, 1, 16), (26, 30, 3, 72, 3, 1, 16),
