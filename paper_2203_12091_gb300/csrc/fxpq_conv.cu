@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(256) s2d_kernel(const __half* __restrict__ x, 
                                                   int W, int K, int R, int S, int pad, long long x_ps, long long w_ps,
                                                   S2dPlan p, int px, int pw, unsigned xb, uint4* __restrict__ x2,
                                                   uint4* __restrict__ w2) {
+    pdl_wait();
     const int c8 = p.C2 / 8;
     if (blockIdx.x < xb) {
         const long long npix = (long long)N * p.H2 * p.W2;
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(256) s2d_kernel(const __half* __restrict__ x, 
 
 template <typename ACC>
 __global__ void splitk_reduce_kernel(const ConvArgs a, const ACC* __restrict__ part, int ks) {
+    pdl_wait();
     const long long total = a.M * a.K;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
@@ -182,9 +184,9 @@ fxpq_status launch_splitk_reduce(const ConvArgs& a, const void* part, int ks, bo
     if (blocks > 152LL * 8) blocks = 152LL * 8;
     if (blocks < 1) blocks = 1;
     if (acc64)
-        splitk_reduce_kernel<long long><<<(unsigned)blocks, 256, 0, st>>>(a, static_cast<const long long*>(part), ks);
+        launch_pdl(splitk_reduce_kernel<long long>, (unsigned)blocks, 256, 0, st, a, static_cast<const long long*>(part), ks);
     else
-        splitk_reduce_kernel<int><<<(unsigned)blocks, 256, 0, st>>>(a, static_cast<const int*>(part), ks);
+        launch_pdl(splitk_reduce_kernel<int>, (unsigned)blocks, 256, 0, st, a, static_cast<const int*>(part), ks);
     return after_launch("splitk_reduce");
 }
 
@@ -423,7 +425,7 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
             char* base = static_cast<char*>(ws);
             const long long npix = (long long)a.N * p.H2 * p.W2 * a.px, nw = (long long)a.K * p.R2 * p.S2 * (p.C2 / 8) * a.pw;
             const unsigned xb = (unsigned)((npix + 255) / 256), wb = (unsigned)((nw + 255) / 256);
-            s2d_kernel<<<xb + wb, 256, 0, st>>>(a.x, a.w, a.N, a.H, a.W, a.K, a.R, a.S, a.pad, a.x_ps, a.w_ps, p, a.px, a.pw,
+            launch_pdl(s2d_kernel, xb + wb, 256, 0, st, a.x, a.w, a.N, a.H, a.W, a.K, a.R, a.S, a.pad, a.x_ps, a.w_ps, p, a.px, a.pw,
                                                 xb, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + p.x_bytes));
             fxpq_status s = after_launch("s2d");
             if (s != FXPQ_OK) return s;

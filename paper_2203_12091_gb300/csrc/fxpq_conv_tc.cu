@@ -522,39 +522,38 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     launched = true;
     if (a.has_scale && P.ksplit == 1) return launch_conv_tc_scaled(P, BN, acc64, grid, st);
     if (P.patch == 3 && (P.w32 || P.wf32))  // window mode, 32-bit two-limb epilogue: its own instance (never split)
-        conv_tc_kernel<64, long long, false, false, false, true>
-            <<<grid, tc_threads_win(), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, long long, false, false, false, true>, grid, tc_threads_win(), tc_smem_bytes<64>(), st, P);
     else if (P.patch == 4 && (P.fast_store || a.out_mode == FXPQ_OUT_F32))
         // 64-channel window mode: the instance with its own shared-memory layout and 16 epilogue warps
-        conv_tc_kernel<64, int, false, false, false, false, true><<<grid, tc_threads_win(), tc_smem_w64(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, int, false, false, false, false, true>, grid, tc_threads_win(), tc_smem_w64(), st, P);
     else if (P.patch == 4) {
         launched = false;  // no TMA store of the output: the CUDA-core kernel runs instead
         return FXPQ_OK;
     }
     else if (P.pk && P.ksplit > 1)
-        conv_tc_kernel<256, int, false, true, true><<<grid, tc_threads_pk(256, true), tc_smem_bytes<256, true>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<256, int, false, true, true>, grid, tc_threads_pk(256, true), tc_smem_bytes<256, true>(), st, P);
     else if (P.pk)
-        conv_tc_kernel<256, int, false, false, true><<<grid, tc_threads_pk(256, true), tc_smem_bytes<256, true>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<256, int, false, false, true>, grid, tc_threads_pk(256, true), tc_smem_bytes<256, true>(), st, P);
     else if (P.ksplit > 1 && BN == 256)
-        conv_tc_kernel<256, int, false, true><<<grid, tc_threads(256), tc_smem_bytes<256>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<256, int, false, true>, grid, tc_threads(256), tc_smem_bytes<256>(), st, P);
     else if (P.ksplit > 1 && acc64)
-        conv_tc_kernel<64, long long, false, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, long long, false, true>, grid, tc_threads(64), tc_smem_bytes<64>(), st, P);
     else if (P.ksplit > 1)
-        conv_tc_kernel<64, int, false, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, int, false, true>, grid, tc_threads(64), tc_smem_bytes<64>(), st, P);
     else if (P.fepi && BN == 64)
-        conv_tc_kernel<64, int, false, false, false, false, false, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, int, false, false, false, false, false, true>, grid, tc_threads(64), tc_smem_bytes<64>(), st, P);
     else if (P.fepi && BN == 128)
-        conv_tc_kernel<128, int, false, false, false, false, false, true><<<grid, tc_threads(128), tc_smem_bytes<128>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<128, int, false, false, false, false, false, true>, grid, tc_threads(128), tc_smem_bytes<128>(), st, P);
     else if (P.fepi)
-        conv_tc_kernel<256, int, false, false, false, false, false, true><<<grid, tc_threads(256), tc_smem_bytes<256>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<256, int, false, false, false, false, false, true>, grid, tc_threads(256), tc_smem_bytes<256>(), st, P);
     else if (acc64)
-        conv_tc_kernel<64, long long, false><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, long long, false>, grid, tc_threads(64), tc_smem_bytes<64>(), st, P);
     else if (BN == 64)
-        conv_tc_kernel<64, int, false><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, int, false>, grid, tc_threads(64), tc_smem_bytes<64>(), st, P);
     else if (BN == 128)
-        conv_tc_kernel<128, int, false><<<grid, tc_threads(128), tc_smem_bytes<128>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<128, int, false>, grid, tc_threads(128), tc_smem_bytes<128>(), st, P);
     else
-        conv_tc_kernel<256, int, false><<<grid, tc_threads(256), tc_smem_bytes<256>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<256, int, false>, grid, tc_threads(256), tc_smem_bytes<256>(), st, P);
     launched = true;
     const fxpq_status s = after_launch("conv_tc");
     if (s != FXPQ_OK || P.ksplit == 1) return s;

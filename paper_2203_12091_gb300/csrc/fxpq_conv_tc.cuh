@@ -109,7 +109,7 @@ struct TcParams {
     CUtensorMap tmap_w;  // weights as [planes][K][R*S*Cp] fp16, box {64, BN, 1}, 128-byte swizzle
     CUtensorMap tmap_w2; // rows2 > 0: the same with a box of rows2 channels, for the last column tile (a TMA box is
     int rows2;           // slow where it lies outside the tensor: 72 channels of 3 x 3 x 64, 1568 row tiles, 54.9 us with
-    uint32_t idesc2;     // 56 of a box's 64 rows past the end, NEWX without); idesc2: MMAs of rows2 columns, rounded to 16
+    uint32_t idesc2;     // 56 of a box's 64 rows past the end, 31.4 without); idesc2: MMAs of rows2 columns, rounded to 16
     CUtensorMap tmap_y;  // output codes: [M][K] box {64, 128} (linear tiles) or [N][P][Q][K] box {64, TW, TH, 1}
     CUtensorMap tmap_x;  // patch tiles: activations [planes][N][H][W][Cp], box {64, TW, TH, 1, 1}; window mode:
                          // [planes][N][H][W * 8], box {8 WW, WH, 1, 1} (a window row is one 16 WW-byte run)
@@ -205,6 +205,9 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
                      reinterpret_cast<uint64_t>(map)),
                  "r"(x), "r"(y), "r"(src)
                  : "memory");
+}
+__device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
@@ -913,11 +916,18 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (threadIdx.x == 32) {  // the descriptors that this launch uses, fetched while the kernel sets up
+        prefetch_tmap(&P.tmap_w);
+        if (P.rows2) prefetch_tmap(&P.tmap_w2);
+        if (P.patch || P.rows_tma) prefetch_tmap(&P.tmap_x);
+        if (P.fast_store) prefetch_tmap(&P.tmap_y);
+    }
     if (warp == MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(TMEM_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
+    pdl_wait();
     // window mode, 32-bit epilogue: per output channel the aligned bias B' = b 2^delta split as
     // (B' >> 16, B' & 0xFFFF), in the last 512 bytes of the B region (the resident weights stay below)
     int2* wtab = reinterpret_cast<int2*>(sB + TC_STAGES * B_BYTES - 512);

@@ -37,19 +37,19 @@ fxpq_status launch_conv_tc_scaled(const TcParams& P, int BN, bool acc64, int gri
         }
     }
     if (P.fepi && BN == 64)
-        conv_tc_kernel<64, int, true, false, false, false, false, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, int, true, false, false, false, false, true>, grid, tc_threads(64), tc_smem_bytes<64>(), st, P);
     else if (P.fepi && BN == 128)
-        conv_tc_kernel<128, int, true, false, false, false, false, true><<<grid, tc_threads(128), tc_smem_bytes<128>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<128, int, true, false, false, false, false, true>, grid, tc_threads(128), tc_smem_bytes<128>(), st, P);
     else if (P.fepi)
-        conv_tc_kernel<256, int, true, false, false, false, false, true><<<grid, tc_threads(256), tc_smem_bytes<256>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<256, int, true, false, false, false, false, true>, grid, tc_threads(256), tc_smem_bytes<256>(), st, P);
     else if (acc64)
-        conv_tc_kernel<64, long long, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, long long, true>, grid, tc_threads(64), tc_smem_bytes<64>(), st, P);
     else if (BN == 64)
-        conv_tc_kernel<64, int, true><<<grid, tc_threads(64), tc_smem_bytes<64>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<64, int, true>, grid, tc_threads(64), tc_smem_bytes<64>(), st, P);
     else if (BN == 128)
-        conv_tc_kernel<128, int, true><<<grid, tc_threads(128), tc_smem_bytes<128>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<128, int, true>, grid, tc_threads(128), tc_smem_bytes<128>(), st, P);
     else
-        conv_tc_kernel<256, int, true><<<grid, tc_threads(256), tc_smem_bytes<256>(), st>>>(P);
+        launch_pdl(conv_tc_kernel<256, int, true>, grid, tc_threads(256), tc_smem_bytes<256>(), st, P);
     return after_launch("conv_tc_scale");
 }
 

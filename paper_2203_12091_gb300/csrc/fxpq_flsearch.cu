@@ -417,6 +417,7 @@ __global__ void __launch_bounds__(FS_THREADS, NRB == 2 ? FS_BLOCKS_PER_SM : 2)
         const int nz = (int)((sizeof(FsSmem) - sizeof(sm.sorted)) / 4);
         for (int i = threadIdx.x; i < nz; i += FS_THREADS) z[i] = 0u;
     }
+    pdl_wait();
     __syncthreads();
     if (threadIdx.x == 0) sm.mn = 0xFFFFFFFFu;
     unsigned tmn = 0xFFFFFFFFu, tmx = 0u;
@@ -901,6 +902,7 @@ __global__ void __launch_bounds__(FIN_T) fl_search_final_kernel(const __grid_con
     const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cell = ((int)blockIdx.x - B.fin0[item]) * FIN_WARPS + warp;
     for (int i = lane; i < COL_WORDS; i += 32) sm.col[warp][i] = 0;
+    pdl_wait();
     fin_stage(sm, g);
     if (cell < ncell + 2) {  // warp-uniform
         fin_cell(sm.col[warp] + (lane & (COL_COPIES - 1)), sm, g, F, cell, ncell, lane, 32);
@@ -1096,24 +1098,24 @@ void fs_bins_launch(int variant, int grid, const FsBatch& B, int i0, int i1, cud
         const size_t hb = HS_SMEM;
         const bool vec = variant & 1, l1 = variant & 8;
         if (vec && !l1)
-            fl_search_hist_kernel<true, false><<<grid, HS_T, hb, s>>>(B, i0, i1);
+            launch_pdl(fl_search_hist_kernel<true, false>, grid, HS_T, hb, s, B, i0, i1);
         else if (!l1)
-            fl_search_hist_kernel<false, false><<<grid, HS_T, hb, s>>>(B, i0, i1);
+            launch_pdl(fl_search_hist_kernel<false, false>, grid, HS_T, hb, s, B, i0, i1);
         else if (vec)
-            fl_search_hist_kernel<true, true><<<grid, HS_T, hb, s>>>(B, i0, i1);
+            launch_pdl(fl_search_hist_kernel<true, true>, grid, HS_T, hb, s, B, i0, i1);
         else
-            fl_search_hist_kernel<false, true><<<grid, HS_T, hb, s>>>(B, i0, i1);
+            launch_pdl(fl_search_hist_kernel<false, true>, grid, HS_T, hb, s, B, i0, i1);
         return;
     }
     const size_t sb = sizeof(FsSmem);
     const bool vec = variant & 1, small = variant & 2, narrow = variant & 4, l1 = variant & 8;
 #define FXPQ_FS_LAUNCH(V, L1)                                                            \
     if (narrow && small)                                                                 \
-        fl_search_bins_kernel<V, 10, 2, L1><<<grid, FS_THREADS, sb, s>>>(B, i0, i1);     \
+        launch_pdl(fl_search_bins_kernel<V, 10, 2, L1>, grid, FS_THREADS, sb, s, B, i0, i1);     \
     else if (narrow)                                                                     \
-        fl_search_bins_kernel<V, NJ, 2, L1><<<grid, FS_THREADS, sb, s>>>(B, i0, i1);     \
+        launch_pdl(fl_search_bins_kernel<V, NJ, 2, L1>, grid, FS_THREADS, sb, s, B, i0, i1);     \
     else                                                                                 \
-        fl_search_bins_kernel<V, NJ, NJ, L1><<<grid, FS_THREADS, sb, s>>>(B, i0, i1);
+        launch_pdl(fl_search_bins_kernel<V, NJ, NJ, L1>, grid, FS_THREADS, sb, s, B, i0, i1);
     if (vec && !l1) {
         FXPQ_FS_LAUNCH(true, false)
     } else if (!l1) {
@@ -1182,7 +1184,7 @@ fxpq_status fs_run(FsItemHost* h, int n, FsGlobal* g, cudaStream_t s) {
         }
         j0 = j1;
     }
-    fl_search_final_kernel<<<fblocks, FIN_T, 0, s>>>(B, O, status_ptr());
+    launch_pdl(fl_search_final_kernel, fblocks, FIN_T, 0, s, B, O, status_ptr());
     return after_launch("fl_search_final");
 }
 }  // namespace

@@ -438,6 +438,7 @@ __global__ void __launch_bounds__(HS_T, 1) fl_search_hist_kernel(const __grid_co
         for (int i = (int)tid; i < HS_O_MISC / 4; i += HS_T) z4[i] = make_uint4(0u, 0u, 0u, 0u);
         if (tid < (unsigned)HS_MISC) misc[tid] = tid == HM_MN ? 0xFFFFFFFFu : 0u;
     }
+    pdl_wait();
     __syncthreads();
 
     HsK K;

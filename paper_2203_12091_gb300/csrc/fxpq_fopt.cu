@@ -47,6 +47,7 @@ __device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
 // the reduction index decoded through a table in shared memory (up to CF_TAB steps).
 template <int BM, bool VEC>
 __global__ void __launch_bounds__(256, 2) conv_f32_kernel(const ConvF32Args a) {
+    pdl_wait();
     constexpr int MT = BM / 8;           // output pixels per thread
     constexpr int AV = BM * CF_BK / 4 / 256;  // float4 of the A stage per thread
     constexpr int BV = CF_BN * CF_BK / 4 / 256;
@@ -255,6 +256,7 @@ __global__ void __launch_bounds__(256, 2) conv_f32_kernel(const ConvF32Args a) {
 
 __global__ void maxpool_f32_kernel(const float* __restrict__ x, int N, int H, int W, int C, int k, int stride, int pad,
                                    int P, int Q, float* __restrict__ y) {
+    pdl_wait();
     const long long total = (long long)N * P * Q * C;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const int c = (int)(i % C);
@@ -276,6 +278,7 @@ __global__ void maxpool_f32_kernel(const float* __restrict__ x, int N, int H, in
 
 __global__ void eltwise_f32_kernel(const float* __restrict__ a, const float* __restrict__ b, long long n, int relu,
                                    float* __restrict__ y) {
+    pdl_wait();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float v = a[i] + b[i];
         y[i] = relu ? fmaxf(v, 0.0f) : v;
@@ -284,6 +287,7 @@ __global__ void eltwise_f32_kernel(const float* __restrict__ a, const float* __r
 
 // one thread per (n, c): the mean over H x W (sum in fp32, then divided by H W)
 __global__ void avgpool_f32_kernel(const float* __restrict__ x, int N, int HW, int C, float* __restrict__ y) {
+    pdl_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)N * C) return;
     const long long n = i / C;
@@ -297,6 +301,7 @@ __global__ void avgpool_f32_kernel(const float* __restrict__ x, int N, int HW, i
 // 0 -> +1, -1 -> -1
 __global__ void dequantize_kernel(const __half* __restrict__ codes, long long npix, int Cp, int C, int planes, float scale,
                                   int binary, float* __restrict__ y) {
+    pdl_wait();
     const long long total = npix * C;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const long long pix = i / C;
@@ -415,6 +420,7 @@ __device__ __forceinline__ void ds_walk(const float* __restrict__ xs, long long 
 }
 
 __global__ void __launch_bounds__(DS_T) ds_sum_kernel(const __grid_constant__ DsBatchDev B, DsUnit* units) {
+    pdl_wait();
     __shared__ double red[DS_T / 32];
     const int u = blockIdx.x;
     const DsItemDev& it = B.it[ds_item_of(B, u)];
@@ -428,6 +434,7 @@ __global__ void __launch_bounds__(DS_T) ds_sum_kernel(const __grid_constant__ Ds
 }
 
 __global__ void __launch_bounds__(DS_T) ds_dev_kernel(const __grid_constant__ DsBatchDev B, DsUnit* units) {
+    pdl_wait();
     __shared__ double red[DS_T / 32];
     __shared__ unsigned kmn, kmx;
     const int u = blockIdx.x;
@@ -515,6 +522,7 @@ __device__ __forceinline__ float ds_key_value(unsigned k) {
 // thread 0 the threads' shares of L in order.
 constexpr int DF_T = 64;
 __global__ void __launch_bounds__(DF_T) ds_finish_kernel(const __grid_constant__ DsBatchDev B, const DsUnit* units) {
+    pdl_wait();
     __shared__ double l2s[DF_T];
     __shared__ unsigned kmn, kmx;
     const DsItemDev& it = B.it[blockIdx.x];
@@ -566,6 +574,7 @@ struct CostTerms {
 __global__ void fopt_cost_kernel(const double* __restrict__ stats, long long cand_stride,
                                  const __grid_constant__ CostTerms T, const int* __restrict__ ties, int N,
                                  int n_classes, double* __restrict__ cost) {
+    pdl_wait();
     const int c = blockIdx.x;
     const double* base = stats + (long long)c * cand_stride;
     __shared__ unsigned n_tied, extra;
@@ -612,6 +621,7 @@ __global__ void fopt_cost_kernel(const double* __restrict__ stats, long long can
 // one warp per sample: the number of classes whose logit equals the sample's largest
 template <typename T>
 __global__ void top1_ties_kernel(const T* __restrict__ logits, int N, int C, int32_t* __restrict__ counts) {
+    pdl_wait();
     const int n = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (n >= N) return;
@@ -669,13 +679,13 @@ extern "C" fxpq_status fxpq_conv_f32(const fxpq_conv_f32_desc* h_desc, const flo
     dim3 grid((unsigned)((a.M + bm - 1) / bm), (unsigned)((d.K + CF_BN - 1) / CF_BN));
     cudaStream_t s = as_stream(stream);
     if (bm == 32 && vec)
-        conv_f32_kernel<32, true><<<grid, 256, 0, s>>>(a);
+        launch_pdl(conv_f32_kernel<32, true>, grid, 256, 0, s, a);
     else if (bm == 32)
-        conv_f32_kernel<32, false><<<grid, 256, 0, s>>>(a);
+        launch_pdl(conv_f32_kernel<32, false>, grid, 256, 0, s, a);
     else if (vec)
-        conv_f32_kernel<64, true><<<grid, 256, 0, s>>>(a);
+        launch_pdl(conv_f32_kernel<64, true>, grid, 256, 0, s, a);
     else
-        conv_f32_kernel<64, false><<<grid, 256, 0, s>>>(a);
+        launch_pdl(conv_f32_kernel<64, false>, grid, 256, 0, s, a);
     return after_launch("conv_f32");
 }
 
@@ -686,7 +696,7 @@ extern "C" fxpq_status fxpq_maxpool_f32(const float* d_x, int32_t N, int32_t H, 
     if (P < 1 || Q < 1 || (N > 0 && (!d_x || !d_y))) return FXPQ_ERR_INVALID_ARG;
     const long long total = (long long)N * P * Q * C;
     if (total == 0) return FXPQ_OK;
-    maxpool_f32_kernel<<<grid_of(total), 256, 0, as_stream(stream)>>>(d_x, N, H, W, C, k, stride, pad, P, Q, d_y);
+    launch_pdl(maxpool_f32_kernel, grid_of(total), 256, 0, as_stream(stream), d_x, N, H, W, C, k, stride, pad, P, Q, d_y);
     return after_launch("maxpool_f32");
 }
 
@@ -694,7 +704,7 @@ extern "C" fxpq_status fxpq_eltwise_f32(const float* d_a, const float* d_b, int6
                                         void* stream) {
     if (n < 0 || (n > 0 && (!d_a || !d_b || !d_y))) return FXPQ_ERR_INVALID_ARG;
     if (n == 0) return FXPQ_OK;
-    eltwise_f32_kernel<<<grid_of(n), 256, 0, as_stream(stream)>>>(d_a, d_b, n, relu, d_y);
+    launch_pdl(eltwise_f32_kernel, grid_of(n), 256, 0, as_stream(stream), d_a, d_b, n, relu, d_y);
     return after_launch("eltwise_f32");
 }
 
@@ -703,7 +713,7 @@ extern "C" fxpq_status fxpq_avgpool_f32(const float* d_x, int32_t N, int32_t H, 
     if (N < 0 || H < 1 || W < 1 || C < 1 || (N > 0 && (!d_x || !d_y))) return FXPQ_ERR_INVALID_ARG;
     const long long total = (long long)N * C;
     if (total == 0) return FXPQ_OK;
-    avgpool_f32_kernel<<<(unsigned)((total + 255) / 256), 256, 0, as_stream(stream)>>>(d_x, N, H * W, C, d_y);
+    launch_pdl(avgpool_f32_kernel, (unsigned)((total + 255) / 256), 256, 0, as_stream(stream), d_x, N, H * W, C, d_y);
     return after_launch("avgpool_f32");
 }
 
@@ -711,7 +721,7 @@ extern "C" fxpq_status fxpq_dequantize(const void* d_codes, int64_t npix, int32_
                                        float* d_y, void* stream) {
     if (npix < 0 || C < 1 || Cp < C || !fmt_ok1(fmt) || (npix > 0 && (!d_codes || !d_y))) return FXPQ_ERR_INVALID_ARG;
     if (npix == 0) return FXPQ_OK;
-    dequantize_kernel<<<grid_of(npix * C), 256, 0, as_stream(stream)>>>(
+    launch_pdl(dequantize_kernel, grid_of(npix * C), 256, 0, as_stream(stream),
         static_cast<const __half*>(d_codes), npix, Cp, C, planes_of(fmt), ldexpf(1.0f, -fmt.fl),
         fmt.bits == 1 && fmt.is_signed == 1, d_y);
     return after_launch("dequantize");
@@ -778,13 +788,13 @@ extern "C" fxpq_status fxpq_ds_stats_batch(const fxpq_ds_item* h_items, int32_t 
         }
         if (u > 0x7FFFFFFFLL) return FXPQ_ERR_INVALID_ARG;
         B.unit_end = (int)u;
-        ds_sum_kernel<<<(unsigned)u, DS_T, 0, s>>>(B, units);
+        launch_pdl(ds_sum_kernel, (unsigned)u, DS_T, 0, s, B, units);
         fxpq_status st = after_launch("ds_sum");
         if (st != FXPQ_OK) return st;
-        ds_dev_kernel<<<(unsigned)u, DS_T, 0, s>>>(B, units);
+        launch_pdl(ds_dev_kernel, (unsigned)u, DS_T, 0, s, B, units);
         st = after_launch("ds_dev");
         if (st != FXPQ_OK) return st;
-        ds_finish_kernel<<<B.n, DF_T, 0, s>>>(B, units);
+        launch_pdl(ds_finish_kernel, B.n, DF_T, 0, s, B, units);
         st = after_launch("ds_finish");
         if (st != FXPQ_OK) return st;
     }
@@ -804,7 +814,7 @@ extern "C" fxpq_status fxpq_fopt_cost(const double* d_stats, int64_t cand_stride
         if (h.offset < 0 || h.nu < 1 || h.n_samples < 1) return FXPQ_ERR_INVALID_ARG;
         T.t[i] = CostTermDev{h.offset, h.nu, h.n_samples, h.layer};
     }
-    fopt_cost_kernel<<<n_cand, 128, 0, as_stream(stream)>>>(d_stats, cand_stride, T, d_ties, N, n_classes, d_cost);
+    launch_pdl(fopt_cost_kernel, n_cand, 128, 0, as_stream(stream), d_stats, cand_stride, T, d_ties, N, n_classes, d_cost);
     return after_launch("fopt_cost");
 }
 
@@ -814,10 +824,10 @@ extern "C" fxpq_status fxpq_top1_ties(const void* d_logits, int32_t is_int64, in
     if (N == 0) return FXPQ_OK;
     const unsigned blocks = (unsigned)((N + 7) / 8);
     if (is_int64)
-        top1_ties_kernel<long long><<<blocks, 256, 0, as_stream(stream)>>>(static_cast<const long long*>(d_logits), N, C,
+        launch_pdl(top1_ties_kernel<long long>, blocks, 256, 0, as_stream(stream), static_cast<const long long*>(d_logits), N, C,
                                                                            d_counts);
     else
-        top1_ties_kernel<float><<<blocks, 256, 0, as_stream(stream)>>>(static_cast<const float*>(d_logits), N, C,
+        launch_pdl(top1_ties_kernel<float>, blocks, 256, 0, as_stream(stream), static_cast<const float*>(d_logits), N, C,
                                                                        d_counts);
     return after_launch("top1_ties");
 }

@@ -68,6 +68,7 @@ __global__ void maxpool_kernel(const __half* __restrict__ x, int N, int H, int W
 // integers in fp16, so the half-precision max is exact.
 __global__ void maxpool_vec8_kernel(const uint4* __restrict__ x, int N, int H, int W, int C8, int k, int stride,
                                     int pad, int P, int Q, uint4* __restrict__ y) {
+    pdl_wait();
     const long long total = (long long)N * P * Q * C8;
     const long long step = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
@@ -130,6 +131,7 @@ constexpr int ELT_U = 2;  // 8-code pieces per thread and iteration (their loads
 template <int MODE>
 __global__ void __launch_bounds__(256) eltwise_vec8_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b,
                                                            long long n8, EltVec e, void* __restrict__ y) {
+    pdl_wait();
     const long long step = (long long)gridDim.x * blockDim.x;
     for (long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x; i0 < n8; i0 += ELT_U * step) {
         uint4 va[ELT_U], vb[ELT_U];
@@ -173,6 +175,7 @@ __global__ void __launch_bounds__(256) eltwise_vec8_kernel(const uint4* __restri
 
 // FxP-QLayer on int64 C-Block values (scale 2^-s): codes (fp16 code tensor), int64 copy, or fp32 image.
 __global__ void qlayer_kernel(const long long* __restrict__ v, long long n, OutArgs o, void* y) {
+    pdl_wait();
     const long long step = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += step)
         store_out(o, y, i, 1, 0, v[i], n);
@@ -180,6 +183,7 @@ __global__ void qlayer_kernel(const long long* __restrict__ v, long long n, OutA
 
 __global__ void avgpool_kernel(const __half* __restrict__ x, int N, int HW, int Cp, int planes, long long recip,
                                OutArgs o, void* y) {
+    pdl_wait();
     const long long total = (long long)N * Cp;
     const long long step = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
@@ -233,7 +237,7 @@ extern "C" fxpq_status fxpq_maxpool(const void* d_x, int32_t N, int32_t H, int32
     if (!d_x || !d_y) return FXPQ_ERR_INVALID_ARG;
     const long long total = (long long)N * P * Q * Cp;
     if (planes_of(fmt) == 1 && aligned(d_x, 16) && aligned(d_y, 16)) {
-        maxpool_vec8_kernel<<<grid_for(total / 8), 256, 0, as_stream(stream)>>>(
+        launch_pdl(maxpool_vec8_kernel, grid_for(total / 8), 256, 0, as_stream(stream),
             static_cast<const uint4*>(d_x), N, H, W, Cp / 8, k, stride, pad, P, Q, static_cast<uint4*>(d_y));
         return after_launch("maxpool_vec8");
     }
@@ -269,11 +273,11 @@ extern "C" fxpq_status fxpq_eltwise(const void* d_a, fxpq_fmt fmt_a, const void*
         const int grid = grid_for((n8 + ELT_U - 1) / ELT_U);
         const uint4 *a = static_cast<const uint4*>(d_a), *b = static_cast<const uint4*>(d_b);
         if (out_mode == FXPQ_OUT_CODES)
-            eltwise_vec8_kernel<FXPQ_OUT_CODES><<<grid, 256, 0, as_stream(stream)>>>(a, b, n8, e, d_y);
+            launch_pdl(eltwise_vec8_kernel<FXPQ_OUT_CODES>, grid, 256, 0, as_stream(stream), a, b, n8, e, d_y);
         else if (out_mode == FXPQ_OUT_F32)
-            eltwise_vec8_kernel<FXPQ_OUT_F32><<<grid, 256, 0, as_stream(stream)>>>(a, b, n8, e, d_y);
+            launch_pdl(eltwise_vec8_kernel<FXPQ_OUT_F32>, grid, 256, 0, as_stream(stream), a, b, n8, e, d_y);
         else
-            eltwise_vec8_kernel<FXPQ_OUT_ACC64><<<grid, 256, 0, as_stream(stream)>>>(a, b, n8, e, d_y);
+            launch_pdl(eltwise_vec8_kernel<FXPQ_OUT_ACC64>, grid, 256, 0, as_stream(stream), a, b, n8, e, d_y);
         return after_launch("eltwise_vec8");
     }
     eltwise_kernel<<<grid_for(n_pix * Cp), 256, 0, as_stream(stream)>>>(
@@ -293,7 +297,7 @@ extern "C" fxpq_status fxpq_avgpool(const void* d_x, int32_t N, int32_t H, int32
     if (st != FXPQ_OK) return st;
     if (N == 0) return FXPQ_OK;
     if (!d_x || !d_y) return FXPQ_ERR_INVALID_ARG;
-    avgpool_kernel<<<grid_for((long long)N * Cp), 256, 0, as_stream(stream)>>>(
+    launch_pdl(avgpool_kernel, grid_for((long long)N * Cp), 256, 0, as_stream(stream),
         static_cast<const __half*>(d_x), N, H * W, Cp, planes_of(fmt_x), (long long)recip_code, o, d_y);
     return after_launch("avgpool");
 }
@@ -306,7 +310,7 @@ extern "C" fxpq_status fxpq_qlayer(const int64_t* d_v, int64_t n, int32_t s, int
     if (st != FXPQ_OK) return st;
     if (n == 0) return FXPQ_OK;
     if (!d_v || !d_y) return FXPQ_ERR_INVALID_ARG;
-    qlayer_kernel<<<grid_for(n), 256, 0, as_stream(stream)>>>(reinterpret_cast<const long long*>(d_v), n, o, d_y);
+    launch_pdl(qlayer_kernel, grid_for(n), 256, 0, as_stream(stream), reinterpret_cast<const long long*>(d_v), n, o, d_y);
     return after_launch("qlayer");
 }
 

@@ -204,6 +204,7 @@ constexpr int QI_PIX = 4;
 template <int PLANES>
 __global__ void __launch_bounds__(256) quantize_images3_kernel(const float* __restrict__ x, unsigned npix, unsigned hw,
                                                                QParams p, uint4* __restrict__ out) {
+    pdl_wait();
     bool bad = false;
     const unsigned T = 256, tile = QI_PIX * T;
     for (unsigned long long t0 = (unsigned long long)blockIdx.x * tile; t0 < npix; t0 += (unsigned long long)gridDim.x * tile) {
@@ -784,9 +785,9 @@ extern "C" fxpq_status fxpq_quantize_images(const float* d_x_nchw, int32_t N, in
         const int g = grid_for((npix + QI_PIX - 1) / QI_PIX, 256);
         uint4* o = static_cast<uint4*>(d_y);
         if (planes_of(f) == 1)
-            quantize_images3_kernel<1><<<g, 256, 0, as_stream(stream)>>>(d_x_nchw, (unsigned)npix, (unsigned)(H * W), p, o);
+            launch_pdl(quantize_images3_kernel<1>, g, 256, 0, as_stream(stream), d_x_nchw, (unsigned)npix, (unsigned)(H * W), p, o);
         else
-            quantize_images3_kernel<2><<<g, 256, 0, as_stream(stream)>>>(d_x_nchw, (unsigned)npix, (unsigned)(H * W), p, o);
+            launch_pdl(quantize_images3_kernel<2>, g, 256, 0, as_stream(stream), d_x_nchw, (unsigned)npix, (unsigned)(H * W), p, o);
         return after_launch("quantize_images3");
     }
     quantize_images_kernel<<<grid_for(npix, 256), 256, 0, as_stream(stream)>>>(d_x_nchw, N, C, H, W, c_pad,
