@@ -375,18 +375,6 @@ fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, con
     return FXPQ_OK;
 }
 
-// FXPQ_CONV_PATH=simt selects the CUDA-core kernel for every shape (tests use it to cover both).
-static bool tc_path_enabled() {
-    const char* e = getenv("FXPQ_CONV_PATH");
-    return !(e && strcmp(e, "simt") == 0);
-}
-
-// FXPQ_CONV_PATH=tc_rows / tc_nos2d keep strided 8-channel layers on their own codes.
-static bool s2d_enabled() {
-    const char* e = getenv("FXPQ_CONV_PATH");
-    return !(e && (strcmp(e, "tc_rows") == 0 || strcmp(e, "tc_nos2d") == 0));
-}
-
 // The layer's arguments in the space-to-depth form.
 static ConvArgs s2d_args(const ConvArgs& a, const S2dPlan& p, const __half* x2, const __half* w2) {
     ConvArgs b = a;
@@ -411,7 +399,11 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
                         size_t ws_bytes) {
     const long long M = (long long)a.N * a.P * a.Q;
     if (M == 0) return FXPQ_OK;
-    if (tc_path_enabled()) {
+    // FXPQ_CONV_PATH=tc_rows / tc_nos2d keep strided 8-channel layers on their own codes, simt keeps every layer off
+    // the tensor cores
+    const char* const path = getenv("FXPQ_CONV_PATH");
+    const bool s2d = !(path && (strcmp(path, "tc_rows") == 0 || strcmp(path, "tc_nos2d") == 0));
+    if (!(path && strcmp(path, "simt") == 0)) {
         bool launched = false;
         // A strided 8-channel layer runs in the space-to-depth form when the workspace holds it: its taps are
         // then whole runs of a pixel row, where gathered rows cost about 2600 cycles per 8 taps (ResNet conv1,
@@ -420,8 +412,8 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
         // Rewriting the input is a launch of its own: worth it where the gathered form's row tiles take more than one
         // round over the SMs (7 x 7 / 2, 98 tiles: 14.0 us rewritten, 11.5 gathered; 196 tiles: 15.0 / 17.3);
         // a chosen alternative takes this form at any size
-        const bool rounds = (M + 127) / 128 * ((a.K + 63) / 64) > num_sms() || getenv("FXPQ_CONV_PATH");
-        if (p.ok && rounds && ws && ws_bytes >= p.x_bytes + p.w_bytes && s2d_enabled()) {
+        const bool rounds = (M + 127) / 128 * ((a.K + 63) / 64) > num_sms() || path;
+        if (p.ok && rounds && ws && ws_bytes >= p.x_bytes + p.w_bytes && s2d) {
             char* base = static_cast<char*>(ws);
             const long long npix = (long long)a.N * p.H2 * p.W2 * a.px, nw = (long long)a.K * p.R2 * p.S2 * (p.C2 / 8) * a.pw;
             const unsigned xb = (unsigned)((npix + 255) / 256), wb = (unsigned)((nw + 255) / 256);

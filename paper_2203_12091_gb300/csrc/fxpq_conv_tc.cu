@@ -19,12 +19,7 @@ std::mutex g_tc_mu;
 // 256-column tiles and "tc_bn256" takes them wherever the layer allows (by default they also need
 // enough tiles to keep every SM busy), "tc_win64" keeps window mode's two-limb epilogue in 64-bit
 // arithmetic, "tc_win32" in 32-bit integers, "tc_iepi" the one-group layers' epilogue in integers.
-bool conv_path_is(const char* name) {
-    const char* e = getenv("FXPQ_CONV_PATH");
-    return e && strcmp(e, name) == 0;
-}
 bool g_tc_attr_set = false;
-
 
 // Largest |limb| of a format's codes: the only plane (k <= 8) or the hi / lo limb (k > 8).
 long long limb_max(const fxpq_fmt& f, int plane) {
@@ -139,6 +134,9 @@ EncodeTiledFn encode_tiled() {
 fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStream_t st, bool& launched, void* ws,
                            size_t ws_bytes) {
     launched = false;
+    // (read once: a search of the environment takes about as long as encoding a tensor map)
+    const char* const path = getenv("FXPQ_CONV_PATH");
+    auto conv_path_is = [path](const char* name) { return path && strcmp(path, name) == 0; };
     TcParams P;
     bool acc64 = false;
     const int sms = num_sms();

@@ -13,12 +13,20 @@ from ._lib import DT_F16, DT_I8, DT_I16, DT_I32, DT_U8, DT_U16, OUT_ACC64, OUT_C
 
 
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# The handle of the current stream without a Stream object around it: that object and the pointers' wrappers took
+# half of a small layer's call (9.2 us on the host, 3.4 of them in the library; 4.8 with plain integers, 3.3 of them there).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _s(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
+    return stream.cuda_stream
 
 
 def fmt(bits: int, is_signed: int, fl: int) -> Fmt:
@@ -268,8 +276,7 @@ def fxpq_conv_fwd(desc: L.ConvDesc, x, w, bias, y, stream=None, ws=None) -> int:
     too few tiles for the SMs."""
     scale = L.I32(0)
     L.check("fxpq_conv_fwd", L.lib().fxpq_conv_fwd(ctypes.byref(desc), _p(x), _p(w), _p(bias), _p(y),
-                                                   ctypes.byref(scale), _p(ws),
-                                                   0 if ws is None else ws.numel() * ws.element_size(), _s(stream)))
+                                                   ctypes.byref(scale), _p(ws), 0 if ws is None else ws.nbytes, _s(stream)))
     return scale.value
 
 
