@@ -64,40 +64,56 @@ __global__ void maxpool_kernel(const __half* __restrict__ x, int N, int H, int W
     }
 }
 
-// One-plane codes: 8 channels per thread with 16-byte loads and stores.  The codes are exact
-// integers in fp16, so the half-precision max is exact.
-__global__ void maxpool_vec8_kernel(const uint4* __restrict__ x, int N, int H, int W, int C8, int k, int stride,
-                                    int pad, int P, int Q, uint4* __restrict__ y) {
+__device__ __forceinline__ uint4 max_f16x8(uint4 a, uint4 b) {
+    uint4 o;
+    const uint32_t x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
+    uint32_t m[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __half2 h = __hmax2(*reinterpret_cast<const __half2*>(&x[i]), *reinterpret_cast<const __half2*>(&y[i]));
+        m[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    o.x = m[0], o.y = m[1], o.z = m[2], o.w = m[3];
+    return o;
+}
+
+// One-plane codes: 8 channels per thread with 16-byte loads and stores.  The codes are exact integers in fp16, so the
+// half-precision max is exact.  The loads of a K x K / ST window are all in flight, and its place in the image is found
+// by 32-bit divisions (64-bit ones and loads one after the other bounded this kernel: 3 x 3 / 2 on 128 images of 112 x
+// 112 x 64, 68 -> 48 us, 38 at the rate of a copy; 2 x 2 / 2 on 64 of 224 x 224 x 64, 97 -> 76 us, 76 at that rate; two
+// or four outputs per thread, which share a row, 64 us for the first).  K = 0: any window.
+template <int K, int ST>
+__global__ void __launch_bounds__(256) maxpool_vec8_kernel(const uint4* __restrict__ x, int N, int H, int W, int C8, int k,
+                                                           int stride, int pad, int P, int Q, uint4* __restrict__ y) {
     pdl_wait();
-    const long long total = (long long)N * P * Q * C8;
-    const long long step = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
-        const int c8 = (int)(i % C8);
-        const long long pix = i / C8;
-        const int q = (int)(pix % Q);
-        const int p = (int)((pix / Q) % P);
-        const long long n = pix / ((long long)P * Q);
-        const __half2 ninf = __halves2half2(__ushort_as_half(0xFC00u), __ushort_as_half(0xFC00u));
-        __half2 m0 = ninf, m1 = ninf, m2 = ninf, m3 = ninf;
-        for (int r = 0; r < k; ++r) {
-            const int h = p * stride + r - pad;
-            if (h < 0 || h >= H) continue;
-            for (int s = 0; s < k; ++s) {
-                const int w = q * stride + s - pad;
-                if (w < 0 || w >= W) continue;
-                const uint4 v = __ldg(x + ((n * H + h) * W + w) * C8 + c8);
-                m0 = __hmax2(m0, *reinterpret_cast<const __half2*>(&v.x));
-                m1 = __hmax2(m1, *reinterpret_cast<const __half2*>(&v.y));
-                m2 = __hmax2(m2, *reinterpret_cast<const __half2*>(&v.z));
-                m3 = __hmax2(m3, *reinterpret_cast<const __half2*>(&v.w));
+    const uint4 ninf = make_uint4(0xFC00FC00u, 0xFC00FC00u, 0xFC00FC00u, 0xFC00FC00u);
+    const unsigned i = blockIdx.x * 256u + threadIdx.x, per = (unsigned)P * Q * C8;
+    if (i >= per) return;
+    const unsigned c8 = i % C8, t = i / C8, q = t % Q, p = t / Q;
+    for (int n = blockIdx.y; n < N; n += gridDim.y) {
+        const uint4* xi = x + (long long)n * H * W * C8 + c8;
+        uint4 m = ninf;
+        if constexpr (K > 0) {
+            const int h0 = (int)p * ST - pad, w0 = (int)q * ST - pad;
+            uint4 in[K * K];
+#pragma unroll
+            for (int j = 0; j < K * K; ++j) {
+                const int h = h0 + j / K, w = w0 + j % K;
+                in[j] = (unsigned)h < (unsigned)H && (unsigned)w < (unsigned)W ? __ldg(xi + (long long)(h * W + w) * C8) : ninf;
+            }
+#pragma unroll
+            for (int j = 0; j < K * K; ++j) m = max_f16x8(m, in[j]);
+        } else {
+            for (int r = 0; r < k; ++r) {
+                const int h = (int)p * stride + r - pad;
+                if (h < 0 || h >= H) continue;
+                for (int c = 0; c < k; ++c) {
+                    const int w = (int)q * stride + c - pad;
+                    if (w >= 0 && w < W) m = max_f16x8(m, __ldg(xi + ((long long)h * W + w) * C8));
+                }
             }
         }
-        uint4 o;
-        o.x = *reinterpret_cast<uint32_t*>(&m0);
-        o.y = *reinterpret_cast<uint32_t*>(&m1);
-        o.z = *reinterpret_cast<uint32_t*>(&m2);
-        o.w = *reinterpret_cast<uint32_t*>(&m3);
-        y[i] = o;
+        y[(long long)n * per + i] = m;
     }
 }
 
@@ -237,9 +253,14 @@ extern "C" fxpq_status fxpq_maxpool(const void* d_x, int32_t N, int32_t H, int32
     if (!d_x || !d_y) return FXPQ_ERR_INVALID_ARG;
     const long long total = (long long)N * P * Q * Cp;
     if (planes_of(fmt) == 1 && aligned(d_x, 16) && aligned(d_y, 16)) {
-        launch_pdl(maxpool_vec8_kernel, grid_for(total / 8), 256, 0, as_stream(stream),
-            static_cast<const uint4*>(d_x), N, H, W, Cp / 8, k, stride, pad, P, Q, static_cast<uint4*>(d_y));
-        return after_launch("maxpool_vec8");
+        const bool two = (k == 2 || k == 3) && stride == 2;
+        const long long per = (long long)P * Q * (Cp / 8);
+        if (per < (1LL << 31) && (long long)H * W < (1LL << 31)) {
+            auto kernel = two ? (k == 3 ? maxpool_vec8_kernel<3, 2> : maxpool_vec8_kernel<2, 2>) : maxpool_vec8_kernel<0, 0>;
+            launch_pdl(kernel, dim3((unsigned)((per + 255) / 256), (unsigned)(N < 65535 ? N : 65535)), 256, 0, as_stream(stream),
+                       static_cast<const uint4*>(d_x), N, H, W, Cp / 8, k, stride, pad, P, Q, static_cast<uint4*>(d_y));
+            return after_launch("maxpool_vec8");
+        }
     }
     maxpool_kernel<<<grid_for(total), 256, 0, as_stream(stream)>>>(static_cast<const __half*>(d_x), N, H, W, Cp,
                                                                    planes_of(fmt), k, stride, pad, P, Q,

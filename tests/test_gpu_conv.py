@@ -319,6 +319,21 @@ def test_gemm_entry_point(F):
     assert np.array_equal(F.codes_to_int(y.cpu(), fy, (M, N)).numpy(), want.reshape(M, N))
 
 
+@pytest.mark.parametrize("N,H,C,k,st,pad", [(1, 3, 8, 3, 2, 0), (3, 8, 8, 3, 2, 2), (2, 2, 264, 2, 2, 1), (70000, 2, 8, 2, 2, 0),
+                                            (2, 33, 72, 3, 2, 1), (2, 9, 16, 2, 1, 1), (1, 20, 40, 5, 3, 2)])
+def test_maxpool_windows_parity(F, N, H, C, k, st, pad):
+    """Windows with their own instances and others, over the edges, of a single output, and more images than a grid row."""
+    if os.environ.get("FXPQ_CONV_PATH") != "tc":
+        pytest.skip("once")
+    rng = np.random.default_rng(N + H + C)
+    x = rand_codes(rng, (N, H, H, C), 7, 1)
+    f = F.fmt(7, 1, 3)
+    P = (H + 2 * pad - k) // st + 1
+    y = torch.empty(N * P * P * C, dtype=torch.float16, device="cuda")
+    F.fxpq_maxpool(to_f16_planes(x, 7, C), N, H, H, C, f, k, st, pad, y)
+    assert np.array_equal(F.codes_to_int(y.cpu(), f, (N, P, P, C)).numpy(), oracle.maxpool(x, k, st, pad))
+
+
 @pytest.mark.parametrize("k,st,pad,bits", [(3, 2, 0, 8), (2, 2, 0, 6), (3, 2, 1, 8), (3, 2, 1, 12), (3, 1, 1, 4)])
 def test_maxpool_parity(F, k, st, pad, bits):
     rng = np.random.default_rng(k + st + pad + bits)
