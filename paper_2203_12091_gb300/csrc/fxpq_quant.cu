@@ -781,7 +781,7 @@ extern "C" fxpq_status fxpq_quantize_images(const float* d_x_nchw, int32_t N, in
     if (!d_x_nchw || !d_y || !aligned(d_y, 16)) return FXPQ_ERR_INVALID_ARG;
     QParams p = make_qparams(f);
     long long npix = (long long)N * H * W;
-    if (C == 3 && c_pad == 8 && npix < (1LL << 31) && !p.binary) {  // RGB images (the binary quantizer does not round)
+    if (C == 3 && c_pad == 8 && npix < (1LL << 31)) {  // RGB images
         const int g = grid_for((npix + QI_PIX - 1) / QI_PIX, 256);
         uint4* o = static_cast<uint4*>(d_y);
         if (planes_of(f) == 1)

@@ -411,17 +411,6 @@ def test_quantize_rgb_images(F, k, S, fl, N, hw):
     assert np.array_equal(got[..., :3], want) and np.all(got[..., 3:] == 0)
 
 
-def test_quantize_rgb_images_binary(F):
-    """Signed 1-bit codes: the sign of each value, not its rounding."""
-    x = torch.tensor([-0.3, 0.3, -0.0, -1e-30, 0.6, -2.0] * 8, device="cuda").reshape(1, 3, 4, 4)
-    f = F.fmt(1, 1, 0)
-    out = torch.full((16 * 8,), 55.0, dtype=torch.float16, device="cuda")
-    F.fxpq_quantize_images(x, f, 8, out)
-    got = F.codes_to_int(out.cpu(), f, (4, 4, 8)).numpy()
-    want = oracle.quantize(np.ascontiguousarray(x.cpu().numpy().transpose(0, 2, 3, 1)), 1, 1, 0).reshape(4, 4, 3)
-    assert np.array_equal(got[..., :3], want) and want.min() == -1
-
-
 def test_quantize_rgb_images_nonfinite(F):
     x = torch.ones(1, 3, 4, 4, device="cuda")
     x[0, 1, 2, 3] = float("nan")
