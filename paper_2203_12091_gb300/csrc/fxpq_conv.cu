@@ -396,9 +396,12 @@ static ConvArgs s2d_args(const ConvArgs& a, const S2dPlan& p, const __half* x2, 
 }
 
 fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64, cudaStream_t st, void* ws,
-                        size_t ws_bytes) {
+                        size_t ws_bytes, const float* images) {
     const long long M = (long long)a.N * a.P * a.Q;
     if (M == 0) return FXPQ_OK;
+    auto codes = [&] {  // a.x, where they are not there yet
+        return images ? fxpq_quantize_images(images, a.N, d.C, a.H, a.W, d.fmt_x, a.Cp, const_cast<__half*>(a.x), st) : FXPQ_OK;
+    };
     // FXPQ_CONV_PATH=tc_rows / tc_nos2d keep strided 8-channel layers on their own codes, simt keeps every layer off
     // the tensor cores
     const char* const path = getenv("FXPQ_CONV_PATH");
@@ -415,11 +418,15 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
         const bool rounds = (M + 127) / 128 * ((a.K + 63) / 64) > num_sms() || path;
         if (p.ok && rounds && ws && ws_bytes >= p.x_bytes + p.w_bytes && s2d) {
             char* base = static_cast<char*>(ws);
-            const long long npix = (long long)a.N * p.H2 * p.W2 * a.px, nw = (long long)a.K * p.R2 * p.S2 * (p.C2 / 8) * a.pw;
+            const bool direct = images && launch_quantize_s2d(images, a.N, a.H, a.W, d.fmt_x, p, a.pad, base, st);
+            fxpq_status s = direct ? after_launch("quantize_s2d") : codes();
+            if (s != FXPQ_OK) return s;
+            if (!direct) images = nullptr;
+            const long long npix = direct ? 0 : (long long)a.N * p.H2 * p.W2 * a.px, nw = (long long)a.K * p.R2 * p.S2 * (p.C2 / 8) * a.pw;
             const unsigned xb = (unsigned)((npix + 255) / 256), wb = (unsigned)((nw + 255) / 256);
             launch_pdl(s2d_kernel, xb + wb, 256, 0, st, a.x, a.w, a.N, a.H, a.W, a.K, a.R, a.S, a.pad, a.x_ps, a.w_ps, p, a.px, a.pw,
                                                 xb, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + p.x_bytes));
-            fxpq_status s = after_launch("s2d");
+            s = after_launch("s2d");
             if (s != FXPQ_OK) return s;
             const ConvArgs b = s2d_args(a, p, reinterpret_cast<const __half*>(base),
                                         reinterpret_cast<const __half*>(base + p.x_bytes));
@@ -427,15 +434,30 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
             s = launch_conv_tc(b, d, st, launched, ws_bytes > used ? base + used : nullptr, ws_bytes - used);
             if (s != FXPQ_OK || launched) return s;
         }
-        fxpq_status s = launch_conv_tc(a, d, st, launched, ws, ws_bytes);
+        fxpq_status s = codes();
+        if (s != FXPQ_OK) return s;
+        images = nullptr;
+        s = launch_conv_tc(a, d, st, launched, ws, ws_bytes);
         if (s != FXPQ_OK || launched) return s;
     }
+    const fxpq_status s = codes();
+    if (s != FXPQ_OK) return s;
     dim3 grid((unsigned)((M + TM - 1) / TM), (unsigned)((a.K + TN - 1) / TN));
     if (need64)
         conv_simt_kernel<long long><<<grid, NT, 0, st>>>(a);
     else
         conv_simt_kernel<int><<<grid, NT, 0, st>>>(a);
     return after_launch("conv_simt");
+}
+
+fxpq_status conv_fwd(const fxpq_conv_desc& d, const float* images, const void* d_x, const void* d_w, const int32_t* d_bias, void* d_y,
+                     int32_t* h_out_scale, void* d_ws, size_t ws_bytes, void* stream) {
+    if (d_ws && !aligned(d_ws, 256)) return FXPQ_ERR_WORKSPACE;
+    ConvArgs a;
+    bool need64 = false;
+    fxpq_status st = plan_conv(d, d_x, d_w, d_bias, d_y, a, h_out_scale, need64);
+    if (st != FXPQ_OK) return st;
+    return launch_conv(a, d, need64, as_stream(stream), d_ws, d_ws ? ws_bytes : 0, images);
 }
 
 }  // namespace fxpq
@@ -450,12 +472,7 @@ extern "C" fxpq_status fxpq_conv_fwd(const fxpq_conv_desc* h_desc, const void* d
                                      const int32_t* d_bias, void* d_y, int32_t* h_out_scale, void* d_ws,
                                      size_t ws_bytes, void* stream) {
     if (!h_desc) return FXPQ_ERR_INVALID_ARG;
-    if (d_ws && !aligned(d_ws, 256)) return FXPQ_ERR_WORKSPACE;
-    ConvArgs a;
-    bool need64 = false;
-    fxpq_status st = plan_conv(*h_desc, d_x, d_w, d_bias, d_y, a, h_out_scale, need64);
-    if (st != FXPQ_OK) return st;
-    return launch_conv(a, *h_desc, need64, as_stream(stream), d_ws, d_ws ? ws_bytes : 0);
+    return conv_fwd(*h_desc, nullptr, d_x, d_w, d_bias, d_y, h_out_scale, d_ws, ws_bytes, stream);
 }
 
 extern "C" fxpq_status fxpq_gemm(const void* d_x, fxpq_fmt fmt_x, const void* d_w, fxpq_fmt fmt_w,

@@ -157,8 +157,12 @@ int num_sms();  // of the current device
 
 fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, const int32_t* bias, void* y,
                       ConvArgs& a, int32_t* out_scale, bool& need64);
+// images (may be null): the fp32 [N, C, H, W] input instead of its codes; a.x then receives the codes unless the layer
+// reads them in the space-to-depth form alone.
 fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64, cudaStream_t st, void* ws,
-                        size_t ws_bytes);
+                        size_t ws_bytes, const float* images = nullptr);
+fxpq_status conv_fwd(const fxpq_conv_desc& d, const float* images, const void* d_x, const void* d_w, const int32_t* d_bias, void* d_y,
+                     int32_t* h_out_scale, void* d_ws, size_t ws_bytes, void* stream);
 // Tensor-core path; sets launched = false when the shape needs the CUDA-core kernel instead.  ws (may be
 // null): scratch for the split reduction of layers with too few tiles for the SMs.
 fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStream_t st, bool& launched, void* ws,
@@ -180,6 +184,8 @@ struct S2dPlan {
     size_t x_bytes, w_bytes;  // 256-byte multiples
 };
 S2dPlan s2d_plan(const fxpq_conv_desc& d);
+bool launch_quantize_s2d(const float* x, int N, int H, int W, const fxpq_fmt& f, const S2dPlan& s, int pad, void* out,
+                         cudaStream_t st);
 // Scratch bytes a conv may use: the space-to-depth copies, then the split reduction's shares.
 size_t conv_ws_bytes(const fxpq_conv_desc& d);
 

@@ -171,8 +171,16 @@ extern "C" fxpq_status fxpq_net_forward(const fxpq_net* h_net, const float* d_im
     const size_t cws = net_conv_ws(h_net, slots, batch);
     void* conv_ws = (cws && ws_bytes >= total + cws) ? static_cast<void*>(base + total) : nullptr;
 
-    st = fxpq_quantize_images(d_images_nchw, batch, h_net->C, h_net->H, h_net->W, h_net->fmt_in, h_net->Cp_in, ptr(0),
-                              stream);
+    // Images that only the first layer reads, a convolution, are quantized as it wants them
+    int readers = 0;
+    for (int i = 0; i < h_net->n_ops; ++i) {
+        const fxpq_op_desc& o = h_net->ops[i];
+        readers += (o.src0 == 0) + (o.op == FXPQ_OP_ELTWISE && o.src1 == 0);
+    }
+    const bool by_conv = readers == 1 && h_net->ops[0].op == FXPQ_OP_CONV && h_net->ops[0].src0 == 0;
+    if (!by_conv)
+        st = fxpq_quantize_images(d_images_nchw, batch, h_net->C, h_net->H, h_net->W, h_net->fmt_in, h_net->Cp_in, ptr(0),
+                                  stream);
     if (st != FXPQ_OK) return st;
     for (int i = 0; i < h_net->n_ops; ++i) {
         const fxpq_op_desc& o = h_net->ops[i];
@@ -204,8 +212,8 @@ extern "C" fxpq_status fxpq_net_forward(const fxpq_net* h_net, const float* d_im
                 d.d_shift = o.d_shift;
                 d.d_wpacked = o.d_wpacked;
                 int32_t scale = 0;
-                st = fxpq_conv_fwd(&d, ptr(o.src0), o.d_w, o.d_bias, last ? (void*)d_logits : ptr(o.dst), &scale,
-                                   conv_ws, conv_ws ? cws : 0, stream);
+                st = fxpq::conv_fwd(d, by_conv && i == 0 ? d_images_nchw : nullptr, ptr(o.src0), o.d_w, o.d_bias,
+                                    last ? (void*)d_logits : ptr(o.dst), &scale, conv_ws, conv_ws ? cws : 0, stream);
                 if (last && h_logits_scale) *h_logits_scale = scale;
                 break;
             }

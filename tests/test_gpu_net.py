@@ -72,6 +72,34 @@ def test_tiny_residual_net(NET):
         assert np.array_equal(got[..., : oenv[l["name"]][0].shape[-1]], oenv[l["name"]][0]), l["name"]
 
 
+@pytest.mark.parametrize("R,st,pad,hw,k", [(7, 2, 3, 28, 8), (7, 2, 3, 29, 16), (3, 3, 0, 31, 6), (5, 3, 2, 28, 12), (11, 4, 2, 32, 8),
+                                           (11, 4, 2, 33, 16), (3, 2, 1, 20, 2)])
+def test_first_layer_from_images(NET, R, st, pad, hw, k, monkeypatch):
+    """A strided first layer reads images quantized straight into its space-to-depth form, or (maps that the form does
+    not cover, other paths) their codes: the same logits, and a value that is not finite is reported."""
+    from paper_2203_12091_gb300 import fxpq as F
+    L = [{"type": "conv", "name": "c1", "C": 3, "K": 16, "R": R, "stride": st, "pad": pad, "relu": True, "src": None},
+         {"type": "avgpool", "name": "gap", "src": "c1"},
+         {"type": "conv", "name": "fc", "C": 16, "K": 24, "R": 1, "stride": 1, "pad": 0, "relu": False, "src": "gap"}]
+    plan = {"input": k, "c1": {"w": 8, "b": 16, "a": 8}, "gap": {"a": 8, "r": 16}, "fc": {"w": 8, "b": 16}}
+    rng = np.random.default_rng(R + hw)
+    W = {"c1": (rng.standard_normal((16, R, R, 3)).astype(np.float32) * 0.1, rng.standard_normal(16).astype(np.float32) * 0.01),
+         "fc": (rng.standard_normal((24, 1, 1, 16)).astype(np.float32) * 0.3, rng.standard_normal(24).astype(np.float32) * 0.01)}
+    imgs = synth.images(5, 2, hw=hw)
+    q = NET.build_qnet(L, W, torch.from_numpy(imgs[:4]).cuda(), plan)
+    fm, qp = onet.calibrate(L, W, imgs[:4], plan)
+    want, ws = onet.forward(L, fm, qp, imgs)
+    bad = imgs.copy()
+    bad[4, 2, hw - 1, hw - 1] = np.nan
+    for path in ("tc", "tc_nos2d", "simt"):
+        monkeypatch.setenv("FXPQ_CONV_PATH", path)
+        logits, s = q.forward(torch.from_numpy(imgs).cuda())
+        assert s == ws and np.array_equal(logits.cpu().numpy(), want), path
+        F.fxpq_get_device_status()
+        q.forward(torch.from_numpy(bad).cuda())
+        assert F.fxpq_get_device_status() == 3
+
+
 def _workload(NET, arch, batch, seed, plan_seed=None, calib=8, sample=(0, -1), pack=False):
     L = synth.ARCHS[arch]()
     W = synth.weights(arch, seed)
