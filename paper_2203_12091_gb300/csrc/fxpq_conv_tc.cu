@@ -234,6 +234,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         }
         P.patch = 0;
         P.rows_tma = 0;
+        P.rows = TC_BM;
         P.w32 = 0;
         P.wf32 = 0;
         P.win_eps = P.win_c[0] = P.win_c[1] = P.win_c[2] = 0.0f;
@@ -365,11 +366,15 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         if (P.patch == 0 && rows_geom) {
             const cuuint64_t xdims[3] = {(cuuint64_t)P.RSC, (cuuint64_t)a.M, (cuuint64_t)a.px};
             const cuuint64_t xstrides[2] = {(cuuint64_t)P.RSC * 2, (cuuint64_t)a.x_ps * 2};
-            const cuuint32_t xbox[3] = {(cuuint32_t)TC_BK, (cuuint32_t)TC_BM, 1};
+            const long long parts = (a.M + TC_BM - 1) / TC_BM;
+            const int rows = (int)(((a.M + parts - 1) / parts + 7) / 8 * 8);
+            const cuuint32_t xbox[3] = {(cuuint32_t)TC_BK, (cuuint32_t)rows, 1};
             if (enc(&P.tmap_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half*>(a.x), xdims, xstrides, xbox, es,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS) {
                 P.rows_tma = 1;
+                P.rows = rows;
+            }
         }
         if (P.patch == 0 && !P.rows_tma && use_patch) {
             const cuuint64_t xdims[5] = {(cuuint64_t)a.Cp, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.N, (cuuint64_t)a.px};
@@ -409,7 +414,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
             } else {
                 const cuuint64_t ydims[2] = {(cuuint64_t)a.K, (cuuint64_t)a.M};
                 const cuuint64_t ystrides[1] = {(cuuint64_t)a.K * 2};
-                const cuuint32_t ybox[2] = {64, (cuuint32_t)TC_BM};
+                const cuuint32_t ybox[2] = {64, (cuuint32_t)P.rows};
                 r = enc(&P.tmap_y, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, a.y, ydims, ystrides, ybox, es,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

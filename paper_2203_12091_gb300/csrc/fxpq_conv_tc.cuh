@@ -125,8 +125,11 @@ struct TcParams {
                          //    every tap and 16-channel step one shifted swizzled MMA
     int rows_tma;        // 128-row tiles whose A tile is one 2-D TMA box of the activations seen as
                          // [planes][M][R*S*Cp] (1x1 stride-1 layers without padding, and kernels that
-                         // cover the whole unpadded map: FC layers), box {64, 128, 1}, 128-byte
-                         // swizzle, rows past M and taps past R*S*Cp zero filled
+                         // cover the whole unpadded map: FC layers), box {64, rows, 1}, 128-byte
+                         // swizzle, taps past R*S*Cp zero filled
+    int rows;            // output rows of a row tile: 128, or with TMA rows M's equal parts (a box is slow where it lies
+                         // outside the tensor; the tile's other rows hold whatever the stage does and are not stored):
+                         // 136 x 4096 outputs of 4096 products 47.8 us with 128-row tiles, 33.4 with two of 72
     int nacc;            // fp32 accumulators per TMEM buffer (window mode: one per limb pair)
     int WW, WH, S2;      // window mode: window width / height in pixels, taps per row rounded up to even
     int w32;             // window mode, two-limb x and w, one-plane codes out: the 32-bit epilogue (the
@@ -282,8 +285,8 @@ __device__ __forceinline__ int row_in_tile(const TcParams& P, int row) {
 // Linear output row of that place in the tile at T (`row` itself in 128-row tiles), or -1 outside the map.
 __device__ __forceinline__ long long row_at(const TcParams& P, const TileIter& T, int place, int row) {
     if (!P.patch) {
-        const long long m = (long long)T.ng * TC_BM + row;
-        return m < P.a.M ? m : -1;
+        const long long m = (long long)T.ng * P.rows + row;
+        return row < P.rows && m < P.a.M ? m : -1;
     }
     const int n = T.ng * P.TN + (place >> 16), p = T.ip * P.TH + ((place >> 8) & 255), q = T.iq * P.TW + (place & 255);
     if (place < 0 || n >= P.a.N || p >= P.a.P || q >= P.a.Q) return -1;
@@ -1053,7 +1056,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
         if (warp < TC_PRODUCERS) {
             const uint32_t me = warp;
             const bool narrow = P.patch == 2;
-            const uint32_t a_bytes = P.rows_tma ? (uint32_t)(TC_BM * 128) : (uint32_t)(P.TH * P.TW * P.TN * (narrow ? 8 * 16 : 128));
+            const uint32_t a_bytes = P.rows_tma ? (uint32_t)P.rows * 128u : (uint32_t)(P.TH * P.TW * P.TN * (narrow ? 8 * 16 : 128));
             uint32_t it = 0, stage = 0, phase = 0;
             bool ok = true;
             TileIter T(P, SPLIT ? 0 : blockIdx.x);
@@ -1092,7 +1095,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                                                 wq0 + s8, hp0 + r8, n_img, g.a_plane, fb);
                                 }
                             } else if (P.rows_tma) {
-                                tma_load_3d(smem_u32(sA + stage * A_BYTES), &P.tmap_x, kb * TC_BK, tm * TC_BM, g.a_plane,
+                                tma_load_3d(smem_u32(sA + stage * A_BYTES), &P.tmap_x, kb * TC_BK, tm * P.rows, g.a_plane,
                                             fb);
                             } else {
                                 tma_load_5d(smem_u32(sA + stage * A_BYTES), &P.tmap_x, cc, wq0 + ss, hp0 + rr, n_img,
@@ -1781,10 +1784,23 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     if (SPLIT && P.ksplit > 1) {
                         // one share of the reduction: its exact integer sums go to the partial buffer
                         if (m >= 0) {
+                            // (16 bytes per store: with one value per store 64 x 4096 outputs of 4096 products took 29 us, 19 so)
                             ACC* dst = static_cast<ACC*>(P.part) + ((long long)sp * a.M + m) * a.K + k0;
+                            constexpr int V = 16 / (int)sizeof(ACC);
+                            if (a.K % V == 0) {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                if (k0 + j < a.K) dst[j] = acc[j];
+                                for (int j = 0; j < 32; j += V)
+                                    if (k0 + j < a.K) {
+                                        if constexpr (V == 4)
+                                            *reinterpret_cast<int4*>(dst + j) = make_int4((int)acc[j], (int)acc[j + 1], (int)acc[j + 2], (int)acc[j + 3]);
+                                        else
+                                            *reinterpret_cast<longlong2*>(dst + j) = make_longlong2((long long)acc[j], (long long)acc[j + 1]);
+                                    }
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < 32; ++j)
+                                    if (k0 + j < a.K) dst[j] = acc[j];
+                            }
                         }
                         continue;
                     }
@@ -1899,7 +1915,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                     if (P.patch)
                         tma_store_4d(&P.tmap_y, T.tn * BN + hb * 64, T.iq * P.TW, T.ip * P.TH, T.ng * P.TN, src);
                     else
-                        tma_store_2d(&P.tmap_y, T.tn * BN + hb * 64, T.ng * TC_BM, src);
+                        tma_store_2d(&P.tmap_y, T.tn * BN + hb * 64, T.ng * P.rows, src);
                 }
                 bulk_commit();
                 if (NSTG == 1) {

@@ -675,6 +675,20 @@ def test_last_column_tile_parity(F, K, mode, N, H, C, R, kx):
     assert s == ws and np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("M", [1, 7, 64, 127, 129, 136, 200, 257])
+@pytest.mark.parametrize("C,K,mode,kx", [(64, 72, 0, 8), (3000, 264, 0, 8), (3000, 258, 2, 8), (3000, 259, 1, 8), (200, 66, 1, 16), (1600, 63, 1, 16)])
+def test_row_parts_parity(F, M, C, K, mode, kx):
+    """Row tiles that are equal parts of M, alone and split over the reduction: 16-byte shares (K a multiple of 4, or of 2
+    for 64-bit sums) and single values."""
+    rng = np.random.default_rng(M + C + K)
+    fx, fw, fb = F.fmt(kx, 0, kx - 3), F.fmt(8, 1, 7), F.fmt(16, 1, 14)
+    fy = F.fmt(8, 0, 2) if mode == 0 else None
+    x, w, b = rand_codes(rng, (M, 1, 1, C), kx, 0), rand_codes(rng, (K, 1, 1, C), 8, 1), rand_codes(rng, (K,), 16, 1)
+    got, s = run_conv(F, x, fx, w, fw, b, fb, 1, 0, True, mode, fy, (C + 7) // 8 * 8)
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, 1, 0, True, mode, fy)
+    assert s == ws and np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("N,H,C,K,R,st,kx", [(2, 30, 16, 64, 3, 1, 7), (26, 30, 16, 64, 3, 1, 7), (2, 30, 24, 64, 5, 1, 7),
                                              (26, 30, 24, 64, 3, 1, 7), (26, 30, 120, 64, 3, 1, 7), (2, 30, 32, 64, 3, 1, 16),
                                              (2, 30, 80, 64, 3, 1, 16), (2, 30, 3, 64, 5, 1, 16), (26, 30, 3, 72, 3, 1, 16),
