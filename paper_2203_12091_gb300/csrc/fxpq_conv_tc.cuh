@@ -11,17 +11,21 @@
 // sums.  The same grouping carries the two-limb split of 9..16-bit codes
 // (v = 256 * v_hi + v_lo): one pass per (A limb, W limb) pair.
 //
-// CTA (one per SM, persistent over tiles): 9 warps.
+// CTA (one per SM, persistent over tiles):
 //   warps 0-3  producers, into 128-byte swizzled K-major shared-memory stages.  The B tile
-//              (BN channels x 64 taps) always comes by TMA.  The A tile takes one of two forms:
+//              (BN channels x 64 taps) always comes by TMA.  The A tile takes one of these forms:
 //              row tiles (128 consecutive output pixels): cp.async gather by 128 threads, with
-//              zero fill for padding and ragged edges;
+//              zero fill for padding and ragged edges, or one box where the layer's im2col rows are
+//              the stored activations;
 //              patch tiles: a TH x TW patch of output pixels of TN images, whose inputs for one tap
 //              and 64 channels are a single 5-D TMA box, strided like the convolution (the
-//              hardware zero-fills the padding); one warp issues both copies.
-//   warp  4-7  epilogue: drain TMEM (tcgen05.ld), integer running sums, final bias / ReLU /
-//              FxP-QLayer (shared with the CUDA-core kernel).
-//   warp  8    TMEM allocation and the single MMA-issuing thread.
+//              hardware zero-fills the padding); the warps that issue copies own the stages in turn;
+//              windows: see the patch values 3 and 4 of TcParams.
+//   next 8 to 16 (BN / 8; 16 in the window instances)
+//              epilogue: drain TMEM (tcgen05.ld), integer running sums, final bias / ReLU /
+//              FxP-QLayer (shared with the CUDA-core kernel), or fp32 codes where the sums allow it.
+//   then one   TMEM allocation and MMA issue (the whole warp, one elected lane per instruction),
+//   one more   the TMA stores of staged tiles (BN <= 128), or five converters of packed weights.
 // Every wait is bounded: on expiry the kernel latches FXPQ_ERR_TIMEOUT, stops issuing work,
 // drains its own copies and MMAs, frees TMEM and returns.
 // The kernel is a template over the tile width, the integer type of the running sums and whether
@@ -293,12 +297,8 @@ __device__ __forceinline__ long long row_at(const TcParams& P, const TileIter& T
     return ((long long)n * P.a.P + p) * P.a.Q + q;
 }
 
-// Output row (linear index into N*P*Q, or -1 when outside the map) of tile row i.
+// Output row (linear index into N*P*Q, or -1 when outside the map) of row i of the window instances' patch tm.
 __device__ __forceinline__ long long tile_row(const TcParams& P, int tm, int i) {
-    if (!P.patch) {
-        const long long m = (long long)tm * 128 + i;
-        return m < P.a.M ? m : -1;
-    }
     const int per_img = P.tiles_p * P.tiles_q, pix = P.TH * P.TW;
     const int ti = i / pix, j = i - ti * pix;
     if (ti >= P.TN) return -1;
