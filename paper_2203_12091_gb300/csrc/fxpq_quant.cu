@@ -68,6 +68,7 @@ __device__ __forceinline__ S code_bits(int c) {
 // element by element by the first threads of the grid.
 template <typename S, bool F16>
 __global__ void quantize_vec16_kernel(const float* __restrict__ x, long long n, QParams p, S* __restrict__ out) {
+    pdl_wait();
     bool bad = false;
     const long long n16 = n / 16;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -99,6 +100,7 @@ __global__ void quantize_vec16_kernel(const float* __restrict__ x, long long n, 
 // rows x C fp32 -> fp16 code tensor: planes of [rows, Cp] (hi plane, then lo plane when k > 8)
 __global__ void quantize_rows_f16_kernel(const float* __restrict__ x, long long rows, int C, int Cp, int planes,
                                          QParams p, __half* __restrict__ out) {
+    pdl_wait();
     bool bad = false;
     long long total = rows * (long long)Cp;
     long long stride = (long long)gridDim.x * blockDim.x;
@@ -115,6 +117,7 @@ __global__ void quantize_rows_f16_kernel(const float* __restrict__ x, long long 
 // thread from two 16-byte loads, one 16-byte store per plane.
 __global__ void quantize_rows_vec8_kernel(const float4* __restrict__ x, long long n8, int planes, QParams p,
                                           uint4* __restrict__ out) {
+    pdl_wait();
     bool bad = false;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n8; i += stride) {
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(256) quantize_s2d3_kernel(const float* __restr
 // max over rows of sum |code|: one block per row (grid-stride over rows), 8 codes per 16-byte load
 __global__ void code_l1max_kernel(const uint4* __restrict__ codes, long long rows, long long L8,
                                   unsigned long long* __restrict__ out) {
+    pdl_wait();
     __shared__ long long red[32];
     for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
         const uint4* row = codes + r * L8;
@@ -356,6 +360,7 @@ struct QbBatch {
 // One block per work unit: an output-channel group (rpg rows) of a row item, or QB_FLAT_UNIT elements of
 // a flat item.  The format (k from the item, S and FL from the device) is read once per block.
 __global__ void __launch_bounds__(256) quantize_batch_kernel(const __grid_constant__ QbBatch B) {
+    pdl_wait();
     int item = 0;
     while (item + 1 < B.n && (int)blockIdx.x >= B.unit0[item + 1]) ++item;
     const QbItem& I = B.it[item];
@@ -566,6 +571,7 @@ __device__ __forceinline__ uint4 fields_to_f16(uint32_t lo, uint32_t hi, uint32_
 // with one code per thread, 66 us.  x 16-byte aligned, out at any code.
 __global__ void __launch_bounds__(256) quantize_planes2_kernel(const float* __restrict__ x, long long n, QParams p,
                                                                __half* __restrict__ out) {
+    pdl_wait();
     bool bad = false;
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -601,6 +607,7 @@ constexpr int PACK_U = 2;  // 256-code pieces per warp and iteration (their load
 template <int PLANES>
 __global__ void __launch_bounds__(256) pack_codes_kernel(const __half* __restrict__ codes, long long n, int k,
                                                          uint32_t* __restrict__ words) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -643,6 +650,7 @@ __global__ void __launch_bounds__(256) pack_codes_kernel(const __half* __restric
 template <int PLANES>
 __global__ void __launch_bounds__(256) unpack_codes_kernel(const uint32_t* __restrict__ words, long long n, int k,
                                                            int is_signed, __half* __restrict__ codes) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -774,22 +782,22 @@ extern "C" fxpq_status fxpq_quantize(const float* d_x, int64_t n, fxpq_fmt f, in
     const bool al16 = aligned(d_x, 16) && aligned(d_codes, 16);
     if (dtype == FXPQ_DT_F16) {
         if (planes_of(f) == 1 && al16) {
-            quantize_vec16_kernel<uint16_t, true><<<grid_for((n + 15) / 16, T), T, 0, s>>>(
+            launch_pdl(quantize_vec16_kernel<uint16_t, true>, grid_for((n + 15) / 16, T), T, 0, s,
                 d_x, n, p, static_cast<uint16_t*>(d_codes));
             return after_launch("quantize_f16");
         }
         // (planes on 16-byte boundaries: 2^25 16-bit codes 49 us here, 54 us through the kernel below)
         if (al16 && n % 8 == 0) {
-            quantize_rows_vec8_kernel<<<grid_for(n / 8, T), T, 0, s>>>(reinterpret_cast<const float4*>(d_x), n / 8,
+            launch_pdl(quantize_rows_vec8_kernel, grid_for(n / 8, T), T, 0, s, reinterpret_cast<const float4*>(d_x), n / 8,
                                                                       planes_of(f), p, static_cast<uint4*>(d_codes));
             return after_launch("quantize_rows_vec8");
         }
         if (planes_of(f) == 2 && aligned(d_x, 16) && aligned(d_codes, 2)) {
-            quantize_planes2_kernel<<<grid_for((n + 7) / 8, T), T, 0, s>>>(d_x, n, p, static_cast<__half*>(d_codes));
+            launch_pdl(quantize_planes2_kernel, grid_for((n + 7) / 8, T), T, 0, s, d_x, n, p, static_cast<__half*>(d_codes));
             return after_launch("quantize_planes2");
         }
         // unaligned: one code per row of one channel
-        quantize_rows_f16_kernel<<<grid_for(n, T), T, 0, s>>>(d_x, n, 1, 1, planes_of(f), p,
+        launch_pdl(quantize_rows_f16_kernel, grid_for(n, T), T, 0, s, d_x, n, 1, 1, planes_of(f), p,
                                                               static_cast<__half*>(d_codes));
         return after_launch("quantize_rows_f16");
     }
@@ -798,14 +806,14 @@ extern "C" fxpq_status fxpq_quantize(const float* d_x, int64_t n, fxpq_fmt f, in
         switch (dtype) {
             case FXPQ_DT_I8:
             case FXPQ_DT_U8:
-                quantize_vec16_kernel<uint8_t, false><<<g, T, 0, s>>>(d_x, n, p, static_cast<uint8_t*>(d_codes));
+                launch_pdl(quantize_vec16_kernel<uint8_t, false>, g, T, 0, s, d_x, n, p, static_cast<uint8_t*>(d_codes));
                 break;
             case FXPQ_DT_I16:
             case FXPQ_DT_U16:
-                quantize_vec16_kernel<uint16_t, false><<<g, T, 0, s>>>(d_x, n, p, static_cast<uint16_t*>(d_codes));
+                launch_pdl(quantize_vec16_kernel<uint16_t, false>, g, T, 0, s, d_x, n, p, static_cast<uint16_t*>(d_codes));
                 break;
             default:
-                quantize_vec16_kernel<uint32_t, false><<<g, T, 0, s>>>(d_x, n, p, static_cast<uint32_t*>(d_codes));
+                launch_pdl(quantize_vec16_kernel<uint32_t, false>, g, T, 0, s, d_x, n, p, static_cast<uint32_t*>(d_codes));
                 break;
         }
         return after_launch("quantize_vec16");
@@ -836,11 +844,11 @@ extern "C" fxpq_status fxpq_quantize_rows(const float* d_x, int64_t rows, int32_
     QParams p = make_qparams(f);
     if (C == Cp && aligned(d_x, 16) && aligned(d_y, 16)) {
         const long long n8 = rows * (long long)C / 8;
-        quantize_rows_vec8_kernel<<<grid_for(n8, 256), 256, 0, as_stream(stream)>>>(
+        launch_pdl(quantize_rows_vec8_kernel, grid_for(n8, 256), 256, 0, as_stream(stream),
             reinterpret_cast<const float4*>(d_x), n8, planes_of(f), p, static_cast<uint4*>(d_y));
         return after_launch("quantize_rows_vec8");
     }
-    quantize_rows_f16_kernel<<<grid_for(rows * Cp, 256), 256, 0, as_stream(stream)>>>(
+    launch_pdl(quantize_rows_f16_kernel, grid_for(rows * Cp, 256), 256, 0, as_stream(stream),
         d_x, rows, C, Cp, planes_of(f), p, static_cast<__half*>(d_y));
     return after_launch("quantize_rows_f16");
 }
@@ -874,7 +882,7 @@ extern "C" fxpq_status fxpq_code_l1max(const void* d_codes, int64_t rows, int64_
     if (cudaMemsetAsync(d_out, 0, sizeof(int64_t), s) != cudaSuccess) return FXPQ_ERR_CUDA;
     if (rows == 0 || L == 0) return FXPQ_OK;
     const int grid = rows < 4096 ? (int)rows : 4096;
-    code_l1max_kernel<<<grid, 256, 0, s>>>(static_cast<const uint4*>(d_codes), rows, L / 8,
+    launch_pdl(code_l1max_kernel, grid, 256, 0, s, static_cast<const uint4*>(d_codes), rows, L / 8,
                                            reinterpret_cast<unsigned long long*>(d_out));
     return after_launch("code_l1max");
 }
@@ -924,7 +932,7 @@ extern "C" fxpq_status fxpq_quantize_batch(const fxpq_quantize_item* h_items, in
         }
         B.unit0[m] = (int)units;
         if (units == 0) continue;
-        quantize_batch_kernel<<<(unsigned)units, 256, 0, s>>>(B);
+        launch_pdl(quantize_batch_kernel, (unsigned)units, 256, 0, s, B);
         const fxpq_status st = after_launch("quantize_batch");
         if (st != FXPQ_OK) return st;
     }
@@ -938,9 +946,9 @@ extern "C" fxpq_status fxpq_pack_codes(const void* d_codes, int64_t n, fxpq_fmt 
     if (n == 0) return FXPQ_OK;
     const int T = 256, grid = grid_for((n + 256 * PACK_U - 1) / (256 * PACK_U) * 32, T);
     if (planes_of(fmt) == 1)
-        pack_codes_kernel<1><<<grid, T, 0, as_stream(stream)>>>(static_cast<const __half*>(d_codes), n, fmt.bits, d_words);
+        launch_pdl(pack_codes_kernel<1>, grid, T, 0, as_stream(stream), static_cast<const __half*>(d_codes), n, fmt.bits, d_words);
     else
-        pack_codes_kernel<2><<<grid, T, 0, as_stream(stream)>>>(static_cast<const __half*>(d_codes), n, fmt.bits, d_words);
+        launch_pdl(pack_codes_kernel<2>, grid, T, 0, as_stream(stream), static_cast<const __half*>(d_codes), n, fmt.bits, d_words);
     return after_launch("pack_codes");
 }
 
@@ -970,10 +978,10 @@ extern "C" fxpq_status fxpq_unpack_codes(const uint32_t* d_words, int64_t n, fxp
     if (n == 0) return FXPQ_OK;
     const int T = 256, grid = grid_for((n + 256 * PACK_U - 1) / (256 * PACK_U) * 32, T);
     if (planes_of(fmt) == 1)
-        unpack_codes_kernel<1><<<grid, T, 0, as_stream(stream)>>>(d_words, n, fmt.bits, fmt.is_signed,
+        launch_pdl(unpack_codes_kernel<1>, grid, T, 0, as_stream(stream), d_words, n, fmt.bits, fmt.is_signed,
                                                                   static_cast<__half*>(d_codes));
     else
-        unpack_codes_kernel<2><<<grid, T, 0, as_stream(stream)>>>(d_words, n, fmt.bits, fmt.is_signed,
+        launch_pdl(unpack_codes_kernel<2>, grid, T, 0, as_stream(stream), d_words, n, fmt.bits, fmt.is_signed,
                                                                   static_cast<__half*>(d_codes));
     return after_launch("unpack_codes");
 }
