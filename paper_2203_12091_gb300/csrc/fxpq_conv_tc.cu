@@ -13,12 +13,13 @@ namespace {
 int g_num_sms = 0;
 std::mutex g_tc_mu;
 
-// FXPQ_CONV_PATH picks among exact alternatives so that tests can compare them on the same shapes:
-// "tc_rows" keeps every layer on 128-row tiles gathered by the producer warps, "tc_patch" takes patch tiles wherever the geometry
-// allows them (by default only while they compute few extra rows), "tc_bn128" never takes
-// 256-column tiles and "tc_bn256" takes them wherever the layer allows (by default they also need
-// enough tiles to keep every SM busy), "tc_win64" keeps window mode's two-limb epilogue in 64-bit
-// arithmetic, "tc_win32" in 32-bit integers, "tc_iepi" the one-group layers' epilogue in integers.
+// FXPQ_CONV_PATH picks among exact alternatives so that tests can compare them on the same shapes: "tc" takes patch
+// tiles up to four times the gathered form's k-blocks (by default the line depends on alignment, limbs and tiles)
+// and space-to-depth at any size, "tc_patch" patch tiles wherever the geometry allows them, "tc_rows" 128-row tiles
+// gathered by the producer warps for every layer, "tc_bn128" no 256-column tiles and "tc_bn256" them wherever the layer
+// allows (by default the width whose rounds take the fewest cycles), "tc_win64" window mode's two-limb epilogue in
+// 64-bit arithmetic, "tc_win32" in 32-bit integers, "tc_nowin" no window mode, "tc_iepi" the one-group layers' epilogue
+// in integers, "tc_nos2d" no space-to-depth, "tc_nosplit" no split reduction, "tc_nopack" no packed weights.
 bool g_tc_attr_set = false;
 
 // Largest |limb| of a format's codes: the only plane (k <= 8) or the hi / lo limb (k > 8).
