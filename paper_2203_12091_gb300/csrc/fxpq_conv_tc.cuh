@@ -1912,7 +1912,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                 if (!wait_bounded(sb ? stg_full2 : stg_full, (u / NSTG) & 1, abort, P.status)) break;
                 for (int hb = 0; hb < BN / 64; ++hb) {
                     const uint32_t src = smem_u32(sO + sb * STG_BYTES + hb * (TC_BM * 128));
-                    if (P.patch)
+                    if (WEPI || P.patch)
                         tma_store_4d(&P.tmap_y, T.tn * BN + hb * 64, T.iq * P.TW, T.ip * P.TH, T.ng * P.TN, src);
                     else
                         tma_store_2d(&P.tmap_y, T.tn * BN + hb * 64, T.ng * P.rows, src);
