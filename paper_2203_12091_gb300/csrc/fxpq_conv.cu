@@ -376,7 +376,7 @@ fxpq_status plan_conv(const fxpq_conv_desc& d, const void* x, const void* w, con
 }
 
 // The layer's arguments in the space-to-depth form.
-static ConvArgs s2d_args(const ConvArgs& a, const S2dPlan& p, const __half* x2, const __half* w2) {
+ConvArgs s2d_args(const ConvArgs& a, const S2dPlan& p, const __half* x2, const __half* w2) {
     ConvArgs b = a;
     b.x = x2;
     b.w = w2;
@@ -393,6 +393,12 @@ static ConvArgs s2d_args(const ConvArgs& a, const S2dPlan& p, const __half* x2, 
     b.x_sh = (long long)p.W2 * p.C2;
     b.x_sn = (long long)p.H2 * p.W2 * p.C2;
     return b;
+}
+
+fxpq_conv_desc s2d_desc(const fxpq_conv_desc& d) {
+    fxpq_conv_desc e = d;
+    e.d_wpacked = nullptr;
+    return e;
 }
 
 fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64, cudaStream_t st, void* ws,
@@ -431,7 +437,7 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
             const ConvArgs b = s2d_args(a, p, reinterpret_cast<const __half*>(base),
                                         reinterpret_cast<const __half*>(base + p.x_bytes));
             const size_t used = p.x_bytes + p.w_bytes;
-            s = launch_conv_tc(b, d, st, launched, ws_bytes > used ? base + used : nullptr, ws_bytes - used);
+            s = launch_conv_tc(b, s2d_desc(d), st, launched, ws_bytes > used ? base + used : nullptr, ws_bytes - used);
             if (s != FXPQ_OK || launched) return s;
         }
         fxpq_status s = codes();

@@ -184,6 +184,10 @@ struct S2dPlan {
     size_t x_bytes, w_bytes;  // 256-byte multiples
 };
 S2dPlan s2d_plan(const fxpq_conv_desc& d);
+// The layer (a, d) in that form, on the rewritten codes x2 and weights w2.  Its packed weights stay behind: their records
+// are the original reduction's.
+ConvArgs s2d_args(const ConvArgs& a, const S2dPlan& p, const __half* x2, const __half* w2);
+fxpq_conv_desc s2d_desc(const fxpq_conv_desc& d);
 bool launch_quantize_s2d(const float* x, int N, int H, int W, const fxpq_fmt& f, const S2dPlan& s, int pad, void* out,
                          cudaStream_t st);
 // Scratch bytes a conv may use: the space-to-depth copies, then the split reduction's shares.

@@ -47,10 +47,6 @@ int num_sms() {
 // Patch shape of a layer's output: TW x TH pixels of TN images, at most 128, with the fewest tiles (a 7 x 7 map
 // of 128 images takes 49 tiles like its 6272 rows do, not 128).  Only widths and heights that divide the map
 // into equal counts matter; among equals the fewest images and the widest rows.
-struct PatchShape {
-    int TW = 0, TH = 0, TN = 0;
-    long long tiles = 0;
-};
 static PatchShape patch_shape(const ConvArgs& a, int max_tn) {
     PatchShape s;
     const long long ideal = (a.M + TC_BM - 1) / TC_BM;
@@ -109,6 +105,80 @@ bool plan_tc(const ConvArgs& a, const fxpq_conv_desc& d, TcParams& P, bool& acc6
     return ng > 0;
 }
 
+// FXPQ_CONV_PATH as `path` (may be null) is one of the names above.
+static bool path_is(const char* path, const char* name) { return path && strcmp(path, name) == 0; }
+
+// The host's choices for a layer: P's exact groups and f.  False: the tensor-core path cannot keep the sums exact.
+bool choose_form(const ConvArgs& a, const fxpq_conv_desc& d, const char* path, int sms, bool has_ws, TcParams& P, TcForm& f) {
+    auto conv_path_is = [path](const char* name) { return path_is(path, name); };
+    bool& acc64 = f.acc64 = false;
+    const long long row_tiles_est = (a.M + TC_BM - 1) / TC_BM;
+    // Layers whose im2col matrix is the stored activations themselves: 1x1 stride-1 convolutions
+    // without padding ([M][Cp] per plane) and kernels covering the whole unpadded map (P = Q = 1,
+    // FC layers: [N][H W Cp]).  A 128-row A tile is then one 2-D box of [M][R S Cp].
+    const bool one_by_one = a.R == 1 && a.S == 1 && a.stride == 1 && a.pad == 0 && a.x_sw == a.Cp;
+    const bool whole_map = a.R == a.H && a.S == a.W && a.pad == 0 && a.P == 1 && a.Q == 1;
+    const bool rows_geom = f.rows_geom = (one_by_one || whole_map) && a.M > 0 && a.M < (1LL << 31) - TC_BM &&
+                           !conv_path_is("tc_rows") && !conv_path_is("tc_patch");
+    // Patch tiles for every other layer whose stride a TMA box can traverse and whose channel count fills its
+    // 64-channel blocks well enough: up to four times the k-blocks of the flattened reduction of the
+    // gathered row tiles, which take about six times as long per k-block (2600 cycles against 410; a 7 x 7
+    // 512-channel layer of 128 images 95 us gathered, 31 us as patches); 8-channel stride-1 inputs take boxes
+    // of one tap each (narrow)
+    const bool narrow = f.narrow = a.Cp == 8;
+    PatchShape& ps = f.ps = PatchShape();
+    if (!rows_geom && a.P > 0 && a.Q > 0 && a.N > 0 && a.stride <= (narrow ? 1 : 8) && !conv_path_is("tc_rows"))
+        ps = patch_shape(a, TC_BM);
+    const int kbt = P.kbt = (a.Cp + TC_BK - 1) / TC_BK;
+    const int kb_flat = (a.R * a.S * a.Cp + TC_BK - 1) / TC_BK;
+    // How many of its k-blocks a layer may spend as patches for one of the flattened reduction (K = 64 / 256, 3x3,
+    // 588 row tiles, us as patches and gathered): 32 channels, 1.8 times as many, 15.8 / 22.4 and 31.5 / 35.2; 16
+    // channels, 3 times, 25.3 / 19.4 and 37.3 / 29.4.  Pixels that are not whole 32-byte sectors cost their boxes
+    // double: 120 channels, 1.06 times, 37.6 / 46.2; 136 channels, 1.35 times, 55.7 / 49.3; 24 channels 63.9 / 35.2.
+    // Where each tile has an SM to itself the latency of a k-block decides instead, and patches win longer (24
+    // channels, 21 tiles: 8.9 / 9.9).  Two-limb reductions drain a group per limb pair, which hides less of the
+    // patches' k-blocks (32 channels, 1.8 times: 68 / 62; 80 channels, 1.5 times: 99.5 / 103; 16-bit 24 channels, 5 x 5,
+    // 2.5 times: 272 / 103).
+    // Eight-channel patches take the gathered form's k-blocks, a box per tap: one-limb layers 1.1 to 1.4 times faster,
+    // two-limb ones only with few taps (128 channels, 3 x 3, 1568 tiles: 134 / 140; 64 channels, 7 x 7: 132 / 114).
+    // (The space-to-depth form has no more k-blocks as patches.)
+    const bool two_limb = a.px * a.pw > 1, lone = row_tiles_est * ((a.K + 63) / 64) <= sms;
+    const bool any_patch = conv_path_is("tc") || conv_path_is("tc_bn256") || a.x_sw != a.Cp;
+    const double most = any_patch ? 4.0 : a.Cp % 16 ? (lone && !two_limb ? 2.3 : 1.15) : two_limb ? 1.55 : lone ? 4.0 : 2.0;
+    const bool use_patch = f.use_patch =
+        ps.TW > 0 && (conv_path_is("tc_patch") || (narrow ? any_patch || !two_limb || (!lone && a.R * a.S <= 16)
+                                                          : (double)ps.tiles * a.R * a.S * kbt <= most * (double)row_tiles_est * kb_flat));
+    if (!plan_tc(a, d, P, acc64, use_patch && !narrow ? a.R * a.S * kbt : kb_flat)) return false;
+    // ... with few row tiles (FC layers at small batches) they take 256-column tiles and a split
+    // reduction fills the SMs: the MMA thread's fixed cost per k-block is then hidden, and the weights
+    // stream at the memory's rate
+    const bool wide_split = rows_geom && !acc64 && !a.has_scale && has_ws && a.K > 128 && !conv_path_is("tc_bn128") &&
+                            !conv_path_is("tc_nosplit") && row_tiles_est * ((a.K + 255) / 256) * 2 <= sms &&
+                            (kb_flat * a.px * a.pw >= 32 || d.d_wpacked);  // (shorter ones are not split, see below)
+    // Tile width: 64 columns for int64 sums and at most 64 output channels, else the width whose whole rounds
+    // over the SMs take the fewest cycles.  A k-block costs what its stage takes from L2 at about 80 bytes
+    // per cycle and SM (24, 32 and 48 KB: 300, 410 and 615 cycles; the MMAs 228, 256 and 512); a 256-column
+    // tile of several exact groups has one accumulator buffer, whose drain is not hidden.
+    const long long tiles_m_est = use_patch ? ps.tiles : row_tiles_est;
+    int& BN = f.BN = 64;
+    if (acc64 || a.K <= 64) {
+        BN = 64;
+    } else if (wide_split || (a.K > 128 && conv_path_is("tc_bn256"))) {
+        BN = 256;
+    } else {
+        auto rounds = [&](int bn) { return (double)((tiles_m_est * ((a.K + bn - 1) / bn) + sms - 1) / sms); };
+        const double c64 = rounds(64) * 300, c128 = rounds(128) * 410, c256 = rounds(256) * (P.n_groups > 1 ? 1100 : 615);
+        BN = c128 <= c64 ? 128 : 64;
+        if (a.K > 128 && !conv_path_is("tc_bn128") && c256 <= (BN == 128 ? c128 : c64)) BN = 256;
+    }
+    // packed k-bit weights (k <= 8, one plane) are read by the 256-column TMA-row instances of the
+    // split (FC) layers, whose weights stream through once; elsewhere every weight tile is expanded
+    // once per row tile and the fp16 codes are read instead
+    f.pk = d.d_wpacked && d.fmt_w.bits <= 8 && BN == 256 && wide_split && (reinterpret_cast<uintptr_t>(d.d_wpacked) & 15) == 0 &&
+           !conv_path_is("tc_nopack");
+    return true;
+}
+
 namespace {
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -137,75 +207,16 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     launched = false;
     // (read once: a search of the environment takes about as long as encoding a tensor map)
     const char* const path = getenv("FXPQ_CONV_PATH");
-    auto conv_path_is = [path](const char* name) { return path && strcmp(path, name) == 0; };
+    auto conv_path_is = [path](const char* name) { return path_is(path, name); };
     TcParams P;
-    bool acc64 = false;
+    TcForm f;
     const int sms = num_sms();
-    const long long row_tiles_est = (a.M + TC_BM - 1) / TC_BM;
-    // Layers whose im2col matrix is the stored activations themselves: 1x1 stride-1 convolutions
-    // without padding ([M][Cp] per plane) and kernels covering the whole unpadded map (P = Q = 1,
-    // FC layers: [N][H W Cp]).  A 128-row A tile is then one 2-D box of [M][R S Cp].
-    const bool one_by_one = a.R == 1 && a.S == 1 && a.stride == 1 && a.pad == 0 && a.x_sw == a.Cp;
-    const bool whole_map = a.R == a.H && a.S == a.W && a.pad == 0 && a.P == 1 && a.Q == 1;
-    const bool rows_geom = (one_by_one || whole_map) && a.M > 0 && a.M < (1LL << 31) - TC_BM &&
-                           !conv_path_is("tc_rows") && !conv_path_is("tc_patch");
-    // Patch tiles for every other layer whose stride a TMA box can traverse and whose channel count fills its
-    // 64-channel blocks well enough: up to four times the k-blocks of the flattened reduction of the
-    // gathered row tiles, which take about six times as long per k-block (2600 cycles against 410; a 7 x 7
-    // 512-channel layer of 128 images 95 us gathered, 31 us as patches); 8-channel stride-1 inputs take boxes
-    // of one tap each (narrow)
-    const bool narrow = a.Cp == 8;
-    PatchShape ps;
-    if (!rows_geom && a.P > 0 && a.Q > 0 && a.N > 0 && a.stride <= (narrow ? 1 : 8) && !conv_path_is("tc_rows"))
-        ps = patch_shape(a, TC_BM);
-    const int kbt = (a.Cp + TC_BK - 1) / TC_BK;
-    const int kb_flat = (a.R * a.S * a.Cp + TC_BK - 1) / TC_BK;
-    // How many of its k-blocks a layer may spend as patches for one of the flattened reduction (K = 64 / 256, 3x3,
-    // 588 row tiles, us as patches and gathered): 32 channels, 1.8 times as many, 15.8 / 22.4 and 31.5 / 35.2; 16
-    // channels, 3 times, 25.3 / 19.4 and 37.3 / 29.4.  Pixels that are not whole 32-byte sectors cost their boxes
-    // double: 120 channels, 1.06 times, 37.6 / 46.2; 136 channels, 1.35 times, 55.7 / 49.3; 24 channels 63.9 / 35.2.
-    // Where each tile has an SM to itself the latency of a k-block decides instead, and patches win longer (24
-    // channels, 21 tiles: 8.9 / 9.9).  Two-limb reductions drain a group per limb pair, which hides less of the
-    // patches' k-blocks (32 channels, 1.8 times: 68 / 62; 80 channels, 1.5 times: 99.5 / 103; 16-bit 24 channels, 5 x 5,
-    // 2.5 times: 272 / 103).
-    // Eight-channel patches take the gathered form's k-blocks, a box per tap: one-limb layers 1.1 to 1.4 times faster,
-    // two-limb ones only with few taps (128 channels, 3 x 3, 1568 tiles: 134 / 140; 64 channels, 7 x 7: 132 / 114).
-    // (The space-to-depth form has no more k-blocks as patches.)
-    const bool two_limb = a.px * a.pw > 1, lone = row_tiles_est * ((a.K + 63) / 64) <= sms;
-    const bool any_patch = conv_path_is("tc") || conv_path_is("tc_bn256") || a.x_sw != a.Cp;
-    const double most = any_patch ? 4.0 : a.Cp % 16 ? (lone && !two_limb ? 2.3 : 1.15) : two_limb ? 1.55 : lone ? 4.0 : 2.0;
-    const bool use_patch =
-        ps.TW > 0 && (conv_path_is("tc_patch") || (narrow ? any_patch || !two_limb || (!lone && a.R * a.S <= 16)
-                                                          : (double)ps.tiles * a.R * a.S * kbt <= most * (double)row_tiles_est * kb_flat));
-    P.kbt = kbt;
-    if (!plan_tc(a, d, P, acc64, use_patch && !narrow ? a.R * a.S * kbt : kb_flat)) return FXPQ_OK;
-    // ... with few row tiles (FC layers at small batches) they take 256-column tiles and a split
-    // reduction fills the SMs: the MMA thread's fixed cost per k-block is then hidden, and the weights
-    // stream at the memory's rate
-    const bool wide_split = rows_geom && !acc64 && !a.has_scale && ws && a.K > 128 && !conv_path_is("tc_bn128") &&
-                            !conv_path_is("tc_nosplit") && row_tiles_est * ((a.K + 255) / 256) * 2 <= sms &&
-                            (kb_flat * a.px * a.pw >= 32 || d.d_wpacked);  // (shorter ones are not split, see below)
-    // Tile width: 64 columns for int64 sums and at most 64 output channels, else the width whose whole rounds
-    // over the SMs take the fewest cycles.  A k-block costs what its stage takes from L2 at about 80 bytes
-    // per cycle and SM (24, 32 and 48 KB: 300, 410 and 615 cycles; the MMAs 228, 256 and 512); a 256-column
-    // tile of several exact groups has one accumulator buffer, whose drain is not hidden.
-    const long long tiles_m_est = use_patch ? ps.tiles : row_tiles_est;
-    int BN = 64;
-    if (acc64 || a.K <= 64) {
-        BN = 64;
-    } else if (wide_split || (a.K > 128 && conv_path_is("tc_bn256"))) {
-        BN = 256;
-    } else {
-        auto rounds = [&](int bn) { return (double)((tiles_m_est * ((a.K + bn - 1) / bn) + sms - 1) / sms); };
-        const double c64 = rounds(64) * 300, c128 = rounds(128) * 410, c256 = rounds(256) * (P.n_groups > 1 ? 1100 : 615);
-        BN = c128 <= c64 ? 128 : 64;
-        if (a.K > 128 && !conv_path_is("tc_bn128") && c256 <= (BN == 128 ? c128 : c64)) BN = 256;
-    }
-    // packed k-bit weights (k <= 8, one plane) are read by the 256-column TMA-row instances of the
-    // split (FC) layers, whose weights stream through once; elsewhere every weight tile is expanded
-    // once per row tile and the fp16 codes are read instead
-    P.pk = d.d_wpacked && d.fmt_w.bits <= 8 && BN == 256 && wide_split && (reinterpret_cast<uintptr_t>(d.d_wpacked) & 15) == 0 &&
-           !conv_path_is("tc_nopack");
+    if (!choose_form(a, d, path, sms, ws != nullptr, P, f)) return FXPQ_OK;
+    const bool rows_geom = f.rows_geom, narrow = f.narrow, use_patch = f.use_patch, two_limb = a.px * a.pw > 1;
+    const PatchShape& ps = f.ps;
+    bool acc64 = f.acc64;
+    int BN = f.BN;
+    P.pk = f.pk;
     P.wpack = static_cast<const uint32_t*>(d.d_wpacked);
     P.wk = d.fmt_w.bits;
     P.wsigned = d.fmt_w.is_signed;

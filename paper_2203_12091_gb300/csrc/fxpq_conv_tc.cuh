@@ -2103,7 +2103,28 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     }
 }
 
+// Patch shape of a layer's output: TW x TH pixels of TN images (see patch_shape).
+struct PatchShape {
+    int TW = 0, TH = 0, TN = 0;
+    long long tiles = 0;
+};
+// What the host chose for a layer, besides its exact groups.
+struct TcForm {
+    bool rows_geom;   // row tiles by TMA: the im2col matrix is the stored activations
+    bool narrow;      // 8 stored channels
+    bool use_patch;   // patch tiles of shape ps, else (without rows_geom) gathered row tiles
+    bool acc64;       // int64 running sums
+    bool pk;          // packed weights are read
+    int BN;           // tile width
+    PatchShape ps;
+};
+
 }  // namespace tc
+
+// The host's choices for a layer on `sms` SMs: P's exact groups (and P.kbt) and f.  path: FXPQ_CONV_PATH or null; has_ws:
+// there is scratch.  False: the tensor-core path cannot keep the sums exact.  Touches no device.
+bool choose_form(const ConvArgs& a, const fxpq_conv_desc& d, const char* path, int sms, bool has_ws, tc::TcParams& P,
+                 tc::TcForm& f);
 
 // Launches the SC = true kernel for tile width BN (acc64: the 64-bit running-sum variant, BN = 64).
 fxpq_status launch_conv_tc_scaled(const tc::TcParams& P, int BN, bool acc64, int grid, cudaStream_t st);

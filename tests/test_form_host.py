@@ -1,0 +1,49 @@
+"""The tensor-core path's choice of a form for a layer, run on the CPU (`tests/form_host.cu`): what each form may be given."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = os.path.join(ROOT, "tests", "form_host.cu")
+BIN = os.path.join(ROOT, "tests", "_build", "form_host")
+IN = ["N", "H", "W", "C", "Cp", "K", "R", "S", "stride", "pad", "xb", "wb", "mode", "packed", "s2d", "path"]
+OUT = ["status", "s2d_ok", "planned", "rows_geom", "narrow", "use_patch", "pk", "BN", "n_groups", "overlap", "TW", "TH", "TN",
+       "tiles"]
+
+
+def choose(layers):
+    """The choices for layers given as dicts (mode 1: int64 sums; missing: no padding, 8 / 7 bits, default path)."""
+    from paper_2203_12091_gb300 import build as B
+    if not os.path.exists(B.nvcc()) and not shutil.which(B.nvcc()):
+        pytest.skip("nvcc not available")
+    B.build()
+    objs = sorted(os.path.join(B.BUILD, f) for f in os.listdir(B.BUILD) if f.endswith(".o"))
+    deps = [SRC] + objs + [os.path.join(B.CSRC, f) for f in os.listdir(B.CSRC) if f.endswith(".cuh")]
+    if not os.path.exists(BIN) or any(os.path.getmtime(d) > os.path.getmtime(BIN) for d in deps):
+        os.makedirs(os.path.dirname(BIN), exist_ok=True)
+        r = subprocess.run([B.nvcc(), *B.ARCH, "-O2", "-std=c++17", "--expt-relaxed-constexpr", f"-I{B.INCLUDE}", f"-I{B.CSRC}", SRC,
+                            *objs, "-o", BIN + ".tmp"], capture_output=True, text=True)
+        assert r.returncode == 0, r.stdout + r.stderr
+        os.replace(BIN + ".tmp", BIN)
+    text = ""
+    for c in layers:
+        c = {"W": c["H"], "S": c["R"], "Cp": (c["C"] + 7) // 8 * 8, "stride": 1, "pad": 0, "xb": 8, "wb": 7, "mode": 1, "packed": 0,
+             "s2d": 0, "path": "-", **c}
+        text += " ".join(str(c[k]) for k in IN) + "\n"
+    r = subprocess.run([BIN], input=text, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    rows = [dict(zip(OUT, map(int, line.split()))) for line in r.stdout.strip().splitlines()]
+    assert len(rows) == len(layers)
+    return rows
+
+
+def test_packed_weights_stay_behind_the_space_to_depth_form():
+    """The records hold the original reduction: the original layer may read them, its rewritten form may not."""
+    layers = [dict(N=3, H=224, C=3, K=192, R=4, stride=4), dict(N=40, H=5, C=8, K=16384, R=5, stride=4),
+              dict(N=40, H=4, C=3, K=16384, R=4, stride=4), dict(N=40, H=7, C=8, K=264, R=7, stride=2, path="tc")]
+    for c, plain, s2d in zip(layers, choose([dict(c, packed=1) for c in layers]), choose([dict(c, packed=1, s2d=1) for c in layers])):
+        assert s2d["s2d_ok"] and s2d["planned"] and s2d["rows_geom"] and not s2d["pk"], c
+        if c["R"] == c["H"] and c["K"] > 300:
+            assert plain["pk"], c

@@ -661,6 +661,20 @@ def test_space_to_depth_parity(F, H, C, K, R, st, pad, kx, kw, mode):
     assert s == ws and np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("N,H,C,K,R,st", [(3, 56, 3, 192, 4, 4), (3, 5, 8, 264, 5, 4), (5, 4, 3, 136, 4, 4), (3, 7, 8, 264, 7, 2),
+                                          (160, 8, 3, 192, 4, 4)])
+@pytest.mark.parametrize("kx", [8, 16])
+def test_strided_layers_with_packed_weights(F, N, H, C, K, R, st, kx):
+    """Packed weights of strided layers on 8 stored channels: 1x1 and whole-map layers once space-to-depth, in which the
+    records (of the original reduction, shorter where the stride does not divide the kernel) stay unread."""
+    rng = np.random.default_rng(N * H + K)
+    fx, fw, fb, fy = F.fmt(kx, 0, kx - 3), F.fmt(7, 1, 6), F.fmt(16, 1, 14), F.fmt(8, 0, 2)
+    x, w, b = rand_codes(rng, (N, H, H, C), kx, 0), rand_codes(rng, (K, R, R, C), 7, 1), rand_codes(rng, (K,), 16, 1)
+    got, s = run_conv(F, x, fx, w, fw, b, fb, st, 0, True, 0, fy, 8, packed_w=w)
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, st, 0, True, 0, fy)
+    assert s == ws and np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("K,mode", [(8, 0), (24, 0), (72, 0), (120, 0), (136, 0), (200, 0), (264, 0), (2, 1), (10, 2), (77, 2), (130, 1)])
 @pytest.mark.parametrize("N,H,C,R,kx", [(3, 12, 64, 3, 7), (3, 12, 72, 1, 7), (5, 1, 700, 1, 8), (2, 9, 24, 3, 16), (40, 20, 64, 3, 8)])
 def test_last_column_tile_parity(F, K, mode, N, H, C, R, kx):
