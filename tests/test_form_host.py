@@ -47,3 +47,17 @@ def test_packed_weights_stay_behind_the_space_to_depth_form():
         assert s2d["s2d_ok"] and s2d["planned"] and s2d["rows_geom"] and not s2d["pk"], c
         if c["R"] == c["H"] and c["K"] > 300:
             assert plain["pk"], c
+
+
+def test_overlapping_pixels_are_read_through_tensor_maps():
+    """The space-to-depth form of a wide enough tap row has overlapping pixels: never gathered, over all its geometries."""
+    layers = [dict(N=N, H=H, W=W, C=C, K=64, R=R, S=S, stride=st, pad=pad, xb=xb, wb=xb - 1, s2d=1, path=path)
+              for st in (2, 3, 4) for R in range(st, 12) for S in range(st, 12) for C in (1, 2, 3, 5, 8)
+              for N, H, W, pad in ((1, 31, 29, 0), (40, 51, 47, 0), (7, 140, 140, 3))
+              for xb in (8, 16) for path in ("-", "tc_patch")]
+    seen = 0
+    for c, r in zip(layers, choose(layers)):
+        if r["s2d_ok"] and r["planned"] and r["overlap"]:
+            seen += 1
+            assert r["use_patch"] or r["rows_geom"], c
+    assert seen > 1000

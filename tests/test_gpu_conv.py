@@ -675,6 +675,29 @@ def test_strided_layers_with_packed_weights(F, N, H, C, K, R, st, kx):
     assert s == ws and np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("N,H,W,C,R,S,st", [(40, 51, 47, 1, 7, 3, 2), (40, 51, 47, 2, 8, 4, 2), (3, 51, 47, 1, 8, 3, 2),
+                                            (9, 30, 141, 2, 7, 4, 2), (5, 60, 60, 1, 11, 5, 3), (4, 45, 50, 3, 3, 8, 2)])
+@pytest.mark.parametrize("kx", [8, 16])
+@pytest.mark.parametrize("path", ["", "tc_patch"])
+def test_space_to_depth_of_rectangular_kernels(F, N, H, W, C, R, S, st, kx, path):
+    """Kernels of unequal sides on few channels: as patches the rewritten layer takes up to four times the k-blocks of the
+    gathered form, which its overlapping pixels may not take.  The default choice, and patches everywhere."""
+    if os.environ.get("FXPQ_CONV_PATH") != "tc":
+        pytest.skip("once")
+    rng = np.random.default_rng(H * W + R)
+    fx, fw, fb, fy = F.fmt(kx, 0, kx - 3), F.fmt(kx, 1, kx - 1), F.fmt(16, 1, 14), F.fmt(8, 0, 2)
+    x, w, b = rand_codes(rng, (N, H, W, C), kx, 0), rand_codes(rng, (64, R, S, C), kx, 1), rand_codes(rng, (64,), 16, 1)
+    del os.environ["FXPQ_CONV_PATH"]
+    if path:
+        os.environ["FXPQ_CONV_PATH"] = path
+    try:
+        got, s = run_conv(F, x, fx, w, fw, b, fb, st, 0, True, 0, fy, 8)
+    finally:
+        os.environ["FXPQ_CONV_PATH"] = "tc"
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, st, 0, True, 0, fy)
+    assert s == ws and np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("K,mode", [(8, 0), (24, 0), (72, 0), (120, 0), (136, 0), (200, 0), (264, 0), (2, 1), (10, 2), (77, 2), (130, 1)])
 @pytest.mark.parametrize("N,H,C,R,kx", [(3, 12, 64, 3, 7), (3, 12, 72, 1, 7), (5, 1, 700, 1, 8), (2, 9, 24, 3, 16), (40, 20, 64, 3, 8)])
 def test_last_column_tile_parity(F, K, mode, N, H, C, R, kx):
