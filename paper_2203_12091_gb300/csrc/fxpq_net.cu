@@ -14,6 +14,7 @@ namespace {
 struct Slot {
     int H = 0, W = 0, Cp = 0;
     int C = 0;  // true channel count (Cp without the padding)
+    int live = 0;  // channels that may hold codes other than zero: C, but for a sum those of both operands
     fxpq_fmt fmt{0, 0, 0};
     bool defined = false;
     size_t offset = 0, bytes = 0;
@@ -30,7 +31,7 @@ fxpq_status plan_net(const fxpq_net* net, int32_t batch, std::vector<Slot>& slot
     slots[0].H = net->H;
     slots[0].W = net->W;
     slots[0].Cp = net->Cp_in;
-    slots[0].C = net->C;
+    slots[0].C = slots[0].live = net->C;
     slots[0].fmt = net->fmt_in;
     slots[0].defined = true;
     for (int i = 0; i < net->n_ops; ++i) {
@@ -47,7 +48,7 @@ fxpq_status plan_net(const fxpq_net* net, int32_t batch, std::vector<Slot>& slot
                 out.H = (s0.H + 2 * o.pad - o.R) / o.stride + 1;
                 out.W = (s0.W + 2 * o.pad - o.S) / o.stride + 1;
                 out.Cp = o.K;
-                out.C = o.K;
+                out.C = out.live = o.K;
                 out.fmt = o.fmt_y;
                 if (last) break;
                 if (!fxpq::fmt_ok(o.fmt_y) || (o.K % 8)) return FXPQ_ERR_INVALID_ARG;
@@ -59,6 +60,7 @@ fxpq_status plan_net(const fxpq_net* net, int32_t batch, std::vector<Slot>& slot
                 out.W = (s0.W + 2 * o.pad - o.R) / o.stride + 1;
                 out.Cp = s0.Cp;
                 out.C = s0.C;
+                out.live = s0.live;
                 out.fmt = s0.fmt;
                 break;
             case FXPQ_OP_ELTWISE: {
@@ -66,6 +68,7 @@ fxpq_status plan_net(const fxpq_net* net, int32_t batch, std::vector<Slot>& slot
                 const Slot& s1 = slots[o.src1];
                 if (s1.H != s0.H || s1.W != s0.W || s1.Cp != s0.Cp) return FXPQ_ERR_INVALID_ARG;
                 out = s0;
+                out.live = std::max(s0.live, s1.live);
                 out.fmt = o.fmt_y;
                 break;
             }
@@ -73,6 +76,7 @@ fxpq_status plan_net(const fxpq_net* net, int32_t batch, std::vector<Slot>& slot
                 out.H = out.W = 1;
                 out.Cp = s0.Cp;
                 out.C = s0.C;
+                out.live = s0.live;
                 out.fmt = o.fmt_y;
                 break;
             default:
@@ -104,7 +108,7 @@ size_t net_conv_ws(const fxpq_net* net, const std::vector<Slot>& slots, int32_t 
         if (o.op != FXPQ_OP_CONV) continue;
         const Slot& s0 = slots[o.src0];
         fxpq_conv_desc d = {};
-        d.N = batch, d.H = s0.H, d.W = s0.W, d.C = s0.C, d.Cp = s0.Cp, d.K = o.K, d.R = o.R, d.S = o.S;
+        d.N = batch, d.H = s0.H, d.W = s0.W, d.C = s0.live, d.Cp = s0.Cp, d.K = o.K, d.R = o.R, d.S = o.S;
         d.stride = o.stride, d.pad = o.pad, d.fmt_x = s0.fmt, d.fmt_w = o.fmt_w;
         const size_t b = fxpq::conv_ws_bytes(d);
         if (b > m) m = b;
@@ -192,7 +196,7 @@ extern "C" fxpq_status fxpq_net_forward(const fxpq_net* h_net, const float* d_im
                 d.N = batch;
                 d.H = s0.H;
                 d.W = s0.W;
-                d.C = s0.C;
+                d.C = s0.live;
                 d.Cp = s0.Cp;
                 d.K = o.K;
                 d.R = o.R;
@@ -412,7 +416,7 @@ extern "C" fxpq_status fxpq_net_calibrate(const fxpq_net* h_net, const float* d_
                 cd.N = n_calib;
                 cd.H = s0.H;
                 cd.W = s0.W;
-                cd.C = s0.C;
+                cd.C = s0.live;
                 cd.Cp = s0.Cp;
                 cd.K = o.K;
                 cd.R = o.R;

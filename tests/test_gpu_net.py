@@ -100,6 +100,30 @@ def test_first_layer_from_images(NET, R, st, pad, hw, k, monkeypatch):
         assert F.fxpq_get_device_status() == 3
 
 
+def test_addition_of_maps_with_different_channel_counts(NET, monkeypatch):
+    """A sum of a 3-channel map (stored as 8) and an 8-channel one has 8 channels whichever comes first: the strided
+    layer behind it, which the space-to-depth form reduces to its true channels, gives the same logits both ways."""
+    monkeypatch.setenv("FXPQ_CONV_PATH", "tc")
+    rng = np.random.default_rng(8)
+    W = {nm: (rng.standard_normal(sh).astype(np.float32) * 0.2, rng.standard_normal(sh[0]).astype(np.float32) * 0.01)
+         for nm, sh in (("c0", (8, 3, 3, 3)), ("c1", (16, 4, 4, 8)), ("fc", (24, 1, 1, 16)))}
+    plan = {"input": 8, "c0": {"w": 8, "b": 16, "a": 8}, "e": {"a": 8}, "c1": {"w": 8, "b": 16, "a": 8}, "gap": {"a": 8, "r": 16},
+            "fc": {"w": 8, "b": 16}}
+    imgs = torch.from_numpy(synth.images(5, 2, hw=28)).cuda()
+    out = []
+    for a, b in (("p0", "c0"), ("c0", "p0")):
+        L = [{"type": "maxpool", "name": "p0", "k": 3, "stride": 1, "pad": 1},
+             {"type": "conv", "name": "c0", "C": 3, "K": 8, "R": 3, "stride": 1, "pad": 1, "relu": True, "src": "p0"},
+             {"type": "eltwise", "name": "e", "a": a, "b": b, "relu": True},
+             {"type": "conv", "name": "c1", "C": 8, "K": 16, "R": 4, "stride": 4, "pad": 0, "relu": True, "src": "e"},
+             {"type": "avgpool", "name": "gap", "src": "c1"},
+             {"type": "conv", "name": "fc", "C": 16, "K": 24, "R": 1, "stride": 1, "pad": 0, "relu": False, "src": "gap"}]
+        q = NET.build_qnet(L, W, imgs, plan)
+        logits, s = q.forward(imgs)
+        out.append((logits.cpu().numpy(), s, q.fmts["c1"]["a"].tup()))
+    assert np.array_equal(out[0][0], out[1][0]) and out[0][1:] == out[1][1:]
+
+
 def _workload(NET, arch, batch, seed, plan_seed=None, calib=8, sample=(0, -1), pack=False):
     L = synth.ARCHS[arch]()
     W = synth.weights(arch, seed)
