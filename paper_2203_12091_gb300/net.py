@@ -98,6 +98,7 @@ class QNet:
         self.qp = {}
         self.pack_weights = pack_weights
         self.qs = {}  # BN conv name -> (aleph1 int32 codes, aleph2 int32 codes)
+        self.w_c = {}  # conv name -> input channels of its weights
         self.w_l1 = {}  # conv name -> max over output channels of sum |weight code| (0: unknown)
         self.names = ["input"] + [L_["name"] for L_ in layers]
         self.slot = {nm: i for i, nm in enumerate(self.names)}
@@ -126,6 +127,7 @@ class QNet:
                 w, b = weights_dev[nm]
                 K, R, _, C = w.shape
                 assert C <= Cp
+                self.w_c[nm] = C
                 searches.append((w, plan[nm]["w"]))
                 owners.append((nm, "w"))
                 if b is not None:
@@ -233,7 +235,7 @@ class QNet:
             sH, sW, sCp = self.shapes[src]
             wq, bq = self.q[nm]
             sq, hq = self.qs.get(nm, (None, None))
-            d = F.conv_desc(N, sH, sW, L_["C"], sCp, L_["K"], L_["R"], L_["R"], L_["stride"], L_["pad"], L_["relu"],
+            d = F.conv_desc(N, sH, sW, self.w_c.get(nm, sCp), sCp, L_["K"], L_["R"], L_["R"], L_["stride"], L_["pad"], L_["relu"],
                             out_mode, fx, self.fmts[nm]["w"], self.fmts[nm].get("b"), fy, self.w_l1.get(nm, 0),
                             scale=sq, fmt_scale=self.fmts[nm].get("s"), shift=hq, fmt_shift=self.fmts[nm].get("h"),
                             wpacked=self.qp.get(nm))

@@ -100,6 +100,19 @@ def test_first_layer_from_images(NET, R, st, pad, hw, k, monkeypatch):
         assert F.fxpq_get_device_status() == 3
 
 
+def test_layer_dicts_without_channel_counts(NET):
+    """A layer's input channels come from its weights: a trace of layers that do not state them equals one of layers that do."""
+    L, plan = _tiny()
+    rng = np.random.default_rng(3)
+    W = {l["name"]: (rng.standard_normal((l["K"], l["R"], l["R"], l["C"])).astype(np.float32) * 0.2,
+                     rng.standard_normal(l["K"]).astype(np.float32) * 0.01) for l in L if l["type"] == "conv"}
+    imgs = torch.from_numpy(synth.images(3, 2, hw=28)).cuda()
+    last = []
+    for layers in (L, [{k: v for k, v in l.items() if k != "C"} for l in L]):
+        last.append(NET.build_qnet(layers, W, imgs, plan).trace(imgs)["fc"][0].cpu())
+    assert torch.equal(*last)
+
+
 def test_addition_of_maps_with_different_channel_counts(NET, monkeypatch):
     """A sum of a 3-channel map (stored as 8) and an 8-channel one has 8 channels whichever comes first: the strided
     layer behind it, which the space-to-depth form reduces to its true channels, gives the same logits both ways."""
