@@ -30,6 +30,7 @@ struct ConvF32Args {
     float* y;
     int N, H, W, C, K, R, S, stride, pad, P, Q, relu;
     long long M;
+    int n_first;  // first output channel of the launch
 };
 
 __device__ __forceinline__ unsigned long long f2_pack(float x, float y) {
@@ -44,8 +45,10 @@ __device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
 }
 
 // VEC: C % 4 == 0 (a float4 of a row stays inside one tap) and 16-byte aligned x and w; otherwise single loads,
-// the reduction index decoded through a table in shared memory (up to CF_TAB steps).
-template <int BM, bool VEC>
+// the reduction index decoded through a table in shared memory (up to CF_TAB steps, whose tap rows and columns are below
+// CF_TAB too and share a word).  Off: the type of an offset within a window, 64-bit where that spans 2^31 elements (a few
+// taps of long rows).
+template <int BM, bool VEC, typename Off = int>
 __global__ void __launch_bounds__(256, 2) conv_f32_kernel(const ConvF32Args a) {
     pdl_wait();
     constexpr int MT = BM / 8;           // output pixels per thread
@@ -55,16 +58,19 @@ __global__ void __launch_bounds__(256, 2) conv_f32_kernel(const ConvF32Args a) {
     // lanes with consecutive k / 4 then fall into different banks, and pieces stay whole for the loads
     __shared__ __align__(16) float sa[2][CF_BK][BM];
     __shared__ __align__(16) float sb[2][CF_BK][CF_BN];
-    __shared__ int2 tab[VEC ? 1 : CF_TAB];
+    __shared__ Off tab_off[VEC ? 1 : CF_TAB];
+    __shared__ int tab_rs[VEC ? 1 : CF_TAB];
+    static_assert(CF_TAB <= 32768, "a tap's row and column share a word");
     const int tid = threadIdx.x, grp = tid >> 6, t64 = tid & 63;
     const int tx = t64 & 7, ty = t64 >> 3;
     const long long m0 = (long long)blockIdx.x * BM;
-    const int n0 = blockIdx.y * CF_BN;
+    const int n0 = a.n_first + (int)blockIdx.y * CF_BN;
     const int RSC = a.R * a.S * a.C;
     if (!VEC) {
         for (int k = tid; k < RSC && k < CF_TAB; k += 256) {
             const int c = k % a.C, rs = k / a.C, s = rs % a.S, r = rs / a.S;
-            tab[k] = make_int2((r * a.W + s) * a.C + c, (r << 16) | s);
+            tab_off[k] = ((Off)r * a.W + s) * a.C + c;
+            tab_rs[k] = (r << 16) | s;
         }
         __syncthreads();
     }
@@ -75,7 +81,7 @@ __global__ void __launch_bounds__(256, 2) conv_f32_kernel(const ConvF32Args a) {
 #pragma unroll
     for (int i = 0; i < AV; ++i) {
         const long long m = m0 + lr + 32 * i;
-        p0[i] = -(1 << 20);  // rows past the end read zeros
+        p0[i] = -(1 << 30);  // rows past the end read zeros
         q0[i] = 0;
         xo[i] = 0;
         if (m < a.M) {
@@ -118,20 +124,23 @@ __global__ void __launch_bounds__(256, 2) conv_f32_kernel(const ConvF32Args a) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int kk = k + e;
-                int2 te = make_int2(0, 0);
-                if (kk < RSC) {
-                    if (kk < CF_TAB) {
-                        te = tab[kk];
-                    } else {
-                        const int c = kk % a.C, rs = kk / a.C, s = rs % a.S, r = rs / a.S;
-                        te = make_int2((r * a.W + s) * a.C + c, (r << 16) | s);
-                    }
+                int r = 0, s = 0;
+                Off off = 0;
+                if (kk < CF_TAB && kk < RSC) {
+                    off = tab_off[kk];
+                    r = tab_rs[kk] >> 16;
+                    s = tab_rs[kk] & 0xFFFF;
+                } else if (kk < RSC) {
+                    const int c = kk % a.C, rs = kk / a.C;
+                    s = rs % a.S;
+                    r = rs / a.S;
+                    off = ((Off)r * a.W + s) * a.C + c;
                 }
 #pragma unroll
                 for (int i = 0; i < AV; ++i) {
-                    const int h = p0[i] + (te.y >> 16), w = q0[i] + (te.y & 0xFFFF);
+                    const int h = p0[i] + r, w = q0[i] + s;
                     const bool in = kk < RSC && (unsigned)h < (unsigned)a.H && (unsigned)w < (unsigned)a.W;
-                    va[i][e] = in ? __ldg(a.x + xo[i] + te.x) : 0.0f;
+                    va[i][e] = in ? __ldg(a.x + xo[i] + off) : 0.0f;
                 }
 #pragma unroll
                 for (int i = 0; i < BV; ++i) {
@@ -673,20 +682,29 @@ extern "C" fxpq_status fxpq_conv_f32(const fxpq_conv_f32_desc* h_desc, const flo
     ConvF32Args a{d_x, d_w, d_bias, d_y, d.N, d.H, d.W, d.C, d.K, d.R, d.S, d.stride, d.pad, P, Q, d.relu ? 1 : 0,
                   (long long)d.N * P * Q};
     if (a.M == 0) return FXPQ_OK;
-    // 32-pixel tiles for few output pixels (FC layers of a calibration slice), where 64-pixel ones are mostly empty
     const bool vec = d.C % 4 == 0 && aligned(d_x, 16) && aligned(d_w, 16);
-    const int bm = a.M <= 32 ? 32 : 64;
-    dim3 grid((unsigned)((a.M + bm - 1) / bm), (unsigned)((d.K + CF_BN - 1) / CF_BN));
+    const bool wide = !vec && ((long long)d.R * d.W + d.S) * d.C >= (1LL << 31);
+    // 32-pixel tiles for few output pixels (FC layers of a calibration slice), where 64-pixel ones are mostly empty
+    const int bm = a.M <= 32 && !wide ? 32 : 64;
+    const long long cols = ((long long)d.K + CF_BN - 1) / CF_BN;
     cudaStream_t s = as_stream(stream);
-    if (bm == 32 && vec)
-        launch_pdl(conv_f32_kernel<32, true>, grid, 256, 0, s, a);
-    else if (bm == 32)
-        launch_pdl(conv_f32_kernel<32, false>, grid, 256, 0, s, a);
-    else if (vec)
-        launch_pdl(conv_f32_kernel<64, true>, grid, 256, 0, s, a);
-    else
-        launch_pdl(conv_f32_kernel<64, false>, grid, 256, 0, s, a);
-    return after_launch("conv_f32");
+    for (long long c0 = 0; c0 < cols; c0 += 65535) {  // (a grid has at most 65535 rows)
+        a.n_first = (int)(c0 * CF_BN);
+        const dim3 grid((unsigned)((a.M + bm - 1) / bm), (unsigned)(cols - c0 < 65535 ? cols - c0 : 65535));
+        if (wide)
+            launch_pdl(conv_f32_kernel<64, false, long long>, grid, 256, 0, s, a);
+        else if (bm == 32 && vec)
+            launch_pdl(conv_f32_kernel<32, true>, grid, 256, 0, s, a);
+        else if (bm == 32)
+            launch_pdl(conv_f32_kernel<32, false>, grid, 256, 0, s, a);
+        else if (vec)
+            launch_pdl(conv_f32_kernel<64, true>, grid, 256, 0, s, a);
+        else
+            launch_pdl(conv_f32_kernel<64, false>, grid, 256, 0, s, a);
+        const fxpq_status st = after_launch("conv_f32");
+        if (st != FXPQ_OK) return st;
+    }
+    return FXPQ_OK;
 }
 
 extern "C" fxpq_status fxpq_maxpool_f32(const float* d_x, int32_t N, int32_t H, int32_t W, int32_t C, int32_t k,

@@ -71,6 +71,25 @@ def test_conv_f32_tiles(M, N, H, C, K, R, st, pad, off):
     assert (np.abs(got[:-1].reshape(want.shape) - want) <= (R * R * C + 2) * 2.0 ** -24 * mag).all()
 
 
+@pytest.mark.parametrize("H,W,R,S,st,K", [(2, 70007, 1, 70000, 1, 3), (40003, 2, 40000, 1, 1, 3), (9, 280_000_000, 9, 1, 999_983, 2),
+                                         (1, 3, 1, 2, 1, 4_200_000)])
+def test_conv_f32_index_ranges(M, H, W, R, S, st, K):
+    """Kernels longer than a table entry's halves, taps more than 2^31 elements apart and more channel tiles than a grid row:
+    one channel (no quads), against fp64 within the bound of a chain of R S additions."""
+    fopt, F = M
+    P, Q = (H - R) // st + 1, (W - S) // st + 1
+    g = torch.Generator(device="cuda").manual_seed(R + S)
+    x = torch.zeros(H, W, device="cuda")
+    x[:, ::st] = torch.randn(H, (W + st - 1) // st, generator=g, device="cuda")
+    w, b = torch.randn(K, R, S, generator=g, device="cuda"), torch.randn(K, generator=g, device="cuda")
+    y = torch.empty(P * Q * K, dtype=torch.float32, device="cuda")
+    F.fxpq_conv_f32(1, H, W, 1, K, R, S, st, 0, False, x, w, b, y)
+    taps = torch.stack([x[p * st:p * st + R, q * st:q * st + S] for p in range(P) for q in range(Q)]).reshape(P * Q, -1).double()
+    w64, b64 = w.reshape(K, -1).double(), b.double()
+    err = (y.reshape(P * Q, K).double() - (taps @ w64.T + b64)).abs()
+    assert (err <= (R * S + 2) * 2.0 ** -24 * (taps.abs() @ w64.abs().T + b64.abs())).all()
+
+
 @pytest.mark.parametrize("fmt", [(8, 1, 5), (8, 0, 30), (16, 1, -3), (4, 1, -20), (24, 1, 10), (1, 1, 2)])
 @pytest.mark.parametrize("kind", ["normal", "relu", "wide", "offset", "constant"])
 def test_ds_stats_against_exact_sums(M, fmt, kind):
