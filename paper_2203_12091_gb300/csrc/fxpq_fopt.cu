@@ -437,8 +437,22 @@ __global__ void __launch_bounds__(DS_T) ds_sum_kernel(const __grid_constant__ Ds
     const float* xs = it.x + (long long)s * it.nu;
     const long long i0 = (long long)c * DS_CHUNK, i1 = min(i0 + DS_CHUNK, it.nu);
     Sum3 acc;
-    ds_walk(xs, i0, i1, [&](float v) { acc.add(v); });
-    const double t = ds_block_sum(acc.value(), red);
+    double big = 0.0;  // steps with a value of 2^100 or more, whose fp32 sums could overflow
+    for (long long i = i0 + threadIdx.x; i < i1; i += (long long)DS_U * DS_T) {
+        float v[DS_U], top = 0.0f;
+#pragma unroll
+        for (int j = 0; j < DS_U; ++j) v[j] = i + (long long)j * DS_T < i1 ? __ldg(xs + i + (long long)j * DS_T) : 0.0f;
+#pragma unroll
+        for (int j = 0; j < DS_U; ++j) top = fmaxf(top, fabsf(v[j]));
+        if (top < 0x1p100f) {
+#pragma unroll
+            for (int j = 0; j < DS_U; ++j) acc.add(v[j]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < DS_U; ++j) big += (double)v[j];
+        }
+    }
+    const double t = ds_block_sum(acc.value() + big, red);
     if (threadIdx.x == 0) units[u].sum = t;
 }
 

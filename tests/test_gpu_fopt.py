@@ -121,6 +121,35 @@ def test_ds_stats_against_exact_sums(M, fmt, kind):
     assert abs(h[4] - float(dev)) <= 1e-15 * float(dev) + n * (4e-16 * float(np.abs(x).max())) ** 2 + 1e-300
 
 
+@pytest.mark.parametrize("kind", ["one sign", "both signs", "beside small ones", "inf", "nan"])
+def test_ds_stats_of_huge_values(M, kind):
+    """Finite values whose sums leave fp32's range keep a finite mean, within the bound of the exact sums' test; an infinity
+    gives an infinite mean."""
+    from fractions import Fraction
+    fopt, F = M
+    rng = np.random.default_rng(9)
+    n = 70001
+    x = (1 + rng.random(n)).astype(np.float32) * np.float32(1.5e38)
+    if kind == "both signs":
+        x *= rng.choice([-1, 1], n).astype(np.float32)
+    elif kind == "beside small ones":
+        x[rng.random(n) < 0.9] = rng.standard_normal()
+    elif kind in ("inf", "nan"):
+        x = rng.standard_normal(n).astype(np.float32)
+        x[4321] = np.float32(kind)
+    out = torch.empty(5, dtype=torch.float64, device="cuda")
+    F.fxpq_ds_stats_batch([(torch.from_numpy(x).cuda(), 1, n, F.fmt(8, 1, 3), out)])
+    h = out.cpu().numpy()
+    if kind in ("inf", "nan"):
+        assert np.array_equal(h[3], np.float64(kind), equal_nan=True)
+        return
+    xs = [Fraction(float(v)) for v in x]
+    mean = sum(xs) / n
+    dev = sum((a - mean) ** 2 for a in xs)
+    assert abs(Fraction(h[3]) - mean) <= Fraction(4e-16) * sum(map(abs, xs)) / n
+    assert h[4] == pytest.approx(float(dev), rel=1e-12)
+
+
 def test_ds_stats_batch_and_ties(M):
     """Statistics records (Eq. DSB_QE's L, the range ends, per-sample mean and sum of squared deviations)
     against float64 numpy, several items in one batch, one of them past one work unit per sample; a
