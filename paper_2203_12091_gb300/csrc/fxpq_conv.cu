@@ -216,7 +216,7 @@ S2dPlan s2d_plan(const fxpq_conv_desc& d) {
     p.flat = (p.S2 * p.C2 + 63) / 64 < p.S2 * ((p.C2 + 63) / 64);
     p.x_bytes = ((size_t)d.N * p.H2 * p.W2 * p.C2 * 2 * planes_of(d.fmt_x) + 255) / 256 * 256;
     p.w_bytes = ((size_t)d.K * p.R2 * p.S2 * p.C2 * 2 * planes_of(d.fmt_w) + 255) / 256 * 256;
-    p.ok = (long long)d.N * p.H2 * p.W2 * 2 < (1LL << 31) * 128;
+    p.ok = (long long)p.H2 * p.W2 < (1LL << 31) && (long long)d.N * p.H2 * p.W2 * 2 < (1LL << 31) * 128;
     return p;
 }
 

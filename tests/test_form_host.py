@@ -61,3 +61,9 @@ def test_overlapping_pixels_are_read_through_tensor_maps():
             seen += 1
             assert r["use_patch"] or r["rows_geom"], c
     assert seen > 1000
+
+
+def test_space_to_depth_maps_have_31_bit_positions():
+    """The copy kernels count a rewritten map's pixels in 32 bits: larger maps keep their own codes."""
+    layers = [dict(N=1, H=H, C=1, K=8, R=2, stride=2) for H in (92_000, 92_800, 131_072, 400_000)]
+    assert [r["s2d_ok"] for r in choose(layers)] == [1, 0, 0, 0]
