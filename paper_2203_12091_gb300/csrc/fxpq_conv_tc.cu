@@ -147,11 +147,16 @@ bool choose_form(const ConvArgs& a, const fxpq_conv_desc& d, const char* path, i
     const bool two_limb = a.px * a.pw > 1, lone = row_tiles_est * ((a.K + 63) / 64) <= sms;
     const bool any_patch = conv_path_is("tc") || conv_path_is("tc_bn256");
     const double most = any_patch ? 4.0 : a.Cp % 16 ? (lone && !two_limb ? 2.3 : 1.15) : two_limb ? 1.55 : lone ? 4.0 : 2.0;
-    const bool use_patch = f.use_patch =
+    bool& use_patch = f.use_patch;
+    use_patch =
         ps.TW > 0 && (overlap || conv_path_is("tc_patch") || (narrow ? any_patch || !two_limb || (!lone && a.R * a.S <= 16)
                                                           : (double)ps.tiles * a.R * a.S * kbt <= most * (double)row_tiles_est * kb_flat));
     if (overlap && !use_patch && !rows_geom) return false;
-    if (!plan_tc(a, d, P, acc64, use_patch && !narrow ? a.R * a.S * kbt : kb_flat)) return false;
+    if (use_patch && !narrow && !plan_tc(a, d, P, acc64, a.R * a.S * kbt)) {  // too many groups: gathered, if that has fewer
+        if (overlap) return false;
+        use_patch = false;
+    }
+    if (!(use_patch && !narrow) && !plan_tc(a, d, P, acc64, kb_flat)) return false;
     // ... with few row tiles (FC layers at small batches) they take 256-column tiles and a split
     // reduction fills the SMs: the MMA thread's fixed cost per k-block is then hidden, and the weights
     // stream at the memory's rate

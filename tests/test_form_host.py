@@ -67,3 +67,11 @@ def test_space_to_depth_maps_have_31_bit_positions():
     """The copy kernels count a rewritten map's pixels in 32 bits: larger maps keep their own codes."""
     layers = [dict(N=1, H=H, C=1, K=8, R=2, stride=2) for H in (92_000, 92_800, 131_072, 400_000)]
     assert [r["s2d_ok"] for r in choose(layers)] == [1, 0, 0, 0]
+
+
+def test_patches_give_way_where_their_groups_are_too_many():
+    """Patches take whole k-blocks per tap and so more exact groups than the gathered reduction: a layer that only the
+    latter keeps exact is gathered, not left to the CUDA cores."""
+    layers = [dict(N=4, H=30, C=48, K=64, R=10, pad=5, xb=16, wb=16), dict(N=2, H=14, C=664, K=64, R=7, pad=3, wb=8)]
+    for c, r in zip(layers, choose(layers)):
+        assert r["planned"] and not r["use_patch"] and r["n_groups"] <= 64, c

@@ -729,7 +729,8 @@ def test_row_parts_parity(F, M, C, K, mode, kx):
 @pytest.mark.parametrize("N,H,C,K,R,st,kx", [(2, 30, 16, 64, 3, 1, 7), (26, 30, 16, 64, 3, 1, 7), (2, 30, 24, 64, 5, 1, 7),
                                              (26, 30, 24, 64, 3, 1, 7), (26, 30, 120, 64, 3, 1, 7), (2, 30, 32, 64, 3, 1, 16),
                                              (2, 30, 80, 64, 3, 1, 16), (2, 30, 3, 64, 5, 1, 16), (26, 30, 3, 72, 3, 1, 16),
-                                             (2, 30, 3, 64, 3, 1, 7), (2, 30, 3, 64, 3, 2, 7), (90, 30, 3, 64, 3, 2, 7)])
+                                             (2, 30, 3, 64, 3, 1, 7), (2, 30, 3, 64, 3, 2, 7), (90, 30, 3, 64, 3, 2, 7),
+                                             (2, 20, 48, 64, 10, 1, 16)])
 def test_chosen_form_parity(F, N, H, C, K, R, st, kx):
     """The form that a layer takes by itself, patches, gathered rows or space-to-depth, on both sides of its lines."""
     if os.environ.get("FXPQ_CONV_PATH") != "tc":
