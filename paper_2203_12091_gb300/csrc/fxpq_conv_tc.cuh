@@ -523,78 +523,6 @@ __device__ __forceinline__ void tmem_st16_nw(uint32_t taddr, const uint32_t (&r)
         "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
 }
-// Final epilogue of 32 consecutive output channels k0.. of row m (generic outputs: two-plane codes,
-// int64 accumulators, fp32 calibration images): bias alignment, ReLU, FxP-QLayer.
-// (This and the next are calls, their values passed in local memory: inlined, they made the 128-column kernels
-// spill 1.2 KB around every path, the codes of several groups among them.  They run in short loops: unrolled over
-// the 32 channels, the int64 logits of a 512 -> 1000 layer, one tile per CTA and each instruction run once,
-// took 25 us, most of it for fetching code and re-reading parameters; 13 us now.)
-template <typename ACC, bool SC>
-__device__ __noinline__ void epilogue_block32(const ConvArgs& a, long long m, int k0, const ACC (&acc)[32]) {
-#pragma unroll 1
-    for (int j = 0; j < 32; ++j) {
-        const int k = k0 + j;
-        if (k >= a.K) break;
-        cblock_epilogue_store<SC>(a, m, k, (long long)acc[j]);
-    }
-}
-
-// The same for fp32-image and int64 outputs through a 2 KiB shared-memory slice of the warp (`wbuf`): every
-// round each lane puts 64 bytes of its row there (16-byte pieces rotated against bank conflicts), then the
-// warp writes 16-byte pieces of whole row segments, eight rows per instruction, rather than 32 rows at one
-// value per lane.  All 32 lanes take part; rows with m < 0 (outside the output) store nothing.  Needs K %
-// 4 == 0 (fp32) or K % 2 == 0 (int64), so that a 16-byte piece is wholly inside or past K.
-template <typename ACC, bool SC>
-__device__ __noinline__ void epilogue_block32_staged(const ConvArgs& a, long long m, int k0, const ACC (&acc)[32],
-                                                        unsigned char* wbuf, int lane) {
-    const bool f32 = a.out_mode == FXPQ_OUT_F32;
-    const int esz = f32 ? 4 : 8;
-    const int per = 64 / esz;  // values per round: 64 bytes of a row
-    const int K = a.K;         // (copies: a lies in memory here, and every store below may alias it)
-    unsigned char* const y = static_cast<unsigned char*>(a.y);
-    const float f32_scale = a.f32_scale;
-    // lane j holds the bias of channel k0 + j, aligned: its one load serves the chunk, and a value costs a shift,
-    // an addition and a shuffle (cblock_value decides on delta, bias and ReLU anew for every one)
-    const int dr = a.has_bias && a.delta < 0 ? -a.delta : 0;
-    const long long bl = a.has_bias && k0 + lane < K ? (long long)__ldg(a.bias + k0 + lane) << max(a.delta, 0) : 0;
-    const long long floor = a.relu ? 0ll : LLONG_MIN;
-    auto value = [&](int j) -> long long {
-        const int k = min(k0 + j, K - 1);
-        if constexpr (SC) return cblock_value<SC>(a, k, (long long)acc[j], a.has_bias ? __ldg(a.bias + k) : 0);
-        return max(((long long)acc[j] << dr) + __shfl_sync(0xffffffffu, bl, j), floor);
-    };
-#pragma unroll 1
-    for (int c0 = 0; c0 < 32 && k0 + c0 < K; c0 += per) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            // one 16-byte piece: four fp32 images or two int64 sums
-            uint32_t wv[4];
-            if (f32) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) wv[e] = __float_as_uint(__ll2float_rn(value(c0 + 4 * q + e)) * f32_scale);
-            } else {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const long long v = value(c0 + 2 * q + e);
-                    wv[2 * e] = (uint32_t)(unsigned long long)v;
-                    wv[2 * e + 1] = (uint32_t)((unsigned long long)v >> 32);
-                }
-            }
-            *reinterpret_cast<uint4*>(wbuf + lane * 64 + 16 * (q ^ ((lane >> 1) & 3))) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-            const int r = (lane >> 2) + 8 * it, pc = lane & 3;
-            const long long mr = __shfl_sync(0xffffffffu, m, r);
-            const uint4 v = *reinterpret_cast<const uint4*>(wbuf + r * 64 + 16 * (pc ^ ((r >> 1) & 3)));
-            const int kk = k0 + c0 + pc * (per / 4);
-            if (mr >= 0 && kk < K) *reinterpret_cast<uint4*>(y + (mr * K + kk) * esz) = v;
-        }
-        __syncwarp();
-    }
-}
-
 // 32 one-plane codes per lane (row m, channels k0 ..) through a 2 KB shared-memory slice of the warp: each
 // lane puts its row's 64 bytes there (16-byte pieces rotated against bank conflicts), then every store
 // instruction writes whole 64-byte row segments of eight rows.  One-plane codes have K % 8 == 0, so a
@@ -728,6 +656,170 @@ __device__ __forceinline__ uint32_t pack_codes_f16(int c0, int c1) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+// Final epilogue of 32 consecutive output channels k0.. of row m, every output that the staged tiles of one-plane codes do
+// not carry (two-plane codes, int64 sums, fp32 images, codes of packed-weight layers): bias alignment, Scale layer, ReLU,
+// FxP-QLayer.  All 32 lanes take part; rows with m < 0 (outside the output) store nothing.  wbuf: epi_buf_bytes<ACC>() of
+// shared memory of the warp, or null.
+//   codes: 16-byte pieces of eight codes per plane (K % 8 == 0);
+//   fp32 (K % 4 == 0) and int64 (K % 2 == 0) with wbuf: every round each lane puts 16 of its row's sums there (16-byte
+//     pieces rotated against bank conflicts), then takes four channels in four rows, four lanes side by side, so that the
+//     warp writes whole row segments rather than 32 rows at one value per lane;
+//   else one value per store.
+// Lane j holds the constants of channel k0 + j, aligned: one load serves the chunk, and shuffles hand them out.  (Loading
+// them per value, one after the other, the 9- to 16-bit codes of a small layer took 10 to 20 us more, and those of 4 x 98 x
+// 98 x 208 outputs 376 us; 172 with one code per store in unrolled code, 66 so.)
+// It is a call, its values passed in local memory: inlined, it made the 128-column kernels spill 1.2 KB around every path,
+// the codes of several groups among them.  It runs in short loops: unrolled over the 32 channels, the int64 logits of a
+// 512 -> 1000 layer, one tile per CTA and each instruction run once, took 25 us, most of it for fetching code and
+// re-reading parameters; 13 us so.
+template <typename ACC>
+__host__ __device__ constexpr int epi_buf_bytes() {
+    return 32 * 16 * (int)sizeof(ACC);
+}
+// a is a copy of what it needs: read through a reference, the kernel's parameters cost a trip to memory each.
+struct EpiBlock {
+    void* y;
+    const int32_t *bias, *scale, *shift;
+    long long M;
+    int K, out_mode, py;
+    float f32_scale;
+    Epi64 e;
+};
+__device__ __forceinline__ EpiBlock make_epi_block(const ConvArgs& a) {
+    return EpiBlock{a.y, a.bias, a.scale, a.shift, a.M, a.K, a.out_mode, a.py, a.f32_scale, make_epi64(a)};
+}
+template <typename ACC, bool SC>
+__device__ __noinline__ void epilogue_block32(const EpiBlock a, long long m, int k0, const ACC (&acc)[32], unsigned char* wbuf,
+                                              int lane) {
+    if (!__any_sync(0xffffffffu, m >= 0)) return;
+    const int mode = a.out_mode, K = a.K;
+    const long long M = a.M;
+    const Epi64& e = a.e;
+    const long long bl = (long long)(e.has_bias && k0 + lane < K ? __ldg(a.bias + k0 + lane) : 0) << e.dl;
+    int32_t ms = 0;
+    long long hl = 0;
+    if constexpr (SC) {
+        ms = k0 + lane < K ? __ldg(a.scale + k0 + lane) : 0;
+        hl = (long long)(k0 + lane < K ? __ldg(a.shift + k0 + lane) : 0) << e.dl2;
+    }
+    auto form = [&](long long v, long long b, int32_t s, long long h) -> long long {
+        v = (v << e.dr) + b;
+        if constexpr (SC) v = ((v * (long long)s) << e.dr2) + h;
+        return max(v, e.floor);
+    };
+    auto value = [&](int j) -> long long {  // of the lane's own row
+        return form((long long)acc[j], __shfl_sync(0xffffffffu, bl, j), SC ? __shfl_sync(0xffffffffu, ms, j) : 0,
+                    SC ? __shfl_sync(0xffffffffu, hl, j) : 0ll);
+    };
+    if (mode == FXPQ_OUT_CODES) {
+        const int py = a.py;
+        const int left = min(-e.sh, 31);  // sh <= 0: past 2^17, or with 31 bits to the left, every value is clipped
+        __half* const y = static_cast<__half*>(a.y) + m * K;
+#pragma unroll 1
+        for (int c0 = 0; c0 < 32 && k0 + c0 < K; c0 += 8) {
+            int c[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const long long v = value(c0 + j);
+                const long long q = e.ok ? (v + e.hm1 + ((v >> e.sh) & 1)) >> e.sh : min(max(v, -(1ll << 17)), 1ll << 17) << left;
+                c[j] = (int)min(max(q, (long long)e.lo), (long long)e.hi);
+            }
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                hi[j] = py == 2 ? pack_codes_f16(c[2 * j] >> 8, c[2 * j + 1] >> 8) : pack_codes_f16(c[2 * j], c[2 * j + 1]);
+                lo[j] = pack_codes_f16(c[2 * j] & 255, c[2 * j + 1] & 255);
+            }
+            if (m >= 0) {
+                *reinterpret_cast<uint4*>(y + k0 + c0) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                if (py == 2) *reinterpret_cast<uint4*>(y + M * K + k0 + c0) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            }
+        }
+        return;
+    }
+    const bool f32 = mode == FXPQ_OUT_F32;
+    const float f32_scale = a.f32_scale;
+    float* const yf = static_cast<float*>(a.y);
+    long long* const yl = static_cast<long long*>(a.y);
+    if (!wbuf || K % (f32 ? 4 : 2) != 0) {
+#pragma unroll 1
+        for (int c0 = 0; c0 < 32 && k0 + c0 < K; c0 += 8) {
+            long long v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = value(c0 + j);
+            if (m >= 0) {
+                const long long o = m * K + k0 + c0;
+                const int n = min(K - k0 - c0, 8);
+                if (f32) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (j < n) yf[o + j] = __ll2float_rn(v[j]) * f32_scale;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (j < n) yl[o + j] = v[j];
+                }
+            }
+            __syncwarp();
+        }
+        return;
+    }
+    // a row's 16 sums take U pieces of 16 bytes, piece u at u ^ swz(row)
+    constexpr int U = (int)sizeof(ACC), ROW = 16 * U;
+    auto swz = [](int row) { return U == 8 ? row & 7 : (row >> 1) & 3; };
+    const int pc = lane & 3;
+#pragma unroll 1
+    for (int c0 = 0; c0 < 32 && k0 + c0 < K; c0 += 16) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            uint4 w;
+            if constexpr (U == 4) {
+                w = make_uint4((uint32_t)acc[c0 + 4 * u], (uint32_t)acc[c0 + 4 * u + 1], (uint32_t)acc[c0 + 4 * u + 2],
+                               (uint32_t)acc[c0 + 4 * u + 3]);
+            } else {
+                const unsigned long long w0 = (unsigned long long)acc[c0 + 2 * u], w1 = (unsigned long long)acc[c0 + 2 * u + 1];
+                w = make_uint4((uint32_t)w0, (uint32_t)(w0 >> 32), (uint32_t)w1, (uint32_t)(w1 >> 32));
+            }
+            *reinterpret_cast<uint4*>(wbuf + lane * ROW + 16 * (u ^ swz(lane))) = w;
+        }
+        __syncwarp();
+        const int kk = k0 + c0 + 4 * pc;
+        long long bv[4], hv[4];
+        int32_t sv[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            bv[i] = __shfl_sync(0xffffffffu, bl, c0 + 4 * pc + i);
+            sv[i] = SC ? __shfl_sync(0xffffffffu, ms, c0 + 4 * pc + i) : 0;
+            hv[i] = SC ? __shfl_sync(0xffffffffu, hl, c0 + 4 * pc + i) : 0ll;
+        }
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const int r = (lane >> 2) + 8 * it;
+            const long long mr = __shfl_sync(0xffffffffu, m, r);
+            ACC raw[4];
+#pragma unroll
+            for (int h = 0; h < U / 4; ++h)
+                *reinterpret_cast<uint4*>(raw + 4 * h / (U / 4)) =
+                    *reinterpret_cast<const uint4*>(wbuf + r * ROW + 16 * ((U / 4 * pc + h) ^ swz(r)));
+            long long v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = form((long long)raw[i], bv[i], sv[i], hv[i]);
+            if (mr >= 0 && kk < K) {
+                if (f32) {
+                    *reinterpret_cast<float4*>(yf + mr * K + kk) =
+                        make_float4(__ll2float_rn(v[0]) * f32_scale, __ll2float_rn(v[1]) * f32_scale,
+                                    __ll2float_rn(v[2]) * f32_scale, __ll2float_rn(v[3]) * f32_scale);
+                } else {
+                    longlong2* const d = reinterpret_cast<longlong2*>(yl + mr * K + kk);
+                    d[0] = make_longlong2(v[0], v[1]);
+                    if (kk + 2 < K) d[1] = make_longlong2(v[2], v[3]);
+                }
+            }
+        }
+        __syncwarp();
+    }
+}
+
 // One code of the two-limb window epilogue in exact 32-bit arithmetic (see the generic window epilogue): bt the
 // aligned bias (high and low 16 bits), m = sh - 16, half = 2^(m-1), mmask = 2^m - 1.
 __device__ __forceinline__ int win_code(uint32_t fhh, uint32_t fhl, uint32_t flh, uint32_t fll, int2 bt, int m, int half,
@@ -857,7 +949,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     static_assert(!FE || (sizeof(ACC) == 4 && !SPLIT && !PK && !WIN && !W64), "fp32 epilogue: plain int32 instances");
     constexpr bool WEPI = WIN || W64;  // the window instances' epilogue (16 warps, two staging tiles)
     constexpr int EPI_WARPS = WEPI ? TC_WIN_EPI_WARPS : tc_epi_warps(BN);
-    static_assert(tc_out_bytes(BN, PK) >= EPI_WARPS * 2048 || WEPI, "the staged fp32 / int64 epilogue takes 2 KB per warp");
+    static_assert(tc_out_bytes(BN, PK) >= EPI_WARPS * (int)(32 * 16 * sizeof(ACC)) || WEPI, "epilogue_block32's buffers fit");
     constexpr int MMA_WARP = 4 + EPI_WARPS;
     constexpr bool STORE_WARP = BN <= 128;  // warp MMA_WARP + 1 stores the staged tiles
     constexpr int STG_BYTES = BN * TC_BM * 2;  // one staging tile
@@ -1876,17 +1968,12 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                             *reinterpret_cast<uint4*>(half_buf + row * 128 + ((chunk ^ (row & 7)) << 4)) =
                                 make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
                         }
-                    } else if (!PK && (a.out_mode == FXPQ_OUT_F32 ? a.K % 4 == 0 : (a.out_mode == FXPQ_OUT_ACC64 && a.K % 2 == 0))) {
-                        // fp32 / int64 outputs through the warp's 2 KiB of the (unused) staging tile
+                    } else {
+                        // everything else, through the warp's 2 KiB of the (unused) staging tile
                         ACC v[32];
 #pragma unroll
                         for (int j = 0; j < 32; ++j) v[j] = acc[j];
-                        epilogue_block32_staged<ACC, SC>(a, m, k0, v, sO + (warp - 4) * 2048, lane);
-                    } else if (m >= 0) {
-                        ACC v[32];
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) v[j] = acc[j];
-                        epilogue_block32<ACC, SC>(a, m, k0, v);
+                        epilogue_block32<ACC, SC>(make_epi_block(a), m, k0, v, PK ? nullptr : sO + (warp - 4) * epi_buf_bytes<ACC>(), lane);
                     }
                     }
                 }

@@ -763,6 +763,24 @@ def test_patch_shapes_parity(F, N, H, C, K, R, st, pad, mode):
     assert s == ws and np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("sh", [37, 1, 0, -1, -9, -30, -31, -35])  # the FxP-QLayer's shift: right, none, left, left by 31 and more
+@pytest.mark.parametrize("N,H,C,K,R,kx,scale", [(2, 9, 16, 72, 3, 8, 0), (3, 5, 24, 8, 1, 16, 0), (2, 7, 64, 264, 3, 7, 1), (1, 6, 16, 40, 3, 16, 1)])
+@pytest.mark.parametrize("ky,Sy", [(16, 1), (12, 0)])
+def test_two_plane_codes(F, sh, N, H, C, K, R, kx, scale, ky, Sy):
+    """Codes of more than 8 bits over the whole range of shifts, sums next to zero and past every clip level among them."""
+    rng = np.random.default_rng(abs(sh) + K)
+    fx, fw, fb, fs, fh = F.fmt(kx, 1, 2), F.fmt(7, 1, 3), F.fmt(16, 1, 4), F.fmt(8, 1, 0), F.fmt(16, 1, 3)
+    s0 = 5  # the accumulator's scale, whatever the bias (coarser) and the Scale layer's shift (coarser) are
+    fy = F.fmt(ky, Sy, s0 - sh)
+    x, w, b = rand_codes(rng, (N, H, H, C), kx, 1), rng.integers(-2, 3, size=(K, R, R, C)), rng.integers(-40, 40, size=K)
+    x[0, :2] = 0
+    w[1], b[1], b[2], w[2] = 0, 0, 1, 0
+    sc = (rng.integers(-3, 4, size=K), fs, rng.integers(-99, 99, size=K), fh) if scale else None
+    got, s = run_conv(F, x, fx, w, fw, b, fb, 1, R // 2, False, 0, fy, C, 0, scale=sc)
+    want, ws = oracle_conv(x, fx, w, fw, b, fb, 1, R // 2, False, 0, fy, scale=sc)
+    assert s == ws == s0 and np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("N,H,C,K,R,st,l1", [(2, 9, 64, 64, 3, 1, 1), (3, 12, 64, 136, 3, 2, 1), (2, 8, 128, 264, 3, 1, 1),
                                              (1, 7, 512, 72, 3, 1, 1), (1, 7, 256, 64, 7, 1, 0)])  # the last two split
 @pytest.mark.parametrize("mode,relu,ty", [(0, True, (8, 0, 2)), (0, False, (5, 1, 1)), (2, True, None), (2, False, None), (1, False, None)])
