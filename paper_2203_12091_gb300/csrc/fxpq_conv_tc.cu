@@ -450,6 +450,10 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         launched = true;
         return FXPQ_OK;
     }
+    // the fp32 epilogue, for a layer of one exact group that is not split
+    const bool fp32_epi = ((a.vf && P.fast_store) || (a.vi && a.K % 4 == 0) ||
+                           (a.vs && (P.fast_store || (a.out_mode == FXPQ_OUT_F32 && a.K % 4 == 0)))) &&
+                          P.n_groups == 1 && P.g[0].shift == 0 && P.patch != 3 && !P.pk && !acc64 && !conv_path_is("tc_iepi");
     // Split reduction for layers whose tiles cannot occupy the SMs (FC layers, small batches) and whose
     // reduction is long: ks units share every tile's k-blocks (share s of every exact group), and their
     // exact integer sums meet in the workspace.
@@ -470,12 +474,16 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         // groups (two-limb layers): each share takes whole groups
         int ks_sub = std::min(cap, std::min(min_len / 4, TC_MAX_GROUPS / ng));
         int ks_whole = std::min(cap, ng);
-        // the second kernel costs about 3 us, a k-block of a tile that has its SM to itself 0.15 us (1 image,
-        // ResNet-18: 21 us for 72 k-blocks, 11 for 1): the split has to shorten the chain by 24
+        // The second kernel costs about 3 us, a k-block of a tile that has its SM to itself 0.15 us (0.33 gathered): a
+        // layer with the fp32 epilogue is split if that shortens the chain by 12.  Other epilogues run once per tile in
+        // one kernel take 4 to 8 us, and the second kernel spreads them: always split (334 small layers: 12 is 0.5% off
+        // the better of both on average, 24 for all 16%; 9 k-blocks to 16-bit codes, 825 x 240 outputs, 14.4 us whole,
+        // 8.5 split; 16-bit, 8 k-blocks, 20 x 120 int64 sums 15.4 / 7.1)
         int total = 0;
         for (int gi = 0; gi < ng; ++gi) total += P.g[gi].kb1 - P.g[gi].kb0;
-        if (total - total / std::max(ks_sub, 1) < 24) ks_sub = 1;
-        if (total - total / std::max(ks_whole, 1) < 24) ks_whole = 1;
+        const int saves = fp32_epi ? 12 : 1;
+        if (total - total / std::max(ks_sub, 1) < saves) ks_sub = 1;
+        if (total - total / std::max(ks_whole, 1) < saves) ks_whole = 1;
         if (ks_sub >= 2 && ks_sub >= ks_whole) {
             TcGroup g0[TC_MAX_GROUPS];
             for (int gi = 0; gi < ng; ++gi) g0[gi] = P.g[gi];
@@ -501,9 +509,7 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         }
     }
     P.n_units = P.n_tiles * P.ksplit;
-    P.fepi = ((a.vf && P.fast_store) || (a.vi && a.K % 4 == 0) ||
-              (a.vs && (P.fast_store || (a.out_mode == FXPQ_OUT_F32 && a.K % 4 == 0)))) && P.n_groups == 1 && P.g[0].shift == 0 && P.patch != 3 &&
-             P.ksplit == 1 && !P.pk && !acc64 && !conv_path_is("tc_iepi");
+    P.fepi = fp32_epi && P.ksplit == 1;
     {
         std::lock_guard<std::mutex> lk(g_tc_mu);
         if (!g_tc_attr_set) {
