@@ -214,6 +214,8 @@ S2dPlan s2d_plan(const fxpq_conv_desc& d) {
     p.H2 = (int)P + p.R2 - 1;
     p.W2 = (int)Q + p.S2 - 1;
     p.flat = (p.S2 * p.C2 + 63) / 64 < p.S2 * ((p.C2 + 63) / 64);
+    p.kb = p.flat ? p.R2 * ((p.S2 * p.C2 + 63) / 64) : p.R2 * p.S2 * ((p.C2 + 63) / 64);
+    p.kb_own = (d.R * d.S * 8 + 63) / 64;
     p.x_bytes = ((size_t)d.N * p.H2 * p.W2 * p.C2 * 2 * planes_of(d.fmt_x) + 255) / 256 * 256;
     p.w_bytes = ((size_t)d.K * p.R2 * p.S2 * p.C2 * 2 * planes_of(d.fmt_w) + 255) / 256 * 256;
     p.ok = (long long)p.H2 * p.W2 < (1LL << 31) && (long long)d.N * p.H2 * p.W2 * 2 < (1LL << 31) * 128;
@@ -419,10 +421,12 @@ fxpq_status launch_conv(const ConvArgs& a, const fxpq_conv_desc& d, bool need64,
         // 7 x 7 / 2 of 128 images, 455 -> 216 us with its copy; AlexNet conv1, 11 x 11 / 4 of 256, 431 -> 336)
         const S2dPlan p = s2d_plan(d);
         // Rewriting the input is a launch of its own: worth it where the gathered form's row tiles take more than one
-        // round over the SMs (7 x 7 / 2, 98 tiles: 14.0 us rewritten, 11.5 gathered; 196 tiles: 15.0 / 17.3);
-        // a chosen alternative takes this form at any size
-        const bool rounds = (M + 127) / 128 * ((a.K + 63) / 64) > num_sms() || path;
-        if (p.ok && rounds && ws && ws_bytes >= p.x_bytes + p.w_bytes && s2d) {
+        // round over the SMs (7 x 7 / 2, 98 tiles: 14.0 us rewritten, 11.5 gathered; 196 tiles: 15.0 / 17.3) and, for
+        // codes that are there already, where it saves a quarter of at least three k-blocks (300 layers: with 7 x 7 / 2
+        // 0.69 times as long on average, 3 x 3 / 2 0.96 to 1.04; 8 channels, 7 x 7 / 4, 185 tiles 24.1 us rewritten,
+        // 13.7 gathered); a chosen alternative takes this form at any size
+        const bool worth = (M + 127) / 128 * ((a.K + 63) / 64) > num_sms() && (images || (4 * p.kb <= 3 * p.kb_own && p.kb_own >= 3));
+        if (p.ok && (worth || path) && ws && ws_bytes >= p.x_bytes + p.w_bytes && s2d) {
             char* base = static_cast<char*>(ws);
             const bool direct = images && launch_quantize_s2d(images, a.N, a.H, a.W, d.fmt_x, p, a.pad, base, st);
             fxpq_status s = direct ? after_launch("quantize_s2d") : codes();

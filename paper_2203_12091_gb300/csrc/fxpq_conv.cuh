@@ -181,6 +181,7 @@ size_t conv_split_ws_bytes(long long M, int K);
 struct S2dPlan {
     bool ok, flat;
     int st, C, R2, S2, C2, H2, W2;
+    int kb, kb_own;           // k-blocks of the rewritten reduction and of the layer's own
     size_t x_bytes, w_bytes;  // 256-byte multiples
 };
 S2dPlan s2d_plan(const fxpq_conv_desc& d);

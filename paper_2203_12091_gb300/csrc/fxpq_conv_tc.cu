@@ -135,22 +135,37 @@ bool choose_form(const ConvArgs& a, const fxpq_conv_desc& d, const char* path, i
     // 588 row tiles, us as patches and gathered): 32 channels, 1.8 times as many, 15.8 / 22.4 and 31.5 / 35.2; 16
     // channels, 3 times, 25.3 / 19.4 and 37.3 / 29.4.  Pixels that are not whole 32-byte sectors cost their boxes
     // double: 120 channels, 1.06 times, 37.6 / 46.2; 136 channels, 1.35 times, 55.7 / 49.3; 24 channels 63.9 / 35.2.
-    // Where each tile has an SM to itself the latency of a k-block decides instead, and patches win longer (24
-    // channels, 21 tiles: 8.9 / 9.9).  Two-limb reductions drain a group per limb pair, which hides less of the
+    // Where each tile has an SM to itself, its split shares fill the others: a one-limb layer's patches cost 0.30 us per
+    // k-block of every SM (0.36 off 32-byte sectors), gathered rows 0.5 and 1 us at the start (400 layers: 0.3 and 0.7%
+    // off the better of both; 40 channels, 11 x 11, 45 tiles 39.6 / 25.6; 24 channels, 7 x 5, one tile 6.1 / 10.4).
+    // Two-limb reductions drain a group per limb pair, which hides less of the
     // patches' k-blocks (32 channels, 1.8 times: 68 / 62; 80 channels, 1.5 times: 99.5 / 103; 16-bit 24 channels, 5 x 5,
     // 2.5 times: 272 / 103).
-    // Eight-channel patches take the gathered form's k-blocks, a box per tap: one-limb layers 1.1 to 1.4 times faster,
-    // two-limb ones only with few taps (128 channels, 3 x 3, 1568 tiles: 134 / 140; 64 channels, 7 x 7: 132 / 114).
+    // Strided two-limb layers of one column tile, whose boxes are read once, are gathered (K = 56, 13 images, 3 x 3 / 2 on
+    // 75 x 75: 64 channels 34.4 / 26.7, 256 channels 83.7 / 72.7; K = 192: 64.9 / 67.8 and 163 / 206).
+    // Eight-channel patches take the gathered form's k-blocks, a box per tap: one-limb layers 1.1 to 1.4 times faster with
+    // up to 40 taps (11 x 11: 17 maps of 46 x 46 33.3 / 20.7; 23 of 28 x 28 23.8 / 12.6), two-limb ones only with few
+    // (128 channels, 3 x 3, 1568 tiles: 134 / 140; 64 channels, 7 x 7: 132 / 114) and up to 256 output channels (344
+    // channels, 3 x 3, 3198 tiles: 235 / 207).
     // Overlapping pixels (the flat space-to-depth form) are read by patches whatever they cost: a tensor map has the
     // strides that the gather does not look at.
     const bool overlap = a.x_sw != a.Cp;
     const bool two_limb = a.px * a.pw > 1, lone = row_tiles_est * ((a.K + 63) / 64) <= sms;
     const bool any_patch = conv_path_is("tc") || conv_path_is("tc_bn256");
-    const double most = any_patch ? 4.0 : a.Cp % 16 ? (lone && !two_limb ? 2.3 : 1.15) : two_limb ? 1.55 : lone ? 4.0 : 2.0;
+    const double kb_patch = (double)ps.tiles * a.R * a.S * kbt, kb_rows = (double)row_tiles_est * kb_flat;
+    bool worth;
+    if (narrow)
+        worth = any_patch || (two_limb ? !lone && a.R * a.S <= 16 && a.K <= 256 : a.R * a.S <= 40);
+    else if (any_patch)
+        worth = kb_patch <= 4.0 * kb_rows;
+    else if (two_limb)
+        worth = (lone || a.stride == 1 || a.K > 64) && kb_patch <= (a.Cp % 16 ? 1.15 : 1.55) * kb_rows;
+    else if (lone)
+        worth = ((a.Cp % 16 ? 0.36 : 0.3) * kb_patch - 0.5 * kb_rows) * ((a.K + 63) / 64) <= 1.0 * sms;
+    else
+        worth = kb_patch <= (a.Cp % 16 ? 1.15 : 2.0) * kb_rows;
     bool& use_patch = f.use_patch;
-    use_patch =
-        ps.TW > 0 && (overlap || conv_path_is("tc_patch") || (narrow ? any_patch || !two_limb || (!lone && a.R * a.S <= 16)
-                                                          : (double)ps.tiles * a.R * a.S * kbt <= most * (double)row_tiles_est * kb_flat));
+    use_patch = ps.TW > 0 && (overlap || conv_path_is("tc_patch") || worth);
     if (overlap && !use_patch && !rows_geom) return false;
     if (use_patch && !narrow && !plan_tc(a, d, P, acc64, a.R * a.S * kbt)) {  // too many groups: gathered, if that has fewer
         if (overlap) return false;

@@ -730,7 +730,8 @@ def test_row_parts_parity(F, M, C, K, mode, kx):
                                              (26, 30, 24, 64, 3, 1, 7), (26, 30, 120, 64, 3, 1, 7), (2, 30, 32, 64, 3, 1, 16),
                                              (2, 30, 80, 64, 3, 1, 16), (2, 30, 3, 64, 5, 1, 16), (26, 30, 3, 72, 3, 1, 16),
                                              (2, 30, 3, 64, 3, 1, 7), (2, 30, 3, 64, 3, 2, 7), (90, 30, 3, 64, 3, 2, 7),
-                                             (2, 20, 48, 64, 10, 1, 16)])
+                                             (2, 20, 48, 64, 10, 1, 16), (90, 30, 3, 64, 7, 2, 7), (90, 30, 3, 64, 7, 2, 16),
+                                             (46, 23, 8, 64, 11, 1, 7), (46, 23, 64, 56, 3, 2, 16), (12, 40, 3, 264, 3, 1, 16)])
 def test_chosen_form_parity(F, N, H, C, K, R, st, kx):
     """The form that a layer takes by itself, patches, gathered rows or space-to-depth, on both sides of its lines."""
     if os.environ.get("FXPQ_CONV_PATH") != "tc":
