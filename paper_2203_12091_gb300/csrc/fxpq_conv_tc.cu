@@ -234,7 +234,8 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
     TcParams P;
     TcForm f;
     const int sms = num_sms();
-    if (!choose_form(a, d, path, sms, ws != nullptr, P, f)) return FXPQ_OK;
+    const bool two_shares = ws && ws_bytes / 2 >= (size_t)a.M * a.K * sizeof(int);  // room for a split
+    if (!choose_form(a, d, path, sms, two_shares, P, f)) return FXPQ_OK;
     const bool rows_geom = f.rows_geom, narrow = f.narrow, use_patch = f.use_patch, two_limb = a.px * a.pw > 1;
     const PatchShape& ps = f.ps;
     bool acc64 = f.acc64;

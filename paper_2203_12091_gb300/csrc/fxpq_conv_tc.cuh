@@ -2209,7 +2209,7 @@ struct TcForm {
 }  // namespace tc
 
 // The host's choices for a layer on `sms` SMs: P's exact groups (and P.kbt) and f.  path: FXPQ_CONV_PATH or null; has_ws:
-// there is scratch.  False: the tensor-core path cannot keep the sums exact.  Touches no device.
+// there is scratch for two shares of a split.  False: the tensor-core path cannot keep the sums exact.  Touches no device.
 bool choose_form(const ConvArgs& a, const fxpq_conv_desc& d, const char* path, int sms, bool has_ws, tc::TcParams& P,
                  tc::TcForm& f);
 

@@ -171,9 +171,9 @@ extern "C" fxpq_status fxpq_net_forward(const fxpq_net* h_net, const float* d_im
     char* base = static_cast<char*>(d_ws);
     auto ptr = [&](int slot) { return static_cast<void*>(base + slots[slot].offset); };
     if (batch == 0) return FXPQ_OK;
-    // the convs' scratch follows the slots when the caller provided it
-    const size_t cws = net_conv_ws(h_net, slots, batch);
-    void* conv_ws = (cws && ws_bytes >= total + cws) ? static_cast<void*>(base + total) : nullptr;
+    // the convs' scratch is what the caller provided behind the slots: a conv takes the forms that it holds
+    const size_t cws = std::min(net_conv_ws(h_net, slots, batch), ws_bytes - total);
+    void* conv_ws = cws ? static_cast<void*>(base + total) : nullptr;
 
     // Images that only the first layer reads, a convolution, are quantized as it wants them
     int readers = 0;
@@ -217,7 +217,7 @@ extern "C" fxpq_status fxpq_net_forward(const fxpq_net* h_net, const float* d_im
                 d.d_wpacked = o.d_wpacked;
                 int32_t scale = 0;
                 st = fxpq::conv_fwd(d, by_conv && i == 0 ? d_images_nchw : nullptr, ptr(o.src0), o.d_w, o.d_bias,
-                                    last ? (void*)d_logits : ptr(o.dst), &scale, conv_ws, conv_ws ? cws : 0, stream);
+                                    last ? (void*)d_logits : ptr(o.dst), &scale, conv_ws, cws, stream);
                 if (last && h_logits_scale) *h_logits_scale = scale;
                 break;
             }

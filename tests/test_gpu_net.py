@@ -100,6 +100,37 @@ def test_first_layer_from_images(NET, R, st, pad, hw, k, monkeypatch):
         assert F.fxpq_get_device_status() == 3
 
 
+def test_smaller_workspaces(NET):
+    """Scratch that holds a split reduction's shares but not the larger copies of the first layer still splits the FC layer;
+    with none at all the logits are the same."""
+    from paper_2203_12091_gb300 import fxpq as F
+    L = [{"type": "conv", "name": "c1", "C": 3, "K": 64, "R": 7, "stride": 2, "pad": 3, "relu": True, "src": None},
+         {"type": "maxpool", "name": "p1", "k": 4, "stride": 4, "pad": 0},
+         {"type": "conv", "name": "fc", "C": 64, "K": 24, "R": 12, "stride": 1, "pad": 0, "relu": False, "src": "p1"}]
+    plan = {"input": 8, "c1": {"w": 8, "b": 16, "a": 8}, "fc": {"w": 8, "b": 16}}
+    rng = np.random.default_rng(4)
+    W = {l["name"]: (rng.standard_normal((l["K"], l["R"], l["R"], l["C"])).astype(np.float32) * 0.05,
+                     rng.standard_normal(l["K"]).astype(np.float32) * 0.01) for l in L if l["type"] == "conv"}
+    N = 12  # 96 x 96 images: 216 row tiles, more than one round of the SMs
+    imgs = torch.from_numpy(synth.images(N, 2, hw=96)).cuda()
+    q = NET.build_qnet(L, W, imgs[:4], plan)
+    f = q.fmts
+    need = [F.fxpq_conv_workspace(F.conv_desc(N, *g, False, F.OUT_ACC64, fx, f[nm]["w"], f[nm]["b"], None))
+            for nm, g, fx in (("c1", (96, 96, 3, 8, 64, 7, 7, 2, 3), f["input"]["a"]), ("fc", (12, 12, 64, 64, 24, 12, 12, 1, 0), f["c1"]["a"]))]
+    full = q.workspace_bytes(N)
+    slots = full - 256 - max((n + 255) // 256 * 256 for n in need)
+    assert need[1] < need[0]
+    out, launches = [], []
+    for nbytes in (full, slots + need[1], slots):
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        assert ws.data_ptr() % 256 == 0
+        n0 = F.fxpq_launch_count()
+        out.append(q.forward(imgs, ws=ws)[0].cpu())
+        launches.append(F.fxpq_launch_count() - n0)
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+    assert launches[1] == launches[2] + 1, launches  # the second kernel of the split
+
+
 def test_layer_dicts_without_channel_counts(NET):
     """A layer's input channels come from its weights: a trace of layers that do not state them equals one of layers that do."""
     L, plan = _tiny()
