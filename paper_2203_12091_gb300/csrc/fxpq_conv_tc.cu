@@ -51,18 +51,21 @@ static PatchShape patch_shape(const ConvArgs& a, int max_tn) {
     PatchShape s;
     const long long ideal = (a.M + TC_BM - 1) / TC_BM;
     const int span = (256 - 1) / a.stride + 1;  // a TMA box spans at most 256 input positions
-    for (int i = 1, tw = 0; i <= a.Q; ++i) {
-        const int w = (a.Q + i - 1) / i;
-        if (w == tw || w > TC_BM || w > span) continue;
-        tw = w;
-        for (int j = 1, th = 0; j <= a.P; ++j) {
-            const int h = (a.P + j - 1) / j;
-            if (h == th || (long long)h * tw > TC_BM || h > span) continue;
-            th = h;
+    const int wmax = span < TC_BM ? span : TC_BM;
+    // i columns of patches are ceil(Q / i) wide: from the widest that fits, each distinct width with its fewest columns (rows
+    // likewise).  Shapes whose padded pixels fill more tiles than the best one has are passed over.  About 1 us for 55 x
+    // 55 and 56 x 56 maps, 0.5 for 112 x 112, 3 for 4095 x 4095 (every i and j tried: 3, 1.7 and 870).
+    for (int i = (a.Q + wmax - 1) / wmax, tw; i <= a.Q; i = tw > 1 ? (a.Q + tw - 2) / (tw - 1) : a.Q + 1) {
+        tw = (a.Q + i - 1) / i;
+        const int hmax = TC_BM / tw < span ? TC_BM / tw : span;
+        if (s.TW && (long long)a.N * a.P * i > s.tiles * (TC_BM / tw)) continue;
+        for (int j = (a.P + hmax - 1) / hmax, th; j <= a.P; j = th > 1 ? (a.P + th - 2) / (th - 1) : a.P + 1) {
+            th = (a.P + j - 1) / j;
+            if (s.TW && (long long)a.N * (i * tw) * (j * th) > s.tiles * TC_BM) continue;
             int tn = TC_BM / (th * tw);
             if (tn > a.N) tn = a.N;
             if (tn > max_tn) tn = max_tn;
-            const long long t = (long long)((a.N + tn - 1) / tn) * ((a.P + th - 1) / th) * ((a.Q + tw - 1) / tw);
+            const long long t = (long long)((a.N + tn - 1) / tn) * j * i;
             if (s.TW == 0 || t < s.tiles || (t == s.tiles && tn < s.TN)) s.TW = tw, s.TH = th, s.TN = tn, s.tiles = t;
             if (s.tiles == ideal && s.TN == 1) return s;
         }

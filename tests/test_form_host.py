@@ -75,3 +75,31 @@ def test_patches_give_way_where_their_groups_are_too_many():
     layers = [dict(N=4, H=30, C=48, K=64, R=10, pad=5, xb=16, wb=16), dict(N=2, H=14, C=664, K=64, R=7, pad=3, wb=8)]
     for c, r in zip(layers, choose(layers)):
         assert r["planned"] and not r["use_patch"] and r["n_groups"] <= 64, c
+
+
+def _patch_shape(N, P, Q, stride):
+    """Every way of cutting a map into equal counts of columns and rows, in the library's order: widest first."""
+    best, ideal, span = None, (N * P * Q + 127) // 128, 255 // stride + 1
+    for w in sorted({-(-Q // i) for i in range(1, Q + 1)}, reverse=True):
+        for h in sorted({-(-P // j) for j in range(1, P + 1)}, reverse=True):
+            if w > min(128, span) or h * w > 128 or h > span:
+                continue
+            tn = min(128 // (h * w), N)
+            t = -(-N // tn) * -(-P // h) * -(-Q // w)
+            if best is None or t < best[3] or (t == best[3] and tn < best[2]):
+                best = (w, h, tn, t)
+            if best[3] == ideal and best[2] == 1:
+                return best
+    return best
+
+
+def test_patch_shapes_are_the_best_of_all():
+    """The search that skips equal and hopeless shapes finds what a full one finds."""
+    import random
+    rng = random.Random(2)
+    sizes = [(1, 1, 1, 1), (7, 1, 300, 1), (5, 300, 1, 1), (128, 7, 7, 1), (64, 56, 55, 1), (1, 1023, 511, 1), (2, 224, 222, 1), (1, 20, 4095, 8)]
+    sizes += [(rng.randint(1, 200), rng.randint(1, 120), rng.randint(1, 120), rng.choice([1, 1, 2, 3, 8])) for _ in range(300)]
+    layers = [dict(N=N, H=(P - 1) * st + 3, W=(Q - 1) * st + 3, C=64, K=64, R=3, stride=st) for N, P, Q, st in sizes]
+    for (N, P, Q, st), r in zip(sizes, choose(layers)):
+        if not r["rows_geom"]:
+            assert (r["TW"], r["TH"], r["TN"], r["tiles"]) == _patch_shape(N, P, Q, st), (N, P, Q, st)
