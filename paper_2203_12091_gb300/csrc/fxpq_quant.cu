@@ -202,8 +202,8 @@ __device__ __forceinline__ uint32_t limb_lo_f16x2(uint32_t b0, uint32_t b1) {
 
 // The same for three-channel images padded to 8: four pixels per thread, 256 apart, so that twelve loads are
 // in flight (one pixel per thread and iteration waited on three), the position in the image found by one
-// division per block tile, codes rounded by one fp32 addition (see f32_codes_f16x2 and the limbs above).  HBM-bound: 12 bytes read, 16 per plane
-// written.  224 x 224, one plane: 128 images 107 -> 33 us, two planes 117 -> 50 us.
+// division per block tile and one per image crossed, codes rounded by one fp32 addition (see f32_codes_f16x2 and the limbs
+// above).  HBM-bound: 12 bytes read, 16 per plane written.  224 x 224, one plane: 128 images 107 -> 33 us, two planes 117 -> 50 us.
 constexpr int QI_PIX = 4;
 template <int PLANES>
 __global__ void __launch_bounds__(256) quantize_images3_kernel(const float* __restrict__ x, unsigned npix, unsigned hw,
@@ -222,9 +222,10 @@ __global__ void __launch_bounds__(256) quantize_images3_kernel(const float* __re
 #pragma unroll
             for (int c = 0; c < 3; ++c) v[j][c] = in ? __ldg(s + (unsigned long long)c * hw) : 0.0f;
             pix += T;
-            while (pix >= hw) {
-                pix -= hw;
-                ++n;
+            if (pix >= hw) {  // (a division, not a loop: images may be of one pixel)
+                const unsigned d = pix / hw;
+                n += d;
+                pix -= d * hw;
             }
         }
 #pragma unroll

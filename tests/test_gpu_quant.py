@@ -399,7 +399,7 @@ def test_pack_unpack_quantize_any_alignment(F, k, S, n, off):
 
 
 @pytest.mark.parametrize("k,S,fl", [(8, 0, 5), (8, 1, 5), (9, 1, 4), (16, 0, 13), (16, 1, 12), (2, 1, 40), (16, 1, -32)])
-@pytest.mark.parametrize("N,hw", [(1, 1), (3, 13), (2, 33), (5, 17)])
+@pytest.mark.parametrize("N,hw", [(1, 1), (3, 13), (2, 33), (5, 17), (1500, 1), (700, 2)])
 def test_quantize_rgb_images(F, k, S, fl, N, hw):
     """Three-channel images: blocks of 1024 pixels that span images and end inside one, every level, ties."""
     x = _adv(k + N, N * 3 * hw * hw)[: N * 3 * hw * hw].reshape(N, 3, hw, hw)
