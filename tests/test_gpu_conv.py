@@ -320,7 +320,8 @@ def test_gemm_entry_point(F):
 
 
 @pytest.mark.parametrize("N,H,C,k,st,pad", [(1, 3, 8, 3, 2, 0), (3, 8, 8, 3, 2, 2), (2, 2, 264, 2, 2, 1), (70000, 2, 8, 2, 2, 0),
-                                            (2, 33, 72, 3, 2, 1), (2, 9, 16, 2, 1, 1), (1, 20, 40, 5, 3, 2)])
+                                            (2, 33, 72, 3, 2, 1), (2, 9, 16, 2, 1, 1), (1, 20, 40, 5, 3, 2),
+                                            (1500, 3, 24, 3, 2, 1), (2001, 5, 8, 5, 3, 2), (1100, 4, 40, 2, 1, 1), (1025, 8, 16, 3, 2, 0)])
 def test_maxpool_windows_parity(F, N, H, C, k, st, pad):
     """Windows with their own instances and others, over the edges, of a single output, and more images than a grid row."""
     if os.environ.get("FXPQ_CONV_PATH") != "tc":
