@@ -820,8 +820,13 @@ __device__ __noinline__ void epilogue_block32(const EpiBlock a, long long m, int
     }
 }
 
-// One code of the two-limb window epilogue in exact 32-bit arithmetic (see the generic window epilogue): bt the
-// aligned bias (high and low 16 bits), m = sh - 16, half = 2^(m-1), mmask = 2^m - 1.
+// One code of the two-limb window epilogue in exact 32-bit arithmetic.  With the limb sums S_hh, S_mid = S_hl + S_lh, S_ll
+// and the aligned bias B' = 2^16 Bh + Bl (0 <= Bl < 2^16; bt = (Bh, Bl)):
+//   v = 2^16 S_hh + 2^8 S_mid + S_ll + B' = 2^16 T + Lo,
+//   L = 2^8 S_mid + S_ll + Bl,  T = S_hh + Bh + (L >> 16),  Lo = L & 0xFFFF
+// (the host keeps |L| and |T| below 2^31).  With sh = 16 + m, floor(v / 2^sh) = T >> m and the remainder is 2^16 (T mod
+// 2^m) + Lo, so round half to even needs T mod 2^m (mmask = 2^m - 1) against half = 2^(m-1), and Lo only to tell a tie
+// (Lo = 0) from above it.  ReLU: v < 0 exactly when T < 0.
 __device__ __forceinline__ int win_code(uint32_t fhh, uint32_t fhl, uint32_t flh, uint32_t fll, int2 bt, int m, int half,
                                         int mmask, int relu, int lo, int hi) {
     const int mid = __float2int_rn(__uint_as_float(fhl)) + __float2int_rn(__uint_as_float(flh));
@@ -1027,7 +1032,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
     // (B' >> 16, B' & 0xFFFF), in the last 512 bytes of the B region (the resident weights stay below)
     int2* wtab = reinterpret_cast<int2*>(sB + TC_STAGES * B_BYTES - 512);
     float* wtabf = reinterpret_cast<float*>(sB + TC_STAGES * B_BYTES - 768);  // B' 2^-sh, the 256 bytes before it
-    if (BN == 64 && sizeof(ACC) == 8 && !SC && P.patch == 3 && (P.w32 || P.wf32) && warp == 1) {
+    if (WIN && P.patch == 3 && (P.w32 || P.wf32) && warp == 1) {
         for (int k = lane; k < 64; k += 32) {
             const long long bb = (a.has_bias && k < a.K) ? ((long long)__ldg(a.bias + k) << (a.delta > 0 ? a.delta : 0)) : 0;
             wtab[k] = make_int2((int)(bb >> 16), (int)(bb & 0xFFFF));
@@ -1559,74 +1564,6 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         continue;
                     }
                     if constexpr (!FE) {
-                    if (BN == 64 && sizeof(ACC) == 8 && !SC && P.patch == 3 && P.w32) {
-                        // window mode, two-limb x and w, 32-bit arithmetic.  With the limb sums S_hh,
-                        // S_mid = S_hl + S_lh, S_ll and the aligned bias B' = 2^16 Bh + Bl (0 <= Bl < 2^16):
-                        //   v = 2^16 S_hh + 2^8 S_mid + S_ll + B' = 2^16 T + Lo,
-                        //   L = 2^8 S_mid + S_ll + Bl,  T = S_hh + Bh + (L >> 16),  Lo = L & 0xFFFF,
-                        // (the host keeps |L| and |T| below 2^31).  With sh = 16 + m, floor(v / 2^sh) =
-                        // T >> m and the remainder is 2^16 (T mod 2^m) + Lo, so round half to even needs
-                        // T mod 2^m against 2^(m-1), and Lo only to tell a tie (Lo = 0) from above it.
-                        // ReLU: v < 0 exactly when T < 0.
-                        const int m = a.sh - 16;
-                        const int half = m > 0 ? 1 << (m - 1) : 0;
-                        const int mmask = (int)((1u << m) - 1u);
-                        const int lo = (int)a.lo, hi = (int)a.hi;
-                        const uint32_t abase = lane_base + buf * (uint32_t)(4 * BN) + cb * 32;
-                        uint32_t w[16];
-#pragma unroll
-                        for (int hf = 0; hf < 2; ++hf) {
-                            uint32_t fhh[16], fhl[16], flh[16], fll[16];
-                            tmem_ld16_nw(abase + 16 * hf, fhh);
-                            tmem_ld16_nw(abase + (uint32_t)BN + 16 * hf, fhl);
-                            tmem_ld16_nw(abase + (uint32_t)(2 * BN) + 16 * hf, flh);
-                            tmem_ld16_nw(abase + (uint32_t)(3 * BN) + 16 * hf, fll);
-                            tmem_wait_ld();
-                            reg_fence(fhh);
-                            reg_fence(fhl);
-                            reg_fence(flh);
-                            reg_fence(fll);
-                            if (hf == 1 && c == CPW - 1) {
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(accempty0 + 8 * buf);
-                            }
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                int c2[2];
-#pragma unroll
-                                for (int h = 0; h < 2; ++h) {
-                                    const int jj = 2 * j + h;
-                                    const int2 bt = wtab[cb * 32 + 16 * hf + jj];
-                                    const int mid = __float2int_rn(__uint_as_float(fhl[jj])) +
-                                                    __float2int_rn(__uint_as_float(flh[jj]));
-                                    const int L = mid * 256 + __float2int_rn(__uint_as_float(fll[jj])) + bt.y;
-                                    const int T = __float2int_rn(__uint_as_float(fhh[jj])) + bt.x + (L >> 16);
-                                    const int Lo = L & 0xFFFF;
-                                    int q, up;
-                                    if (m > 0) {
-                                        q = T >> m;
-                                        const int rem = T & mmask;
-                                        up = (rem > half) | ((rem == half) & ((Lo != 0) | (q & 1)));
-                                    } else {
-                                        q = T;
-                                        up = (Lo > 0x8000) | ((Lo == 0x8000) & (q & 1));
-                                    }
-                                    int cc = (a.relu && T < 0) ? 0 : q + up;
-                                    c2[h] = min(max(cc, lo), hi);
-                                }
-                                w[8 * hf + j] = pack_codes_f16(c2[0], c2[1]);
-                            }
-                        }
-                        unsigned char* half_buf = stg + (cb >> 1) * (TC_BM * 128);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int chunk = (cb & 1) * 4 + q;
-                            *reinterpret_cast<uint4*>(half_buf + row * 128 + ((chunk ^ (row & 7)) << 4)) =
-                                make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-                        }
-                        continue;
-                    }
                     if (sizeof(ACC) == 8 && P.patch == 3 && P.nacc == 4 && P.fast_store && a.sh >= 1 && a.sh <= 62) {
                         // window mode, two-limb x and w, one-plane codes out: each 16-column half goes
                         // from the four limb accumulators to packed codes before the next is loaded
@@ -1873,7 +1810,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                         if (lane == 0) mbar_arrive(accempty0 + 8 * buf);
                     }
                     if (!last) continue;
-                    if (SPLIT && P.ksplit > 1) {
+                    if constexpr (SPLIT) {
                         // one share of the reduction: its exact integer sums go to the partial buffer
                         if (m >= 0) {
                             // (16 bytes per store: with one value per store 64 x 4096 outputs of 4096 products took 29 us, 19 so)
@@ -1894,9 +1831,7 @@ __global__ void __launch_bounds__((WIN || W64) ? tc_threads_win() : tc_threads_p
                                     if (k0 + j < a.K) dst[j] = acc[j];
                             }
                         }
-                        continue;
-                    }
-                    if (P.fast_store) {
+                    } else if (P.fast_store) {
                         // 32 one-plane codes -> 4 swizzled 16-byte chunks of this row in the staging buffer
                         // (the epilogue constants are rebuilt here from the parameters rather than kept
                         // live across the tile loop)
