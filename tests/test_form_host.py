@@ -7,32 +7,38 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SRC = os.path.join(ROOT, "tests", "form_host.cu")
-BIN = os.path.join(ROOT, "tests", "_build", "form_host")
 IN = ["N", "H", "W", "C", "Cp", "K", "R", "S", "stride", "pad", "xb", "wb", "mode", "packed", "s2d", "path"]
 OUT = ["status", "s2d_ok", "planned", "rows_geom", "narrow", "use_patch", "pk", "BN", "n_groups", "overlap", "TW", "TH", "TN",
        "tiles"]
 
 
-def choose(layers):
-    """The choices for layers given as dicts (mode 1: int64 sums; missing: no padding, 8 / 7 bits, default path)."""
+def build_harness(src):
+    """A host program of this folder, compiled against the library's objects."""
     from paper_2203_12091_gb300 import build as B
     if not os.path.exists(B.nvcc()) and not shutil.which(B.nvcc()):
         pytest.skip("nvcc not available")
     B.build()
+    exe = os.path.join(ROOT, "tests", "_build", os.path.basename(src)[:-3])
     objs = sorted(os.path.join(B.BUILD, f) for f in os.listdir(B.BUILD) if f.endswith(".o"))
-    deps = [SRC] + objs + [os.path.join(B.CSRC, f) for f in os.listdir(B.CSRC) if f.endswith(".cuh")]
-    if not os.path.exists(BIN) or any(os.path.getmtime(d) > os.path.getmtime(BIN) for d in deps):
-        os.makedirs(os.path.dirname(BIN), exist_ok=True)
-        r = subprocess.run([B.nvcc(), *B.ARCH, "-O2", "-std=c++17", "--expt-relaxed-constexpr", f"-I{B.INCLUDE}", f"-I{B.CSRC}", SRC,
-                            *objs, "-o", BIN + ".tmp"], capture_output=True, text=True)
+    deps = [src] + objs + [os.path.join(B.CSRC, f) for f in os.listdir(B.CSRC) if f.endswith(".cuh")]
+    if not os.path.exists(exe) or any(os.path.getmtime(d) > os.path.getmtime(exe) for d in deps):
+        os.makedirs(os.path.dirname(exe), exist_ok=True)
+        r = subprocess.run([B.nvcc(), *B.ARCH, "-O2", "-std=c++17", "--expt-relaxed-constexpr", f"-I{B.INCLUDE}", f"-I{B.CSRC}", src,
+                            *objs, "-o", exe + ".tmp"], capture_output=True, text=True)
         assert r.returncode == 0, r.stdout + r.stderr
-        os.replace(BIN + ".tmp", BIN)
+        os.replace(exe + ".tmp", exe)
+    return exe
+
+
+def choose(layers):
+    """The choices for layers given as dicts (mode 1: int64 sums; missing: no padding, 8 / 7 bits, default path)."""
+    exe = build_harness(SRC)
     text = ""
     for c in layers:
         c = {"W": c["H"], "S": c["R"], "Cp": (c["C"] + 7) // 8 * 8, "stride": 1, "pad": 0, "xb": 8, "wb": 7, "mode": 1, "packed": 0,
              "s2d": 0, "path": "-", **c}
         text += " ".join(str(c[k]) for k in IN) + "\n"
-    r = subprocess.run([BIN], input=text, capture_output=True, text=True, timeout=300)
+    r = subprocess.run([exe], input=text, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr
     rows = [dict(zip(OUT, map(int, line.split()))) for line in r.stdout.strip().splitlines()]
     assert len(rows) == len(layers)

@@ -100,6 +100,53 @@ def test_first_layer_from_images(NET, R, st, pad, hw, k, monkeypatch):
         assert F.fxpq_get_device_status() == 3
 
 
+def _small_net(NET):
+    """A net of chained kernels of every kind, its quantized form and two batches of images with their logits."""
+    L, plan = _tiny()
+    rng = np.random.default_rng(12)
+    W = {l["name"]: (rng.standard_normal((l["K"], l["R"], l["R"], l["C"])).astype(np.float32) * 0.2,
+                     rng.standard_normal(l["K"]).astype(np.float32) * 0.01) for l in L if l["type"] == "conv"}
+    imgs = [torch.from_numpy(synth.images(6, seed, hw=28)).cuda() for seed in (2, 3)]
+    q = NET.build_qnet(L, W, imgs[0], plan)
+    want = [q.forward(x)[0].clone() for x in imgs]
+    torch.cuda.synchronize()
+    assert not torch.equal(*want)
+    return q, imgs, want
+
+
+def test_forward_in_a_captured_graph(NET):
+    """Chained launches captured as a graph: replays read the inputs of the moment."""
+    from paper_2203_12091_gb300 import fxpq as F
+    q, imgs, want = _small_net(NET)
+    x, ws = imgs[0].clone(), F.workspace(q.workspace_bytes(6), "cuda")
+    logits = torch.empty_like(want[0])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(3):
+            q.forward(x, logits, ws)
+    for i in (1, 0, 1):
+        x.copy_(imgs[i])
+        logits.fill_(-1)
+        graph.replay()
+        assert torch.equal(logits, want[i]), i
+
+
+def test_forwards_on_two_streams(NET):
+    """Chained launches of two streams, each with its own workspace, interleaved."""
+    from paper_2203_12091_gb300 import fxpq as F
+    q, imgs, want = _small_net(NET)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    ws = [F.workspace(q.workspace_bytes(6), "cuda") for _ in range(2)]
+    got = [[torch.empty_like(want[0]) for _ in range(20)] for _ in range(2)]
+    torch.cuda.synchronize()
+    for j in range(20):
+        for i in range(2):
+            q.forward(imgs[i], got[i][j], ws[i], streams[i])
+    torch.cuda.synchronize()
+    for i in range(2):
+        assert all(torch.equal(g, want[i]) for g in got[i]), i
+
+
 def test_smaller_workspaces(NET):
     """Scratch that holds a split reduction's shares but not the larger copies of the first layer still splits the FC layer;
     with none at all the logits are the same."""
