@@ -308,7 +308,7 @@ FXPQ_API fxpq_status fxpq_avgpool(const void* d_x, int32_t N, int32_t H, int32_t
 /* Packed k-bit code storage (the footprint of Sec. V-E.2's memory model: k bits per code, Eq. mfp).
  * Codes are taken in groups of 32 (the last zero-padded); group g occupies k = fmt.bits uint32 words,
  * word g*k + b holding bit b of the k-bit two's-complement field of code 32g + i at bit i (a bit-plane
- * layout: a warp packs a group with k ballots and unpacks it with k shuffles).  Unpacking sign-extends
+ * layout).  Unpacking sign-extends
  * when fmt.is_signed.  d_codes: fp16 code tensor of n codes (plane-major when fmt.bits > 8), 2-byte
  * aligned; d_words: ceil(n / 32) * fmt.bits words, 4-byte aligned.  Codes outside fmt's range are
  * truncated to their low k bits (they cannot come from the quantizer). */

@@ -885,11 +885,6 @@ struct FsOutBatch {
     FsOut o[FS_MAX_ITEMS];
 };
 
-// Finalize: one warp per cell of one item (the cells of every S, k, FL, then the two stats cells),
-// FIN_WARPS cells per block.  The block stages the item's keys once; each warp's lanes score their
-// share of the keys into the warp's columns, and lane 0 turns them into the exact 768-bit value and
-// its nearest double.  The item's last block to finish (completion ticket) writes the scores, the
-// argmin per wordlength (exact ties keep the smaller FL) and the stats.
 // Clears the bins.  (A kernel rather than a memset: the next one is then set up, its shared bins cleared, meanwhile;
 // a one-row search of 16M values 63.0 -> 60.4 us.)
 __global__ void __launch_bounds__(256) fs_clear_kernel(uint4* g, size_t n) {
@@ -898,6 +893,11 @@ __global__ void __launch_bounds__(256) fs_clear_kernel(uint4* g, size_t n) {
     if (i < n) g[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+// Finalize: one warp per cell of one item (the cells of every S, k, FL, then the two stats cells),
+// FIN_WARPS cells per block.  The block stages the item's keys once; each warp's lanes score their
+// share of the keys into the warp's columns, and the warp together turns them into the exact 768-bit
+// value and its nearest double.  The item's last block to finish (completion ticket) writes the scores, the
+// argmin per wordlength (exact ties keep the smaller FL) and the stats.
 __global__ void __launch_bounds__(FIN_T) fl_search_final_kernel(const __grid_constant__ FsBatch B,
                                                                  const __grid_constant__ FsOutBatch O, int* status) {
     const int item = batch_item(B.fin0, B.n_items, (int)blockIdx.x);
