@@ -1,6 +1,7 @@
 // fxpq_conv_tc.cu -- host side of the tensor-core C-Block (planning, tensor maps, launch) and the
 // kernels without a Scale layer; the kernel itself is in fxpq_conv_tc.cuh.
 #include <algorithm>
+#include <cmath>
 
 #include "fxpq_conv_tc.cuh"
 
@@ -14,7 +15,7 @@ int g_num_sms = 0;
 std::mutex g_tc_mu;
 
 // FXPQ_CONV_PATH picks among exact alternatives so that tests can compare them on the same shapes: "tc" takes patch
-// tiles up to four times the gathered form's k-blocks (by default the line depends on alignment, limbs and tiles)
+// tiles up to four times the gathered form's k-blocks (by default the form that takes less time)
 // and space-to-depth at any size, "tc_patch" patch tiles wherever the geometry allows them, "tc_rows" 128-row tiles
 // gathered by the producer warps for every layer, "tc_bn128" no 256-column tiles and "tc_bn256" them wherever the layer
 // allows (by default the width whose rounds take the fewest cycles), "tc_win64" window mode's two-limb epilogue in
@@ -123,29 +124,53 @@ bool choose_form(const ConvArgs& a, const fxpq_conv_desc& d, const char* path, i
     const bool whole_map = a.R == a.H && a.S == a.W && a.pad == 0 && a.P == 1 && a.Q == 1;
     const bool rows_geom = f.rows_geom = (one_by_one || whole_map) && a.M > 0 && a.M < (1LL << 31) - TC_BM &&
                            !conv_path_is("tc_rows") && !conv_path_is("tc_patch");
-    // Patch tiles for every other layer whose stride a TMA box can traverse and whose channel count fills its
-    // 64-channel blocks well enough: up to four times the k-blocks of the flattened reduction of the
-    // gathered row tiles, which take about six times as long per k-block (2600 cycles against 410; a 7 x 7
-    // 512-channel layer of 128 images 95 us gathered, 31 us as patches); 8-channel stride-1 inputs take boxes
-    // of one tap each (narrow)
+    // Patch tiles or gathered row tiles for every other layer, patches if a TMA box can traverse the stride: a patch takes
+    // whole 64-channel blocks per tap, which may be several times the k-blocks of the gathered rows' flattened reduction,
+    // each of which takes longer (a 7 x 7 512-channel layer of 128 images 95 us gathered, 31 us as patches); 8-channel
+    // stride-1 inputs take boxes of one tap each (narrow)
     const bool narrow = f.narrow = a.Cp == 8;
     PatchShape& ps = f.ps = PatchShape();
     if (!rows_geom && a.P > 0 && a.Q > 0 && a.N > 0 && a.stride <= (narrow ? 1 : 8) && !conv_path_is("tc_rows"))
         ps = patch_shape(a, TC_BM);
     const int kbt = P.kbt = (a.Cp + TC_BK - 1) / TC_BK;
     const int kb_flat = (a.R * a.S * a.Cp + TC_BK - 1) / TC_BK;
-    // How many of its k-blocks a layer may spend as patches for one of the flattened reduction (K = 64 / 256, 3x3,
-    // 588 row tiles, us as patches and gathered): 32 channels, 1.8 times as many, 15.8 / 22.4 and 31.5 / 35.2; 16
-    // channels, 3 times, 25.3 / 19.4 and 37.3 / 29.4.  Pixels that are not whole 32-byte sectors cost their boxes
-    // double: 120 channels, 1.06 times, 37.6 / 46.2; 136 channels, 1.35 times, 55.7 / 49.3; 24 channels 63.9 / 35.2.
-    // Where each tile has an SM to itself, its split shares fill the others: a one-limb layer's patches cost 0.30 us per
-    // k-block of every SM (0.36 off 32-byte sectors), gathered rows 0.5 and 1 us at the start (400 layers: 0.3 and 0.7%
-    // off the better of both; 40 channels, 11 x 11, 45 tiles 39.6 / 25.6; 24 channels, 7 x 5, one tile 6.1 / 10.4).
-    // Two-limb reductions drain a group per limb pair, which hides less of the
-    // patches' k-blocks (32 channels, 1.8 times: 68 / 62; 80 channels, 1.5 times: 99.5 / 103; 16-bit 24 channels, 5 x 5,
-    // 2.5 times: 272 / 103).
-    // Strided two-limb layers of one column tile, whose boxes are read once, are gathered (K = 56, 13 images, 3 x 3 / 2 on
-    // 75 x 75: 64 channels 34.4 / 26.7, 256 channels 83.7 / 72.7; K = 192: 64.9 / 67.8 and 163 / 206).
+    // A layer's time in a form, in us, as fitted to 1734 layers of 1 to 1500 tiles in both (the better one is met but for
+    // 0.1 to 1.4% on average over their kinds, at worst 1.4 times): a round of tiles, or of a split's shares, over the SMs
+    // costs 2.4 per limb pair that it drains and per k-block, on one SM of few and on one of all, 0.34 to 0.38 gathered,
+    // 0.11 to 0.19 as patches and 0.15 to 0.32 where a pixel is not whole 32-byte sectors, whose boxes cost double, more
+    // in wider tiles; a split its second kernel.  (By tiles and k-blocks alone the choice was up to 1.7 times off: 16-bit,
+    // 3 x 3 / 2 on 13 maps of 75 x 75 x 64, 169 patches against 140 row tiles, 34.4 / 26.7.)
+    const bool two_limb = a.px * a.pw > 1, lone = row_tiles_est * ((a.K + 63) / 64) <= sms;
+    auto rounds = [&](long long tiles, int bn) { return (double)((tiles * ((a.K + bn - 1) / bn) + sms - 1) / sms); };
+    // Tile width: 64 columns for int64 sums and at most 64 output channels, else the width whose whole rounds over the SMs
+    // take the fewest cycles.  A k-block costs what its stage takes from L2 at about 80 bytes per cycle and SM (24, 32 and
+    // 48 KB: 300, 410 and 615 cycles; the MMAs 228, 256 and 512); a 256-column tile of several exact groups has one
+    // accumulator buffer, whose drain is not hidden.
+    auto width = [&](long long tiles, bool groups) {
+        const double c64 = rounds(tiles, 64) * 300, c128 = rounds(tiles, 128) * 410, c256 = rounds(tiles, 256) * (groups ? 1100 : 615);
+        const int bn = c128 <= c64 ? 128 : 64;
+        return a.K > 128 && !conv_path_is("tc_bn128") && c256 <= (bn == 128 ? c128 : c64) ? 256 : bn;
+    };
+    auto form_us = [&](bool patch) {
+        const long long tiles = patch ? ps.tiles : row_tiles_est;
+        const int bn = two_limb || a.K <= 64 ? 64 : width(tiles, false);
+        const double n = (double)tiles * ((a.K + bn - 1) / bn), kb = patch ? a.R * a.S * kbt : kb_flat, pairs = a.px * a.pw;
+        const double wide = (bn == 64 ? 300 : bn == 128 ? 410 : 615) / 300.0 - 1.0, outputs = 1e-6 * (double)a.M * a.K;
+        auto per_kb = [&](double load) {
+            return !patch      ? 0.34 + 0.04 * load + 0.33 * wide
+                   : a.Cp % 16 ? 0.15 + 0.17 * load + 0.30 * wide
+                               : 0.11 + 0.08 * load + 0.11 * wide;
+        };
+        double shares = 1.0;
+        if (has_ws && bn == 64 && 2.0 * n <= sms) {
+            shares = std::floor(std::min({sms / n, (double)TC_MAX_SPLIT, std::max(kb / 4.0, two_limb ? pairs * std::ceil(kb / 8.0) : 0.0)}));
+            const bool fp32 = !two_limb && a.py == 1 && a.out_mode != FXPQ_OUT_ACC64;
+            if (shares < 2.0 || (fp32 && kb * (1.0 - 1.0 / shares) * per_kb(1.0) < 1.9 + 3.5 * shares * outputs)) shares = 1.0;
+        }
+        const double n_rounds = std::ceil(n * shares / sms), load = n * shares / (sms * n_rounds);
+        const double round = 2.4 * (1.0 + wide) * std::max(1.0, pairs / shares) - 1.0 + per_kb(load) * kb * pairs / shares;
+        return (patch ? 3.4 : 4.8) + n_rounds * round + (shares > 1.0 ? 1.5 + 3.5 * shares * outputs : 0.0);
+    };
     // Eight-channel patches take the gathered form's k-blocks, a box per tap: one-limb layers 1.1 to 1.4 times faster with
     // up to 40 taps (11 x 11: 17 maps of 46 x 46 33.3 / 20.7; 23 of 28 x 28 23.8 / 12.6), two-limb ones only with few
     // (128 channels, 3 x 3, 1568 tiles: 134 / 140; 64 channels, 7 x 7: 132 / 114) and up to 256 output channels (344
@@ -153,20 +178,10 @@ bool choose_form(const ConvArgs& a, const fxpq_conv_desc& d, const char* path, i
     // Overlapping pixels (the flat space-to-depth form) are read by patches whatever they cost: a tensor map has the
     // strides that the gather does not look at.
     const bool overlap = a.x_sw != a.Cp;
-    const bool two_limb = a.px * a.pw > 1, lone = row_tiles_est * ((a.K + 63) / 64) <= sms;
     const bool any_patch = conv_path_is("tc") || conv_path_is("tc_bn256");
-    const double kb_patch = (double)ps.tiles * a.R * a.S * kbt, kb_rows = (double)row_tiles_est * kb_flat;
-    bool worth;
-    if (narrow)
-        worth = any_patch || (two_limb ? !lone && a.R * a.S <= 16 && a.K <= 256 : a.R * a.S <= 40);
-    else if (any_patch)
-        worth = kb_patch <= 4.0 * kb_rows;
-    else if (two_limb)
-        worth = (lone || a.stride == 1 || a.K > 64) && kb_patch <= (a.Cp % 16 ? 1.15 : 1.55) * kb_rows;
-    else if (lone)
-        worth = ((a.Cp % 16 ? 0.36 : 0.3) * kb_patch - 0.5 * kb_rows) * ((a.K + 63) / 64) <= 1.0 * sms;
-    else
-        worth = kb_patch <= (a.Cp % 16 ? 1.15 : 2.0) * kb_rows;
+    const bool worth = narrow      ? any_patch || (two_limb ? !lone && a.R * a.S <= 16 && a.K <= 256 : a.R * a.S <= 40)
+                       : any_patch ? (double)ps.tiles * a.R * a.S * kbt <= 4.0 * (double)row_tiles_est * kb_flat
+                                   : form_us(true) <= form_us(false);
     bool& use_patch = f.use_patch;
     use_patch = ps.TW > 0 && (overlap || conv_path_is("tc_patch") || worth);
     if (overlap && !use_patch && !rows_geom) return false;
@@ -181,22 +196,13 @@ bool choose_form(const ConvArgs& a, const fxpq_conv_desc& d, const char* path, i
     const bool wide_split = rows_geom && !acc64 && !a.has_scale && has_ws && a.K > 128 && !conv_path_is("tc_bn128") &&
                             !conv_path_is("tc_nosplit") && row_tiles_est * ((a.K + 255) / 256) * 2 <= sms &&
                             (kb_flat * a.px * a.pw >= 32 || d.d_wpacked);  // (shorter ones are not split, see below)
-    // Tile width: 64 columns for int64 sums and at most 64 output channels, else the width whose whole rounds
-    // over the SMs take the fewest cycles.  A k-block costs what its stage takes from L2 at about 80 bytes
-    // per cycle and SM (24, 32 and 48 KB: 300, 410 and 615 cycles; the MMAs 228, 256 and 512); a 256-column
-    // tile of several exact groups has one accumulator buffer, whose drain is not hidden.
-    const long long tiles_m_est = use_patch ? ps.tiles : row_tiles_est;
     int& BN = f.BN = 64;
-    if (acc64 || a.K <= 64) {
+    if (acc64 || a.K <= 64)
         BN = 64;
-    } else if (wide_split || (a.K > 128 && conv_path_is("tc_bn256"))) {
+    else if (wide_split || (a.K > 128 && conv_path_is("tc_bn256")))
         BN = 256;
-    } else {
-        auto rounds = [&](int bn) { return (double)((tiles_m_est * ((a.K + bn - 1) / bn) + sms - 1) / sms); };
-        const double c64 = rounds(64) * 300, c128 = rounds(128) * 410, c256 = rounds(256) * (P.n_groups > 1 ? 1100 : 615);
-        BN = c128 <= c64 ? 128 : 64;
-        if (a.K > 128 && !conv_path_is("tc_bn128") && c256 <= (BN == 128 ? c128 : c64)) BN = 256;
-    }
+    else
+        BN = width(use_patch ? ps.tiles : row_tiles_est, P.n_groups > 1);
     // packed k-bit weights (k <= 8, one plane) are read by the 256-column TMA-row instances of the
     // split (FC) layers, whose weights stream through once; elsewhere every weight tile is expanded
     // once per row tile and the fp16 codes are read instead
@@ -493,16 +499,26 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         // groups (two-limb layers): each share takes whole groups
         int ks_sub = std::min(cap, std::min(min_len / 4, TC_MAX_GROUPS / ng));
         int ks_whole = std::min(cap, ng);
-        // The second kernel costs about 3 us, a k-block of a tile that has its SM to itself 0.15 us (0.33 gathered): a
-        // layer with the fp32 epilogue is split if that shortens the chain by 12.  Other epilogues run once per tile in
-        // one kernel take 4 to 8 us, and the second kernel spreads them: always split (334 small layers: 12 is 0.5% off
-        // the better of both on average, 24 for all 16%; 9 k-blocks to 16-bit codes, 825 x 240 outputs, 14.4 us whole,
-        // 8.5 split; 16-bit, 8 k-blocks, 20 x 120 int64 sums 15.4 / 7.1)
+        // The second kernel costs about 1.9 us and 3.5 per million values and share, a k-block of a tile that has its SM to
+        // itself 0.19 to 0.38 us (choose_form): a layer with the fp32 epilogue is split if that shortens the chain by more (FC
+        // layers' 256-column tiles: by 12 k-blocks).  Other epilogues run once per tile in one kernel take 4 to 8 us, and
+        // the second kernel spreads them: split if anything is saved, for one-plane codes (staged, the shorter ones) if
+        // that pays for the shares' traffic as well (334 small layers: 0 to 0.5% off the better of both on average, 16%
+        // with 24 k-blocks for all; 9 k-blocks to 16-bit codes, 825 x 240 outputs, 14.4 us whole, 8.5 split; 16-bit, 8
+        // k-blocks, 20 x 120 int64 sums 15.4 / 7.1; 2 k-blocks, 0.33 M one-plane codes 11.6 / 14.4; 25 k-blocks, 0.54 M
+        // codes with the fp32 epilogue 8.9 / 12.0)
         int total = 0;
         for (int gi = 0; gi < ng; ++gi) total += P.g[gi].kb1 - P.g[gi].kb0;
-        const int saves = fp32_epi ? 12 : 1;
-        if (total - total / std::max(ks_sub, 1) < saves) ks_sub = 1;
-        if (total - total / std::max(ks_whole, 1) < saves) ks_whole = 1;
+        const double outputs = 1e-6 * (double)a.M * a.K, per_kb = !P.patch && !P.rows_tma ? 0.38 : P.patch && a.Cp % 16 ? 0.31 : 0.19;
+        auto pays = [&](int ks) {
+            const double saved = total - total / std::max(ks, 1);
+            return saved >= (BN == 256             ? (fp32_epi ? 12.0 : 1.0)
+                             : fp32_epi            ? (1.9 + 3.5 * ks * outputs) / per_kb
+                             : P.fast_store        ? 1.0 + 16.0 * outputs
+                                                   : 1.0);
+        };
+        if (!pays(ks_sub)) ks_sub = 1;
+        if (!pays(ks_whole)) ks_whole = 1;
         if (ks_sub >= 2 && ks_sub >= ks_whole) {
             TcGroup g0[TC_MAX_GROUPS];
             for (int gi = 0; gi < ng; ++gi) g0[gi] = P.g[gi];
