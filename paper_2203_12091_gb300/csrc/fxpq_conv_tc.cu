@@ -499,23 +499,25 @@ fxpq_status launch_conv_tc(const ConvArgs& a, const fxpq_conv_desc& d, cudaStrea
         // groups (two-limb layers): each share takes whole groups
         int ks_sub = std::min(cap, std::min(min_len / 4, TC_MAX_GROUPS / ng));
         int ks_whole = std::min(cap, ng);
-        // The second kernel costs about 1.9 us and 3.5 per million values and share, a k-block of a tile that has its SM to
-        // itself 0.19 to 0.38 us (choose_form): a layer with the fp32 epilogue is split if that shortens the chain by more (FC
-        // layers' 256-column tiles: by 12 k-blocks).  Other epilogues run once per tile in one kernel take 4 to 8 us, and
-        // the second kernel spreads them: split if anything is saved, for one-plane codes (staged, the shorter ones) if
-        // that pays for the shares' traffic as well (334 small layers: 0 to 0.5% off the better of both on average, 16%
-        // with 24 k-blocks for all; 9 k-blocks to 16-bit codes, 825 x 240 outputs, 14.4 us whole, 8.5 split; 16-bit, 8
-        // k-blocks, 20 x 120 int64 sums 15.4 / 7.1; 2 k-blocks, 0.33 M one-plane codes 11.6 / 14.4; 25 k-blocks, 0.54 M
-        // codes with the fp32 epilogue 8.9 / 12.0)
+        // The second kernel costs about 1.9 us and 3.5 per million values and share, 1.6 and 2.5 where it takes a Scale layer's
+        // work off the tiles; a k-block of a tile that has its SM to itself 0.19 to 0.38 us (choose_form): a layer with the
+        // fp32 epilogue is split if that shortens the chain by more (FC layers' 256-column tiles: by 12 k-blocks).  Other
+        // epilogues run once per tile in one kernel take 4 to 8 us, and the second kernel spreads them: split if anything is
+        // saved, for one-plane codes (staged, the shorter ones) if that pays for the shares' traffic as well (334 small
+        // layers: 0 to 0.5% off the better of both on average, 16% with 24 k-blocks for all; 9 k-blocks to 16-bit codes, 825
+        // x 240 outputs, 14.4 us whole, 8.5 split; 16-bit, 8 k-blocks, 20 x 120 int64 sums 15.4 / 7.1; 2 k-blocks, 0.33 M
+        // one-plane codes 11.6 / 14.4; 25 k-blocks, 0.54 M codes with the fp32 epilogue 8.9 / 12.0, 18 and 0.1 M 7.0 / 7.4;
+        // ResNet-18's Scale layers of one image, where only those of 14 and more saved k-blocks are split, 172 us, none of
+        // 14 177, all 179)
         int total = 0;
         for (int gi = 0; gi < ng; ++gi) total += P.g[gi].kb1 - P.g[gi].kb0;
         const double outputs = 1e-6 * (double)a.M * a.K, per_kb = !P.patch && !P.rows_tma ? 0.38 : P.patch && a.Cp % 16 ? 0.31 : 0.19;
         auto pays = [&](int ks) {
             const double saved = total - total / std::max(ks, 1);
-            return saved >= (BN == 256             ? (fp32_epi ? 12.0 : 1.0)
-                             : fp32_epi            ? (1.9 + 3.5 * ks * outputs) / per_kb
-                             : P.fast_store        ? 1.0 + 16.0 * outputs
-                                                   : 1.0);
+            return saved >= (BN == 256      ? (fp32_epi ? 12.0 : 1.0)
+                             : fp32_epi     ? (a.has_scale ? 1.6 + 2.5 * ks * outputs : 1.9 + 3.5 * ks * outputs) / per_kb
+                             : P.fast_store ? 1.0 + 16.0 * outputs
+                                            : 1.0);
         };
         if (!pays(ks_sub)) ks_sub = 1;
         if (!pays(ks_whole)) ks_whole = 1;
